@@ -185,6 +185,10 @@ cudaError_t launch_stage2_w32(const float2* t1, const float* lam, int nk, int n,
 // ends.  The slow request of the serving tests.
 cudaError_t launch_delay(cudaStream_t st, double ms);
 
+// dst[i] = src[i] by a kernel, one end page-locked host memory that the device can address: a copy that
+// does not wait in a copy engine's queue behind the copies of other streams.
+cudaError_t launch_host_copy(float* dst, const float* src, size_t floats, cudaStream_t st);
+
 // Twiddle table of the 512-point adjoint-rows kernel (ilt.cu): kAdj512TableLen entries.
 constexpr int kAdj512TableLen = 31 * 16 + 15 * 32;
 void adj512_table(float2* out);
