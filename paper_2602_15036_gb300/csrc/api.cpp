@@ -50,22 +50,16 @@ struct Carve {
 };
 
 litho_status upload(litho_kernels* h) {
-  const int F = h->n_focus, K = h->k, C = h->crop, N = h->n;
+  const int C = h->crop, N = h->n;
   LITHO_TRY_CUDA(cudaGetDevice(&h->device));
-  std::vector<float> lam(size_t(F) * K);
-  for (size_t i = 0; i < lam.size(); ++i) lam[i] = float(h->lambda[i]);
-  std::vector<float2> phi(size_t(F) * K * C * C);
-  for (size_t i = 0; i < phi.size(); ++i) phi[i] = make_float2(float(h->phi_host[2 * i]), float(h->phi_host[2 * i + 1]));
   std::vector<float2> tw(N);
   if (!fft_twiddle_table(N, tw.data())) {
     set_error("no FFT plan for n = %d", N);
     return LITHO_EINVAL;
   }
-  LITHO_TRY_CUDA(cudaMalloc(&h->d_lambda, lam.size() * sizeof(float)));
-  LITHO_TRY_CUDA(cudaMalloc(&h->d_phi, phi.size() * sizeof(float2)));
+  litho_status ks = build_kernel_set(h);
+  if (ks != LITHO_OK) return ks;
   LITHO_TRY_CUDA(cudaMalloc(&h->d_tw, tw.size() * sizeof(float2)));
-  LITHO_TRY_CUDA(cudaMemcpy(h->d_lambda, lam.data(), lam.size() * sizeof(float), cudaMemcpyHostToDevice));
-  LITHO_TRY_CUDA(cudaMemcpy(h->d_phi, phi.data(), phi.size() * sizeof(float2), cudaMemcpyHostToDevice));
   LITHO_TRY_CUDA(cudaMemcpy(h->d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice));
   // coarse grid: I has no frequency at or beyond C along either axis, so
   // nc >= 2C samples determine it exactly
@@ -91,18 +85,6 @@ litho_status upload(litho_kernels* h) {
     LITHO_TRY_CUDA(cudaMemcpy(h->d_tw512, t512.data(), t512.size() * sizeof(float2), cudaMemcpyHostToDevice));
   }
   if (N == 1024 || h->nc == 1024) {
-    // sqrt(lam_fk) Phi_fk for the aerial path's stage 1 (FP64 product, then rounded)
-    std::vector<float2> phs(phi.size());
-    const size_t cc = size_t(C) * C;
-    for (size_t fk = 0; fk < size_t(F) * K; ++fk) {
-      const double r = std::sqrt(std::max(0.0, h->lambda[fk]));
-      for (size_t i = 0; i < cc; ++i) {
-        const size_t e = fk * cc + i;
-        phs[e] = make_float2(float(r * h->phi_host[2 * e]), float(r * h->phi_host[2 * e + 1]));
-      }
-    }
-    LITHO_TRY_CUDA(cudaMalloc(&h->d_phi_s, phs.size() * sizeof(float2)));
-    LITHO_TRY_CUDA(cudaMemcpy(h->d_phi_s, phs.data(), phs.size() * sizeof(float2), cudaMemcpyHostToDevice));
     std::vector<float2> t32(kStage2W32TableLen);
     stage2_w32_table(t32.data());
     LITHO_TRY_CUDA(cudaMalloc(&h->d_tw32, t32.size() * sizeof(float2)));
@@ -142,13 +124,12 @@ void litho_free_kernels(litho_kernels* h) {
   int cur = 0;
   cudaGetDevice(&cur);
   cudaSetDevice(h->device);
-  cudaFree(h->d_lambda);
-  cudaFree(h->d_phi);
+  cudaFree(h->d_psi);
+  cudaFree(h->d_power);
   cudaFree(h->d_tw);
   if (h->d_twc_tc != h->d_twc) cudaFree(h->d_twc_tc);
   cudaFree(h->d_twc);
   cudaFree(h->d_tw32);
-  cudaFree(h->d_phi_s);
   cudaFree(h->d_tw512);
   for (auto& s : h->host_streams)
     if (s) cudaStreamDestroy(s);
@@ -406,12 +387,13 @@ struct FusedResist {
   uint8_t* printed;
 };
 
-// `planes` coarse images in L.ic -> N x N planes at `out` (plane offset `p0`
-// of the call for the fused resist outputs).
+// The coarse images in L.ic, one per clip and kernel set -> the N x N planes of
+// `clips` clips at `out` (plane offset `p0` of the call for the fused resist outputs).
 // rows_done: stage 2 has already written the coarse images' row spectra to L.rowbuf2.
-static litho_status upsample(const litho_kernels* h, litho_precision p, const AerialLayout& L, int planes, float* out,
+static litho_status upsample(const litho_kernels* h, litho_precision p, const AerialLayout& L, int clips, float* out,
                              const FusedResist* fr, size_t p0, cudaStream_t st, bool rows_done = false) {
-  const int N = h->n, NC = coarse_n(h, p), C2 = 2 * h->crop;
+  const int N = h->n, NC = coarse_n(h, p), C2 = 2 * h->crop, planes = clips * h->n_sets;
+  const PlaneOut po = plane_out(h);
   const float2* twc = coarse_tw(h, p);
   const float* gain = fr ? L.gain : nullptr;
   ProfScope ps(fr ? kStageUpsampleResist : kStageUpsample, st, rows_done ? 2 : 3);
@@ -423,12 +405,12 @@ static litho_status upsample(const litho_kernels* h, litho_precision p, const Ae
     LITHO_TRY_CUDA(launch_stage1_fft(L.spec, nullptr, planes, N, C2, h->d_tw, L.q, st));
   }
   if (!fr) {
-    LITHO_TRY_CUDA(launch_band_rows_real(L.q, planes, N, C2, 1.0f, h->d_tw, out, st));
+    LITHO_TRY_CUDA(launch_band_rows_real(L.q, clips, h->n_sets, N, C2, 1.0f, h->d_tw, out, po, st));
     return LITHO_OK;
   }
   const size_t nn = size_t(N) * N;
-  LITHO_TRY_CUDA(launch_band_rows_resist(L.q, planes, N, C2, h->d_tw, fr->threshold, out, fr->iblur + p0 * nn,
-                                         fr->printed ? fr->printed + p0 * nn : nullptr, st));
+  LITHO_TRY_CUDA(launch_band_rows_resist(L.q, clips, h->n_sets, N, C2, h->d_tw, fr->threshold, out, fr->iblur + p0 * nn,
+                                         fr->printed ? fr->printed + p0 * nn : nullptr, po, st));
   return LITHO_OK;
 }
 
@@ -473,7 +455,7 @@ static litho_status aerial_prepare(const litho_kernels* h, const float* mask_dev
 static litho_status aerial_run(const litho_kernels* h, const float* mask_dev, int b, double dose, litho_precision p,
                                bool coarse, float* intensity_dev, const AerialLayout& L, const FusedResist* fr,
                                cudaStream_t st) {
-  const int N = h->n, C = h->crop, F = h->n_focus, K = h->k;
+  const int N = h->n, C = h->crop, F = h->n_focus;
   {
     ProfScope ps(kStageMaskSpectrum, st, 2);
     LITHO_TRY_CUDA(launch_mask_spectrum(mask_dev, b, N, C, h->d_tw, L.rowbuf, L.mhat, st));
@@ -486,33 +468,31 @@ static litho_status aerial_run(const litho_kernels* h, const float* mask_dev, in
       litho_status s =
           gemm_aerial_group(h, L.mhat + size_t(c0) * C * C, g, float(dose), p, coarse, coarse ? L.ic : dst, L.gws, st);
       if (s != LITHO_OK) return s;
-      if (coarse && (s = upsample(h, p, L, g * F, dst, fr, size_t(c0) * F, st)) != LITHO_OK) return s;
+      if (coarse && (s = upsample(h, p, L, g, dst, fr, size_t(c0) * F, st)) != LITHO_OK) return s;
     }
     return LITHO_OK;
   }
   const int NE = coarse ? coarse_n(h, p) : N;
   const float2* tw = coarse ? coarse_tw(h, p) : h->d_tw;
-  // On a 1024-point grid stage 1 takes sqrt(lam) Phi and the warp-per-row stage 2 sums |E|^2 unweighted
-  const bool folded = h->d_phi_s && h->d_tw32 && stage2_w32_supported(NE, C);
   // with the warp-per-row stage 2 on the coarse grid, stage 2 writes the row spectra that the
   // interpolation's column pass reads, in place of the coarse images
-  const bool rows_in_stage2 = coarse && folded && interp_cols_supported(NE, N);
+  const bool rows_in_stage2 = coarse && h->d_tw32 && stage2_w32_supported(NE, C) && interp_cols_supported(NE, N);
+  const FieldSet fs = field_set(h, 0, h->n_sets);
+  const PlaneOut po = coarse ? plane_out_identity(h->n_sets) : plane_out(h);
   for (int c0 = 0; c0 < b; c0 += G) {
     const int g = std::min(G, b - c0);
     float* img = intensity_dev + size_t(c0) * F * N * N;
     {
       ProfScope ps(kStageStage1Fft, st, 1);
-      LITHO_TRY_CUDA(launch_stage1_fft(L.mhat + size_t(c0) * C * C, folded ? h->d_phi_s : h->d_phi, F * K, NE, C, tw,
-                                       L.t1, st, g));
+      LITHO_TRY_CUDA(launch_stage1_fft(L.mhat + size_t(c0) * C * C, h->d_psi, fs.fields(), NE, C, tw, L.t1, st, g));
     }
     {
       ProfScope ps(kStageStage2Fft, st, 1);
-      LITHO_TRY_CUDA(launch_stage2_fft(L.t1, h->d_lambda, K, NE, C, float(dose), tw, coarse ? L.ic : img, g * F,
-                                       (long long)K * NE * C, (long long)NE * NE, st, F, h->d_tw32, h->d_tw512,
-                                       folded, rows_in_stage2 ? L.rowbuf2 : nullptr, 2 * C));
+      LITHO_TRY_CUDA(launch_stage2_fft(L.t1, fs, g, NE, C, float(dose), tw, coarse ? L.ic : img, po, st, h->d_tw32,
+                                       h->d_tw512, rows_in_stage2 ? L.rowbuf2 : nullptr, 2 * C));
     }
     if (coarse) {
-      litho_status s = upsample(h, p, L, g * F, img, fr, size_t(c0) * F, st, rows_in_stage2);
+      litho_status s = upsample(h, p, L, g, img, fr, size_t(c0) * F, st, rows_in_stage2);
       if (s != LITHO_OK) return s;
     }
   }

@@ -1,6 +1,6 @@
 // FFT-based kernels: mask spectrum (crop), stage 1 (band multiply + inverse
 // transform over v), and stage 2 of the FP32 path (inverse transform over u
-// fused with the lam_k |E_k|^2 accumulation over all kernels).
+// fused with the |E_k|^2 accumulation over all kernels).
 //
 // Paper Section III.A: the object spectrum O(f) of Eq. (1) (thin-mask reading:
 // the mask's DFT), and the SOCS image of Eq. (4), I = sum_k lam_k |O (x) phi_k|^2,
@@ -147,10 +147,9 @@ struct OutC64 {
 
 // ---- stage 2 (FP32 path): one image row per CTA, all kernels of the plane ------------------------
 template <int N, bool BANDED>
-__global__ void __launch_bounds__(Plan<N>::NT, 512 / Plan<N>::NT) k_stage2(const float2* __restrict__ t1, const float* __restrict__ lam,
-                                                        int nk, int crop, float dose,
-                                                        const float2* __restrict__ tw_g, float* __restrict__ img,
-                                                        long long t1_plane, long long img_plane, int lam_period) {
+__global__ void __launch_bounds__(Plan<N>::NT, 512 / Plan<N>::NT) k_stage2(const float2* __restrict__ t1, const __grid_constant__ FieldSet fs,
+                                                        int crop, float dose, const float2* __restrict__ tw_g,
+                                                        float* __restrict__ img, const __grid_constant__ PlaneOut po) {
   using PL = Plan<N>;
   constexpr int NT = PL::NT;
   constexpr int RL = PL::R[PL::P - 1];
@@ -160,8 +159,8 @@ __global__ void __launch_bounds__(Plan<N>::NT, 512 / Plan<N>::NT) k_stage2(const
   load_twiddles<N>(tw, tw_g);
   __syncthreads();
   const int y = blockIdx.x, plane = blockIdx.y, t = threadIdx.x, half = crop / 2;
-  const float2* base = t1 + plane * t1_plane + (size_t)y * crop;
-  const float* lp = lam + (plane % lam_period) * nk;  // planes repeat every lam_period (clips of a batch)
+  const int clip = plane / fs.planes, pl = plane - clip * fs.planes, nk = fs.start[pl + 1] - fs.start[pl];
+  const float2* base = t1 + ((size_t)(clip * fs.fields() + fs.start[pl]) * N + y) * crop;
   float acc[PERL][RL];
 #pragma unroll
   for (int p = 0; p < PERL; ++p)
@@ -174,26 +173,26 @@ __global__ void __launch_bounds__(Plan<N>::NT, 512 / Plan<N>::NT) k_stage2(const
   MidTwiddles<N, +1> mid;
   if constexpr (kMid) mid.load(tw, t);
   for (int j = 0; j < nk; ++j) {
-    const float l = __ldg(lp + j);
-    if (l == 0.f) continue;  // uniform across the block
     const float2* row = base + (size_t)j * N * crop;
     auto load = [&](int, int r, int idx) {
       const int c = (r < PL::R[0] / 2 ? idx : idx - N) + half;  // first pass: idx < N/2 exactly when r < R/2
       return (c >= 0 && c < crop) ? __ldg(row + c) : make_float2(0.f, 0.f);
     };
-    auto use = [&](int p, int q, int, float2 v) { acc[p][q] = fmaf(l, fmaf(v.x, v.x, v.y * v.y), acc[p][q]); };
+    auto use = [&](int p, int q, int, float2 v) { acc[p][q] = fmaf(v.x, v.x, fmaf(v.y, v.y, acc[p][q])); };
     if constexpr (kMid)
       fft_load_use_mid<N, +1, decltype(load), decltype(use), BANDED>(buf, tw, t, load, use, mid);
     else
       fft_load_use<N, +1, decltype(load), decltype(use), BANDED>(buf, tw, t, load, use);
   }
-  float* out = img + plane * img_plane + (size_t)y * N;
+  for (int d = po.first[pl]; d < po.first[pl + 1]; ++d) {
+    float* out = img + ((size_t)(clip * po.out_planes + po.list[d]) * N + y) * N;
 #pragma unroll
-  for (int p = 0; p < PERL; ++p) {
-    const int jj = t + p * NT;
-    if (jj < N / RL) {
+    for (int p = 0; p < PERL; ++p) {
+      const int jj = t + p * NT;
+      if (jj < N / RL) {
 #pragma unroll
-      for (int q = 0; q < RL; ++q) out[jj + q * (N / RL)] = dose * acc[p][q];
+        for (int q = 0; q < RL; ++q) out[jj + q * (N / RL)] = dose * acc[p][q];
+      }
     }
   }
 }
@@ -203,20 +202,27 @@ __global__ void __launch_bounds__(Plan<N>::NT, 512 / Plan<N>::NT) k_stage2(const
 template <int N, bool BANDED>
 __global__ void __launch_bounds__(Plan<N>::NT) k_band_rows_real(const float2* __restrict__ q, int crop, float scale,
                                                                 const float2* __restrict__ tw_g,
-                                                                float* __restrict__ out, int rows_per_cta) {
+                                                                float* __restrict__ out, int planes,
+                                                                const __grid_constant__ PlaneOut po,
+                                                                int rows_per_cta) {
   __shared__ float2 buf[PadLen<N>::value];
   __shared__ float2 tw[N];
   load_twiddles<N>(tw, tw_g);
   __syncthreads();
-  const int p = blockIdx.y, half = crop / 2;
+  const int p = blockIdx.y, half = crop / 2, clip = p / planes, pl = p - clip * planes;
+  const int d0 = po.first[pl], d1 = po.first[pl + 1];
+  const size_t p0 = (size_t)(clip * po.out_planes + po.list[d0]) * N;  // rows before the first output plane
   for (int y = blockIdx.x * rows_per_cta; y < min(N, (blockIdx.x + 1) * rows_per_cta); ++y) {
     const float2* row = q + ((size_t)p * N + y) * crop;
     auto load = [&](int, int r, int idx) {
       const int c = (r < Plan<N>::R[0] / 2 ? idx : idx - N) + half;  // first pass: idx < N/2 exactly when r < R/2
       return (c >= 0 && c < crop) ? __ldg(row + c) : make_float2(0.f, 0.f);
     };
-    float* o = out + ((size_t)p * N + y) * N;
-    auto use = [&](int, int, int x, float2 v) { o[x] = scale * v.x; };
+    float* o = out + (p0 + y) * N;
+    auto use = [&](int, int, int x, float2 v) {
+      o[x] = scale * v.x;
+      for (int d = d0 + 1; d < d1; ++d) o[(po.list[d] - po.list[d0]) * (N * N) + x] = scale * v.x;
+    };
     fft_load_use<N, +1, decltype(load), decltype(use), BANDED>(buf, tw, threadIdx.x, load, use);
   }
 }
@@ -228,23 +234,31 @@ template <int N, bool BANDED>
 __global__ void __launch_bounds__(Plan<N>::NT) k_band_rows_resist(const float2* __restrict__ q, int crop,
                                                                   const float2* __restrict__ tw_g, float thr,
                                                                   float* __restrict__ img, float* __restrict__ iblur,
-                                                                  uint8_t* __restrict__ printed, int rows_per_cta) {
+                                                                  uint8_t* __restrict__ printed, int planes,
+                                                                  const __grid_constant__ PlaneOut po,
+                                                                  int rows_per_cta) {
   __shared__ float2 buf[PadLen<N>::value];
   __shared__ float2 tw[N];
   load_twiddles<N>(tw, tw_g);
   __syncthreads();
-  const int p = blockIdx.y, half = crop / 2;
+  const int p = blockIdx.y, half = crop / 2, clip = p / planes, pl = p - clip * planes;
+  const int d0 = po.first[pl], d1 = po.first[pl + 1];
+  const size_t p0 = (size_t)(clip * po.out_planes + po.list[d0]) * N;  // rows before the first output plane
   for (int y = blockIdx.x * rows_per_cta; y < min(N, (blockIdx.x + 1) * rows_per_cta); ++y) {
     const float2* row = q + ((size_t)p * N + y) * crop;
     auto load = [&](int, int r, int idx) {
       const int c = (r < Plan<N>::R[0] / 2 ? idx : idx - N) + half;  // first pass: idx < N/2 exactly when r < R/2
       return (c >= 0 && c < crop) ? __ldg(row + c) : make_float2(0.f, 0.f);
     };
-    const size_t o = ((size_t)p * N + y) * N;
+    const size_t o = (p0 + y) * N;
+    auto put = [&](size_t at, float2 v) {
+      if (img) img[at] = v.x;
+      iblur[at] = v.y;
+      if (printed) printed[at] = v.y >= thr ? 1 : 0;
+    };
     auto use = [&](int, int, int x, float2 v) {
-      if (img) img[o + x] = v.x;
-      iblur[o + x] = v.y;
-      if (printed) printed[o + x] = v.y >= thr ? 1 : 0;
+      put(o + x, v);
+      for (int d = d0 + 1; d < d1; ++d) put(o + (po.list[d] - po.list[d0]) * (N * N) + x, v);
     };
     fft_load_use<N, +1, decltype(load), decltype(use), BANDED>(buf, tw, threadIdx.x, load, use);
   }
@@ -277,7 +291,9 @@ template <int N, bool BANDED>
 __global__ void __launch_bounds__(Plan<N>::NT, N >= 512 ? 640 / Plan<N>::NT : 1) k_resist_grad_rows(const float2* __restrict__ band, int crop,
                                                                    const float2* __restrict__ tw_g,
                                                                    const float* __restrict__ target,
-                                                                   int planes_per_clip, float beta, float thr,
+                                                                   int planes_per_clip,
+                                                                   const __grid_constant__ PlaneWeight weight,
+                                                                   float beta, float thr,
                                                                    float2* __restrict__ rowbuf,
                                                                    double* __restrict__ partial, int pairs_per_cta) {
   using SH = GradRowsShape<N>;
@@ -293,6 +309,7 @@ __global__ void __launch_bounds__(Plan<N>::NT, N >= 512 ? 640 / Plan<N>::NT : 1)
   __syncthreads();
   const int p = blockIdx.y, t = threadIdx.x, half = crop / 2;
   const float* tg = target + (size_t)(p / planes_per_clip) * N * N;
+  const float wgt = weight.w[p % planes_per_clip], beta2 = 2.0f * wgt * beta;
   for (int pr = blockIdx.x * pairs_per_cta; pr < min(N / 2, (blockIdx.x + 1) * pairs_per_cta); ++pr) {
     const int y0 = 2 * pr;
     const float2* r0 = band + ((size_t)p * N + y0) * crop;
@@ -315,7 +332,7 @@ __global__ void __launch_bounds__(Plan<N>::NT, N >= 512 ? 640 / Plan<N>::NT : 1)
       const float z1 = 1.0f / (1.0f + expf(-beta * (v.y - thr)));
       const float d0 = z0 - __ldg(t0 + x), d1 = z1 - __ldg(t1 + x);
       racc = fmaf(d0, d0, fmaf(d1, d1, racc));
-      const float2 q = make_float2(2.0f * d0 * beta * z0 * (1.0f - z0), 2.0f * d1 * beta * z1 * (1.0f - z1));
+      const float2 q = make_float2(beta2 * d0 * z0 * (1.0f - z0), beta2 * d1 * z1 * (1.0f - z1));
       if constexpr (SH::kRegs)
         qreg[pp + PERL * qq] = q;
       else
@@ -342,7 +359,7 @@ __global__ void __launch_bounds__(Plan<N>::NT, N >= 512 ? 640 / Plan<N>::NT : 1)
     if (t == 0) {
       double sum = 0.0;
       for (int w = 0; w < NW; ++w) sum += wsum[w];
-      partial[(size_t)p * (N / 2) + pr] = sum;
+      partial[(size_t)p * (N / 2) + pr] = wgt * sum;
     }
     float2* o0 = rowbuf + ((size_t)p * N + y0) * crop;
     float2* o1 = o0 + crop;
@@ -372,47 +389,35 @@ inline int rows_per_cta(int rows, int planes, int per_sm) {
 }
 
 template <int N>
-cudaError_t band_rows_resist_n(const float2* q, int planes, int crop, const float2* tw, float thr, float* img,
-                               float* iblur, uint8_t* printed, cudaStream_t st) {
-  const int rpc = rows_per_cta(N, planes, 2048 / Plan<N>::NT), grid = (N + rpc - 1) / rpc;
-  if (2 * crop <= N)
-    k_band_rows_resist<N, true><<<dim3(grid, planes), Plan<N>::NT, 0, st>>>(q, crop, tw, thr, img, iblur, printed,
-                                                                           rpc);
-  else
-    k_band_rows_resist<N, false><<<dim3(grid, planes), Plan<N>::NT, 0, st>>>(q, crop, tw, thr, img, iblur, printed,
-                                                                            rpc);
+cudaError_t band_rows_resist_n(const float2* q, int clips, int planes, int crop, const float2* tw, float thr,
+                               float* img, float* iblur, uint8_t* printed, const PlaneOut& po, cudaStream_t st) {
+  const int rpc = rows_per_cta(N, clips * planes, 2048 / Plan<N>::NT), grid = (N + rpc - 1) / rpc;
+  auto kern = 2 * crop <= N ? k_band_rows_resist<N, true> : k_band_rows_resist<N, false>;
+  kern<<<dim3(grid, clips * planes), Plan<N>::NT, 0, st>>>(q, crop, tw, thr, img, iblur, printed, planes, po, rpc);
   return cudaGetLastError();
 }
 
 template <int N>
 cudaError_t resist_grad_rows_n(const float2* band, int planes, int crop, const float2* tw, const float* target,
-                               int planes_per_clip, float beta, float thr, float2* rowbuf, double* partial,
-                               cudaStream_t st) {
+                               int planes_per_clip, const PlaneWeight& weight, float beta, float thr, float2* rowbuf,
+                               double* partial, cudaStream_t st) {
   static_assert(Plan<N>::NT % 32 == 0, "whole warps");
   const size_t sm = sizeof(float2) * (N + PadLen<N>::value + (GradRowsShape<N>::kRegs ? crop + 1 : N + 1));
   const int ppc = rows_per_cta(N / 2, planes, 2048 / Plan<N>::NT), grid = (N / 2 + ppc - 1) / ppc;
-  cudaError_t e;
-  if (2 * crop <= N) {
-    if ((e = smem_attrs(k_resist_grad_rows<N, true>, sm)) != cudaSuccess) return e;
-    k_resist_grad_rows<N, true><<<dim3(grid, planes), Plan<N>::NT, sm, st>>>(band, crop, tw, target, planes_per_clip,
-                                                                            beta, thr, rowbuf, partial, ppc);
-  } else {
-    if ((e = smem_attrs(k_resist_grad_rows<N, false>, sm)) != cudaSuccess) return e;
-    k_resist_grad_rows<N, false><<<dim3(grid, planes), Plan<N>::NT, sm, st>>>(band, crop, tw, target,
-                                                                             planes_per_clip, beta, thr, rowbuf,
-                                                                             partial, ppc);
-  }
+  auto kern = 2 * crop <= N ? k_resist_grad_rows<N, true> : k_resist_grad_rows<N, false>;
+  cudaError_t e = smem_attrs(kern, sm);
+  if (e != cudaSuccess) return e;
+  kern<<<dim3(grid, planes), Plan<N>::NT, sm, st>>>(band, crop, tw, target, planes_per_clip, weight, beta, thr, rowbuf,
+                                                    partial, ppc);
   return cudaGetLastError();
 }
 
 template <int N>
-cudaError_t band_rows_real_n(const float2* q, int planes, int crop, float scale, const float2* tw, float* out,
-                             cudaStream_t st) {
-  const int rpc = rows_per_cta(N, planes, 2048 / Plan<N>::NT), grid = (N + rpc - 1) / rpc;
-  if (2 * crop <= N)
-    k_band_rows_real<N, true><<<dim3(grid, planes), Plan<N>::NT, 0, st>>>(q, crop, scale, tw, out, rpc);
-  else
-    k_band_rows_real<N, false><<<dim3(grid, planes), Plan<N>::NT, 0, st>>>(q, crop, scale, tw, out, rpc);
+cudaError_t band_rows_real_n(const float2* q, int clips, int planes, int crop, float scale, const float2* tw,
+                             float* out, const PlaneOut& po, cudaStream_t st) {
+  const int rpc = rows_per_cta(N, clips * planes, 2048 / Plan<N>::NT), grid = (N + rpc - 1) / rpc;
+  auto kern = 2 * crop <= N ? k_band_rows_real<N, true> : k_band_rows_real<N, false>;
+  kern<<<dim3(grid, clips * planes), Plan<N>::NT, 0, st>>>(q, crop, scale, tw, out, planes, po, rpc);
   return cudaGetLastError();
 }
 
@@ -465,14 +470,10 @@ cudaError_t stage1_n(const float2* mhat, const float2* phi, int nk, int crop, co
 }
 
 template <int N>
-cudaError_t stage2_n(const float2* t1, const float* lam, int nk, int crop, float dose, const float2* tw, float* img,
-                     int planes, long long t1_plane, long long img_plane, int lam_period, cudaStream_t st) {
-  if (2 * crop <= N)
-    k_stage2<N, true><<<dim3(N, planes), Plan<N>::NT, 0, st>>>(t1, lam, nk, crop, dose, tw, img, t1_plane,
-                                                               img_plane, lam_period);
-  else
-    k_stage2<N, false><<<dim3(N, planes), Plan<N>::NT, 0, st>>>(t1, lam, nk, crop, dose, tw, img, t1_plane,
-                                                                img_plane, lam_period);
+cudaError_t stage2_n(const float2* t1, const FieldSet& fs, int clips, int crop, float dose, const float2* tw,
+                     float* img, const PlaneOut& po, cudaStream_t st) {
+  auto kern = 2 * crop <= N ? k_stage2<N, true> : k_stage2<N, false>;
+  kern<<<dim3(N, clips * fs.planes), Plan<N>::NT, 0, st>>>(t1, fs, crop, dose, tw, img, po);
   return cudaGetLastError();
 }
 
@@ -526,9 +527,9 @@ cudaError_t launch_mask_spectrum(const float* m, int b, int n, int crop, const f
 #undef CALL
 }
 
-cudaError_t launch_band_rows_real(const float2* q, int planes, int n, int crop, float scale, const float2* tw,
-                                  float* out, cudaStream_t st) {
-#define CALL(N) band_rows_real_n<N>(q, planes, crop, scale, tw, out, st)
+cudaError_t launch_band_rows_real(const float2* q, int clips, int planes, int n, int crop, float scale,
+                                  const float2* tw, float* out, const PlaneOut& po, cudaStream_t st) {
+#define CALL(N) band_rows_real_n<N>(q, clips, planes, crop, scale, tw, out, po, st)
   LITHO_DISPATCH_N(n, CALL)
 #undef CALL
 }
@@ -547,9 +548,10 @@ cudaError_t launch_blur_gain(const ResistTaps& taps, int n, int crop, float* gai
 }
 
 cudaError_t launch_resist_grad_rows(const float2* band, int planes, int n, int crop, const float2* tw,
-                                    const float* target, int planes_per_clip, float beta, float thr, float2* rowbuf,
-                                    double* partial, cudaStream_t st) {
-#define CALL(N) resist_grad_rows_n<N>(band, planes, crop, tw, target, planes_per_clip, beta, thr, rowbuf, partial, st)
+                                    const float* target, int planes_per_clip, const PlaneWeight& weight, float beta,
+                                    float thr, float2* rowbuf, double* partial, cudaStream_t st) {
+#define CALL(N) \
+  resist_grad_rows_n<N>(band, planes, crop, tw, target, planes_per_clip, weight, beta, thr, rowbuf, partial, st)
   LITHO_DISPATCH_N(n, CALL)
 #undef CALL
 }
@@ -559,34 +561,31 @@ cudaError_t launch_mask_cols(const float2* rowbuf, int b, int n, int crop, const
   LITHO_DISPATCH_NC(n, CALL)
 #undef CALL
 }
-cudaError_t launch_band_rows_resist(const float2* q, int planes, int n, int crop, const float2* tw, float threshold,
-                                    float* img, float* iblur, uint8_t* printed, cudaStream_t st) {
-#define CALL(N) band_rows_resist_n<N>(q, planes, crop, tw, threshold, img, iblur, printed, st)
+cudaError_t launch_band_rows_resist(const float2* q, int clips, int planes, int n, int crop, const float2* tw,
+                                    float threshold, float* img, float* iblur, uint8_t* printed, const PlaneOut& po,
+                                    cudaStream_t st) {
+#define CALL(N) band_rows_resist_n<N>(q, clips, planes, crop, tw, threshold, img, iblur, printed, po, st)
   LITHO_DISPATCH_N(n, CALL)
 #undef CALL
 }
 
 cudaError_t launch_stage1_fft(const float2* mhat, const float2* phi, int nk, int n, int crop, const float2* tw,
                               float2* t1, cudaStream_t st, int clips) {
+  if (nk == 0) return cudaSuccess;  // every kernel has lambda = 0: no field
 #define CALL(N) stage1_n<N>(mhat, phi, nk, crop, tw, t1, st, clips)
   LITHO_DISPATCH_N(n, CALL)
 #undef CALL
 }
 
-cudaError_t launch_stage2_fft(const float2* t1, const float* lam, int nk, int n, int crop, float dose,
-                              const float2* tw, float* img, int planes, long long t1_plane_stride,
-                              long long img_plane_stride, cudaStream_t st, int lam_period, const float2* tw32,
-                              const float2* tw512, bool folded, float2* spec, int spec_crop) {
-  if (lam_period <= 0) lam_period = planes;
+cudaError_t launch_stage2_fft(const float2* t1, const FieldSet& fs, int clips, int n, int crop, float dose,
+                              const float2* tw, float* img, const PlaneOut& po, cudaStream_t st, const float2* tw32,
+                              const float2* tw512, float2* spec, int spec_crop) {
   if (tw32 && stage2_w32_supported(n, crop))
-    return launch_stage2_w32(t1, lam, nk, n, crop, dose, tw32, img, planes, t1_plane_stride, img_plane_stride,
-                             lam_period, st, folded, spec, spec_crop);
-  // only the warp-per-row kernel sums unweighted or writes row spectra
-  if (folded || spec) return cudaErrorInvalidValue;
+    return launch_stage2_w32(t1, fs, clips, n, crop, dose, tw32, img, po, st, spec, spec_crop);
+  if (spec) return cudaErrorInvalidValue;  // only the warp-per-row kernel writes row spectra
   if (tw512 && stage2_w512_supported(n, crop))
-    return launch_stage2_w512(t1, lam, nk, n, crop, dose, tw512, img, planes, t1_plane_stride, img_plane_stride,
-                              lam_period, st);
-#define CALL(N) stage2_n<N>(t1, lam, nk, crop, dose, tw, img, planes, t1_plane_stride, img_plane_stride, lam_period, st)
+    return launch_stage2_w512(t1, fs, clips, n, crop, dose, tw512, img, po, st);
+#define CALL(N) stage2_n<N>(t1, fs, clips, crop, dose, tw, img, po, st)
   LITHO_DISPATCH_N(n, CALL)
 #undef CALL
 }

@@ -160,10 +160,12 @@ __host__ __device__ constexpr uint32_t idesc_f16(int fmt, int m, int n) {
 }
 
 struct GemmParams {
-  int n, nk, n_focus, planes, tiles_y, tiles_x, chunks, split, fmt;
-  const float* lamp;  // [F][K] lambda / scale^2
+  int n, planes, tiles_y, tiles_x, chunks, split, fmt;  // planes: of all clips
+  FieldSet fs;        // the planes and fields of one clip
+  PlaneOut po;        // output planes of each plane
+  const float* lamp;  // [fields] 1 / scale^2
   float dose;
-  float* img;         // [planes][n][n]
+  float* img;         // [clips][out_planes][n][n]
   int* err;
 };
 
@@ -200,7 +202,8 @@ __global__ void k_wait_selftest(int* err, long long limit, int code) {
 __global__ void __launch_bounds__(THREADS, 1)
     k_dft_gemm(const __grid_constant__ CUtensorMap ta_hi, const __grid_constant__ CUtensorMap ta_lo,
                const __grid_constant__ CUtensorMap ta_s, const __grid_constant__ CUtensorMap tb_hi,
-               const __grid_constant__ CUtensorMap tb_lo, const __grid_constant__ CUtensorMap tb_s, GemmParams p) {
+               const __grid_constant__ CUtensorMap tb_lo, const __grid_constant__ CUtensorMap tb_s,
+               const __grid_constant__ GemmParams p) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + RING_BYTES);
@@ -250,10 +253,9 @@ __global__ void __launch_bounds__(THREADS, 1)
       for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
         const int plane = t / tiles_per_plane, rem = t % tiles_per_plane;
         const int yt = rem / p.tiles_x, xt = rem % p.tiles_x;
-        const float* lam = p.lamp + (plane % p.n_focus) * p.nk;
-        for (int k = 0; k < p.nk && ok; ++k) {
-          if (lam[k] == 0.f) continue;
-          const int arow = (plane * p.nk + k) * p.n + yt * BM;
+        const int clip = plane / p.fs.planes, pl = plane - clip * p.fs.planes;
+        for (int k = p.fs.start[pl]; k < p.fs.start[pl + 1] && ok; ++k) {
+          const int arow = (clip * p.fs.fields() + k) * p.n + yt * BM;
           for (int ch = 0; ch < p.chunks; ++ch, ++it) {
             const int s = it % STAGES;
             const uint32_t use = it / STAGES;
@@ -295,10 +297,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       uint32_t it = 0, acc_it = 0;
       bool ok = true;
       for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
-        const int plane = t / tiles_per_plane;
-        const float* lam = p.lamp + (plane % p.n_focus) * p.nk;
-        for (int k = 0; k < p.nk && ok; ++k) {
-          if (lam[k] == 0.f) continue;
+        const int pl = t / tiles_per_plane % p.fs.planes, nk = p.fs.start[pl + 1] - p.fs.start[pl];
+        for (int k = 0; k < nk && ok; ++k) {
           if (!wait_bar(acc_empty, (acc_it & 1) ^ 1, abort_flag, p.err, 2)) {
             ok = false;
             break;
@@ -367,13 +367,12 @@ __global__ void __launch_bounds__(THREADS, 1)
     for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
       const int plane = t / tiles_per_plane, rem = t % tiles_per_plane;
       const int yt = rem / p.tiles_x, xt = rem % p.tiles_x;
-      const float* lam = p.lamp + (plane % p.n_focus) * p.nk;
+      const int clip = plane / p.fs.planes, pl = plane - clip * p.fs.planes;
       float acc[64];
 #pragma unroll
       for (int i = 0; i < 64; ++i) acc[i] = 0.f;
-      for (int k = 0; k < p.nk; ++k) {
-        const float l = lam[k];
-        if (l == 0.f) continue;
+      for (int k = p.fs.start[pl]; k < p.fs.start[pl + 1]; ++k) {
+        const float l = __ldg(p.lamp + k);
         if (!wait_bar(acc_full, acc_it & 1, abort_flag, p.err, 4)) {
           ok = false;
           break;
@@ -408,11 +407,14 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
       if (!ok) break;
       const int row = yt * BM + q * 32 + lane;
-      float4* out = reinterpret_cast<float4*>(p.img + ((size_t)plane * p.n + row) * p.n + xt * XT + half * 64);
+      for (int d = p.po.first[pl]; d < p.po.first[pl + 1]; ++d) {
+        const size_t dst = clip * p.po.out_planes + p.po.list[d];
+        float4* out = reinterpret_cast<float4*>(p.img + (dst * p.n + row) * p.n + xt * XT + half * 64);
 #pragma unroll
-      for (int i = 0; i < 16; ++i)
-        out[i] = make_float4(p.dose * acc[4 * i], p.dose * acc[4 * i + 1], p.dose * acc[4 * i + 2],
-                             p.dose * acc[4 * i + 3]);
+        for (int i = 0; i < 16; ++i)
+          out[i] = make_float4(p.dose * acc[4 * i], p.dose * acc[4 * i + 1], p.dose * acc[4 * i + 2],
+                               p.dose * acc[4 * i + 3]);
+      }
     }
   }
   tc_fence_before();
@@ -549,8 +551,8 @@ struct GemmOperands {
   void* b_lo[kModes][2] = {};
   void* b_s[kModes][2] = {};  // [Ws_hi 32 | Ws_lo 32] chunks, split modes
   CUtensorMap map_hi[kModes][2], map_lo[kModes][2], map_s[kModes][2];
-  float* d_lamp[kModes] = {};   // lambda / scale^2 per (f, k)
-  float* d_scale[kModes] = {};  // stage-1 scale per (f, k)
+  float* d_lamp[kModes] = {};   // 1 / scale^2 per kernel of the device's sets
+  float* d_scale[kModes] = {};  // stage-1 scale per kernel
   int* d_err = nullptr;
   int sm_count = 0;
 };
@@ -568,6 +570,29 @@ int arrays_of(int mode) { return is_split(mode) ? 3 : 1; }  // A_hi (+ A_lo, AS 
 
 size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 
+// bound[j] = max over the columns u of sum_v |psi_j(v, u)|; one block per kernel.
+__global__ void __launch_bounds__(256) k_column_bound(const float2* __restrict__ psi, int crop,
+                                                      float* __restrict__ bound) {
+  psi += (size_t)blockIdx.x * crop * crop;
+  float top = 0.f;
+  for (int u = threadIdx.x; u < crop; u += blockDim.x) {
+    float col = 0.f;
+    for (int v = 0; v < crop; ++v) {
+      const float2 x = psi[(size_t)v * crop + u];
+      col += hypotf(x.x, x.y);
+    }
+    top = fmaxf(top, col);
+  }
+  __shared__ float s[256];
+  s[threadIdx.x] = top;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (threadIdx.x < o) s[threadIdx.x] = fmaxf(s[threadIdx.x], s[threadIdx.x + o]);
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) bound[blockIdx.x] = s[0];
+}
+
 // Builds the twiddle operand B (cos | sin chunks, split) and the per-kernel
 // scales for one precision mode.  Host FP64, then rounded.
 litho_status build_operands(const litho_kernels* hc, int mode, bool coarse) {
@@ -581,7 +606,7 @@ litho_status build_operands(const litho_kernels* hc, int mode, bool coarse) {
   std::lock_guard<std::mutex> lk(g->mu);
   const int gi = coarse ? 1 : 0;
   if (g->built[mode][gi]) return LITHO_OK;
-  const int N = eval_n(h, coarse), C = h->crop, F = h->n_focus, K = h->k;
+  const int N = eval_n(h, coarse), C = h->crop, total = h->set_start[h->n_sets];
   const size_t cols = size_t(2) * C, count = size_t(N) * cols;
   std::vector<uint16_t> hi(count), lo(count), sum(count);
   auto split = [&](double w, uint16_t& h16, uint16_t& l16) {
@@ -608,25 +633,24 @@ litho_status build_operands(const litho_kernels* hc, int mode, bool coarse) {
       sum[size_t(x) * cols + kk] = part ? sl : sh;
     }
   }
-  // per-kernel scales: |T_k| <= max_u sum_v |Phi_k(v, u)| for masks with |m| <= 1
-  std::vector<float> scale(size_t(F) * K, 1.f), lamp(size_t(F) * K, 0.f);
-  for (int f = 0; f < F; ++f)
-    for (int k = 0; k < K; ++k) {
-      const size_t fk = size_t(f) * K + k;
+  // per-kernel scales: |T_k| <= max_u sum_v |Psi_k(v, u)| for masks with |m| <= 1
+  std::vector<float> scale(std::max(1, total), 1.f), lamp(std::max(1, total), 1.f);
+  if (is_fp16(mode) && total > 0) {
+    std::vector<float> bound(total);
+    float* d_bound = nullptr;
+    LITHO_TRY_CUDA(cudaMalloc(&d_bound, total * sizeof(float)));
+    k_column_bound<<<total, 256>>>(h->d_psi, C, d_bound);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpy(bound.data(), d_bound, total * sizeof(float), cudaMemcpyDeviceToHost);
+    cudaFree(d_bound);
+    LITHO_TRY_CUDA(e);
+    for (int j = 0; j < total; ++j) {
       double s = 1.0;
-      if (is_fp16(mode)) {
-        double bound = 0.0;
-        const double* ph = &h->phi_host[fk * size_t(C) * C * 2];
-        for (int u = 0; u < C; ++u) {
-          double col = 0.0;
-          for (int v = 0; v < C; ++v) col += std::hypot(ph[(size_t(v) * C + u) * 2], ph[(size_t(v) * C + u) * 2 + 1]);
-          bound = std::max(bound, col);
-        }
-        if (bound > 0.0) s = std::ldexp(1.0, int(std::floor(std::log2(8192.0 / bound))));
-      }
-      scale[fk] = float(s);
-      lamp[fk] = float(h->lambda[fk] / (s * s));
+      if (bound[j] > 0.f) s = std::ldexp(1.0, int(std::floor(std::log2(8192.0 / bound[j]))));
+      scale[j] = float(s);
+      lamp[j] = float(1.0 / (s * s));
     }
+  }
   LITHO_TRY_CUDA(cudaMalloc(&g->b_hi[mode][gi], count * 2));
   LITHO_TRY_CUDA(cudaMemcpy(g->b_hi[mode][gi], hi.data(), count * 2, cudaMemcpyHostToDevice));
   if (is_split(mode)) {
@@ -692,7 +716,9 @@ litho_status gemm_aerial_group(const litho_kernels* h, const float2* mhat, int c
                                litho_precision prec, bool coarse, float* img, void* ws, cudaStream_t st) {
   const int mode = mode_of(prec), gi = coarse ? 1 : 0;
   GemmOperands* g = h->gemm;
-  const int N = eval_n(h, coarse), C = h->crop, F = h->n_focus, K = h->k;
+  const int N = eval_n(h, coarse), C = h->crop;
+  const FieldSet fs = field_set(h, 0, h->n_sets);
+  const int nk = fs.fields();
   const float2* tw = coarse ? h->d_twc_tc : h->d_tw;
   const size_t arr = up256(size_t(std::min(clips, GROUP_CLIPS)) * per_clip_array_bytes(h, coarse));
   char* a_hi = static_cast<char*>(ws);
@@ -700,21 +726,22 @@ litho_status gemm_aerial_group(const litho_kernels* h, const float2* mhat, int c
   char* a_s = is_split(mode) ? a_hi + 2 * arr : a_hi;
   {
     ProfScope ps(kStageGemmOperands, st, 1);  // one launch for the group
-    cudaError_t e;
-    if (mode == kBF16)
-      e = stage1_split_mode<kBF16>(N, mhat, h->d_phi, F * K, C, tw, g->d_scale[mode], a_hi, nullptr, nullptr, clips,
+    cudaError_t e = cudaSuccess;
+    if (nk == 0) {  // every kernel has lambda = 0: no operand rows
+    } else if (mode == kBF16)
+      e = stage1_split_mode<kBF16>(N, mhat, h->d_psi, nk, C, tw, g->d_scale[mode], a_hi, nullptr, nullptr, clips,
                                    st);
     else if (mode == kFP16)
-      e = stage1_split_mode<kFP16>(N, mhat, h->d_phi, F * K, C, tw, g->d_scale[mode], a_hi, nullptr, nullptr, clips,
+      e = stage1_split_mode<kFP16>(N, mhat, h->d_psi, nk, C, tw, g->d_scale[mode], a_hi, nullptr, nullptr, clips,
                                    st);
     else if (mode == kBF16X3)
-      e = stage1_split_mode<kBF16X3>(N, mhat, h->d_phi, F * K, C, tw, g->d_scale[mode], a_hi, a_lo, a_s, clips, st);
+      e = stage1_split_mode<kBF16X3>(N, mhat, h->d_psi, nk, C, tw, g->d_scale[mode], a_hi, a_lo, a_s, clips, st);
     else
-      e = stage1_split_mode<kFP16X3>(N, mhat, h->d_phi, F * K, C, tw, g->d_scale[mode], a_hi, a_lo, a_s, clips, st);
+      e = stage1_split_mode<kFP16X3>(N, mhat, h->d_psi, nk, C, tw, g->d_scale[mode], a_hi, a_lo, a_s, clips, st);
     LITHO_TRY_CUDA(e);
   }
   const int fmt = is_fp16(mode) ? 0 : 1;
-  const unsigned long long rows = (unsigned long long)clips * F * K * N;
+  const unsigned long long rows = (unsigned long long)clips * std::max(1, nk) * N;
   CUtensorMap ta_hi, ta_lo, ta_s;
   if (!make_map(&ta_hi, a_hi, fmt, rows, 2ull * C) || !make_map(&ta_lo, a_lo, fmt, rows, 2ull * C) ||
       !make_map(&ta_s, a_s, fmt, rows, 2ull * C)) {
@@ -723,9 +750,9 @@ litho_status gemm_aerial_group(const litho_kernels* h, const float2* mhat, int c
   }
   GemmParams p;
   p.n = N;
-  p.nk = K;
-  p.n_focus = F;
-  p.planes = clips * F;
+  p.fs = fs;
+  p.po = coarse ? plane_out_identity(h->n_sets) : plane_out(h);
+  p.planes = clips * fs.planes;
   p.tiles_y = N / BM;
   p.tiles_x = N / XT;
   p.chunks = C / CH;

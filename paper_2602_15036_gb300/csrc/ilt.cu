@@ -9,6 +9,7 @@
 //   q_f = 2 (Z_f - target) b Z_f (1 - Z_f),  G_f = g (x) q_f          (= dL/dI_f)
 //   H_fk(u) = sum_x G_f(x) E_fk(x) e^{-2 pi i u.x/N}    on the crop
 //   S(u) = sum_f sum_k lam_fk conj(Phi_fk(u)) H_fk(u)
+// with sqrt(lam) Phi replaced by the kernel set's Psi, which give the same I (kernelset.cu).
 //   dL/dm(x) = 2 D N^-2 Re sum_u S(u) e^{+2 pi i u.x/N},  dL/dtheta = dL/dm a m (1 - m).
 //
 // Kernels (per clip, for a group of P focus planes at a time):
@@ -21,7 +22,7 @@
 //   k_adj_rows       per image row: E_fk from the stage-1 field (inverse FFT),
 //                    times G_f, forward FFT, crop columns -> U_fk[y][c]
 //   k_adj_cols       per crop column block and run of a clip's fields: forward
-//                    FFT over y, crop rows, times lam conj(Phi), summed over
+//                    FFT over y, crop rows, times conj(Psi), summed over
 //                    the run in registers -> one partial S per run
 //   k_sum_planes     S = sum of a clip's runs in fixed order
 //   k_grad_rows      band-to-full inverse of S along x (after stage 1 along y),
@@ -54,8 +55,9 @@ __global__ void k_sigmoid(const float4* __restrict__ theta, float alpha, float4*
 // Clip blockIdx.y: its `planes` planes of ib and q, its target, its
 // kPartials partial sums (the same partition for every group size).
 __global__ void __launch_bounds__(256) k_resist_grad(const float* __restrict__ ib, const float* __restrict__ target,
-                                                     size_t nn, int planes, float beta, float thr,
-                                                     float* __restrict__ q, double* __restrict__ partial) {
+                                                     size_t nn, int planes, const __grid_constant__ PlaneWeight weight,
+                                                     float beta, float thr, float* __restrict__ q,
+                                                     double* __restrict__ partial) {
   const size_t clip = blockIdx.y;
   ib += clip * planes * nn;
   q += clip * planes * nn;
@@ -64,14 +66,18 @@ __global__ void __launch_bounds__(256) k_resist_grad(const float* __restrict__ i
   double acc = 0.0;
   const size_t total = nn * planes, stride = (size_t)gridDim.x * blockDim.x;
   size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  size_t pix = i % nn;  // i mod nn, carried along instead of recomputed
+  int pl = int(i / nn);
+  size_t pix = i - pl * nn;  // i mod nn and i div nn, carried along instead of recomputed
   for (; i < total; i += stride) {
     const float z = 1.0f / (1.0f + expf(-beta * (ib[i] - thr)));
-    const float d = z - target[pix];
-    acc += double(d) * double(d);
-    q[i] = 2.0f * d * beta * z * (1.0f - z);
+    const float d = z - target[pix], w = weight.w[pl];
+    acc += double(w) * double(d) * double(d);
+    q[i] = 2.0f * w * d * beta * z * (1.0f - z);
     pix += stride;
-    while (pix >= nn) pix -= nn;
+    while (pix >= nn) {
+      pix -= nn;
+      ++pl;
+    }
   }
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
   __shared__ double ws[8];
@@ -103,13 +109,13 @@ __global__ void __launch_bounds__(1024) k_reduce_loss(const double* __restrict__
 
 // Backward rows: for every kernel of the plane, E = inverse FFT of the band row
 // T[y][:], P = G[y][:] E, U[y][c] = forward FFT of P on the crop columns.
-// Plane p takes lam[(p mod lam_period) nk ...] (clips of a group repeat the focus planes).
+// Planes of a clip and their fields as in `fs`; plane pl of clip i takes G at plane i g_planes + pl of g.
 // BANDED (2 crop <= N): the band row's zero half is skipped in the first pass.
 template <int N, bool BANDED>
-__global__ void __launch_bounds__(Plan<N>::NT) k_adj_rows(const float2* __restrict__ t1, const float* __restrict__ lam,
-                                                          int nk, int crop, const float* __restrict__ g,
-                                                          const float2* __restrict__ tw_g, float2* __restrict__ u,
-                                                          int lam_period) {
+__global__ void __launch_bounds__(Plan<N>::NT) k_adj_rows(const float2* __restrict__ t1,
+                                                          const __grid_constant__ FieldSet fs, int crop,
+                                                          const float* __restrict__ g, int g_planes,
+                                                          const float2* __restrict__ tw_g, float2* __restrict__ u) {
   using PL = Plan<N>;
   constexpr int NT = PL::NT, RL = PL::R[PL::P - 1];
   constexpr int PERL = PassShape<N, NT, RL>::PER;
@@ -119,8 +125,9 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_adj_rows(const float2* __restri
   float2* bufb = sm + N + PadLen<N>::value;
   load_twiddles<N>(tw, tw_g);
   const int y = blockIdx.x, plane = blockIdx.y, t = threadIdx.x, half = crop / 2;
+  const int clip = plane / fs.planes, pl = plane - clip * fs.planes;
   float gv[PERL][RL];
-  const float* grow = g + ((size_t)plane * N + y) * N;
+  const float* grow = g + ((size_t)(clip * g_planes + pl) * N + y) * N;
 #pragma unroll
   for (int p = 0; p < PERL; ++p)
 #pragma unroll
@@ -129,9 +136,8 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_adj_rows(const float2* __restri
       gv[p][q] = jj < N / RL ? grow[jj + q * (N / RL)] : 0.f;
     }
   __syncthreads();
-  for (int k = 0; k < nk; ++k) {
-    if (lam[(plane % lam_period) * nk + k] == 0.f) continue;
-    const size_t rowoff = (((size_t)plane * nk + k) * N + y) * crop;
+  for (int k = fs.start[pl]; k < fs.start[pl + 1]; ++k) {
+    const size_t rowoff = ((size_t)(clip * fs.fields() + k) * N + y) * crop;
     const float2* row = t1 + rowoff;
     auto load_band = [&](int, int r, int idx) {
       const int c = (r < PL::R[0] / 2 ? idx : idx - N) + half;  // first pass: idx < N/2 exactly when r < R/2
@@ -182,9 +188,9 @@ __device__ __forceinline__ void adj_cp16(void* smem_dst, const void* gmem_src) {
 
 template <bool BANDED>
 __global__ void __launch_bounds__(32 * kAdjWarps, 2)
-    k_adj_rows_w512(const float2* __restrict__ t1, const float* __restrict__ lam, int nk, int crop,
-                    const float* __restrict__ g, const float2* __restrict__ tw_g, float2* __restrict__ u,
-                    int lam_period) {
+    k_adj_rows_w512(const float2* __restrict__ t1, const __grid_constant__ FieldSet fs, int crop,
+                    const float* __restrict__ g, int g_planes, const float2* __restrict__ tw_g,
+                    float2* __restrict__ u) {
   constexpr int N = 512;
   extern __shared__ float4 smem_raw[];
   float2* tw1 = reinterpret_cast<float2*>(smem_raw);  // inverse pass 2: (r - 1) 16 + j
@@ -198,15 +204,15 @@ __global__ void __launch_bounds__(32 * kAdjWarps, 2)
   if (y0 >= N) return;  // no block barrier below
   float2* buf = bufs + wp * 2 * kAdjBuf;
   float2* stage = stage0 + (size_t)wp * 2 * crop;
-  const float* lp = lam + (plane % lam_period) * nk;
-  const size_t field = (size_t)N * crop;
-  const float2* t1p = t1 + (size_t)plane * nk * field;
-  float2* up = u + (size_t)plane * nk * field;
+  const int clip = plane / fs.planes, pl = plane - clip * fs.planes, nk = fs.start[pl + 1] - fs.start[pl];
+  const size_t field = (size_t)N * crop, first = (size_t)(clip * fs.fields() + fs.start[pl]) * field;
+  const float2* t1p = t1 + first;
+  float2* up = u + first;
   // this lane's row in passes 2 and 3 (inverse pass 2, forward pass 1) and its butterfly
   const int rsel = lane / 16, jj = lane % 16;
   float gv[32];  // G(y, jj + 16 q) of the lane's row
   {
-    const float* grow = g + ((size_t)plane * N + y0 + rsel) * N;
+    const float* grow = g + ((size_t)(clip * g_planes + pl) * N + y0 + rsel) * N;
 #pragma unroll
     for (int q = 0; q < 32; ++q) gv[q] = __ldg(grow + jj + 16 * q);
   }
@@ -215,7 +221,7 @@ __global__ void __launch_bounds__(32 * kAdjWarps, 2)
     for (int i = lane; i < crop; i += 32) adj_cp16(stage + 2 * i, src + 2 * i);
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  fetch(0);
+  if (nk > 0) fetch(0);
   for (int k = 0; k < nk; ++k) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncwarp();
@@ -237,7 +243,6 @@ __global__ void __launch_bounds__(32 * kAdjWarps, 2)
     }
     __syncwarp();  // both band rows are in registers: the staging buffer takes kernel k + 1
     if (k + 1 < nk) fetch(k + 1);
-    if (lp[k] == 0.f) continue;  // a zero kernel: U is not written (the column pass skips it)
 #pragma unroll
     for (int row = 0; row < 2; ++row) {
       dft_reg<16, +1, BANDED>(a[row]);
@@ -287,7 +292,7 @@ __global__ void __launch_bounds__(32 * kAdjWarps, 2)
   }
 }
 
-// Backward columns: forward FFT over y of U_j[:, c], crop rows, times lam_j conj(Phi_j);
+// Backward columns: forward FFT over y of U_j[:, c], crop rows, times conj(Psi_j);
 // field j uses kernel j mod period.  W columns per CTA with the lanes of a
 // warp interleaved over them (as in stage 1): the first pass reads U straight
 // from global memory (W adjacent columns of 32/W rows per warp load: whole
@@ -301,27 +306,24 @@ template <int N> struct AdjW { static constexpr int W = Plan<N>::NT <= 64 ? 8 : 
 // cost the 1024-point one (twice the slots); so shared memory up to 512.
 template <int N> struct AdjAccInSmem { static constexpr bool value = N <= 512; };
 
-// Runs of fields per clip in the adjoint columns: the largest divisor of the
-// clip's field count that is at most 8 (a function of that count alone, so a
-// clip's sums do not depend on how many clips a launch holds).
+// Runs of fields per clip in the adjoint columns: at most 8, of equal length
+// but for the last (a function of the clip's field count alone, so a clip's
+// sums do not depend on how many clips a launch holds).
 int adj_col_splits(int period) {
-  for (int d = 8; d > 1; --d)
-    if (period % d == 0) return d;
-  return 1;
+  const int per = std::max(1, (period + 7) / 8);
+  return std::max(1, (period + per - 1) / per);
 }
 
 // Per crop column block and run of fields j in [j0, j1) of one clip (the
-// clip's `period` fields split into `splits` runs of period / splits): the
-// forward transform over y of each field's column, the crop, lam conj(Phi)
-// times it, summed over the run (in registers, or up to 512 points in shared
+// clip's `period` fields split into `splits` runs): the forward transform over
+// y of each field's column, the crop, conj(Psi) times it, summed over the run (in registers, or up to 512 points in shared
 // memory, one slot per thread and output position) and written once, to
 // part[clip splits + split][cv][c].  k_sum_planes then adds a clip's runs in
 // order, so the sum's order depends on the clip's own field count only.
 template <int N>
 __global__ void __launch_bounds__(Plan<N>::NT * AdjW<N>::W, AdjAccInSmem<N>::value ? 2 : 1) k_adj_cols(const float2* __restrict__ u,
                                                                         const float2* __restrict__ phi,
-                                                                        const float* __restrict__ lam, int crop,
-                                                                        const float2* __restrict__ tw_g,
+                                                                        int crop, const float2* __restrict__ tw_g,
                                                                         float2* __restrict__ part, int period,
                                                                         int splits) {
   constexpr int W = AdjW<N>::W, NT = Plan<N>::NT, LD = (PadLen<N>::value + 15) / 16 * 16 + 16 / W;
@@ -334,7 +336,7 @@ __global__ void __launch_bounds__(Plan<N>::NT * AdjW<N>::W, AdjAccInSmem<N>::val
   constexpr int R0 = Plan<N>::R[0], NB0 = N / R0;
   static_assert(PassShape<N, NT, R0>::PER == 1, "one first-pass butterfly per thread");
   const int tid = threadIdx.x, g = tid % W, t = tid / W, c0 = blockIdx.x * W, half = crop / 2;
-  const int clip = blockIdx.y / splits, split = blockIdx.y % splits, jb = period / splits;
+  const int clip = blockIdx.y / splits, split = blockIdx.y % splits, jb = (period + splits - 1) / splits;
   float2* acc_s = buf + W * LD;  // kSmem: this thread's PERL x RL sums at (pp RL + q) T + tid
   float2 acc_r[kSmem ? 1 : PERL * RL];
   auto acc = [&](int i) -> float2& {
@@ -343,7 +345,7 @@ __global__ void __launch_bounds__(Plan<N>::NT * AdjW<N>::W, AdjAccInSmem<N>::val
     else
       return acc_r[i];
   };
-  const int j0 = clip * period + split * jb, j1 = j0 + jb;
+  const int j0 = clip * period + split * jb, j1 = min(j0 + jb, (clip + 1) * period);
   load_twiddles<N>(tw, tw_g);
   // this thread's first-pass inputs (rows t + r N/R0) of a field, loaded one field ahead
   float2 nxt[R0];
@@ -352,17 +354,12 @@ __global__ void __launch_bounds__(Plan<N>::NT * AdjW<N>::W, AdjAccInSmem<N>::val
 #pragma unroll
     for (int r = 0; r < R0; ++r) nxt[r] = t < NB0 ? __ldg(src + (size_t)(t + r * NB0) * crop) : make_float2(0.f, 0.f);
   };
-  prefetch(j0);
+  if (j0 < j1) prefetch(j0);
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < PERL * RL; ++i) acc(i) = make_float2(0.f, 0.f);
   for (int j = j0; j < j1; ++j) {
     const int jk = j % period;
-    const float l = lam[jk];
-    if (l == 0.f) {  // uniform across the block: nothing to add
-      if (j + 1 < j1) prefetch(j + 1);
-      continue;
-    }
     const float2* ph = phi + (size_t)jk * crop * crop + c0 + g;
     float2 cur[R0];
 #pragma unroll
@@ -376,9 +373,9 @@ __global__ void __launch_bounds__(Plan<N>::NT * AdjW<N>::W, AdjAccInSmem<N>::val
       const int cv = freq_of_idx(idx, N) + half;
       if (cv >= 0 && cv < crop) {
         const float2 p = __ldg(ph + (size_t)cv * crop);
-        // += lam conj(p) h
+        // += conj(p) h
         float2& a = acc(pp * RL + q);
-        a = make_float2(fmaf(l, p.x * h.x + p.y * h.y, a.x), fmaf(l, p.x * h.y - p.y * h.x, a.y));
+        a = make_float2(fmaf(p.x, h.x, fmaf(p.y, h.y, a.x)), fmaf(p.x, h.y, fmaf(-p.y, h.x, a.y)));
       }
     };
     fft_load_use<N, -1, decltype(load), decltype(use), false>(buf + g * LD, tw, t, load, use, after_first);
@@ -411,24 +408,40 @@ __global__ void k_to_channel(const float* __restrict__ img, float* __restrict__ 
 // rows and columns form for G = 1 collapses to
 //   S(v,u) = N^2 sum_k lam_k |Phi_k(v,u)|^2 mhat(v,u),
 // exactly (on the coarse grid too: there G is the constant (N/nc)^2 and the
-// transforms are on nc).  No field is transformed.  Clip blockIdx.y; the nk
-// kernels of phi and lam (all planes of the call) are summed in order.
-__global__ void k_ones_adjoint(const float2* __restrict__ mhat, const float2* __restrict__ phi,
-                               const float* __restrict__ lam, int nk, size_t cc, float n2, float2* __restrict__ s,
-                               int accumulate) {
+// transforms are on nc).  No field is transformed.  The sum over a plane's
+// kernels does not depend on the mask: the kernel set keeps it (`power`, per
+// set, rounded once from FP64).  Clip blockIdx.y; the planes' sets are listed
+// in `sets`.
+__global__ void k_ones_adjoint(const float2* __restrict__ mhat, const float* __restrict__ power,
+                               const __grid_constant__ PlaneOut sets, size_t cc, float n2, float2* __restrict__ s) {
   mhat += (size_t)blockIdx.y * cc;
   s += (size_t)blockIdx.y * cc;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < cc; i += (size_t)gridDim.x * blockDim.x) {
     float d = 0.f;
-    for (int k = 0; k < nk; ++k) {
-      const float2 p = __ldg(phi + (size_t)k * cc + i);
-      d = fmaf(__ldg(lam + k), fmaf(p.x, p.x, p.y * p.y), d);
-    }
+    for (int f = 0; f < sets.out_planes; ++f) d += __ldg(power + sets.list[f] * cc + i);
     const float2 m = mhat[i];
-    float2 a = accumulate ? s[i] : make_float2(0.f, 0.f);
-    a.x = fmaf(n2 * d, m.x, a.x);
-    a.y = fmaf(n2 * d, m.y, a.y);
-    s[i] = a;
+    s[i] = make_float2(n2 * d * m.x, n2 * d * m.y);
+  }
+}
+
+// The sets of focus planes [f0, f0 + count), for k_ones_adjoint.
+PlaneOut sets_of(const litho_kernels* h, int f0, int count) {
+  PlaneOut o{};
+  o.out_planes = count;
+  for (int i = 0; i < count; ++i) o.list[i] = h->set_of[f0 + i];
+  return o;
+}
+
+// out[i nu + u] = the sum of clip i's upstream planes list[first[u]] ... (blockIdx.y = i nu + u).
+__global__ void k_sum_upstream(const float* __restrict__ up, size_t nn, int nu, const __grid_constant__ PlaneOut planes,
+                               float* __restrict__ out) {
+  const int clip = blockIdx.y / nu, u = blockIdx.y - clip * nu;
+  up += (size_t)clip * planes.out_planes * nn;
+  out += (size_t)blockIdx.y * nn;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nn; i += (size_t)gridDim.x * blockDim.x) {
+    float a = up[planes.list[planes.first[u]] * nn + i];
+    for (int d = planes.first[u] + 1; d < planes.first[u + 1]; ++d) a += up[planes.list[d] * nn + i];
+    out[i] = a;
   }
 }
 
@@ -483,37 +496,37 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_grad_rows(const float2* __restr
 }
 
 template <int N>
-cudaError_t adj_rows_n(const float2* t1, const float* lam, int nk, int crop, const float* g, const float2* tw,
-                       float2* u, int planes, int lam_period, cudaStream_t st, const float2* tw512) {
+cudaError_t adj_rows_n(const float2* t1, const FieldSet& fs, int clips, int crop, const float* g, int g_planes,
+                       const float2* tw, float2* u, cudaStream_t st, const float2* tw512) {
+  const int planes = clips * fs.planes;
   if (N == 512 && tw512 && crop % 2 == 0 && crop / 2 <= 128) {  // two rows per warp
     const size_t sm = sizeof(float2) * (kAdjTw1 + kAdjTw2 + kAdjWarps * 2 * (size_t(kAdjBuf) + crop));
     cudaError_t e = smem_attrs(k_adj_rows_w512<true>, sm);
     if (e != cudaSuccess) return e;
-    k_adj_rows_w512<true><<<dim3(N / (2 * kAdjWarps), planes), 32 * kAdjWarps, sm, st>>>(t1, lam, nk, crop, g,
-                                                                                          tw512, u, lam_period);
+    k_adj_rows_w512<true><<<dim3(N / (2 * kAdjWarps), planes), 32 * kAdjWarps, sm, st>>>(t1, fs, crop, g, g_planes,
+                                                                                          tw512, u);
     return cudaGetLastError();
   }
   const size_t sm = sizeof(float2) * (N + 2 * PadLen<N>::value);
   auto kern = 2 * crop <= N ? k_adj_rows<N, true> : k_adj_rows<N, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  kern<<<dim3(N, planes), Plan<N>::NT, sm, st>>>(t1, lam, nk, crop, g, tw, u, lam_period);
+  kern<<<dim3(N, planes), Plan<N>::NT, sm, st>>>(t1, fs, crop, g, g_planes, tw, u);
   return cudaGetLastError();
 }
 
 template <int N>
-cudaError_t adj_cols_n(const float2* u, const float2* phi, const float* lam, int crop, const float2* tw, float2* part,
-                       int fields, int period, cudaStream_t st) {
+cudaError_t adj_cols_n(const float2* u, const float2* phi, int crop, const float2* tw, float2* part, int clips,
+                       int period, cudaStream_t st) {
   constexpr int W = AdjW<N>::W;
-  if (crop % W != 0 || period < 1 || fields % period != 0) return cudaErrorInvalidValue;
+  if (crop % W != 0) return cudaErrorInvalidValue;
   constexpr int LD = (PadLen<N>::value + 15) / 16 * 16 + 16 / W;
   constexpr int RL = Plan<N>::R[Plan<N>::P - 1], PERL = PassShape<N, Plan<N>::NT, RL>::PER;
   const size_t sm = sizeof(float2) * (N + W * LD + (AdjAccInSmem<N>::value ? size_t(PERL) * RL * Plan<N>::NT * W : 0));
   cudaError_t e = smem_attrs(k_adj_cols<N>, sm);
   if (e != cudaSuccess) return e;
   const int splits = adj_col_splits(period);
-  k_adj_cols<N><<<dim3(crop / W, (fields / period) * splits), Plan<N>::NT * W, sm, st>>>(u, phi, lam, crop, tw, part,
-                                                                                          period, splits);
+  k_adj_cols<N><<<dim3(crop / W, clips * splits), Plan<N>::NT * W, sm, st>>>(u, phi, crop, tw, part, period, splits);
   return cudaGetLastError();
 }
 
@@ -539,17 +552,16 @@ cudaError_t grad_rows_n(const float2* qf, int crop, float scale, const float* m,
     default: return cudaErrorInvalidValue; \
   }
 
-cudaError_t launch_adj_rows(int n, const float2* t1, const float* lam, int nk, int crop, const float* g,
-                            const float2* tw, float2* u, int planes, int lam_period, cudaStream_t st,
-                            const float2* tw512) {
-#define CALL(N) adj_rows_n<N>(t1, lam, nk, crop, g, tw, u, planes, lam_period, st, tw512)
+cudaError_t launch_adj_rows(int n, const float2* t1, const FieldSet& fs, int clips, int crop, const float* g,
+                            int g_planes, const float2* tw, float2* u, cudaStream_t st, const float2* tw512) {
+#define CALL(N) adj_rows_n<N>(t1, fs, clips, crop, g, g_planes, tw, u, st, tw512)
   ILT_DISPATCH(n, CALL)
 #undef CALL
 }
-// fields = clips x period; part receives clips x adj_col_splits(period) crop x crop sums.
-cudaError_t launch_adj_cols(int n, const float2* u, const float2* phi, const float* lam, int crop, const float2* tw,
-                            float2* part, int fields, int period, cudaStream_t st) {
-#define CALL(N) adj_cols_n<N>(u, phi, lam, crop, tw, part, fields, period, st)
+// part receives clips x adj_col_splits(period) crop x crop sums.
+cudaError_t launch_adj_cols(int n, const float2* u, const float2* phi, int crop, const float2* tw, float2* part,
+                            int clips, int period, cudaStream_t st) {
+#define CALL(N) adj_cols_n<N>(u, phi, crop, tw, part, clips, period, st)
   ILT_DISPATCH(n, CALL)
 #undef CALL
 }
@@ -664,14 +676,16 @@ size_t ai_channels_bytes(const litho_kernels* h, int b) { return ilt_layout(h, b
 
 litho_status ai_channels(const litho_kernels* h, const float* target, int b, double dose, int focus, bool coarse,
                          float* x, void* workspace, cudaStream_t st) {
-  const int G = ilt_group(h, b), K = h->k, N = h->n, C = h->crop;
+  const int G = ilt_group(h, b), N = h->n, C = h->crop;
   IltLayout L = ilt_layout(h, b, 1, G, workspace);
   const size_t nn = size_t(N) * N;
   coarse = coarse && h->nc > 0 && interp_cols_supported(h->nc, N);
   const int NE = coarse ? h->nc : N, C2 = 2 * C;
   const float2* twe = coarse ? h->d_twc : h->d_tw;
-  const float2* phi = h->d_phi + size_t(focus) * K * C * C;
-  const float* lam = h->d_lambda + size_t(focus) * K;
+  const int set = h->set_of[focus];
+  const FieldSet fs = field_set(h, set, 1);
+  const PlaneOut one = plane_out_identity(1);
+  const float2* psi = h->d_psi + h->set_start[set] * (size_t(C) * C);
   const float scale = float(2.0 * dose / (double(N) * double(N)));
   // a 1024-point coarse grid: the warp-per-row stage 2 writes the coarse image's row spectra itself
   const bool rows2 = coarse && h->d_tw32 && stage2_w32_supported(NE, C);
@@ -680,22 +694,21 @@ litho_status ai_channels(const litho_kernels* h, const float* target, int b, dou
     {  // channel 1: the aerial image of the targets (interpolated from the coarse grid)
       ProfScope ps(kStageIltForward, st, coarse ? (rows2 ? 6 : 7) : 4);
       LITHO_TRY_CUDA(launch_mask_spectrum(target + c0 * nn, g, N, C, h->d_tw, L.rowbuf, L.mhat, st));
-      LITHO_TRY_CUDA(launch_stage1_fft(L.mhat, phi, K, NE, C, twe, L.t1, st, g));
-      LITHO_TRY_CUDA(launch_stage2_fft(L.t1, lam, K, NE, C, float(dose), twe, coarse ? L.ic : L.img, g,
-                                       (long long)K * NE * C, (long long)NE * NE, st, 1, h->d_tw32, h->d_tw512, false,
-                                       rows2 ? L.mid : nullptr, C2));
+      LITHO_TRY_CUDA(launch_stage1_fft(L.mhat, psi, fs.fields(), NE, C, twe, L.t1, st, g));
+      LITHO_TRY_CUDA(launch_stage2_fft(L.t1, fs, g, NE, C, float(dose), twe, coarse ? L.ic : L.img, one, st,
+                                       h->d_tw32, h->d_tw512, rows2 ? L.mid : nullptr, C2));
       if (coarse) {
         if (!rows2) LITHO_TRY_CUDA(launch_mask_rows(L.ic, g, NE, C2, twe, L.mid, st));
         LITHO_TRY_CUDA(launch_interp_cols(L.mid, g, NE, N, C2, twe, h->d_tw, nullptr, L.big, st));
-        LITHO_TRY_CUDA(launch_band_rows_real(L.big, g, N, C2, 1.0f, h->d_tw, L.img, st));
+        LITHO_TRY_CUDA(launch_band_rows_real(L.big, g, 1, N, C2, 1.0f, h->d_tw, L.img, one, st));
       }
       k_to_channel<<<512, 256, 0, st>>>(L.img, x + size_t(c0) * 3 * nn, g, nn, 1);
       LITHO_TRY_CUDA(cudaGetLastError());
     }
     {  // channel 2: the adjoint applied to dL/dI = 1, in closed form (k_ones_adjoint)
       ProfScope ps(kStageIltBackward, st, 3);
-      k_ones_adjoint<<<dim3(128, g), 256, 0, st>>>(L.mhat, phi, lam, K, size_t(C) * C,
-                                                   float(double(N) * double(N)), L.s, 0);
+      k_ones_adjoint<<<dim3(128, g), 256, 0, st>>>(L.mhat, h->d_power, sets_of(h, focus, 1), size_t(C) * C,
+                                                   float(double(N) * double(N)), L.s);
       LITHO_TRY_CUDA(cudaGetLastError());
       LITHO_TRY_CUDA(launch_stage1_fft(L.s, nullptr, g, N, C, h->d_tw, L.qf, st));
       LITHO_TRY_CUDA(launch_grad_rows(N, L.qf, C, scale, nullptr, 0.f, h->d_tw, x + (size_t(c0) * 3 + 2) * nn, g,
@@ -756,7 +769,7 @@ litho_status litho_ilt_grad(const litho_kernels* h, const float* theta_dev, cons
     set_error("blur radius must be below n/2");
     return LITHO_EINVAL;
   }
-  const int F = h->n_focus, K = h->k, N = h->n, C = h->crop;
+  const int F = h->n_focus, N = h->n, C = h->crop;
   int P, G;
   if (!ilt_plan(h, b, F, workspace_bytes, &P, &G)) {
     set_error("workspace too small: %zu bytes given, at least %zu needed", workspace_bytes,
@@ -788,11 +801,14 @@ litho_status litho_ilt_grad(const litho_kernels* h, const float* theta_dev, cons
     return LITHO_EINVAL;
   }
   float2* qrows = reinterpret_cast<float2*>(L.img);
-  // Groups of g clips: every launch covers the group's g x P planes (plane
-  // i P + p is focus plane f0 + p of clip c0 + i; its fields follow the
-  // plane's K kernels).
+  // Focus planes that share an image are evaluated once and counted as often as they occur (their
+  // q = dL/dI adds up): with the full workspace all kernel sets at a time, else one.
+  const int U = h->n_sets, PU = P == F ? U : 1;
+  const PlaneOut each = plane_out_identity(PU);
+  // Groups of g clips: every launch covers the group's g x PU planes (plane
+  // i PU + p is set u0 + p of clip c0 + i).
   for (int c0 = 0; c0 < b; c0 += G) {
-    const int g = std::min(G, b - c0), gp = g * P;
+    const int g = std::min(G, b - c0), gp = g * PU;
     {
       ProfScope ps(kStageIltForward, st, 3);
       {
@@ -804,29 +820,31 @@ litho_status litho_ilt_grad(const litho_kernels* h, const float* theta_dev, cons
       LITHO_TRY_CUDA(cudaGetLastError());
       LITHO_TRY_CUDA(launch_mask_spectrum(L.m, g, N, C, h->d_tw, L.rowbuf, L.mhat, st));
     }
-    for (int f0 = 0; f0 < F; f0 += P) {
-      const float2* phi = h->d_phi + size_t(f0) * K * C * C;
-      const float* lam = h->d_lambda + size_t(f0) * K;
+    for (int u0 = 0; u0 < U; u0 += PU) {
+      const FieldSet fs = field_set(h, u0, PU);
+      const float2* psi = h->d_psi + h->set_start[u0] * (size_t(C) * C);
+      PlaneWeight weight{};
+      for (int f = 0; f < F; ++f)
+        if (h->set_of[f] >= u0 && h->set_of[f] < u0 + PU) ++weight.w[h->set_of[f] - u0];
       {
         ProfScope ps(kStageIltForward, st, coarse ? (rows2 ? 5 : 6) : 5);
-        LITHO_TRY_CUDA(launch_stage1_fft(L.mhat, phi, P * K, NE, C, twe, L.t1, st, g));
-        LITHO_TRY_CUDA(launch_stage2_fft(L.t1, lam, K, NE, C, float(dose), twe, coarse ? L.ic : L.img, gp,
-                                         (long long)K * NE * C, (long long)NE * NE, st, P, h->d_tw32, h->d_tw512,
-                                         false, rows2 ? L.mid : nullptr, C2));
+        LITHO_TRY_CUDA(launch_stage1_fft(L.mhat, psi, fs.fields(), NE, C, twe, L.t1, st, g));
+        LITHO_TRY_CUDA(launch_stage2_fft(L.t1, fs, g, NE, C, float(dose), twe, coarse ? L.ic : L.img, each, st,
+                                         h->d_tw32, h->d_tw512, rows2 ? L.mid : nullptr, C2));
         if (coarse) {  // the blurred image straight from the interpolation (blur applied to the spectrum)
           if (!rows2) LITHO_TRY_CUDA(launch_mask_rows(L.ic, gp, NE, C2, twe, L.mid, st));
           LITHO_TRY_CUDA(launch_interp_cols(L.mid, gp, NE, N, C2, twe, h->d_tw, L.gain, L.big, st));
           // blurred rows, resist, dL/dI and its row spectra on the 2C band (into the free image
           // buffer), partial losses per row pair
-          LITHO_TRY_CUDA(launch_resist_grad_rows(L.big, gp, N, C2, h->d_tw, target_dev + c0 * nn, P,
+          LITHO_TRY_CUDA(launch_resist_grad_rows(L.big, gp, N, C2, h->d_tw, target_dev + c0 * nn, PU, weight,
                                                  float(resist_steep), float(threshold), qrows, L.partial, st));
-          k_reduce_loss<<<g, 1024, 0, st>>>(L.partial, P * N / 2, L.loss + c0, f0 > 0 ? 1 : 0);
+          k_reduce_loss<<<g, 1024, 0, st>>>(L.partial, PU * N / 2, L.loss + c0, u0 > 0 ? 1 : 0);
         } else {
           LITHO_TRY_CUDA(launch_resist(L.img, gp, N, taps, float(threshold), L.blur, nullptr, st));
-          k_resist_grad<<<dim3(kPartials, g), 256, 0, st>>>(L.blur, target_dev + c0 * nn, nn, P,
+          k_resist_grad<<<dim3(kPartials, g), 256, 0, st>>>(L.blur, target_dev + c0 * nn, nn, PU, weight,
                                                            float(resist_steep), float(threshold), L.img, L.partial);
           LITHO_TRY_CUDA(cudaGetLastError());
-          k_reduce_loss<<<g, 1024, 0, st>>>(L.partial, kPartials, L.loss + c0, f0 > 0 ? 1 : 0);
+          k_reduce_loss<<<g, 1024, 0, st>>>(L.partial, kPartials, L.loss + c0, u0 > 0 ? 1 : 0);
         }
         LITHO_TRY_CUDA(cudaGetLastError());
       }
@@ -836,14 +854,15 @@ litho_status litho_ilt_grad(const litho_kernels* h, const float* theta_dev, cons
         if (coarse) {  // low-pass of g (x) q: the spectrum of q on the 2C band times the blur's transfer function
           LITHO_TRY_CUDA(launch_mask_cols(qrows, gp, N, C2, h->d_tw, L.spec, L.gain, true, st));
           LITHO_TRY_CUDA(launch_stage1_fft(L.spec, nullptr, gp, NE, C2, twe, L.mid, st));
-          LITHO_TRY_CUDA(launch_band_rows_real(L.mid, gp, NE, C2, lp_scale, twe, L.ic, st));
+          LITHO_TRY_CUDA(launch_band_rows_real(L.mid, g, PU, NE, C2, lp_scale, twe, L.ic, each, st));
           gsrc = L.ic;
         } else {
           LITHO_TRY_CUDA(launch_resist(L.img, gp, N, taps, float(threshold), L.blur, nullptr, st));
         }
-        LITHO_TRY_CUDA(launch_adj_rows(NE, L.t1, lam, K, C, gsrc, twe, L.u, gp, P, st, h->d_tw512));
-        LITHO_TRY_CUDA(launch_adj_cols(NE, L.u, phi, lam, C, twe, L.sk, gp * K, P * K, st));
-        k_sum_planes<<<dim3(256, g), 256, 0, st>>>(L.sk, adj_col_splits(P * K), size_t(C) * C, L.s, f0 > 0 ? 1 : 0);
+        LITHO_TRY_CUDA(launch_adj_rows(NE, L.t1, fs, g, C, gsrc, PU, twe, L.u, st, h->d_tw512));
+        LITHO_TRY_CUDA(launch_adj_cols(NE, L.u, psi, C, twe, L.sk, g, fs.fields(), st));
+        k_sum_planes<<<dim3(256, g), 256, 0, st>>>(L.sk, adj_col_splits(fs.fields()), size_t(C) * C, L.s,
+                                                   u0 > 0 ? 1 : 0);
         LITHO_TRY_CUDA(cudaGetLastError());
       }
     }
@@ -883,7 +902,7 @@ litho_status litho_intensity_vjp(const litho_kernels* h, const float* mask_dev, 
     set_error("workspace must be 256-byte aligned");
     return LITHO_EINVAL;
   }
-  const int F = h->n_focus, K = h->k, N = h->n, C = h->crop;
+  const int F = h->n_focus, N = h->n, C = h->crop;
   int P, G;
   if (!ilt_plan(h, b, f_count, workspace_bytes, &P, &G)) {
     set_error("workspace too small: %zu bytes given, at least %zu needed", workspace_bytes,
@@ -908,28 +927,55 @@ litho_status litho_intensity_vjp(const litho_kernels* h, const float* mask_dev, 
     const int g = std::min(G, b - c0);
     LITHO_TRY_CUDA(launch_mask_spectrum(mask_dev + c0 * nn, g, N, C, h->d_tw, L.rowbuf, L.mhat, st));
     if (!upstream_dev) {  // dL/dI = 1 on every pixel of the selected planes: the closed form
-      k_ones_adjoint<<<dim3(128, g), 256, 0, st>>>(L.mhat, h->d_phi + size_t(f_first) * K * C * C,
-                                                   h->d_lambda + size_t(f_first) * K, f_count * K, size_t(C) * C,
-                                                   float(double(N) * double(N)), L.s, 0);
+      k_ones_adjoint<<<dim3(128, g), 256, 0, st>>>(L.mhat, h->d_power, sets_of(h, f_first, f_count), size_t(C) * C,
+                                                   float(double(N) * double(N)), L.s);
       LITHO_TRY_CUDA(cudaGetLastError());
     }
     for (int f0 = f_first; upstream_dev && f0 < f_first + f_count; f0 += P) {
-      const int p = std::min(P, f_first + f_count - f0);
+      int p = std::min(P, f_first + f_count - f0);
       const float* up = upstream_dev + (size_t(c0) * F + f0) * nn;
+      // the kernel sets of these planes in order, and the planes of each
+      int sets[kMaxPlanes], nu = 0;
+      for (int f = 0; f < p; ++f) sets[f] = h->set_of[f0 + f];
+      std::sort(sets, sets + p);
+      nu = int(std::unique(sets, sets + p) - sets);
+      PlaneOut planes{};
+      planes.out_planes = p;
+      bool in_order = nu == p;
+      for (int i = 0, at = 0; i < nu; ++i) {
+        for (int f = 0; f < p; ++f)
+          if (h->set_of[f0 + f] == sets[i]) {
+            in_order = in_order && f == i;
+            planes.list[at++] = (unsigned char)f;
+          }
+        planes.first[i + 1] = (unsigned char)at;
+      }
+      if (!in_order) {  // planes with the same fields: their upstreams add up
+        k_sum_upstream<<<dim3(unsigned(std::min<size_t>((nn + 255) / 256, 1024)), g * nu), 256, 0, st>>>(up, nn, nu,
+                                                                                                       planes, L.img);
+        LITHO_TRY_CUDA(cudaGetLastError());
+        up = L.img;
+        p = nu;
+      }
       if (coarse) {
         LITHO_TRY_CUDA(launch_mask_spectrum(up, g * p, N, C2, h->d_tw, L.big, L.spec, st));
         LITHO_TRY_CUDA(launch_stage1_fft(L.spec, nullptr, g * p, NE, C2, twe, L.mid, st));
-        LITHO_TRY_CUDA(launch_band_rows_real(L.mid, g * p, NE, C2, lp_scale, twe, L.ic, st));
+        LITHO_TRY_CUDA(launch_band_rows_real(L.mid, g, p, NE, C2, lp_scale, twe, L.ic, plane_out_identity(p), st));
         up = L.ic;
       }
-      LITHO_TRY_CUDA(launch_stage1_fft(L.mhat, h->d_phi + size_t(f0) * K * C * C, p * K, NE, C, twe, L.t1, st, g));
-      LITHO_TRY_CUDA(
-          launch_adj_rows(NE, L.t1, h->d_lambda + size_t(f0) * K, K, C, up, twe, L.u, g * p, p, st, h->d_tw512));
-      LITHO_TRY_CUDA(launch_adj_cols(NE, L.u, h->d_phi + size_t(f0) * K * C * C, h->d_lambda + size_t(f0) * K, C,
-                                     twe, L.sk, g * p * K, p * K, st));
-      k_sum_planes<<<dim3(256, g), 256, 0, st>>>(L.sk, adj_col_splits(p * K), size_t(C) * C, L.s,
-                                                 f0 > f_first ? 1 : 0);
-      LITHO_TRY_CUDA(cudaGetLastError());
+      // sets that follow one another in the kernel set share their launches
+      for (int r0 = 0, r1; r0 < p; r0 = r1) {
+        for (r1 = r0 + 1; r1 < p && sets[r1] == sets[r0] + (r1 - r0);) ++r1;
+        const FieldSet fs = field_set(h, sets[r0], r1 - r0);
+        const float2* psi = h->d_psi + h->set_start[sets[r0]] * (size_t(C) * C);
+        LITHO_TRY_CUDA(launch_stage1_fft(L.mhat, psi, fs.fields(), NE, C, twe, L.t1, st, g));
+        LITHO_TRY_CUDA(
+            launch_adj_rows(NE, L.t1, fs, g, C, up + size_t(r0) * NE * NE, p, twe, L.u, st, h->d_tw512));
+        LITHO_TRY_CUDA(launch_adj_cols(NE, L.u, psi, C, twe, L.sk, g, fs.fields(), st));
+        k_sum_planes<<<dim3(256, g), 256, 0, st>>>(L.sk, adj_col_splits(fs.fields()), size_t(C) * C, L.s,
+                                                   f0 > f_first || r0 > 0 ? 1 : 0);
+        LITHO_TRY_CUDA(cudaGetLastError());
+      }
     }
     LITHO_TRY_CUDA(launch_stage1_fft(L.s, nullptr, g, N, C, h->d_tw, L.qf, st));
     LITHO_TRY_CUDA(launch_grad_rows(N, L.qf, C, scale, nullptr, 0.f, h->d_tw, dm_dev + c0 * nn, g, (long long)nn,

@@ -1,0 +1,371 @@
+// The SOCS kernels as the device evaluates them: for every focus plane the
+// smallest set of fields that gives the plane's image, with sqrt(lambda)
+// folded in, so that I = dose sum_p |IDFT(M Psi_p)|^2.
+//
+// The object is a real mask, so M(-u) = conj M(u), and a kernel with
+// Psi(-u) = conj Psi(u) gives a real field.  Every kernel is
+// sqrt(lam) Phi = h + i h' with h, h' of that form, and its |E|^2 is the sum
+// of the squares of the two real fields of h and h'.  The plane's image is
+// thus the quadratic form Q = sum h h^T of 2 K real fields, and any set of
+// fields with the same Q gives the same image (Eq. (4)) and the same
+// gradient.  Where Q has rank r < 2 K, its r eigenvectors, scaled by the roots
+// of their eigenvalues and taken two to a complex kernel (|e + i e'|^2 =
+// e^2 + e'^2), are ceil(r/2) < K kernels.  That is the case in focus: with an
+// unaberrated pupil and a centrosymmetric source the TCC is real and even,
+// each h or h' is zero up to a phase, and half the transforms suffice.  Planes
+// whose Q agree (+z and -z of such a system) share one set.  Nothing is
+// assumed about the optics: the Gram matrix of the h decides, in FP64, once
+// per kernel set; a plane that does not reduce keeps sqrt(lam) Phi.
+//
+// Measured (K = 24, planes at -50/0/+50 nm: 36 fields a clip instead of 72):
+// 64 clips of 2048^2 with resist 15.50 -> 9.78 ms, 8 clips on the full grid
+// 5.96 -> 3.27 ms, on the tensor cores 5.18 -> 3.12 ms; ILT step of 16 clips
+// of 1024^2, K = 16, 5 planes 3.62 -> 2.16 ms; one 2048^2 clip in focus 149 ->
+// 117 us.  Error against 64 bits unchanged (3.7e-7, 2.7e-7, 3.0e-6, 1.2e-6, 3.7e-7).
+#include <algorithm>
+#include <cmath>
+#include <new>
+
+#include "litho_internal.h"
+
+namespace litho {
+
+namespace {
+
+constexpr int kMaxReduceK = 64;                       // kernels per plane the reduction considers (2 K-square Jacobi)
+constexpr size_t kMaxReduceBytes = size_t(2) << 30;   // FP64 kernels held on the device while the set is built
+constexpr double kRankTol = 1e-12;                    // eigenvalues of Q below this share of the largest are rounding
+constexpr double kSameTol = 3.552713678800501e-15;    // 2^-48: planes with |Q - Q'|_F <= 2^-24 |Q|_F share a set
+
+// Crop index of -u: entry 0 is u = -C/2, its own mirror on a full-width crop
+// (C = N) and required to be zero otherwise.
+__device__ __forceinline__ int mirror(int i, int crop) {
+  const int v = i / crop, u = i - v * crop;
+  return (v ? crop - v : 0) * crop + (u ? crop - u : 0);
+}
+
+// out[k][l] = (Re, Im) of sum_u A_k(u) conj B_l(u), then of sum_u A_k(u) B_l(-u); block (l, k).
+__global__ void __launch_bounds__(256) k_gram(const double2* __restrict__ a, const double2* __restrict__ b, int crop,
+                                              double4* __restrict__ out) {
+  const int cc = crop * crop;
+  a += (size_t)blockIdx.y * cc;
+  b += (size_t)blockIdx.x * cc;
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int i = threadIdx.x; i < cc; i += blockDim.x) {
+    const double2 x = a[i], y = b[i], z = b[mirror(i, crop)];
+    s[0] += x.x * y.x + x.y * y.y;
+    s[1] += x.y * y.x - x.x * y.y;
+    s[2] += x.x * z.x - x.y * z.y;
+    s[3] += x.x * z.y + x.y * z.x;
+  }
+  __shared__ double w[8][4];
+  for (int q = 0; q < 4; ++q) {
+    for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_down_sync(0xffffffffu, s[q], o);
+    if (threadIdx.x % 32 == 0) w[threadIdx.x / 32][q] = s[q];
+  }
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    double t = 0.0;
+    for (int i = 0; i < 8; ++i) t += w[i][threadIdx.x];
+    reinterpret_cast<double*>(out + (size_t)blockIdx.y * gridDim.x + blockIdx.x)[threadIdx.x] = t;
+  }
+}
+
+// flag[f] = 1 when a kernel of plane f is nonzero at u = -C/2 (no mirror on the crop); block per kernel.
+__global__ void k_edge(const double2* __restrict__ phi, int crop, int nk, int* __restrict__ flag) {
+  const double2* p = phi + (size_t)blockIdx.x * crop * crop;
+  bool any = false;
+  for (int i = threadIdx.x; i < crop; i += blockDim.x) {
+    const double2 x = p[i], y = p[(size_t)i * crop];
+    any = any || x.x != 0.0 || x.y != 0.0 || y.x != 0.0 || y.y != 0.0;
+  }
+  if (any) flag[blockIdx.x / nk] = 1;
+}
+
+// psi_p(u) = sum_k alpha[p][k] Phi_k(u) + beta[p][k] conj Phi_k(-u); blockIdx.y = p.
+__global__ void __launch_bounds__(256) k_combine(const double2* __restrict__ phi, int nk, int crop,
+                                                 const double2* __restrict__ alpha, const double2* __restrict__ beta,
+                                                 float2* __restrict__ psi) {
+  const int cc = crop * crop, p = blockIdx.y, i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= cc) return;
+  const int m = mirror(i, crop);
+  double re = 0.0, im = 0.0;
+  for (int k = 0; k < nk; ++k) {
+    const double2 x = phi[(size_t)k * cc + i], y = phi[(size_t)k * cc + m];
+    const double2 a = alpha[p * nk + k], b = beta[p * nk + k];
+    re += a.x * x.x - a.y * x.y + b.x * y.x + b.y * y.y;
+    im += a.x * x.y + a.y * x.x + b.y * y.x - b.x * y.y;
+  }
+  psi[(size_t)p * cc + i] = make_float2(float(re), float(im));
+}
+
+// One kernel that is kept: psi = root Phi.
+__global__ void __launch_bounds__(256) k_scale(const double2* __restrict__ phi, double root, size_t cc,
+                                               float2* __restrict__ psi) {
+  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (i < cc) psi[i] = make_float2(float(root * phi[i].x), float(root * phi[i].y));
+}
+// power += lam |Phi|^2 (the closed-form adjoint of ones, see k_ones_adjoint).
+__global__ void __launch_bounds__(256) k_add_power(const double2* __restrict__ phi, double lam, size_t cc,
+                                                   double* __restrict__ dsum) {
+  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (i < cc) dsum[i] += lam * (phi[i].x * phi[i].x + phi[i].y * phi[i].y);
+}
+__global__ void __launch_bounds__(256) k_round(const double* __restrict__ x, size_t n, float* __restrict__ y) {
+  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (i < n) y[i] = float(x[i]);
+}
+
+// Eigenvalues (descending) and eigenvectors (columns of v) of a real symmetric
+// matrix by cyclic Jacobi rotations; false when it does not settle.
+bool jacobi(std::vector<double>& a, int n, std::vector<double>& ev, std::vector<double>& v) {
+  v.assign(size_t(n) * n, 0.0);
+  for (int i = 0; i < n; ++i) v[size_t(i) * n + i] = 1.0;
+  double norm = 0.0;
+  for (double x : a) norm += x * x;
+  bool done = false;
+  for (int sweep = 0; sweep < 60 && !done; ++sweep) {
+    double off = 0.0;
+    for (int p = 0; p < n; ++p)
+      for (int q = p + 1; q < n; ++q) off += a[size_t(p) * n + q] * a[size_t(p) * n + q];
+    done = off <= 1e-34 * norm;
+    for (int p = 0; p < n && !done; ++p)
+      for (int q = p + 1; q < n; ++q) {
+        const double g = a[size_t(p) * n + q];
+        if (g == 0.0) continue;
+        const double th = (a[size_t(q) * n + q] - a[size_t(p) * n + p]) / (2.0 * g);
+        const double t = (th >= 0 ? 1.0 : -1.0) / (std::fabs(th) + std::sqrt(th * th + 1.0));
+        const double c = 1.0 / std::sqrt(t * t + 1.0), s = t * c;
+        for (int i = 0; i < n; ++i) {
+          const double x = a[size_t(i) * n + p], y = a[size_t(i) * n + q];
+          a[size_t(i) * n + p] = c * x - s * y;
+          a[size_t(i) * n + q] = s * x + c * y;
+        }
+        for (int i = 0; i < n; ++i) {
+          const double x = a[size_t(p) * n + i], y = a[size_t(q) * n + i];
+          a[size_t(p) * n + i] = c * x - s * y;
+          a[size_t(q) * n + i] = s * x + c * y;
+        }
+        for (int i = 0; i < n; ++i) {
+          const double x = v[size_t(i) * n + p], y = v[size_t(i) * n + q];
+          v[size_t(i) * n + p] = c * x - s * y;
+          v[size_t(i) * n + q] = s * x + c * y;
+        }
+      }
+  }
+  std::vector<int> order(n);
+  for (int i = 0; i < n; ++i) order[i] = i;
+  std::sort(order.begin(), order.end(), [&](int x, int y) { return a[size_t(x) * n + x] > a[size_t(y) * n + y]; });
+  ev.resize(n);
+  std::vector<double> w(size_t(n) * n);
+  for (int j = 0; j < n; ++j) {
+    ev[j] = a[size_t(order[j]) * n + order[j]];
+    for (int i = 0; i < n; ++i) w[size_t(i) * n + j] = v[size_t(i) * n + order[j]];
+  }
+  v.swap(w);
+  return done;
+}
+
+// Inner products of the real fields' kernels h_2k + i h_2k+1 = root_k Phi_k of
+// two planes, from k_gram's sums P = sum A conj B and R = sum A B(-u):
+// <h, h> = Re(P + R)/2, <h', h'> = Re(P - R)/2, <h, h'> = Im(R - P)/2,
+// <h', h> = Im(R + P)/2.
+std::vector<double> real_gram(const std::vector<double4>& g, const double* root_a, int ka, const double* root_b,
+                              int kb) {
+  std::vector<double> out(size_t(4) * ka * kb);
+  for (int k = 0; k < ka; ++k)
+    for (int l = 0; l < kb; ++l) {
+      const double4 e = g[size_t(k) * kb + l];
+      const double r = 0.5 * root_a[k] * root_b[l];
+      double* o = &out[size_t(2 * k) * (2 * kb) + 2 * l];
+      o[0] = r * (e.x + e.z);
+      o[1] = r * (e.w - e.y);
+      o[2 * kb] = r * (e.w + e.y);
+      o[2 * kb + 1] = r * (e.x - e.z);
+    }
+  return out;
+}
+
+double sum_sq(const std::vector<double>& a) {
+  double s = 0.0;
+  for (double x : a) s += x * x;
+  return s;
+}
+
+struct DeviceBuffer {
+  void* p = nullptr;
+  ~DeviceBuffer() { cudaFree(p); }
+  template <class T>
+  T* as() const {
+    return static_cast<T*>(p);
+  }
+};
+
+litho_status build(litho_kernels* h) {
+  const int F = h->n_focus, K = h->k, C = h->crop;
+  const size_t cc = size_t(C) * C, plane_len = size_t(K) * cc;
+  const double2* host = reinterpret_cast<const double2*>(h->phi_host.data());
+  std::vector<double> root(size_t(F) * K);  // sqrt(lambda); 0 for the kernels the FP32 path leaves out
+  for (size_t i = 0; i < root.size(); ++i) root[i] = float(h->lambda[i]) > 0.f ? std::sqrt(h->lambda[i]) : 0.0;
+
+  struct Set {
+    int plane;                         // its first focus plane
+    bool reduced = false;
+    std::vector<double> gram;          // 2K x 2K, when the plane can be reduced or shared
+    std::vector<double2> alpha, beta;  // [kernels][K] when reduced
+    int kernels = 0;
+  };
+  std::vector<Set> sets;
+  DeviceBuffer phi64, gram_d, flag_d, coef, power;
+  const bool whole = K <= kMaxReduceK && F * plane_len * sizeof(double2) <= kMaxReduceBytes;
+  std::vector<int> edge(F, 1);
+  if (whole) {
+    LITHO_TRY_CUDA(cudaMalloc(&phi64.p, F * plane_len * sizeof(double2)));
+    LITHO_TRY_CUDA(cudaMemcpy(phi64.p, host, F * plane_len * sizeof(double2), cudaMemcpyHostToDevice));
+    LITHO_TRY_CUDA(cudaMalloc(&gram_d.p, size_t(K) * K * sizeof(double4)));
+    LITHO_TRY_CUDA(cudaMalloc(&coef.p, size_t(2) * K * K * sizeof(double2)));
+    LITHO_TRY_CUDA(cudaMalloc(&flag_d.p, F * sizeof(int)));
+    LITHO_TRY_CUDA(cudaMemset(flag_d.p, 0, F * sizeof(int)));
+    if (C < h->n) k_edge<<<F * K, 128>>>(phi64.as<double2>(), C, K, flag_d.as<int>());
+    LITHO_TRY_CUDA(cudaGetLastError());
+    LITHO_TRY_CUDA(cudaMemcpy(edge.data(), flag_d.p, F * sizeof(int), cudaMemcpyDeviceToHost));
+  } else {
+    LITHO_TRY_CUDA(cudaMalloc(&phi64.p, cc * sizeof(double2)));  // one kernel at a time
+  }
+  auto gram = [&](int fa, int fb, std::vector<double>* out) -> litho_status {
+    std::vector<double4> g(size_t(K) * K);
+    k_gram<<<dim3(K, K), 256>>>(phi64.as<double2>() + fa * plane_len, phi64.as<double2>() + fb * plane_len, C,
+                                gram_d.as<double4>());
+    LITHO_TRY_CUDA(cudaGetLastError());
+    LITHO_TRY_CUDA(cudaMemcpy(g.data(), gram_d.p, g.size() * sizeof(double4), cudaMemcpyDeviceToHost));
+    *out = real_gram(g, &root[size_t(fa) * K], K, &root[size_t(fb) * K], K);
+    return LITHO_OK;
+  };
+  for (int f = 0; f < F; ++f) {
+    Set t;
+    t.plane = f;
+    int nonzero = 0;
+    for (int k = 0; k < K; ++k) nonzero += root[size_t(f) * K + k] > 0.0;
+    t.kernels = nonzero;
+    int shared = -1;
+    if (!edge[f]) {
+      litho_status s = gram(f, f, &t.gram);
+      if (s != LITHO_OK) return s;
+      const double na = sum_sq(t.gram);
+      if (!std::isfinite(na)) t.gram.clear();
+      for (size_t e = 0; e < sets.size() && shared < 0 && !t.gram.empty(); ++e) {
+        if (sets[e].gram.empty()) continue;
+        const double nb = sum_sq(sets[e].gram);
+        if (std::fabs(na - nb) > 1e-6 * std::max(na, nb)) continue;
+        std::vector<double> x;
+        if ((s = gram(sets[e].plane, f, &x)) != LITHO_OK) return s;
+        // |Q - Q'|^2 = |G|^2 + |G'|^2 - 2 |X|^2
+        if (na + nb - 2.0 * sum_sq(x) <= kSameTol * std::max(na, nb)) shared = int(e);
+      }
+    }
+    if (shared >= 0) {
+      h->set_of[f] = (unsigned char)shared;
+      continue;
+    }
+    h->set_of[f] = (unsigned char)sets.size();
+    std::vector<double> a = t.gram, ev, v;
+    if (!a.empty() && jacobi(a, 2 * K, ev, v) && ev[0] > 0.0) {
+      int r = 0;
+      while (r < 2 * K && ev[r] > kRankTol * ev[0]) ++r;
+      if ((r + 1) / 2 < nonzero) {
+        t.reduced = true;
+        t.kernels = (r + 1) / 2;
+        t.alpha.resize(size_t(t.kernels) * K);
+        t.beta.resize(size_t(t.kernels) * K);
+        auto at = [&](int row, int col) { return col < r ? v[size_t(row) * (2 * K) + col] : 0.0; };
+        for (int q = 0; q < t.kernels; ++q)
+          for (int k = 0; k < K; ++k) {
+            // eigenvectors (a1, b1) and (a2, b2) on h_2k, h_2k+1; a h + b h' = root ((a - i b) Phi + (a + i b) conj Phi(-u))/2
+            const double a1 = at(2 * k, 2 * q), b1 = at(2 * k + 1, 2 * q);
+            const double a2 = at(2 * k, 2 * q + 1), b2 = at(2 * k + 1, 2 * q + 1), w = 0.5 * root[size_t(f) * K + k];
+            t.alpha[size_t(q) * K + k] = make_double2(w * (a1 + b2), w * (a2 - b1));
+            t.beta[size_t(q) * K + k] = make_double2(w * (a1 - b2), w * (a2 + b1));
+          }
+      }
+    }
+    sets.push_back(std::move(t));
+  }
+
+  h->n_sets = int(sets.size());
+  h->set_start[0] = 0;
+  for (int u = 0; u < h->n_sets; ++u) h->set_start[u + 1] = h->set_start[u] + sets[u].kernels;
+  const size_t total = std::max(1, h->set_start[h->n_sets]);
+  LITHO_TRY_CUDA(cudaMalloc(&h->d_psi, total * cc * sizeof(float2)));
+  LITHO_TRY_CUDA(cudaMalloc(&h->d_power, h->n_sets * cc * sizeof(float)));
+  LITHO_TRY_CUDA(cudaMalloc(&power.p, cc * sizeof(double)));
+  const unsigned blocks = unsigned((cc + 255) / 256);
+  for (int u = 0; u < h->n_sets; ++u) {
+    const Set& t = sets[u];
+    float2* psi = h->d_psi + h->set_start[u] * cc;
+    LITHO_TRY_CUDA(cudaMemset(power.p, 0, cc * sizeof(double)));
+    int at = 0;
+    for (int k = 0; k < K; ++k) {
+      const double r = root[size_t(t.plane) * K + k];
+      if (r == 0.0) continue;
+      const double2* src = phi64.as<double2>() + (whole ? t.plane * plane_len + k * cc : 0);
+      if (!whole)
+        LITHO_TRY_CUDA(cudaMemcpy(phi64.p, host + t.plane * plane_len + k * cc, cc * sizeof(double2),
+                                  cudaMemcpyHostToDevice));
+      if (!t.reduced) k_scale<<<blocks, 256>>>(src, r, cc, psi + (at++) * cc);
+      k_add_power<<<blocks, 256>>>(src, h->lambda[size_t(t.plane) * K + k], cc, power.as<double>());
+    }
+    if (t.reduced) {
+      double2* d_alpha = coef.as<double2>();
+      double2* d_beta = d_alpha + size_t(K) * K;
+      LITHO_TRY_CUDA(cudaMemcpy(d_alpha, t.alpha.data(), t.alpha.size() * sizeof(double2), cudaMemcpyHostToDevice));
+      LITHO_TRY_CUDA(cudaMemcpy(d_beta, t.beta.data(), t.beta.size() * sizeof(double2), cudaMemcpyHostToDevice));
+      k_combine<<<dim3(blocks, t.kernels), 256>>>(phi64.as<double2>() + t.plane * plane_len, K, C, d_alpha, d_beta, psi);
+    }
+    k_round<<<blocks, 256>>>(power.as<double>(), cc, h->d_power + u * cc);
+    LITHO_TRY_CUDA(cudaGetLastError());
+  }
+  LITHO_TRY_CUDA(cudaStreamSynchronize(nullptr));  // the set is read from any stream afterwards
+  return LITHO_OK;
+}
+
+}  // namespace
+
+litho_status build_kernel_set(litho_kernels* h) {
+  try {
+    return build(h);
+  } catch (const std::bad_alloc&) {
+    set_error("host allocation failed while building the kernel set");
+    return LITHO_ENOMEM;
+  }
+}
+
+// Planes [0, count) of the sets [first, first + count): their fields in order.
+FieldSet field_set(const litho_kernels* h, int first, int count) {
+  FieldSet s{};
+  s.planes = count;
+  for (int p = 0; p <= count; ++p) s.start[p] = h->set_start[first + p] - h->set_start[first];
+  return s;
+}
+
+PlaneOut plane_out(const litho_kernels* h) {
+  PlaneOut o{};
+  o.out_planes = h->n_focus;
+  int at = 0;
+  for (int u = 0; u < h->n_sets; ++u) {
+    o.first[u] = (unsigned char)at;
+    for (int f = 0; f < h->n_focus; ++f)
+      if (h->set_of[f] == u) o.list[at++] = (unsigned char)f;
+  }
+  o.first[h->n_sets] = (unsigned char)at;
+  return o;
+}
+
+PlaneOut plane_out_identity(int planes) {
+  PlaneOut o{};
+  o.out_planes = planes;
+  for (int u = 0; u < planes; ++u) o.first[u] = o.list[u] = (unsigned char)u;
+  o.first[planes] = (unsigned char)planes;
+  return o;
+}
+
+}  // namespace litho

@@ -27,6 +27,22 @@ void set_error(const char* fmt, ...);
 
 using cd = std::complex<double>;
 
+constexpr int kMaxPlanes = 64;  // focus planes of a kernel set
+
+// The planes a launch evaluates per clip and the fields of each: plane p of
+// clip i sums the fields [start[p], start[p + 1]) of the clip's start[planes].
+struct FieldSet {
+  int planes;
+  int start[kMaxPlanes + 1];
+  __host__ __device__ int fields() const { return start[planes]; }
+};
+// Where a launch's planes go: plane p of clip i is written to the output
+// planes list[first[p]] ... of the clip's out_planes.
+struct PlaneOut {
+  int out_planes;
+  unsigned char first[kMaxPlanes + 1], list[kMaxPlanes];
+};
+
 // ---- per-stage device timing (prof.cpp) ------------------------------------------------------
 enum Stage {
   kStageMaskSpectrum = 0,
@@ -91,8 +107,12 @@ struct litho_kernels {
   std::vector<int> rank;
   std::vector<double> lambda, trace, gap;  // [F*K], [F], [F]
   std::vector<double> phi_host;            // [F][K][C][C][2]
-  float* d_lambda = nullptr;               // [F*K]
-  float2* d_phi = nullptr;                 // [F][K][C][C]
+  // The fields the device evaluates (kernelset.cu): n_sets sets of kernels Psi with
+  // sqrt(lambda) folded in, set u at d_psi + set_start[u] C^2; plane f is the image of set set_of[f].
+  int n_sets = 0, set_start[litho::kMaxPlanes + 1] = {};
+  unsigned char set_of[litho::kMaxPlanes] = {};
+  float2* d_psi = nullptr;                 // [set_start[n_sets]][C][C]
+  float* d_power = nullptr;                // [n_sets][C][C]: sum_k lam_k |Phi_k|^2
   float2* d_tw = nullptr;                  // FFT twiddle table for N
   int nc = 0;                              // FP32 FFT coarse grid: smallest power of two >= 2 crop (0: not below N)
   float2* d_twc = nullptr;                 // FFT twiddle table for nc
@@ -100,8 +120,6 @@ struct litho_kernels {
   float2* d_twc_tc = nullptr;              // FFT twiddle table for nc_tc (d_twc when nc_tc == nc)
   float2* d_tw32 = nullptr;                // second-pass twiddles of the warp-per-row 1024-point stage 2
                                            // (when N or nc is 1024, else NULL)
-  float2* d_phi_s = nullptr;               // sqrt(lam_fk) Phi_fk [F][K][C][C]: the aerial path's stage 1 on a
-                                           // 1024-point grid, so that stage 2 sums |E|^2 unweighted (with d_tw32)
   float2* d_tw512 = nullptr;               // twiddles of the 512-point adjoint rows, two rows per warp
                                            // (when N or nc is 512, else NULL)
   litho::GemmOperands* gemm = nullptr;     // lazily built per precision
@@ -127,6 +145,16 @@ inline const float2* coarse_tw(const litho_kernels* h, litho_precision p) {
   return p == LITHO_PREC_FFT32 ? h->d_twc : h->d_twc_tc;
 }
 
+// ---- the device's kernel sets (kernelset.cu) --------------------------------------------------
+// Fills n_sets, set_start, set_of, d_psi and d_power from lambda and phi_host.
+litho_status build_kernel_set(litho_kernels* h);
+// The planes of sets [first, first + count) as a launch's planes.
+FieldSet field_set(const litho_kernels* h, int first, int count);
+// Set u of a launch over all sets goes to every focus plane it is the image of.
+PlaneOut plane_out(const litho_kernels* h);
+// Plane p goes to output plane p (library intermediates).
+PlaneOut plane_out_identity(int planes);
+
 // ---- launchers (fft.cu) ---------------------------------------------------------------------
 // The N-entry per-pass twiddle table the FFT kernels expect (false if n unsupported).
 bool fft_twiddle_table(int n, float2* out);
@@ -143,42 +171,38 @@ cudaError_t launch_mask_rows(const float* m, int b, int n, int crop, const float
 bool interp_cols_supported(int nc, int n);
 cudaError_t launch_interp_cols(const float2* rspec, int planes, int nc, int n, int c2, const float2* tw_nc,
                                const float2* tw_n, const float* gain, float2* q, cudaStream_t st);
-// Stage 1 (band multiply + inverse DFT over v): for kernels phi[nk][C][C],
-// t1[j][y][c] = sum_v mhat[v][c] phi_j[v][c] e^{+2 pi i v y/N}, j in [0, nk).
-// phi == NULL transforms nk spectra mhat[j][C][C] themselves.  With kernels,
+// Stage 1 (band multiply + inverse DFT over v): for kernels psi[nk][C][C],
+// t1[j][y][c] = sum_v mhat[v][c] psi_j[v][c] e^{+2 pi i v y/N}, j in [0, nk).
+// psi == NULL transforms nk spectra mhat[j][C][C] themselves.  With kernels,
 // `clips` spectra mhat[clips][C][C] are imaged in one launch; clip i writes
 // t1[j + i nk].
-cudaError_t launch_stage1_fft(const float2* mhat, const float2* phi, int nk, int n, int crop, const float2* tw,
+cudaError_t launch_stage1_fft(const float2* mhat, const float2* psi, int nk, int n, int crop, const float2* tw,
                               float2* t1, cudaStream_t st, int clips = 1);
-// Stage 2 FFT path: I[y][x] = dose * sum_j lam[j] |sum_c t1[j][y][c] e^{+2 pi i u_c x/N}|^2
-// for each of `planes` planes; plane p takes lam[(p mod lam_period) nk ...]
-// (lam_period <= 0: planes, no repetition).  With tw32 (the kernel set's
-// d_tw32) a 1024-point row takes the warp-per-row radix-32 kernel, with
-// tw512 (d_tw512) 512-point rows the two-rows-per-warp kernel.  folded (with
-// tw32 only): the fields were made from sqrt(lam) Phi, so |E|^2 is summed
-// without the weight (lam still marks the zero kernels, which are skipped).
-// spec (with tw32 only): instead of the image, each image row's forward
-// transform on the spec_crop frequencies |u| < spec_crop/2, laid out as
-// launch_mask_rows writes them ([planes][n][spec_crop]); img is not written.
-cudaError_t launch_stage2_fft(const float2* t1, const float* lam, int nk, int n, int crop, float dose,
-                              const float2* tw, float* img, int planes, long long t1_plane_stride,
-                              long long img_plane_stride, cudaStream_t st, int lam_period = 0,
-                              const float2* tw32 = nullptr, const float2* tw512 = nullptr, bool folded = false,
-                              float2* spec = nullptr, int spec_crop = 0);
+// Stage 2 FFT path: I[y][x] = dose * sum_j |sum_c t1[j][y][c] e^{+2 pi i u_c x/N}|^2
+// over the fields of each plane of `fs`, for `clips` clips whose fields follow
+// one another in t1; the image of a plane goes to its planes of `po` in img
+// (planes of n^2).  With tw32 (the kernel set's d_tw32) a 1024-point row takes
+// the warp-per-row radix-32 kernel, with tw512 (d_tw512) 512-point rows the
+// two-rows-per-warp kernel.  spec (with tw32 only): instead of the image, each
+// image row's forward transform on the spec_crop frequencies |u| < spec_crop/2,
+// laid out as launch_mask_rows writes them ([clips][planes][n][spec_crop]);
+// img is not written.
+cudaError_t launch_stage2_fft(const float2* t1, const FieldSet& fs, int clips, int n, int crop, float dose,
+                              const float2* tw, float* img, const PlaneOut& po, cudaStream_t st,
+                              const float2* tw32 = nullptr, const float2* tw512 = nullptr, float2* spec = nullptr,
+                              int spec_crop = 0);
 // The warp-per-row stage 2 for 1024-point rows (stage2_w32.cu) and its
 // second-pass twiddle table (31 x 32 entries w^(r l), r in [1, 32), l in [0, 32)).
 bool stage2_w32_supported(int n, int crop);
 // The two-rows-per-warp stage 2 for 512-point rows (twiddles: the kernel set's d_tw512).
 bool stage2_w512_supported(int n, int crop);
-cudaError_t launch_stage2_w512(const float2* t1, const float* lam, int nk, int n, int crop, float dose,
-                               const float2* tw512, float* img, int planes, long long t1_plane, long long img_plane,
-                               int lam_period, cudaStream_t st);
+cudaError_t launch_stage2_w512(const float2* t1, const FieldSet& fs, int clips, int n, int crop, float dose,
+                               const float2* tw512, float* img, const PlaneOut& po, cudaStream_t st);
 void stage2_w32_table(float2* out);
 constexpr int kStage2W32TableLen = 31 * 32;
-cudaError_t launch_stage2_w32(const float2* t1, const float* lam, int nk, int n, int crop, float dose,
-                              const float2* tw2, float* img, int planes, long long t1_plane, long long img_plane,
-                              int lam_period, cudaStream_t st, bool folded = false, float2* spec = nullptr,
-                              int c2 = 0);
+cudaError_t launch_stage2_w32(const float2* t1, const FieldSet& fs, int clips, int n, int crop, float dose,
+                              const float2* tw2, float* img, const PlaneOut& po, cudaStream_t st,
+                              float2* spec = nullptr, int c2 = 0);
 
 // A device-side delay of about `ms` milliseconds on `st` (util.cu): one
 // thread spinning on the SM clock for a fixed number of cycles, which always
@@ -205,9 +229,10 @@ size_t ai_channels_bytes(const litho_kernels* h, int b);
 litho_status ai_channels(const litho_kernels* h, const float* target, int b, double dose, int focus, bool coarse,
                          float* x, void* workspace, cudaStream_t st);
 
-// out[p][y][x] = scale Re(sum_c q[p][y][c] e^{+2 pi i u_c x/N}) for band rows q[p][N][C].
-cudaError_t launch_band_rows_real(const float2* q, int planes, int n, int crop, float scale, const float2* tw,
-                                  float* out, cudaStream_t st);
+// out[plane][y][x] = scale Re(sum_c q[p][y][c] e^{+2 pi i u_c x/N}) for band rows q[p][N][C] of `clips` x `planes`
+// planes p; plane p of a clip goes to its planes of `po`.
+cudaError_t launch_band_rows_real(const float2* q, int clips, int planes, int n, int crop, float scale,
+                                  const float2* tw, float* out, const PlaneOut& po, cudaStream_t st);
 
 struct ResistTaps;
 // gain[i] = sum_a g[a] cos(2 pi (i - crop/2) a / n): the blur's transfer function on the crop.
@@ -217,15 +242,20 @@ cudaError_t launch_blur_gain(const ResistTaps& taps, int n, int crop, float* gai
 // ILT forward end on the coarse grid, per pair of full-grid rows: blurred rows from the
 // band rows, sigmoid resist, dL/dI and its row spectra on the crop (rowbuf, as
 // launch_mask_rows), and one FP64 partial loss per row pair at partial[plane][pair]
-// (planes x n/2 doubles).  Plane p uses target clip p / planes_per_clip.
+// (planes x n/2 doubles).  Plane p uses target clip p / planes_per_clip and counts weight.w[p mod planes_per_clip]
+// times (the focus planes that share its image).
+struct PlaneWeight {
+  unsigned char w[kMaxPlanes];
+};
 cudaError_t launch_resist_grad_rows(const float2* band, int planes, int n, int crop, const float2* tw,
-                                    const float* target, int planes_per_clip, float beta, float thr, float2* rowbuf,
-                                    double* partial, cudaStream_t st);
+                                    const float* target, int planes_per_clip, const PlaneWeight& weight, float beta,
+                                    float thr, float2* rowbuf, double* partial, cudaStream_t st);
 // Column half of launch_mask_spectrum on row spectra already in rowbuf.
 cudaError_t launch_mask_cols(const float2* rowbuf, int b, int n, int crop, const float2* tw, float2* mhat,
                              const float* gain, bool gain_real, cudaStream_t st);
-cudaError_t launch_band_rows_resist(const float2* q, int planes, int n, int crop, const float2* tw, float threshold,
-                                    float* img, float* iblur, uint8_t* printed, cudaStream_t st);
+cudaError_t launch_band_rows_resist(const float2* q, int clips, int planes, int n, int crop, const float2* tw,
+                                    float threshold, float* img, float* iblur, uint8_t* printed, const PlaneOut& po,
+                                    cudaStream_t st);
 
 // ---- rectangle rasterisation (raster.cu) -----------------------------------------------------
 long long raster_tiles_per_rect(int max_side);

@@ -108,7 +108,9 @@ litho_status litho_aerial_noalloc(const litho_kernels* h, const float* mask_dev,
   litho_status s = scratch_address(&base);
   if (s != LITHO_OK) return s;
   const size_t N = h->n, C = h->crop;
-  const int F = h->n_focus, K = h->k;
+  const int F = h->n_focus;
+  const FieldSet fs = field_set(h, 0, h->n_sets);
+  const PlaneOut po = plane_out(h);
   // Every byte of the three regions is written before it is read within each
   // clip, so nothing carries over from an earlier call and nothing is cleared.
   char* p = static_cast<char*>(base);
@@ -120,9 +122,8 @@ litho_status litho_aerial_noalloc(const litho_kernels* h, const float* mask_dev,
     const float* m = mask_dev + size_t(clip) * N * N;
     float* img = intensity_dev + size_t(clip) * F * N * N;
     LITHO_TRY_CUDA(launch_mask_spectrum(m, 1, int(N), int(C), h->d_tw, rowbuf, mhat, st));
-    LITHO_TRY_CUDA(launch_stage1_fft(mhat, h->d_phi, F * K, int(N), int(C), h->d_tw, t1, st));
-    LITHO_TRY_CUDA(launch_stage2_fft(t1, h->d_lambda, K, int(N), int(C), float(dose), h->d_tw, img, F,
-                                     (long long)K * N * C, (long long)N * N, st));
+    LITHO_TRY_CUDA(launch_stage1_fft(mhat, h->d_psi, fs.fields(), int(N), int(C), h->d_tw, t1, st));
+    LITHO_TRY_CUDA(launch_stage2_fft(t1, fs, 1, int(N), int(C), float(dose), h->d_tw, img, po, st));
   }
   return LITHO_OK;
 }

@@ -1,6 +1,6 @@
 // Stage 2 of the FP32 path for 1024-point rows, one warp per row, and for
 // 512-point rows, two rows per warp (paper
-// Eq. (4): I(y, x) = dose sum_k lam_k |sum_u T_k(y, u) e^{+2 pi i u x / N}|^2).
+// Eq. (4): I(y, x) = dose sum_k |sum_u T_k(y, u) e^{+2 pi i u x / N}|^2, sqrt(lam_k) in T_k).
 //
 // The 1024-point inverse transform of a row is two radix-32 passes
 // (1024 = 32 x 32, Stockham order, as in fft_common.cuh):
@@ -13,7 +13,7 @@
 // through a padded shared-memory buffer (element i at i + i/32, so that both
 // the write, lanes at stride 33, and the read, lanes consecutive, are free of
 // bank conflicts).  The kernel loop runs inside the warp: each lane keeps
-// lam_k |E_k|^2 of its 32 samples in registers across all kernels of the
+// |E_k|^2 of its 32 samples in registers across all kernels of the
 // plane and writes them once, coalesced.  Compared with the three-pass
 // block kernel this halves the shared-memory traffic per row, whose pipe was
 // that kernel's bound.
@@ -53,11 +53,11 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // the row x = lane + 32 q is already where the four-step forward transform
 // wants it (pass 1 over q, twiddle e^{-2 pi i lane u1 / 1024}, exchange,
 // pass 2 over the lanes, output u1 + 32 u2 in lane u1).
-template <bool BANDED, int kWarps, bool FOLDED, bool SPEC>
+template <bool BANDED, int kWarps, bool SPEC>
 __global__ void __launch_bounds__(32 * kWarps, 1)
-    k_stage2_w32(const float2* __restrict__ t1, const float* __restrict__ lam, int nk, int crop, float dose,
-                 const float2* __restrict__ tw2_g, float* __restrict__ img, long long t1_plane, long long img_plane,
-                 int lam_period, float2* __restrict__ spec, int c2) {
+    k_stage2_w32(const float2* __restrict__ t1, const __grid_constant__ FieldSet fs, int crop, float dose,
+                 const float2* __restrict__ tw2_g, float* __restrict__ img, const __grid_constant__ PlaneOut po,
+                 float2* __restrict__ spec, int c2) {
   extern __shared__ float4 smem_raw[];
   float2* tw2 = reinterpret_cast<float2*>(smem_raw);  // w^(r l) at (r - 1) 32 + l
   float2* rowbuf = tw2 + (kR - 1) * kR;                // [kWarps][kRowLd]
@@ -67,8 +67,8 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
   const int lane = threadIdx.x % 32, wp = threadIdx.x / 32;
   const int y = blockIdx.x * kWarps + wp, plane = blockIdx.y, half = crop / 2;
   if (y >= kN) return;  // no barrier below
-  const float2* base = t1 + plane * t1_plane + (size_t)y * crop;
-  const float* lp = lam + (plane % lam_period) * nk;
+  const int clip = plane / fs.planes, pl = plane - clip * fs.planes, nk = fs.start[pl + 1] - fs.start[pl];
+  const float2* base = t1 + ((size_t)(clip * fs.fields() + fs.start[pl]) * kN + y) * crop;
   float2* buf = rowbuf + wp * kRowLd;
   float2* stage = stage0 + (size_t)wp * crop;
   // band row of kernel j into the staging buffer: crop / 2 pieces of 16 bytes
@@ -80,11 +80,10 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
   float acc[kR];
 #pragma unroll
   for (int q = 0; q < kR; ++q) acc[q] = 0.f;
-  fetch(0);
+  if (nk > 0) fetch(0);
   for (int j = 0; j < nk; ++j) {
     cp_async_wait<0>();
     __syncwarp();  // row j visible to every lane
-    const float l = __ldg(lp + j);
     const float2* row = stage;
     float2 v[kR];
 #pragma unroll
@@ -99,7 +98,6 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
     }
     __syncwarp();  // every lane has read row j: the buffer takes row j + 1 during the transform
     if (j + 1 < nk) fetch(j + 1);
-    if (l == 0.f) continue;  // a zero kernel (beyond the rank): uniform across the warp
     dft32<+1, BANDED>(v);
 #pragma unroll
     for (int q = 0; q < kR; ++q) buf[lane * (kR + 1) + q] = v[q];  // position 32 lane + q, padded
@@ -112,9 +110,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
     __syncwarp();  // every lane has read buf before the next kernel's pass 1 writes it
     dft32<+1, false>(v);
 #pragma unroll
-    for (int q = 0; q < kR; ++q)
-      acc[q] = FOLDED ? fmaf(v[q].x, v[q].x, fmaf(v[q].y, v[q].y, acc[q]))  // sqrt(lam) is in the field
-                      : fmaf(l, fmaf(v[q].x, v[q].x, v[q].y * v[q].y), acc[q]);
+    for (int q = 0; q < kR; ++q) acc[q] = fmaf(v[q].x, v[q].x, fmaf(v[q].y, v[q].y, acc[q]));
   }
   if constexpr (SPEC) {
     float2 v[kR];
@@ -142,38 +138,32 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
       if (us >= -h2 && us < h2) srow[us + h2] = v[u2];
     }
   } else {
-    float* out = img + plane * img_plane + (size_t)y * kN;
+    for (int d = po.first[pl]; d < po.first[pl + 1]; ++d) {
+      float* out = img + ((size_t)(clip * po.out_planes + po.list[d]) * kN + y) * kN;
 #pragma unroll
-    for (int q = 0; q < kR; ++q) out[lane + kR * q] = dose * acc[q];
+      for (int q = 0; q < kR; ++q) out[lane + kR * q] = dose * acc[q];
+    }
   }
 }
 
-template <bool BANDED, int kWarps, bool FOLDED, bool SPEC>
-cudaError_t launch_w32_k(const float2* t1, const float* lam, int nk, int crop, float dose, const float2* tw2,
-                         float* img, int planes, long long t1_plane, long long img_plane, int lam_period,
-                         cudaStream_t st, float2* spec, int c2) {
-  const dim3 grid((kN + kWarps - 1) / kWarps, planes);
+template <bool BANDED, int kWarps, bool SPEC>
+cudaError_t launch_w32_k(const float2* t1, const FieldSet& fs, int clips, int crop, float dose, const float2* tw2,
+                         float* img, const PlaneOut& po, cudaStream_t st, float2* spec, int c2) {
+  const dim3 grid((kN + kWarps - 1) / kWarps, clips * fs.planes);
   const size_t sm = sizeof(float2) * ((kR - 1) * kR + kWarps * kRowLd + size_t(kWarps) * crop);
-  cudaError_t e = smem_attrs(k_stage2_w32<BANDED, kWarps, FOLDED, SPEC>, sm);
+  cudaError_t e = smem_attrs(k_stage2_w32<BANDED, kWarps, SPEC>, sm);
   if (e != cudaSuccess) return e;
-  k_stage2_w32<BANDED, kWarps, FOLDED, SPEC><<<grid, 32 * kWarps, sm, st>>>(t1, lam, nk, crop, dose, tw2, img,
-                                                                            t1_plane, img_plane, lam_period, spec, c2);
+  k_stage2_w32<BANDED, kWarps, SPEC><<<grid, 32 * kWarps, sm, st>>>(t1, fs, crop, dose, tw2, img, po, spec, c2);
   return cudaGetLastError();
 }
 
 template <int kWarps>
-cudaError_t launch_w32_t(const float2* t1, const float* lam, int nk, int crop, float dose, const float2* tw2,
-                         float* img, int planes, long long t1_plane, long long img_plane, int lam_period,
-                         cudaStream_t st, bool folded, float2* spec, int c2) {
+cudaError_t launch_w32_t(const float2* t1, const FieldSet& fs, int clips, int crop, float dose, const float2* tw2,
+                         float* img, const PlaneOut& po, cudaStream_t st, float2* spec, int c2) {
   const bool banded = crop / 2 <= kN / 4;  // the band leaves indices [N/4, 3N/4) empty
-#define W32(B, F, S) \
-  launch_w32_k<B, kWarps, F, S>(t1, lam, nk, crop, dose, tw2, img, planes, t1_plane, img_plane, lam_period, st, spec, c2)
-  if (spec) {
-    if (banded) return folded ? W32(true, true, true) : W32(true, false, true);
-    return folded ? W32(false, true, true) : W32(false, false, true);
-  }
-  if (banded) return folded ? W32(true, true, false) : W32(true, false, false);
-  return folded ? W32(false, true, false) : W32(false, false, false);
+#define W32(B, S) launch_w32_k<B, kWarps, S>(t1, fs, clips, crop, dose, tw2, img, po, st, spec, c2)
+  if (spec) return banded ? W32(true, true) : W32(false, true);
+  return banded ? W32(true, false) : W32(false, false);
 #undef W32
 }
 
@@ -182,16 +172,15 @@ cudaError_t launch_w32_t(const float2* t1, const float* lam, int nk, int crop, f
 // second (radix-32) pass lanes 0-15 take row A and lanes 16-31 row B, lane j
 // applying w^(r j) to positions j + 16 r and forming the 32-point DFT whose
 // output q is the sample x = j + 16 q.  One padded exchange (i + i/16) per
-// row and kernel; lam |E|^2 accumulates in registers.  The second-pass
+// row and kernel; |E|^2 accumulates in registers.  The second-pass
 // twiddles are the first 31 x 16 entries of the kernel set's 512-point
 // table (w^(r j), r in [1, 32), j in [0, 16)).
 constexpr int kW512Warps = 8, kW512Buf = 512 + 32;
 
 template <bool BANDED>
 __global__ void __launch_bounds__(32 * kW512Warps, 2)
-    k_stage2_w512(const float2* __restrict__ t1, const float* __restrict__ lam, int nk, int crop, float dose,
-                  const float2* __restrict__ tw_g, float* __restrict__ img, long long t1_plane, long long img_plane,
-                  int lam_period) {
+    k_stage2_w512(const float2* __restrict__ t1, const __grid_constant__ FieldSet fs, int crop, float dose,
+                  const float2* __restrict__ tw_g, float* __restrict__ img, const __grid_constant__ PlaneOut po) {
   constexpr int N = 512;
   extern __shared__ float4 smem_raw[];
   float2* tw = reinterpret_cast<float2*>(smem_raw);  // (r - 1) 16 + j
@@ -204,8 +193,8 @@ __global__ void __launch_bounds__(32 * kW512Warps, 2)
   if (y0 >= N) return;  // no block barrier below
   float2* buf = bufs + wp * 2 * kW512Buf;
   float2* stage = stage0 + (size_t)wp * 2 * crop;
-  const float* lp = lam + (plane % lam_period) * nk;
-  const float2* base = t1 + plane * t1_plane + (size_t)y0 * crop;
+  const int clip = plane / fs.planes, pl = plane - clip * fs.planes, nk = fs.start[pl + 1] - fs.start[pl];
+  const float2* base = t1 + ((size_t)(clip * fs.fields() + fs.start[pl]) * N + y0) * crop;
   const int rsel = lane / 16, jj = lane % 16;
   auto fetch = [&](int k) {  // band rows y0, y0 + 1 of kernel k
     const float2* src = base + (size_t)k * N * crop;
@@ -215,7 +204,7 @@ __global__ void __launch_bounds__(32 * kW512Warps, 2)
   float acc[32];
 #pragma unroll
   for (int q = 0; q < 32; ++q) acc[q] = 0.f;
-  fetch(0);
+  if (nk > 0) fetch(0);
   for (int k = 0; k < nk; ++k) {
     cp_async_wait<0>();
     __syncwarp();
@@ -236,8 +225,6 @@ __global__ void __launch_bounds__(32 * kW512Warps, 2)
     }
     __syncwarp();  // both rows are in registers: the staging buffer takes kernel k + 1
     if (k + 1 < nk) fetch(k + 1);
-    const float l = __ldg(lp + k);
-    if (l == 0.f) continue;  // a zero kernel (beyond the rank): uniform across the warp
 #pragma unroll
     for (int row = 0; row < 2; ++row) {
       dft_reg<16, +1, BANDED>(a[row]);
@@ -255,11 +242,13 @@ __global__ void __launch_bounds__(32 * kW512Warps, 2)
     __syncwarp();  // the row buffers are free for the next kernel
     dft32<+1, false>(v);
 #pragma unroll
-    for (int q = 0; q < 32; ++q) acc[q] = fmaf(l, fmaf(v[q].x, v[q].x, v[q].y * v[q].y), acc[q]);
+    for (int q = 0; q < 32; ++q) acc[q] = fmaf(v[q].x, v[q].x, fmaf(v[q].y, v[q].y, acc[q]));
   }
-  float* out = img + plane * img_plane + (size_t)(y0 + rsel) * N;
+  for (int d = po.first[pl]; d < po.first[pl + 1]; ++d) {
+    float* out = img + ((size_t)(clip * po.out_planes + po.list[d]) * N + y0 + rsel) * N;
 #pragma unroll
-  for (int q = 0; q < 32; ++q) out[jj + 16 * q] = dose * acc[q];
+    for (int q = 0; q < 32; ++q) out[jj + 16 * q] = dose * acc[q];
+  }
 }
 
 }  // namespace
@@ -277,38 +266,28 @@ void stage2_w32_table(float2* out) {
 
 bool stage2_w512_supported(int n, int crop) { return n == 512 && crop >= 2 && crop <= 256 && crop % 2 == 0; }
 
-cudaError_t launch_stage2_w512(const float2* t1, const float* lam, int nk, int n, int crop, float dose,
-                               const float2* tw512, float* img, int planes, long long t1_plane, long long img_plane,
-                               int lam_period, cudaStream_t st) {
+cudaError_t launch_stage2_w512(const float2* t1, const FieldSet& fs, int clips, int n, int crop, float dose,
+                               const float2* tw512, float* img, const PlaneOut& po, cudaStream_t st) {
   if (!stage2_w512_supported(n, crop) || !tw512) return cudaErrorInvalidValue;
-  if (lam_period <= 0) lam_period = planes;
-  const dim3 grid(512 / (2 * kW512Warps), planes);
+  const dim3 grid(512 / (2 * kW512Warps), clips * fs.planes);
   const size_t sm = sizeof(float2) * (31 * 16 + kW512Warps * 2 * (size_t(kW512Buf) + crop));
-  if (crop / 2 <= 128) {  // the band leaves indices [N/4, 3N/4) empty
-    cudaError_t e = smem_attrs(k_stage2_w512<true>, sm);
-    if (e != cudaSuccess) return e;
-    k_stage2_w512<true><<<grid, 32 * kW512Warps, sm, st>>>(t1, lam, nk, crop, dose, tw512, img, t1_plane, img_plane,
-                                                           lam_period);
-  } else {
-    cudaError_t e = smem_attrs(k_stage2_w512<false>, sm);
-    if (e != cudaSuccess) return e;
-    k_stage2_w512<false><<<grid, 32 * kW512Warps, sm, st>>>(t1, lam, nk, crop, dose, tw512, img, t1_plane,
-                                                            img_plane, lam_period);
-  }
+  auto kern = crop / 2 <= 128 ? k_stage2_w512<true>  // the band leaves indices [N/4, 3N/4) empty
+                              : k_stage2_w512<false>;
+  cudaError_t e = smem_attrs(kern, sm);
+  if (e != cudaSuccess) return e;
+  kern<<<grid, 32 * kW512Warps, sm, st>>>(t1, fs, crop, dose, tw512, img, po);
   return cudaGetLastError();
 }
 
-cudaError_t launch_stage2_w32(const float2* t1, const float* lam, int nk, int n, int crop, float dose,
-                              const float2* tw2, float* img, int planes, long long t1_plane, long long img_plane,
-                              int lam_period, cudaStream_t st, bool folded, float2* spec, int c2) {
+cudaError_t launch_stage2_w32(const float2* t1, const FieldSet& fs, int clips, int n, int crop, float dose,
+                              const float2* tw2, float* img, const PlaneOut& po, cudaStream_t st, float2* spec,
+                              int c2) {
   if (!stage2_w32_supported(n, crop) || !tw2) return cudaErrorInvalidValue;
   if (spec && (c2 < 2 || c2 > kN || c2 % 2 != 0)) return cudaErrorInvalidValue;
-  if (lam_period <= 0) lam_period = planes;
   // 12 warps per CTA: one CTA of 384 threads fits the SM's registers (about 160 per thread);
   // measured on the 2048^2 workload's 1024-point rows: 5.90 ms per step against 6.29 with 8
   // warps and 6.04 with 16 (128 registers)
-  return launch_w32_t<12>(t1, lam, nk, crop, dose, tw2, img, planes, t1_plane, img_plane, lam_period, st, folded,
-                          spec, c2);
+  return launch_w32_t<12>(t1, fs, clips, crop, dose, tw2, img, po, st, spec, c2);
 }
 
 }  // namespace litho

@@ -1,0 +1,105 @@
+"""The reduced kernel sets the device images with (kernelset.cu) against the FP64 oracle with the
+kernels as given: planes that reduce (in focus), planes that share a set (+z and -z), planes that do
+neither, and kernels without any symmetry, on every path that reads a set.  Bounds as in the parity
+tests of each path: image 1e-5, gradient 1e-4 relative."""
+import numpy as np
+import pytest
+
+import synth
+from oracle import ilt as OL
+from oracle import imaging as OI
+from tests.gpu_util import DUV_ANNULAR, DUV_QUAD21, oracle_kernel_set
+
+pytestmark = pytest.mark.gpu
+PIXEL = 8.0
+
+
+def _random_set(n, c, planes, k, edge):
+    """Complex kernels with no symmetry, decaying from DC, |E|^2 of order 1; `edge`: nonzero at u = -C/2."""
+    rng = np.random.default_rng(7)
+    u = np.arange(c) - c // 2
+    r2 = u[:, None] ** 2 + u ** 2
+    phi = (rng.standard_normal((planes, k, c, c)) + 1j * rng.standard_normal((planes, k, c, c))) * np.exp(-r2 / (c * c / 18))
+    if not edge:
+        phi[..., 0, :] = 0
+        phi[..., :, 0] = 0
+    else:
+        phi[..., 0, :] += 0.1j
+    lam = np.sort(rng.uniform(0.05, 0.2, (planes, k)))[:, ::-1].copy()
+    lam[-1, -2:] = 0.0
+    return lam, phi
+
+
+def _set(name, n):
+    if name == "random":
+        return _random_set(n, 32, 2, 4, False)
+    if name == "edge":
+        return _random_set(n, 32, 1, 3, True)
+    if name == "full width":  # crop = n: u = -n/2 is its own mirror
+        return _random_set(n, n, 1, 3, True)
+    if name == "dark plane":
+        lam, phi = oracle_kernel_set(DUV_QUAD21, n, PIXEL, [0.0, 30.0], 5)
+        lam[0] = 0.0
+        return lam, phi
+    focus, k, optics = {"nominal": ([0.0], 7, DUV_QUAD21), "one kernel": ([0.0], 1, DUV_ANNULAR),
+                        "through focus": ([-40.0, 0.0, 40.0], 8, DUV_ANNULAR),
+                        "reordered": ([30.0, -60.0, 60.0, 0.0, -30.0], 5, DUV_ANNULAR),
+                        "repeated": ([20.0, 20.0, 0.0, 0.0], 6, DUV_QUAD21)}[name]
+    lam, phi = oracle_kernel_set(optics, n, PIXEL, focus, k)
+    return lam, phi * np.exp(1j * np.arange(k))[:, None, None]  # eigenvectors have no phase of their own
+
+
+SETS = ["nominal", "one kernel", "through focus", "reordered", "repeated", "dark plane", "random", "edge"]
+
+
+@pytest.mark.parametrize("precision", ["fft32", "fft32/coarse", "fp16x3", "fp16x3/coarse"])
+@pytest.mark.parametrize("name", SETS + ["full width"])
+def test_images_match_the_given_kernels(litho_lib, cuda, name, precision):
+    import torch
+    n = 32 if name == "full width" else 256
+    if name == "full width" and precision.startswith("fp16"):
+        pytest.skip("the tensor-core path needs a grid of 128 points")
+    if precision == "fp16x3/coarse" and name in ("random", "edge"):
+        pytest.skip("a coarse grid of 64 points")
+    lam, phi = _set(name, n)
+    kern = litho_lib.litho_upload_kernels(n, PIXEL, lam, phi)
+    masks = np.stack([synth.random_rect_mask(n, seed=3 + i, count=6 if n == 32 else 40) for i in range(3)])
+    img = litho_lib.litho_aerial(kern, torch.from_numpy(masks).to(cuda), precision=precision).cpu().numpy()
+    for i, m in enumerate(masks):
+        for f in range(len(lam)):
+            ref = OI.socs_image(m.astype(np.float64), lam[f], phi[f])
+            assert np.abs(img[i, f] - ref).max() <= 1e-5 * max(1.0, ref.max())
+
+
+@pytest.mark.parametrize("precision", ["fft32", "fft32/coarse"])
+@pytest.mark.parametrize("name", SETS)
+def test_gradients_match_the_given_kernels(litho_lib, cuda, name, precision):
+    import torch
+    n, b = 128, 2
+    lam, phi = _set(name, n)
+    planes = len(lam)
+    kern = litho_lib.litho_upload_kernels(n, PIXEL, lam, phi)
+    pairs = [(lam[f], phi[f]) for f in range(planes)]
+    clips = [synth.ilt_clip(n, PIXEL, seed=40 + i) for i in range(b)]
+    theta = torch.from_numpy(np.stack([c[0] for c in clips])).to(cuda)
+    target = torch.from_numpy(np.stack([c[1] for c in clips])).to(cuda)
+    full, small = litho_lib.litho_ilt_workspace_size(kern, b)
+    for size in (full, small):
+        ws = torch.empty(size, dtype=torch.uint8, device=cuda)
+        grad, loss = litho_lib.litho_ilt_grad(kern, theta, target, precision=precision, workspace=ws)
+        for i in range(b):
+            ref_loss, ref = OL.loss_and_grad(clips[i][0].astype(np.float64), clips[i][1].astype(np.float64), pairs)
+            assert abs(loss[i] - ref_loss) <= 1e-5 * ref_loss
+            assert np.linalg.norm(grad[i].cpu().numpy() - ref) <= 1e-4 * np.linalg.norm(ref)
+    rng = np.random.default_rng(1)
+    up = rng.standard_normal((b, planes, n, n)).astype(np.float32)
+    masks = torch.sigmoid(4 * theta)
+    m64 = masks.cpu().numpy().astype(np.float64)
+    for f0, count in {(0, planes), (planes // 2, planes - planes // 2), (planes - 1, 1)}:
+        for given in (up, None):
+            dm = litho_lib.litho_intensity_vjp(kern, masks, None if given is None else torch.from_numpy(up).to(cuda),
+                                               f_first=f0, f_count=count, precision=precision).cpu().numpy()
+            for i in range(b):
+                g = [up[i, f] if given is not None else np.ones((n, n)) for f in range(f0, f0 + count)]
+                ref = OL.intensity_vjp(m64[i], pairs[f0:f0 + count], g)
+                assert np.linalg.norm(dm[i] - ref) <= 1e-4 * np.linalg.norm(ref)
