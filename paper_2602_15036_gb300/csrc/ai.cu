@@ -21,116 +21,123 @@ namespace litho {
 
 namespace {
 
-constexpr int kReduceBlocks = 304, kReduceThreads = 256;
+constexpr int kReduceThreads = 256;
 
-// Per-block minimum and maximum of channel `ch` of X[b][3][nn]: block
-// (x, clip) scans its share of the clip's channel (16-byte loads when nn is a
-// multiple of 4); partials [b][gridDim.x].
-__global__ void __launch_bounds__(kReduceThreads) k_minmax(const float* __restrict__ x, int b, size_t nn, int ch,
-                                                           float2* __restrict__ part) {
-  __shared__ float smin[kReduceThreads], smax[kReduceThreads];
-  float lo = FLT_MAX, hi = -FLT_MAX;
-  const float* src = x + (size_t(blockIdx.y) * 3 + ch) * nn;
-  const size_t t0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
-  if (nn % 4 == 0) {
-    const float4* s4 = reinterpret_cast<const float4*>(src);
-    for (size_t i = t0; i < nn / 4; i += stride) {
-      const float4 v = s4[i];
-      lo = fminf(lo, fminf(fminf(v.x, v.y), fminf(v.z, v.w)));
-      hi = fmaxf(hi, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
-    }
-  } else {
-    for (size_t i = t0; i < nn; i += stride) {
-      lo = fminf(lo, src[i]);
-      hi = fmaxf(hi, src[i]);
-    }
-  }
-  smin[threadIdx.x] = lo;
-  smax[threadIdx.x] = hi;
-  __syncthreads();
-  for (int o = kReduceThreads / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) {
-      smin[threadIdx.x] = fminf(smin[threadIdx.x], smin[threadIdx.x + o]);
-      smax[threadIdx.x] = fmaxf(smax[threadIdx.x], smax[threadIdx.x + o]);
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) part[size_t(blockIdx.y) * gridDim.x + blockIdx.x] = make_float2(smin[0], smax[0]);
+// Blocks per clip of a pass over b clips: about eight CTAs of kReduceThreads per SM in all.
+unsigned blocks_per_clip(int b, size_t items) {
+  const size_t want = std::max<size_t>(1, size_t(8) * 152 / b);
+  return unsigned(std::max<size_t>(1, std::min(want, (items + kReduceThreads - 1) / kReduceThreads)));
 }
 
-// Channel ch of every clip: v -> (v - lo) * s, with lo and s from the
-// `nparts` block partials (mode 0: lo = 0, s = 1/max; mode 1: lo = min,
-// s = 1/(max - min); s = 0 when the range is empty).  Block (x, clip).
-__global__ void k_normalize(float* __restrict__ x, int b, size_t nn, int ch, const float2* __restrict__ part,
-                            int nparts, int mode) {
-  __shared__ float smin[kReduceThreads], smax[kReduceThreads];
+// Floats as unsigned integers of the same order, for integer atomics.
+__device__ __forceinline__ unsigned ordered(float x) {
+  const unsigned u = __float_as_uint(x);
+  return u & 0x80000000u ? ~u : u | 0x80000000u;
+}
+__device__ __forceinline__ float from_ordered(unsigned u) {
+  return __uint_as_float(u & 0x80000000u ? u & 0x7fffffffu : ~u);
+}
+
+// X[c][0] = target[c]; clip blockIdx.y.
+template <class T>
+__global__ void __launch_bounds__(kReduceThreads) k_copy_channel(const T* __restrict__ src, T* __restrict__ x,
+                                                                 size_t n) {
+  src += (size_t)blockIdx.y * n;
+  x += (size_t)blockIdx.y * 3 * n;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+    x[i] = src[i];
+}
+
+// Extremes of channels 1 and 2 of X[b][3][nn] (clip blockIdx.y, channel 1 + blockIdx.z) into
+// ext[channel - 1] = (min, max), as ordered integers: ~0 and 0 on entry.  nn is a multiple of 4.
+__global__ void __launch_bounds__(kReduceThreads) k_minmax(const float4* __restrict__ x, size_t nn4,
+                                                           uint2* __restrict__ ext) {
+  __shared__ float smin[kReduceThreads / 32], smax[kReduceThreads / 32];
   float lo = FLT_MAX, hi = -FLT_MAX;
-  for (int k = threadIdx.x; k < nparts; k += blockDim.x) {
-    lo = fminf(lo, part[k].x);
-    hi = fmaxf(hi, part[k].y);
+  const float4* src = x + (size_t(blockIdx.y) * 3 + 1 + blockIdx.z) * nn4;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nn4; i += (size_t)gridDim.x * blockDim.x) {
+    const float4 v = src[i];
+    lo = fminf(lo, fminf(fminf(v.x, v.y), fminf(v.z, v.w)));
+    hi = fmaxf(hi, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
   }
-  smin[threadIdx.x] = lo;
-  smax[threadIdx.x] = hi;
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fminf(lo, __shfl_down_sync(0xffffffffu, lo, o));
+    hi = fmaxf(hi, __shfl_down_sync(0xffffffffu, hi, o));
+  }
+  if (threadIdx.x % 32 == 0) {
+    smin[threadIdx.x / 32] = lo;
+    smax[threadIdx.x / 32] = hi;
+  }
   __syncthreads();
-  for (int o = kReduceThreads / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) {
-      smin[threadIdx.x] = fminf(smin[threadIdx.x], smin[threadIdx.x + o]);
-      smax[threadIdx.x] = fmaxf(smax[threadIdx.x], smax[threadIdx.x + o]);
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kReduceThreads / 32; ++w) {
+      lo = fminf(lo, smin[w]);
+      hi = fmaxf(hi, smax[w]);
     }
-    __syncthreads();
+    atomicMin(&ext[blockIdx.z].x, ordered(lo));
+    atomicMax(&ext[blockIdx.z].y, ordered(hi));
   }
-  lo = mode == 0 ? 0.f : smin[0];
-  hi = smax[0];
+}
+
+// Channels 1 and 2 of every clip: v -> (v - lo) s with lo = 0, s = 1/max (channel 1) or lo = min,
+// s = 1/(max - min) (channel 2); s = 0 when the range is empty.
+__global__ void __launch_bounds__(kReduceThreads) k_normalize(float4* __restrict__ x, size_t nn4,
+                                                              const uint2* __restrict__ ext) {
+  const uint2 e = ext[blockIdx.z];
+  const float lo = blockIdx.z == 0 ? 0.f : from_ordered(e.x), hi = from_ordered(e.y);
   const float s = hi > lo ? 1.0f / (hi - lo) : 0.f;
-  float* dst = x + (size_t(blockIdx.y) * 3 + ch) * nn;
-  const size_t t0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
-  if (nn % 4 == 0) {
-    float4* d4 = reinterpret_cast<float4*>(dst);
-    for (size_t i = t0; i < nn / 4; i += stride) {
-      float4 v = d4[i];
-      v.x = (v.x - lo) * s;
-      v.y = (v.y - lo) * s;
-      v.z = (v.z - lo) * s;
-      v.w = (v.w - lo) * s;
-      d4[i] = v;
-    }
-  } else {
-    for (size_t i = t0; i < nn; i += stride) dst[i] = (dst[i] - lo) * s;
+  float4* dst = x + (size_t(blockIdx.y) * 3 + 1 + blockIdx.z) * nn4;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nn4; i += (size_t)gridDim.x * blockDim.x) {
+    float4 v = dst[i];
+    v.x = (v.x - lo) * s;
+    v.y = (v.y - lo) * s;
+    v.z = (v.z - lo) * s;
+    v.w = (v.w - lo) * s;
+    dst[i] = v;
   }
 }
 
-__global__ void k_copy_channel(const float* __restrict__ src, float* __restrict__ x, int b, size_t nn, int ch) {
-  const size_t total = size_t(b) * nn;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x)
-    x[(i / nn) * 3 * nn + size_t(ch) * nn + i % nn] = src[i];
-}
-
-__global__ void k_threshold(const float* __restrict__ img, size_t count, float thr, uint8_t* __restrict__ z) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
-    z[i] = img[i] >= thr ? 1 : 0;
-}
-
-// Number of pixels where the two 0/1 prints differ, per clip (grid y): each
-// block counts 16-byte pieces (the XOR of two 0/1 bytes is one bit) and adds
-// its count to the clip's total with an integer atomic (exact, so the result
-// does not depend on the order).  out must be zero on entry.
-constexpr int kL1Blocks = 64;
-__global__ void __launch_bounds__(kReduceThreads) k_l1_count(const uint4* __restrict__ a, const uint4* __restrict__ b,
-                                                             size_t pieces, unsigned long long* __restrict__ out) {
-  __shared__ unsigned long long s[kReduceThreads];
+// z_print = [I >= thr], 16 pixels a step and thread, and, with `out`, the number of pixels where it
+// differs from z_round, per clip (grid y): the XOR of two 0/1 bytes is one bit; each block adds its
+// count to the clip's total with an integer atomic (exact, so the result does not depend on the
+// order).  out must be zero on entry.  VEC: I is 16-byte aligned.  HBM-bound: 5 bytes a pixel read, 1
+// written (a threshold kernel and a counting one that read both prints again took 150 us for 16
+// planes of 2048^2, this one 62 us).
+template <bool VEC>
+__global__ void __launch_bounds__(kReduceThreads) k_print(const float* __restrict__ img, float thr,
+                                                          const uint4* __restrict__ z_round, size_t pieces,
+                                                          uint4* __restrict__ z_print,
+                                                          unsigned long long* __restrict__ out) {
+  __shared__ unsigned warp_sum[kReduceThreads / 32];
   const size_t base = size_t(blockIdx.y) * pieces;
-  unsigned long long c = 0;
+  unsigned c = 0;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < pieces; i += (size_t)gridDim.x * blockDim.x) {
-    const uint4 x = a[base + i], y = b[base + i];
-    c += __popc(x.x ^ y.x) + __popc(x.y ^ y.y) + __popc(x.z ^ y.z) + __popc(x.w ^ y.w);
+    unsigned z[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float4 v;
+      const float* s = img + (base + i) * 16 + 4 * q;
+      if constexpr (VEC)
+        v = __ldg(reinterpret_cast<const float4*>(s));
+      else
+        v = make_float4(__ldg(s), __ldg(s + 1), __ldg(s + 2), __ldg(s + 3));
+      z[q] = unsigned(v.x >= thr) | unsigned(v.y >= thr) << 8 | unsigned(v.z >= thr) << 16 | unsigned(v.w >= thr) << 24;
+    }
+    z_print[base + i] = make_uint4(z[0], z[1], z[2], z[3]);
+    if (out) {
+      const uint4 r = z_round[base + i];
+      c += __popc(z[0] ^ r.x) + __popc(z[1] ^ r.y) + __popc(z[2] ^ r.z) + __popc(z[3] ^ r.w);
+    }
   }
-  s[threadIdx.x] = c;
+  if (!out) return;
+  for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
+  if (threadIdx.x % 32 == 0) warp_sum[threadIdx.x / 32] = c;
   __syncthreads();
-  for (int o = kReduceThreads / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
-    __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long t = 0;
+    for (int w = 0; w < kReduceThreads / 32; ++w) t += warp_sum[w];
+    if (t) atomicAdd(out + blockIdx.y, t);
   }
-  if (threadIdx.x == 0) atomicAdd(out + blockIdx.y, s[0]);
 }
 
 size_t up256(size_t x) { return (x + 255) / 256 * 256; }
@@ -148,7 +155,7 @@ litho_status litho_ai_inputs_workspace_size(const litho_kernels* h, int b, size_
     set_error("null argument or b < 1");
     return LITHO_EINVAL;
   }
-  *bytes = up256(ai_channels_bytes(h, b)) + up256(size_t(std::max(kReduceBlocks, b)) * sizeof(float2));
+  *bytes = up256(ai_channels_bytes(h, b)) + up256(2 * sizeof(uint2));
   return LITHO_OK;
 }
 
@@ -176,21 +183,27 @@ litho_status litho_ai_inputs(const litho_kernels* h, const float* target_dev, in
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t nn = size_t(h->n) * h->n;
-  float2* part = reinterpret_cast<float2*>(static_cast<char*>(workspace_dev) + up256(ai_channels_bytes(h, b)));
+  uint2* ext = reinterpret_cast<uint2*>(static_cast<char*>(workspace_dev) + up256(ai_channels_bytes(h, b)));
   {
     ProfScope ps(kStageIltForward, st, 1);
-    k_copy_channel<<<512, 256, 0, st>>>(target_dev, x_dev, b, nn, 0);
+    const bool vec = ((reinterpret_cast<uintptr_t>(target_dev) | reinterpret_cast<uintptr_t>(x_dev)) & 15) == 0;
+    if (vec)
+      k_copy_channel<<<dim3(blocks_per_clip(b, nn / 4), b), kReduceThreads, 0, st>>>(
+          reinterpret_cast<const float4*>(target_dev), reinterpret_cast<float4*>(x_dev), nn / 4);
+    else
+      k_copy_channel<<<dim3(blocks_per_clip(b, nn), b), kReduceThreads, 0, st>>>(target_dev, x_dev, nn);
     LITHO_TRY_CUDA(cudaGetLastError());
   }
   s = ai_channels(h, target_dev, b, dose, focus, (int(prec) & LITHO_GRID_COARSE) != 0, x_dev, workspace_dev, st);
   if (s != LITHO_OK) return s;
-  ProfScope ps(kStageIltReduce, st, 4);
-  const int per_clip = std::max(1, kReduceBlocks / b);  // partials per clip: at most kReduceBlocks in all
-  for (int ch = 1; ch <= 2; ++ch) {
-    k_minmax<<<dim3(per_clip, b), kReduceThreads, 0, st>>>(x_dev, b, nn, ch, part);
-    k_normalize<<<dim3(std::max(1, 1216 / b), b), kReduceThreads, 0, st>>>(x_dev, b, nn, ch, part, per_clip * b,
-                                                                          ch == 1 ? 0 : 1);
+  ProfScope ps(kStageIltReduce, st, 2);
+  for (int ch = 0; ch < 2; ++ch) {  // (~0, 0): nothing seen yet
+    LITHO_TRY_CUDA(cudaMemsetAsync(&ext[ch].x, 0xff, sizeof(unsigned), st));
+    LITHO_TRY_CUDA(cudaMemsetAsync(&ext[ch].y, 0, sizeof(unsigned), st));
   }
+  const dim3 grid(blocks_per_clip(2 * b, nn / 4), b, 2);
+  k_minmax<<<grid, kReduceThreads, 0, st>>>(reinterpret_cast<const float4*>(x_dev), nn / 4, ext);
+  k_normalize<<<grid, kReduceThreads, 0, st>>>(reinterpret_cast<float4*>(x_dev), nn / 4, ext);
   LITHO_TRY_CUDA(cudaGetLastError());
   return LITHO_OK;
 }
@@ -222,15 +235,15 @@ litho_status litho_print_images(const float* target_dev, const float* intensity_
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t nn = size_t(n) * n;
-  ProfScope ps(kStageResist, st, loss_dev ? 3 : 2);
+  ProfScope ps(kStageResist, st, 2);
   LITHO_TRY_CUDA(launch_resist(target_dev, b, n, taps, float(tau_round), blur_dev, z_round_dev, st));
-  k_threshold<<<1024, 256, 0, st>>>(intensity_dev, size_t(b) * nn, float(tau_print), z_print_dev);
-  if (loss_dev) {
-    LITHO_TRY_CUDA(cudaMemsetAsync(loss_dev, 0, size_t(b) * sizeof(int64_t), st));
-    k_l1_count<<<dim3(kL1Blocks, b), kReduceThreads, 0, st>>>(
-        reinterpret_cast<const uint4*>(z_print_dev), reinterpret_cast<const uint4*>(z_round_dev), nn / 16,
-        reinterpret_cast<unsigned long long*>(loss_dev));
-  }
+  if (loss_dev) LITHO_TRY_CUDA(cudaMemsetAsync(loss_dev, 0, size_t(b) * sizeof(int64_t), st));
+  const size_t pieces = nn / 16;
+  const dim3 grid(blocks_per_clip(b, pieces), b);
+  auto kern = (reinterpret_cast<uintptr_t>(intensity_dev) & 15) == 0 ? k_print<true> : k_print<false>;
+  kern<<<grid, kReduceThreads, 0, st>>>(intensity_dev, float(tau_print), reinterpret_cast<const uint4*>(z_round_dev),
+                                        pieces, reinterpret_cast<uint4*>(z_print_dev),
+                                        reinterpret_cast<unsigned long long*>(loss_dev));
   LITHO_TRY_CUDA(cudaGetLastError());
   return LITHO_OK;
 }

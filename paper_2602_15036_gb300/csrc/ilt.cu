@@ -395,13 +395,6 @@ __global__ void __launch_bounds__(Plan<N>::NT * AdjW<N>::W, AdjAccInSmem<N>::val
   }
 }
 
-// x[i][ch] = img[i] for the planes i of a group (x: [.][3][nn]).
-__global__ void k_to_channel(const float* __restrict__ img, float* __restrict__ x, int planes, size_t nn, int ch) {
-  const size_t total = size_t(planes) * nn;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x)
-    x[(i / nn) * 3 * nn + size_t(ch) * nn + i % nn] = img[i];
-}
-
 // The adjoint for dL/dI = 1 on every pixel (the AI input's gradient channel,
 // Eq. (9), and the intensity VJP without an upstream).  By Parseval,
 // sum_x |E_k(x)|^2 = N^2 sum_v |mhat(v) Phi_k(v)|^2, so the sum the adjoint
@@ -685,6 +678,9 @@ litho_status ai_channels(const litho_kernels* h, const float* target, int b, dou
   const int set = h->set_of[focus];
   const FieldSet fs = field_set(h, set, 1);
   const PlaneOut one = plane_out_identity(1);
+  PlaneOut channel1 = one;  // straight into x[.][1], a clip's second of three planes
+  channel1.out_planes = 3;
+  channel1.list[0] = 1;
   const float2* psi = h->d_psi + h->set_start[set] * (size_t(C) * C);
   const float scale = float(2.0 * dose / (double(N) * double(N)));
   // a 1024-point coarse grid: the warp-per-row stage 2 writes the coarse image's row spectra itself
@@ -695,15 +691,14 @@ litho_status ai_channels(const litho_kernels* h, const float* target, int b, dou
       ProfScope ps(kStageIltForward, st, coarse ? (rows2 ? 6 : 7) : 4);
       LITHO_TRY_CUDA(launch_mask_spectrum(target + c0 * nn, g, N, C, h->d_tw, L.rowbuf, L.mhat, st));
       LITHO_TRY_CUDA(launch_stage1_fft(L.mhat, psi, fs.fields(), NE, C, twe, L.t1, st, g));
-      LITHO_TRY_CUDA(launch_stage2_fft(L.t1, fs, g, NE, C, float(dose), twe, coarse ? L.ic : L.img, one, st,
-                                       h->d_tw32, h->d_tw512, rows2 ? L.mid : nullptr, C2));
+      float* dst = x + size_t(c0) * 3 * nn;
+      LITHO_TRY_CUDA(launch_stage2_fft(L.t1, fs, g, NE, C, float(dose), twe, coarse ? L.ic : dst,
+                                       coarse ? one : channel1, st, h->d_tw32, h->d_tw512, rows2 ? L.mid : nullptr, C2));
       if (coarse) {
         if (!rows2) LITHO_TRY_CUDA(launch_mask_rows(L.ic, g, NE, C2, twe, L.mid, st));
         LITHO_TRY_CUDA(launch_interp_cols(L.mid, g, NE, N, C2, twe, h->d_tw, nullptr, L.big, st));
-        LITHO_TRY_CUDA(launch_band_rows_real(L.big, g, 1, N, C2, 1.0f, h->d_tw, L.img, one, st));
+        LITHO_TRY_CUDA(launch_band_rows_real(L.big, g, 1, N, C2, 1.0f, h->d_tw, dst, channel1, st));
       }
-      k_to_channel<<<512, 256, 0, st>>>(L.img, x + size_t(c0) * 3 * nn, g, nn, 1);
-      LITHO_TRY_CUDA(cudaGetLastError());
     }
     {  // channel 2: the adjoint applied to dL/dI = 1, in closed form (k_ones_adjoint)
       ProfScope ps(kStageIltBackward, st, 3);
