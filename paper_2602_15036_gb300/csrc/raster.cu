@@ -12,9 +12,10 @@
 // reaches at most (ceil(S/16) + 5)^2 tiles; a larger or empty rectangle
 // marks its clip, whose mask is then written as NaN.  A pixel's value is
 // exact up to FP32 rounding: empty and fully covered pixels are recognised
-// directly; otherwise the pixel is swept in x
-// between consecutive piece edges, and in each slab the union length in y of
-// the pieces spanning it is measured by walking up through their intervals.
+// directly, pixels of one or two pieces measured in closed form; otherwise the
+// pixel is swept in x between consecutive piece edges, and in each slab the
+// union length in y of the pieces spanning it is measured by walking up
+// through their intervals.
 // The result does not depend on the order of a tile's list.
 #include <cstdint>
 
@@ -24,10 +25,10 @@ namespace litho {
 
 namespace {
 
-constexpr int kTile = 16, kTileThreads = kTile * kTile;
-// tile kernel: 64 threads, 4 pixels each, and a 256-piece cache (larger
-// lists are read from global memory), so that 32 tiles fit on an SM
-constexpr int kRastThreads = 64, kRastPix = kTile * kTile / kRastThreads, kTileCache = 256;
+constexpr int kTile = 16;
+constexpr int kScanThreads = 1024, kScanRun = 4;  // tiles a thread of the scan takes in a row
+// tile kernel: a warp per tile with a 64-piece cache (larger lists are read from global memory)
+constexpr int kRastWarps = 8, kTileCache = 64, kTilePix = kTile * kTile;
 
 // Pieces of rectangle r (x0, y0, x1, y1) after the shift into [0, n) and the
 // split at n; calls f(piece) for each nonempty one.
@@ -74,17 +75,24 @@ __global__ void k_rast_bin(const float4* __restrict__ rects, const long long* __
   });
 }
 
-// One CTA per clip: exclusive scan of its tile counts (cursor cleared).
-__global__ void __launch_bounds__(kTileThreads) k_rast_scan(const int* __restrict__ count, int tiles2, int* __restrict__ tile_start,
+// One CTA per clip: exclusive scan of its tile counts (cursor cleared), kScanRun tiles per thread and
+// round (256 threads with one tile each took 50 us for 64 clips of 16384 tiles: 64 rounds of two block
+// barriers; now 14).
+__global__ void __launch_bounds__(kScanThreads) k_rast_scan(const int* __restrict__ count, int tiles2, int* __restrict__ tile_start,
                                                             int* __restrict__ cursor, int* __restrict__ total) {
-  __shared__ int warp_sums[kTileThreads / 32];
+  __shared__ int warp_sums[kScanThreads / 32];
   const int c = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const size_t base = (size_t)c * tiles2;
   int run = 0;
-  for (int t0 = 0; t0 < tiles2; t0 += kTileThreads) {
-    const int t = t0 + threadIdx.x;
-    const int v = t < tiles2 ? count[base + t] : 0;
-    int x = v;
+  for (int t0 = 0; t0 < tiles2; t0 += kScanThreads * kScanRun) {
+    const int t = t0 + threadIdx.x * kScanRun;
+    int v[kScanRun], sum = 0;
+#pragma unroll
+    for (int k = 0; k < kScanRun; ++k) {
+      v[k] = t + k < tiles2 ? count[base + t + k] : 0;
+      sum += v[k];
+    }
+    int x = sum;
     for (int o = 1; o < 32; o <<= 1) {
       const int y = __shfl_up_sync(0xffffffffu, x, o);
       if (lane >= o) x += y;
@@ -92,19 +100,23 @@ __global__ void __launch_bounds__(kTileThreads) k_rast_scan(const int* __restric
     if (lane == 31) warp_sums[w] = x;
     __syncthreads();
     if (w == 0) {
-      int s = lane < kTileThreads / 32 ? warp_sums[lane] : 0;
+      int s = warp_sums[lane];
       for (int o = 1; o < 32; o <<= 1) {
         const int y = __shfl_up_sync(0xffffffffu, s, o);
         if (lane >= o) s += y;
       }
-      if (lane < kTileThreads / 32) warp_sums[lane] = s;
+      warp_sums[lane] = s;
     }
     __syncthreads();
-    if (t < tiles2) {
-      tile_start[base + t] = run + (w > 0 ? warp_sums[w - 1] : 0) + x - v;
-      cursor[base + t] = 0;
-    }
-    run += warp_sums[kTileThreads / 32 - 1];
+    int at = run + (w > 0 ? warp_sums[w - 1] : 0) + x - sum;
+#pragma unroll
+    for (int k = 0; k < kScanRun; ++k)
+      if (t + k < tiles2) {
+        tile_start[base + t + k] = at;
+        cursor[base + t + k] = 0;
+        at += v[k];
+      }
+    run += warp_sums[kScanThreads / 32 - 1];
     __syncthreads();
   }
   if (threadIdx.x == 0) total[c] = run;
@@ -118,19 +130,6 @@ __global__ void k_rast_base(const int* __restrict__ total, int b, long long* __r
     run += total[c];
   }
   clip_base[b] = run;
-}
-
-// 1 when one piece covers the unit pixel at (px, py), 0 when none reaches
-// into it, else -1 (a grey pixel: pixel_area measures it).
-__device__ __forceinline__ float pixel_class(const float4* pcs, int np, float px, float py) {
-  const float X1 = px + 1.f, Y1 = py + 1.f;
-  bool any = false;
-  for (int k = 0; k < np; ++k) {
-    const float4 p = pcs[k];
-    if (p.x <= px && p.z >= X1 && p.y <= py && p.w >= Y1) return 1.f;
-    any |= p.x < X1 && p.z > px && p.y < Y1 && p.w > py;
-  }
-  return any ? -1.f : 0.f;
 }
 
 // Union area of the pieces within the unit pixel at (px, py).
@@ -168,54 +167,125 @@ __device__ float pixel_area(const float4* pcs, int np, float px, float py) {
   return area;
 }
 
-__global__ void __launch_bounds__(kRastThreads) k_rast_tiles(const float4* __restrict__ list, const int* __restrict__ count,
-                                                             const int* __restrict__ tile_start,
-                                                             const long long* __restrict__ clip_base,
-                                                             const int* __restrict__ bad, int n,
-                                                             float* __restrict__ mask) {
-  __shared__ float4 cache[kTileCache];
-  __shared__ int grey[kTile * kTile];
-  __shared__ int n_grey;
-  const int tiles = n / kTile, c = blockIdx.y, t = blockIdx.x;
+// Area of a piece within the unit pixel at (px, py), which it reaches.
+__device__ __forceinline__ float overlap(const float4& p, float px, float py) {
+  return (fminf(p.z, px + 1.f) - fmaxf(p.x, px)) * (fminf(p.w, py + 1.f) - fmaxf(p.y, py));
+}
+
+// A warp per 16 x 16 tile.  A lane takes a column of 8 pixels: the rows a piece covers or reaches are
+// bit masks from its rounded edges, tested once per piece instead of once per pixel.  Pixels that no
+// piece reaches are 0, those that one covers 1; the grey ones are gathered, so that whole warps
+// measure them: one or two pieces in closed form (A + B - A B), the rest, pooled over the CTA's
+// tiles, by the sweep of pixel_area.  The tile is put together in shared memory and written by rows.
+// 64 clips of 2048^2, 18 k rectangles each:
+// 2062 -> 783 us (a CTA of 64 threads per tile that tested every pixel against every piece and
+// swept every grey pixel).
+template <bool VEC>
+__global__ void __launch_bounds__(32 * kRastWarps) k_rast_tiles(const float4* __restrict__ list,
+                                                                const int* __restrict__ count,
+                                                                const int* __restrict__ tile_start,
+                                                                const long long* __restrict__ clip_base,
+                                                                const int* __restrict__ bad, int n,
+                                                                float* __restrict__ mask) {
+  __shared__ float4 cache[kRastWarps][kTileCache];
+  __shared__ __align__(16) float value[kRastWarps][kTilePix];
+  __shared__ unsigned char grey[kRastWarps][kTilePix];
+  __shared__ unsigned short pool[kRastWarps * kTilePix];  // warp << 8 | pixel
+  __shared__ const float4* pieces[kRastWarps];
+  __shared__ int n_pieces[kRastWarps], n_pool;
+  const int tiles = n / kTile, c = blockIdx.y, lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int t0 = blockIdx.x * kRastWarps, t = t0 + wp;
+  const bool live = t < tiles * tiles;
   const size_t ti = (size_t)c * tiles * tiles + t;
-  const int ty = t / tiles, tx = t % tiles;
-  // pixel q = threadIdx.x + r * kRastThreads of the tile (row q / 16, column q % 16)
-  auto at = [&](int q) -> float* { return mask + ((size_t)c * n + ty * kTile + q / kTile) * n + tx * kTile + q % kTile; };
-  // the flag and the tile's list are fetched together (a flagged clip's
-  // counts are read but its list is not)
-  const int flagged = bad[c], np = count[ti];
-  const float4* pcs = list + clip_base[c] + tile_start[ti];
-  if (flagged) {  // uniform across the block
-#pragma unroll
-    for (int r = 0; r < kRastPix; ++r) *at(threadIdx.x + r * kRastThreads) = __int_as_float(0x7fc00000);
-    return;
-  }
-  if (threadIdx.x == 0) n_grey = 0;
+  const int flagged = bad[c], np = live && !flagged ? count[ti] : 0;
+  const float4* pcs = list + clip_base[c] + (np > 0 ? tile_start[ti] : 0);
+  if (threadIdx.x == 0) n_pool = 0;
+  const int ty = t / tiles, tx = t - ty * tiles;
+  const float bx = float(tx * kTile), by = float(ty * kTile);  // the tile's corner
   if (np <= kTileCache) {
-    for (int k = threadIdx.x; k < np; k += kRastThreads) cache[k] = pcs[k];
-    pcs = cache;
+    for (int k = lane; k < np; k += 32) cache[wp][k] = pcs[k];
+    pcs = cache[wp];
   }
-  __syncthreads();
-  // empty and fully covered pixels at once; the grey ones are gathered so
-  // that whole warps run their sweeps
-  const int lane = threadIdx.x & 31;
+  if (lane == 0) {
+    pieces[wp] = pcs;
+    n_pieces[wp] = np;
+  }
+  __syncthreads();  // n_pool and the caches
+  // rows 8 (lane / 16) ... + 7 of column lane % 16
+  const int col = lane % kTile, row0 = lane / kTile * 8;
+  const float px = bx + float(col), py0 = by + float(row0);
+  unsigned full = 0, touch = 0;
+  for (int k = 0; k < np; ++k) {
+    const float4 p = pcs[k];
+    // rows r with p.y <= y and p.w >= y + 1, and with p.y < y + 1 and p.w > y (y = py0 + r)
+    const int f0 = max(0, int(ceilf(p.y - py0))), f1 = min(8, int(floorf(p.w - py0)));
+    const int g0 = max(0, int(floorf(p.y - py0))), g1 = min(8, int(ceilf(p.w - py0)));
+    const unsigned mf = f1 > f0 ? (1u << f1) - (1u << f0) : 0u, mg = g1 > g0 ? (1u << g1) - (1u << g0) : 0u;
+    if (p.x <= px && p.z >= px + 1.f) full |= mf;
+    if (p.x < px + 1.f && p.z > px) touch |= mg;
+  }
+  const unsigned g = touch & ~full;
 #pragma unroll
-  for (int r = 0; r < kRastPix; ++r) {
-    const int q = threadIdx.x + r * kRastThreads;
-    const float cls = pixel_class(pcs, np, float(tx * kTile + q % kTile), float(ty * kTile + q / kTile));
-    const unsigned m = __ballot_sync(0xffffffffu, cls < 0.f);
-    int slot = 0;
-    if (lane == 0 && m) slot = atomicAdd(&n_grey, __popc(m));
-    slot = __shfl_sync(0xffffffffu, slot, 0) + __popc(m & ((1u << lane) - 1u));
-    if (cls < 0.f)
-      grey[slot] = q;
-    else
-      *at(q) = cls;
+  for (int r = 0; r < 8; ++r) value[wp][(row0 + r) * kTile + col] = full >> r & 1u ? 1.f : 0.f;
+  int x = __popc(g);  // inclusive warp scan of the grey counts
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  const int n_grey = __shfl_sync(0xffffffffu, x, 31);
+  int at = x - __popc(g);
+  for (unsigned m = g; m; m &= m - 1) grey[wp][at++] = (unsigned char)((row0 + __ffs(m) - 1) * kTile + col);
+  __syncwarp();
+  for (int i = lane; i < n_grey; i += 32) {
+    const int q = grey[wp][i];
+    const float qx = bx + float(q % kTile), qy = by + float(q / kTile);
+    int hits = 0;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+    for (int k = 0; k < np; ++k) {
+      const float4 p = pcs[k];
+      if (p.x < qx + 1.f && p.z > qx && p.y < qy + 1.f && p.w > qy) {
+        if (hits == 0)
+          a = p;
+        else
+          b = p;
+        ++hits;
+      }
+    }
+    if (hits <= 2) {
+      float area = overlap(a, qx, qy);
+      if (hits == 2) {
+        area += overlap(b, qx, qy);
+        const float4 i2 = make_float4(fmaxf(a.x, b.x), fmaxf(a.y, b.y), fminf(a.z, b.z), fminf(a.w, b.w));
+        const float w = fminf(i2.z, qx + 1.f) - fmaxf(i2.x, qx), h = fminf(i2.w, qy + 1.f) - fmaxf(i2.y, qy);
+        if (w > 0.f && h > 0.f) area -= w * h;
+      }
+      value[wp][q] = area;
+    } else {
+      pool[atomicAdd(&n_pool, 1)] = (unsigned short)(wp << 8 | q);
+    }
   }
   __syncthreads();
-  for (int g = threadIdx.x; g < n_grey; g += kRastThreads) {
-    const int q = grey[g];
-    *at(q) = pixel_area(pcs, np, float(tx * kTile + q % kTile), float(ty * kTile + q / kTile));
+  for (int i = threadIdx.x; i < n_pool; i += blockDim.x) {
+    const int w = pool[i] >> 8, q = pool[i] & 255, tt = t0 + w, wy = tt / tiles, wx = tt - wy * tiles;
+    value[w][q] = pixel_area(pieces[w], n_pieces[w], float(wx * kTile + q % kTile), float(wy * kTile + q / kTile));
+  }
+  __syncthreads();
+  if (!live) return;
+  float* dst = mask + ((size_t)c * n + ty * kTile) * n + tx * kTile;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {  // four pixels of row 8 k + lane / 4
+    const int row = 8 * k + lane / 4, cx = lane % 4 * 4;
+    float4 v = *reinterpret_cast<const float4*>(&value[wp][row * kTile + cx]);
+    if (flagged) v.x = v.y = v.z = v.w = __int_as_float(0x7fc00000);
+    float* o = dst + (size_t)row * n + cx;
+    if constexpr (VEC) {
+      *reinterpret_cast<float4*>(o) = v;
+    } else {
+      o[0] = v.x;
+      o[1] = v.y;
+      o[2] = v.z;
+      o[3] = v.w;
+    }
   }
 }
 
@@ -278,15 +348,16 @@ cudaError_t launch_raster(const float4* rects, const long long* rect_start, int 
     k_rast_bin<false><<<grid, 256, 0, st>>>(rects, rect_start, n, max_rects, float(max_side), L.count, nullptr, nullptr,
                                             nullptr, nullptr, L.bad);
   }
-  k_rast_scan<<<b, kTileThreads, 0, st>>>(L.count, int(tiles2), L.tile_start, L.cursor, L.total);
+  k_rast_scan<<<b, kScanThreads, 0, st>>>(L.count, int(tiles2), L.tile_start, L.cursor, L.total);
   k_rast_base<<<1, 1, 0, st>>>(L.total, b, L.clip_base);
   if (max_rects > 0) {
     const dim3 grid(unsigned((max_rects + 255) / 256), b);
     k_rast_bin<true><<<grid, 256, 0, st>>>(rects, rect_start, n, max_rects, float(max_side), L.count, L.tile_start,
                                            L.clip_base, L.cursor, L.list, L.bad);
   }
-  k_rast_tiles<<<dim3(unsigned(tiles2), b), kRastThreads, 0, st>>>(L.list, L.count, L.tile_start, L.clip_base, L.bad,
-                                                                   n, mask);
+  auto kern = (reinterpret_cast<uintptr_t>(mask) & 15) == 0 ? k_rast_tiles<true> : k_rast_tiles<false>;
+  kern<<<dim3(unsigned((tiles2 + kRastWarps - 1) / kRastWarps), b), 32 * kRastWarps, 0, st>>>(
+      L.list, L.count, L.tile_start, L.clip_base, L.bad, n, mask);
   return cudaGetLastError();
 }
 
