@@ -353,7 +353,7 @@ litho_status litho_rasterize(const float* rects_dev, const int64_t* rect_start_d
  * the total; segments at or beyond `capacity` are counted but not written,
  * so a caller that sees total > capacity calls again with more room.
  * Workspace: litho_contours_workspace_size bytes, 256-byte aligned; seg_dev
- * 16-byte aligned.  Asynchronous on `stream` (four launches).  Errors:
+ * 16-byte aligned.  Asynchronous on `stream` (five launches).  Errors:
  * EINVAL, ENOMEM (workspace too small), ECUDA. */
 litho_status litho_contours_workspace_size(int planes, int n, size_t* bytes);
 litho_status litho_contours(const float* iblur_dev, int planes, int n, double threshold, float* seg_dev,
