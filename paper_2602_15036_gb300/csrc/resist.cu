@@ -12,7 +12,7 @@
 // over the taps in the same order as the loop version (k_resist_any, larger
 // radii), so a pixel's value does not depend on the tile.  Bound by the FMA
 // pipe for R = 10 (2 (2R + 1) FMAs a pixel), by HBM for small radii.
-// Measured: 16 planes of 2048^2, R = 10, 503 -> 218 us; 24 planes, R = 5, 471 -> 192 us
+// Measured: 16 planes of 2048^2, R = 10, 503 -> 168 us; 24 planes, R = 5, 471 -> 192 us
 // (32 x 128 strips that loaded 2R + 1 shared values per pixel and row).
 #include <cmath>
 
@@ -26,8 +26,8 @@ constexpr int kThreads = 256;
 
 // ALIGNED: 16-byte loads and paired stores; n a multiple of TW and SH.
 template <int R, int TW, int SH, bool ALIGNED>
-__global__ void __launch_bounds__(kThreads) k_resist(const float* __restrict__ img, int n,
-                                                     const __grid_constant__ ResistTaps taps, float thr,
+__global__ void __launch_bounds__(kThreads, R > 10 ? 2 : 3) k_resist(const float* __restrict__ img, int n,
+                                                        const __grid_constant__ ResistTaps taps, float thr,
                                                      float* __restrict__ iblur, uint8_t* __restrict__ printed) {
   constexpr int ROWS = SH + 2 * R, SEG = TW / 8, HR = (R + 3) / 4 * 4, WIN = 8 + 2 * HR;
   constexpr int PAIRS = TW / 2, GROUPS = kThreads / PAIRS, PER = SH / GROUPS;
@@ -71,26 +71,30 @@ __global__ void __launch_bounds__(kThreads) k_resist(const float* __restrict__ i
   }
   __syncthreads();
   // columns: rows y0 + grp PER ... of columns x0 + 2 cp, x0 + 2 cp + 1
-  const int cp = threadIdx.x % PAIRS, yy = (threadIdx.x / PAIRS) * PER;
-  float2 win[PER + 2 * R];
+  const int cp = threadIdx.x % PAIRS;
+  constexpr int STEP = R > 6 && PER > 8 ? 8 : PER;  // rows per window: three CTAs per SM without spills
+#pragma unroll 1
+  for (int yy = (threadIdx.x / PAIRS) * PER, y1 = yy + PER; yy < y1; yy += STEP) {
+    float2 win[STEP + 2 * R];
 #pragma unroll
-  for (int j = 0; j < PER + 2 * R; ++j) win[j] = *reinterpret_cast<const float2*>(hb + (yy + j) * TW + 2 * cp);
+    for (int j = 0; j < STEP + 2 * R; ++j) win[j] = *reinterpret_cast<const float2*>(hb + (yy + j) * TW + 2 * cp);
 #pragma unroll
-  for (int i = 0; i < PER; ++i) {
-    float2 acc = make_float2(0.f, 0.f);
+    for (int i = 0; i < STEP; ++i) {
+      float2 acc = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int a = -R; a <= R; ++a) acc = __ffma2_rn(make_float2(taps.g[a + R], taps.g[a + R]), win[i + R - a], acc);
-    const size_t o = plane + (size_t)(y0 + yy + i) * n + x0 + 2 * cp;
-    const uint8_t pa = acc.x >= thr ? 1 : 0, pb = acc.y >= thr ? 1 : 0;
-    if constexpr (ALIGNED) {
-      *reinterpret_cast<float2*>(iblur + o) = acc;
-      if (printed) *reinterpret_cast<uchar2*>(printed + o) = make_uchar2(pa, pb);
-    } else {
-      iblur[o] = acc.x;
-      iblur[o + 1] = acc.y;
-      if (printed) {
-        printed[o] = pa;
-        printed[o + 1] = pb;
+      for (int a = -R; a <= R; ++a) acc = __ffma2_rn(make_float2(taps.g[a + R], taps.g[a + R]), win[i + R - a], acc);
+      const size_t o = plane + (size_t)(y0 + yy + i) * n + x0 + 2 * cp;
+      const uint8_t pa = acc.x >= thr ? 1 : 0, pb = acc.y >= thr ? 1 : 0;
+      if constexpr (ALIGNED) {
+        *reinterpret_cast<float2*>(iblur + o) = acc;
+        if (printed) *reinterpret_cast<uchar2*>(printed + o) = make_uchar2(pa, pb);
+      } else {
+        iblur[o] = acc.x;
+        iblur[o + 1] = acc.y;
+        if (printed) {
+          printed[o] = pa;
+          printed[o + 1] = pb;
+        }
       }
     }
   }
