@@ -397,19 +397,24 @@ static litho_status upsample(const litho_kernels* h, litho_precision p, const Ae
   const float2* twc = coarse_tw(h, p);
   const float* gain = fr ? L.gain : nullptr;
   ProfScope ps(fr ? kStageUpsampleResist : kStageUpsample, st, rows_done ? 2 : 3);
+  const int C = h->crop;  // half of the image's band
+  if (!rows_done) LITHO_TRY_CUDA(launch_mask_rows(L.ic, planes, NC, C2, twc, L.rowbuf2, false, st));
   if (interp_cols_supported(NC, N)) {
-    if (!rows_done) LITHO_TRY_CUDA(launch_mask_rows(L.ic, planes, NC, C2, twc, L.rowbuf2, st));
-    LITHO_TRY_CUDA(launch_interp_cols(L.rowbuf2, planes, NC, N, C2, twc, h->d_tw, gain, L.q, st));
+    LITHO_TRY_CUDA(launch_interp_cols(L.rowbuf2, planes, NC, N, C, twc, h->d_tw, gain, true, L.q, st));
   } else {
-    LITHO_TRY_CUDA(launch_mask_spectrum(L.ic, planes, NC, C2, twc, L.rowbuf2, L.spec, st, gain));
-    LITHO_TRY_CUDA(launch_stage1_fft(L.spec, nullptr, planes, N, C2, h->d_tw, L.q, st));
+    LITHO_TRY_CUDA(launch_mask_cols(L.rowbuf2, planes, NC, C2, twc, L.spec, nullptr, false, st));
+    LITHO_TRY_CUDA(launch_stage1_half(L.spec, planes, N, C2, h->d_tw, L.q, gain ? C2 : C, st));
+    if (gain) {
+      LITHO_TRY_CUDA(launch_mask_cols(L.rowbuf2, planes, NC, C2, twc, L.spec, gain, false, st));
+      LITHO_TRY_CUDA(launch_stage1_half(L.spec, planes, N, C2, h->d_tw, L.q + C, C2, st));
+    }
   }
   if (!fr) {
-    LITHO_TRY_CUDA(launch_band_rows_real(L.q, clips, h->n_sets, N, C2, 1.0f, h->d_tw, out, po, st));
+    LITHO_TRY_CUDA(launch_band_rows_real(L.q, clips, h->n_sets, N, C, 1.0f, h->d_tw, out, po, st));
     return LITHO_OK;
   }
   const size_t nn = size_t(N) * N;
-  LITHO_TRY_CUDA(launch_band_rows_resist(L.q, clips, h->n_sets, N, C2, h->d_tw, fr->threshold, out, fr->iblur + p0 * nn,
+  LITHO_TRY_CUDA(launch_band_rows_resist(L.q, clips, h->n_sets, N, C, h->d_tw, fr->threshold, out, fr->iblur + p0 * nn,
                                          fr->printed ? fr->printed + p0 * nn : nullptr, po, st));
   return LITHO_OK;
 }
@@ -813,7 +818,7 @@ litho_status litho_contours(const float* iblur_dev, int planes, int n, double th
     return LITHO_ENOMEM;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  ProfScope ps(kStageContours, st, 4);
+  ProfScope ps(kStageContours, st, 5);
   LITHO_TRY_CUDA(launch_contours(iblur_dev, planes, n, float(threshold), reinterpret_cast<float4*>(seg_dev), cell_dev,
                                  capacity, reinterpret_cast<long long*>(plane_start_dev), workspace_dev, st));
   return LITHO_OK;

@@ -24,17 +24,25 @@ namespace {
 
 __device__ __forceinline__ int freq_of(int idx, int n) { return idx < n / 2 ? idx : idx - n; }
 
+// Spectra of real planes are kept for u >= 0 only ("half"): S(-v, -u) = conj S(v, u), so the column
+// transforms run on half the columns.  A half row holds k = u in [0, crop/2); the mask spectrum, whose
+// crop has u = -crop/2 but not u = crop/2, keeps k = crop/2 as well (stride crop/2 + 8).
+
 // ---- mask spectrum, pass 1: two real rows per complex transform ----------------------------
-// z = m[y0] + i m[y1]; Z = DFT(z); X(u) = (Z(u) + conj Z(-u))/2, Y(u) = (Z(u) - conj Z(-u))/(2i).
+// z = m[y0] + i m[y1]; Z = DFT(z); X(u) = (Z(u) + conj Z(-u))/2, Y(u) = (Z(u) - conj Z(-u))/(2i),
+// written for u in [0, cols) with row stride ld.
 template <int N>
 __global__ void __launch_bounds__(Plan<N>::NT) k_mask_rows(const float* __restrict__ m, int crop,
                                                             const float2* __restrict__ tw_g,
-                                                            float2* __restrict__ rowbuf, int pairs_per_cta) {
+                                                            float2* __restrict__ rowbuf, int cols, int ld,
+                                                            int pairs_per_cta) {
   extern __shared__ float2 smem[];
   float2* tw = smem;
   float2* buf = smem + N;
   float2* zc = smem + N + PadLen<N>::value;  // Z(u) for u in [-C/2, C/2], index u + C/2 (crop + 1 <= N + 1 entries)
+  pdl_start();
   load_twiddles<N>(tw, tw_g);
+  pdl_wait(m);
   __syncthreads();
   const int b = blockIdx.y, t = threadIdx.x, half = crop / 2;
   constexpr int R0 = Plan<N>::R[0], NB0 = N / R0;
@@ -45,7 +53,7 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_mask_rows(const float* __restri
     const float* r0 = m + ((size_t)b * N + 2 * pr) * N;
 #pragma unroll
     for (int r = 0; r < R0; ++r)
-      nxt[r] = t < NB0 ? make_float2(__ldg(r0 + t + r * NB0), __ldg(r0 + N + t + r * NB0)) : make_float2(0.f, 0.f);
+      nxt[r] = t < NB0 ? make_float2(ld_dep(r0 + t + r * NB0), ld_dep(r0 + N + t + r * NB0)) : make_float2(0.f, 0.f);
   };
   const int pr0 = blockIdx.x * pairs_per_cta, pr1 = min(N / 2, (blockIdx.x + 1) * pairs_per_cta);
   if (pr0 < pr1) prefetch(pr0);
@@ -68,55 +76,60 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_mask_rows(const float* __restri
     };
     fft_load_use<N, -1, decltype(load), decltype(use), false>(buf, tw, t, load, use, after_first);
     __syncthreads();
-    float2* o0 = rowbuf + ((size_t)b * N + y0) * crop;
-    float2* o1 = o0 + crop;
-    for (int c = t; c < crop; c += blockDim.x) {
-      const float2 zp = zc[c], zm = zc[crop - c];
-      o0[c] = make_float2(0.5f * (zp.x + zm.x), 0.5f * (zp.y - zm.y));
-      o1[c] = make_float2(0.5f * (zp.y + zm.y), -0.5f * (zp.x - zm.x));
+    float2* o0 = rowbuf + ((size_t)b * N + y0) * ld;
+    float2* o1 = o0 + ld;
+    for (int k = t; k < cols; k += blockDim.x) {
+      const float2 zp = zc[half + k], zm = zc[half - k];
+      o0[k] = make_float2(0.5f * (zp.x + zm.x), 0.5f * (zp.y - zm.y));
+      o1[k] = make_float2(0.5f * (zp.y + zm.y), -0.5f * (zp.x - zm.x));
     }
   }
 }
 
 
-// ---- mask spectrum, pass 2: column DFTs of the crop columns, crop rows kept ------------------
-// With `gain` (per crop index, real and even in the frequency), the stored
-// value is S (1 + i gain[v] gain[u]): an image whose spectrum is S comes out
-// of the inverse transform as I + i (g (x) I) for the separable filter with
-// transfer function gain (x) gain, because both I and g (x) I are real.
-template <int N>
-__global__ void __launch_bounds__(Plan<N>::NT * ColW<N>::W) k_mask_cols(const float2* __restrict__ rowbuf, int crop,
-                                                                         const float2* __restrict__ tw_g,
-                                                                         const float* __restrict__ gain,
-                                                                         float2* __restrict__ mhat, int gain_real) {
-  constexpr int W = ColW<N>::W, NT = Plan<N>::NT, LD = ColLD<N>::value;
+// ---- mask spectrum, pass 2: column DFTs of the columns u >= 0, crop rows kept ------------------
+// Columns u = k for k in [0, cols) of half rows with stride ld.  MIRROR (the mask spectrum on its whole
+// crop): a column u also gives the column -u, S(-v, -u) = conj S(v, u).  Without it only the columns
+// u >= 0 are written (index u + crop/2), times gain[v] gain[u] when gain is given: the spectrum of the
+// plane's blur, |v| < crop/2.  W columns per CTA with the lanes interleaved over them: the first pass reads from global
+// memory and the last one writes there, 8 W bytes of a row at a time, with no copy through shared memory.
+// 64 masks of 2048^2: 330 -> 182 us (every column transformed, and staged in shared memory).
+template <int N, int W, bool MIRROR>
+__global__ void __launch_bounds__(Plan<N>::NT * W) k_mask_cols(const float2* __restrict__ rowbuf, int crop, int cols,
+                                                               int ld, const float2* __restrict__ tw_g,
+                                                               const float* __restrict__ gain,
+                                                               float2* __restrict__ mhat) {
+  constexpr int NT = Plan<N>::NT, LD = (PadLen<N>::value + 15) / 16 * 16 + 16 / W;
   extern __shared__ float2 smem[];
   float2* tw = smem;
   float2* buf = smem + N;
+  pdl_start();
   load_twiddles<N>(tw, tw_g);
-  const int b = blockIdx.y, u0 = blockIdx.x * W, tid = threadIdx.x;
-  const float2* src = rowbuf + (size_t)b * N * crop + u0;
-  for (int i = tid; i < N * W; i += blockDim.x) {
-    const int y = i / W, w = i % W;
-    buf[w * LD + pad16(y)] = src[(size_t)y * crop + w];
-  }
+  pdl_wait(rowbuf, gain);
   __syncthreads();
-  fft_smem<N, -1>(buf + (tid / NT) * LD, tw, tid % NT);
+  const int b = blockIdx.y, tid = threadIdx.x, g = tid % W, t = tid / W, k = blockIdx.x * W + g, half = crop / 2;
+  const bool live = k < cols;
+  const float2* src = rowbuf + (size_t)b * N * ld + k;
+  auto load = [&](int, int, int y) { return live ? ld_dep(src + (size_t)y * ld) : make_float2(0.f, 0.f); };
   const float scale = 1.0f / (float(N) * float(N));
-  float2* dst = mhat + (size_t)b * crop * crop + u0;
-  const int half = crop / 2;
-  for (int i = tid; i < crop * W; i += blockDim.x) {
-    const int cv = i / W, w = i % W;
-    const int idx = (cv - half + N) % N;
-    float2 v = buf[w * LD + pad16(idx)];
-    v = make_float2(v.x * scale, v.y * scale);
-    if (gain) {
-      const float g = __ldg(gain + cv) * __ldg(gain + u0 + w);
-      v = gain_real ? make_float2(g * v.x, g * v.y)  // the blurred plane's spectrum
-                    : make_float2(fmaf(-g, v.y, v.x), fmaf(g, v.x, v.y));  // the plane + i its blur
+  const float gu = gain && live ? scale * ld_dep(gain + half + k) : scale;
+  float2* dst = mhat + (size_t)b * crop * crop;
+  auto use = [&](int, int, int idx, float2 v) {
+    const int f = freq_of(idx, N), cv = half + f, cm = half - f;
+    if (!live) return;
+    if (MIRROR) {
+      v = make_float2(v.x * scale, v.y * scale);
+      if (k < half && cv >= 0 && cv < crop) dst[(size_t)cv * crop + half + k] = v;
+      if (k > 0 && cm >= 0 && cm < crop) dst[(size_t)cm * crop + half - k] = make_float2(v.x, -v.y);
+      // crop == N: v = -N/2 is its own mirror
+      if (k > 0 && f == -N / 2 && crop == N) dst[half - k] = make_float2(v.x, -v.y);
+    } else if (cv >= 0 && cv < crop) {
+      // v = -crop/2 has no mirror on the crop: without it the plane stays real (no consumer reads it)
+      const float s = cv == 0 ? 0.f : gain ? gu * ld_dep(gain + cv) : gu;
+      dst[(size_t)cv * crop + half + k] = make_float2(s * v.x, s * v.y);
     }
-    dst[(size_t)cv * crop + w] = v;
-  }
+  };
+  fft_load_use<N, -1, decltype(load), decltype(use), false>(buf + g * LD, tw, t, load, use);
 }
 
 // Transfer function of the periodic separable blur on an n-point grid:
@@ -125,6 +138,8 @@ __global__ void __launch_bounds__(Plan<N>::NT * ColW<N>::W) k_mask_cols(const fl
 // exactly in integers before cospi.
 __global__ void k_blur_gain(ResistTaps taps, int n, int crop, float* __restrict__ gain) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_start();
+  pdl_wait();
   if (i >= crop) return;
   const int f = i - crop / 2, r = taps.radius;
   float acc = taps.g[r];
@@ -140,7 +155,21 @@ struct OutC64 {
   static constexpr bool kRowWise = false;
   float2* t1;
   int n, crop;
+  __device__ __forceinline__ int first() const { return 0; }  // first crop column, and the rows' stride
+  __device__ __forceinline__ int ld(int c) const { return c; }
   __device__ __forceinline__ float2* column(int j, int c) const { return t1 + (size_t)j * n * crop + c; }
+  template <int W>
+  __device__ void store_row(int, int, int, const float2 (&)[W]) const {}
+};
+
+// The columns u >= 0 alone, as half rows of stride `stride` (any spectra, no kernels).
+struct OutHalf {
+  static constexpr bool kRowWise = false;
+  float2* q;
+  int n, half, stride;
+  __device__ __forceinline__ int first() const { return half; }
+  __device__ __forceinline__ int ld(int) const { return stride; }
+  __device__ __forceinline__ float2* column(int j, int c) const { return q + (size_t)j * n * stride + (c - half); }
   template <int W>
   __device__ void store_row(int, int, int, const float2 (&)[W]) const {}
 };
@@ -156,7 +185,9 @@ __global__ void __launch_bounds__(Plan<N>::NT, 512 / Plan<N>::NT) k_stage2(const
   constexpr int PERL = PassShape<N, NT, RL>::PER;
   __shared__ float2 buf[PadLen<N>::value];
   __shared__ float2 tw[N];
+  pdl_start();
   load_twiddles<N>(tw, tw_g);
+  pdl_wait(t1);
   __syncthreads();
   const int y = blockIdx.x, plane = blockIdx.y, t = threadIdx.x, half = crop / 2;
   const int clip = plane / fs.planes, pl = plane - clip * fs.planes, nk = fs.start[pl + 1] - fs.start[pl];
@@ -176,7 +207,7 @@ __global__ void __launch_bounds__(Plan<N>::NT, 512 / Plan<N>::NT) k_stage2(const
     const float2* row = base + (size_t)j * N * crop;
     auto load = [&](int, int r, int idx) {
       const int c = (r < PL::R[0] / 2 ? idx : idx - N) + half;  // first pass: idx < N/2 exactly when r < R/2
-      return (c >= 0 && c < crop) ? __ldg(row + c) : make_float2(0.f, 0.f);
+      return (c >= 0 && c < crop) ? ld_dep(row + c) : make_float2(0.f, 0.f);
     };
     auto use = [&](int p, int q, int, float2 v) { acc[p][q] = fmaf(v.x, v.x, fmaf(v.y, v.y, acc[p][q])); };
     if constexpr (kMid)
@@ -197,82 +228,76 @@ __global__ void __launch_bounds__(Plan<N>::NT, 512 / Plan<N>::NT) k_stage2(const
   }
 }
 
-// ---- band rows to real image rows: out[p][y][x] = scale Re(sum_c q[p][y][c] e^{2 pi i u_c x/N}) ----------
-// Second half of the exact Fourier interpolation from the coarse grid.
-template <int N, bool BANDED>
-__global__ void __launch_bounds__(Plan<N>::NT) k_band_rows_real(const float2* __restrict__ q, int crop, float scale,
-                                                                const float2* __restrict__ tw_g,
-                                                                float* __restrict__ out, int planes,
-                                                                const __grid_constant__ PlaneOut po,
-                                                                int rows_per_cta) {
-  __shared__ float2 buf[PadLen<N>::value];
-  __shared__ float2 tw[N];
-  load_twiddles<N>(tw, tw_g);
-  __syncthreads();
-  const int p = blockIdx.y, half = crop / 2, clip = p / planes, pl = p - clip * planes;
-  const int d0 = po.first[pl], d1 = po.first[pl + 1];
-  const size_t p0 = (size_t)(clip * po.out_planes + po.list[d0]) * N;  // rows before the first output plane
-  for (int y = blockIdx.x * rows_per_cta; y < min(N, (blockIdx.x + 1) * rows_per_cta); ++y) {
-    const float2* row = q + ((size_t)p * N + y) * crop;
-    auto load = [&](int, int r, int idx) {
-      const int c = (r < Plan<N>::R[0] / 2 ? idx : idx - N) + half;  // first pass: idx < N/2 exactly when r < R/2
-      return (c >= 0 && c < crop) ? __ldg(row + c) : make_float2(0.f, 0.f);
-    };
-    float* o = out + (p0 + y) * N;
-    auto use = [&](int, int, int x, float2 v) {
-      o[x] = scale * v.x;
-      for (int d = d0 + 1; d < d1; ++d) o[(po.list[d] - po.list[d0]) * (N * N) + x] = scale * v.x;
-    };
-    fft_load_use<N, +1, decltype(load), decltype(use), BANDED>(buf, tw, threadIdx.x, load, use);
-  }
+// ---- band rows to image rows: the inverse transform along x ----------------------------------------------
+// Second half of the exact Fourier interpolation from the coarse grid, from half rows: with the spectra
+// A(u) and B(u) of two real rows, one transform of A + i B (A(-u) = conj A(u)) gives both as its real and
+// imaginary parts.
+
+// Element u of A + i B from the half rows a, b of `h` columns.
+__device__ __forceinline__ float2 two_rows(const float2* __restrict__ a, const float2* __restrict__ b, int h, int u) {
+  const int k = u < 0 ? -u : u;
+  if (k >= h) return make_float2(0.f, 0.f);
+  const float2 x = ld_dep(a + k), y = ld_dep(b + k);
+  return u < 0 ? make_float2(x.x + y.y, y.x - x.y) : make_float2(x.x - y.y, x.y + y.x);
 }
 
-// Same transform for band rows carrying S (1 + i gain (x) gain) (see
-// k_mask_cols): the real part is the image, the imaginary part its blur, and
-// printed = [blur >= threshold].  `img` may be NULL (not written).
-template <int N, bool BANDED>
-__global__ void __launch_bounds__(Plan<N>::NT) k_band_rows_resist(const float2* __restrict__ q, int crop,
-                                                                  const float2* __restrict__ tw_g, float thr,
-                                                                  float* __restrict__ img, float* __restrict__ iblur,
-                                                                  uint8_t* __restrict__ printed, int planes,
-                                                                  const __grid_constant__ PlaneOut po,
-                                                                  int rows_per_cta) {
+// Band rows q of h columns two by two (unit i: rows 2 i and 2 i + 1 of q).  RESIST: the two are a row's image
+// and its blur: img = Re (skipped when NULL), iblur = Im, printed = [Im >= threshold] (skipped when NULL).
+// Otherwise they are two rows of the image: img rows 2 i and 2 i + 1, times scale.  Plane p of `planes`
+// per clip goes to its planes of `po`.  Bound by HBM (the rows written).
+template <int N, bool BANDED, bool RESIST>
+__global__ void __launch_bounds__(Plan<N>::NT) k_band_rows(const float2* __restrict__ q, int h, float scale,
+                                                           const float2* __restrict__ tw_g, float thr,
+                                                           float* __restrict__ img, float* __restrict__ iblur,
+                                                           uint8_t* __restrict__ printed, int planes,
+                                                           const __grid_constant__ PlaneOut po, int units_per_cta) {
+  constexpr int NT = Plan<N>::NT, RL = Plan<N>::R[Plan<N>::P - 1], PERL = PassShape<N, NT, RL>::PER;
+  constexpr int UNITS = RESIST ? N : N / 2;
   __shared__ float2 buf[PadLen<N>::value];
   __shared__ float2 tw[N];
+  pdl_start();
   load_twiddles<N>(tw, tw_g);
+  pdl_wait(q);
   __syncthreads();
-  const int p = blockIdx.y, half = crop / 2, clip = p / planes, pl = p - clip * planes;
+  const int p = blockIdx.y, t = threadIdx.x, clip = p / planes, pl = p - clip * planes;
   const int d0 = po.first[pl], d1 = po.first[pl + 1];
-  const size_t p0 = (size_t)(clip * po.out_planes + po.list[d0]) * N;  // rows before the first output plane
-  for (int y = blockIdx.x * rows_per_cta; y < min(N, (blockIdx.x + 1) * rows_per_cta); ++y) {
-    const float2* row = q + ((size_t)p * N + y) * crop;
-    auto load = [&](int, int r, int idx) {
-      const int c = (r < Plan<N>::R[0] / 2 ? idx : idx - N) + half;  // first pass: idx < N/2 exactly when r < R/2
-      return (c >= 0 && c < crop) ? __ldg(row + c) : make_float2(0.f, 0.f);
+  for (int i = blockIdx.x * units_per_cta; i < min(UNITS, (blockIdx.x + 1) * units_per_cta); ++i) {
+    const float2* row = q + ((size_t)p * UNITS + i) * 2 * h;
+    auto load = [&](int, int r, int idx) {  // first pass: idx < N/2 exactly when r < R/2
+      return two_rows(row, row + h, h, r < Plan<N>::R[0] / 2 ? idx : idx - N);
     };
-    const size_t o = (p0 + y) * N;
-    auto put = [&](size_t at, float2 v) {
-      if (img) img[at] = v.x;
-      iblur[at] = v.y;
-      if (printed) printed[at] = v.y >= thr ? 1 : 0;
-    };
-    auto use = [&](int, int, int x, float2 v) {
-      put(o + x, v);
-      for (int d = d0 + 1; d < d1; ++d) put(o + (po.list[d] - po.list[d0]) * (N * N) + x, v);
-    };
-    fft_load_use<N, +1, decltype(load), decltype(use), BANDED>(buf, tw, threadIdx.x, load, use);
+    float2 res[PERL][RL];
+    auto use = [&](int pp, int qq, int, float2 v) { res[pp][qq] = v; };
+    fft_load_use<N, +1, decltype(load), decltype(use), BANDED>(buf, tw, t, load, use);
+    for (int d = d0; d < d1; ++d) {
+      const size_t o = ((size_t)(clip * po.out_planes + po.list[d]) * N + (RESIST ? i : 2 * i)) * N + t;
+#pragma unroll
+      for (int pp = 0; pp < PERL; ++pp)
+        if (t + pp * NT < N / RL) {
+#pragma unroll
+          for (int qq = 0; qq < RL; ++qq) {
+            const size_t at = o + pp * NT + qq * (N / RL);
+            if (RESIST) {
+              if (img) img[at] = res[pp][qq].x;
+              iblur[at] = res[pp][qq].y;
+              if (printed) printed[at] = res[pp][qq].y >= thr ? 1 : 0;
+            } else {
+              img[at] = scale * res[pp][qq].x;
+              img[at + N] = scale * res[pp][qq].y;
+            }
+          }
+        }
+    }
   }
 }
 
 // ILT forward end on the coarse grid, for a pair of rows (y0, y0 + 1) of a
-// full-grid plane whose band rows R_y carry S (1 + i gain (x) gain), so that
-// the imaginary part of IDFT(R_y) is the blurred row.  The blurred row's
-// spectrum is (R_y(u) - conj R_y(-u)) / 2i, so one inverse transform of
-// Bl_y0 + i Bl_y1 gives both blurred rows as its real and imaginary parts.
+// full-grid plane from the half band rows of its blur: one inverse transform
+// of Bl_y0 + i Bl_y1 gives both blurred rows as its real and imaginary parts.
 // The sigmoid resist z = 1 / (1 + e^{-beta (blur - thr)}) (a smooth Eq. (5)),
 // the residual d = z - target of the squared-residual ILT loss and
 // dL/dI = 2 d beta z (1 - z) follow on the spot; the two dL/dI rows go forward as one complex row
-// q[y0] + i q[y1] and leave as their two band spectra, as k_mask_rows writes
+// q[y0] + i q[y1] and leave as their two half spectra, as k_mask_rows writes
 // them.  The pair's sum of d^2 goes to partial[plane][pair] in FP64: one
 // partial per row pair, whatever the launch shape, so the loss does not
 // depend on how clips are grouped.  Plane p belongs to clip
@@ -297,7 +322,7 @@ __global__ void __launch_bounds__(Plan<N>::NT, N >= 512 ? 640 / Plan<N>::NT : 1)
                                                                    float2* __restrict__ rowbuf,
                                                                    double* __restrict__ partial, int pairs_per_cta) {
   using SH = GradRowsShape<N>;
-  constexpr int NT = SH::NT, NW = (NT + 31) / 32, PERL = SH::PERL;
+  constexpr int NT = SH::NT, NW = (NT + 31) / 32, PERL = SH::PERL, RL = SH::RL;
   extern __shared__ float2 smem[];
   float2* tw = smem;
   float2* buf = smem + N;
@@ -305,32 +330,37 @@ __global__ void __launch_bounds__(Plan<N>::NT, N >= 512 ? 640 / Plan<N>::NT : 1)
   // the pair's dL/dI rows (N entries: x row y0, y row y0 + 1)
   float2* zq = smem + N + PadLen<N>::value;
   __shared__ double wsum[NW];
+  pdl_start();
   load_twiddles<N>(tw, tw_g);
+  pdl_wait(band, target);
   __syncthreads();
   const int p = blockIdx.y, t = threadIdx.x, half = crop / 2;
   const float* tg = target + (size_t)(p / planes_per_clip) * N * N;
   const float wgt = weight.w[p % planes_per_clip], beta2 = 2.0f * wgt * beta;
   for (int pr = blockIdx.x * pairs_per_cta; pr < min(N / 2, (blockIdx.x + 1) * pairs_per_cta); ++pr) {
     const int y0 = 2 * pr;
-    const float2* r0 = band + ((size_t)p * N + y0) * crop;
-    const float2* r1 = r0 + crop;
+    const float2* r0 = band + ((size_t)p * N + y0) * half;
     const float* t0 = tg + (size_t)y0 * N;
     const float* t1 = t0 + N;
-    auto load = [&](int, int r, int idx) {
-      const int u = r < Plan<N>::R[0] / 2 ? idx : idx - N;  // first pass: idx < N/2 exactly when r < R/2
-      const int c = u + half, cm = half - u;
-      const bool in = c >= 0 && c < crop, inm = cm >= 0 && cm < crop;
-      const float2 a = in ? __ldg(r0 + c) : make_float2(0.f, 0.f), b = inm ? __ldg(r0 + cm) : make_float2(0.f, 0.f);
-      const float2 e = in ? __ldg(r1 + c) : make_float2(0.f, 0.f), f = inm ? __ldg(r1 + cm) : make_float2(0.f, 0.f);
-      // Bl0 + i Bl1 = ((R1(u) - conj R1(-u)) - i (R0(u) - conj R0(-u))) / 2
-      return make_float2(0.5f * (e.x - f.x + a.y + b.y), 0.5f * (e.y + f.y + b.x - a.x));
+    auto load = [&](int, int r, int idx) {  // first pass: idx < N/2 exactly when r < R/2
+      return two_rows(r0, r0 + half, half, r < Plan<N>::R[0] / 2 ? idx : idx - N);
     };
     float racc = 0.f;  // this thread's residuals of the pair, summed in FP32 before the FP64 sum
+    float2 want[PERL][RL];  // the targets at this thread's outputs, loaded while the later passes run
+    auto after_first = [&]() {
+#pragma unroll
+      for (int pp = 0; pp < PERL; ++pp)
+#pragma unroll
+        for (int qq = 0; qq < RL; ++qq) {
+          const int x = t + pp * NT + qq * (N / RL);
+          want[pp][qq] = t + pp * NT < N / RL ? make_float2(ld_dep(t0 + x), ld_dep(t1 + x)) : make_float2(0.f, 0.f);
+        }
+    };
     float2 qreg[SH::kRegs ? SH::R0 : 1];
     auto use = [&](int pp, int qq, int x, float2 v) {
       const float z0 = 1.0f / (1.0f + expf(-beta * (v.x - thr)));
       const float z1 = 1.0f / (1.0f + expf(-beta * (v.y - thr)));
-      const float d0 = z0 - __ldg(t0 + x), d1 = z1 - __ldg(t1 + x);
+      const float d0 = z0 - want[pp][qq].x, d1 = z1 - want[pp][qq].y;
       racc = fmaf(d0, d0, fmaf(d1, d1, racc));
       const float2 q = make_float2(beta2 * d0 * z0 * (1.0f - z0), beta2 * d1 * z1 * (1.0f - z1));
       if constexpr (SH::kRegs)
@@ -338,7 +368,7 @@ __global__ void __launch_bounds__(Plan<N>::NT, N >= 512 ? 640 / Plan<N>::NT : 1)
       else
         zq[x] = q;
     };
-    fft_load_use<N, +1, decltype(load), decltype(use), BANDED>(buf, tw, t, load, use);
+    fft_load_use<N, +1, decltype(load), decltype(use), BANDED>(buf, tw, t, load, use, after_first);
     double acc = double(racc);
     auto usez = [&](int, int, int idx, float2 v) {
       const int u = freq_of(idx, N);
@@ -361,12 +391,12 @@ __global__ void __launch_bounds__(Plan<N>::NT, N >= 512 ? 640 / Plan<N>::NT : 1)
       for (int w = 0; w < NW; ++w) sum += wsum[w];
       partial[(size_t)p * (N / 2) + pr] = wgt * sum;
     }
-    float2* o0 = rowbuf + ((size_t)p * N + y0) * crop;
-    float2* o1 = o0 + crop;
-    for (int c = t; c < crop; c += NT) {
-      const float2 zp = zq[c], zm = zq[crop - c];
-      o0[c] = make_float2(0.5f * (zp.x + zm.x), 0.5f * (zp.y - zm.y));
-      o1[c] = make_float2(0.5f * (zp.y + zm.y), -0.5f * (zp.x - zm.x));
+    float2* o0 = rowbuf + ((size_t)p * N + y0) * half;
+    float2* o1 = o0 + half;
+    for (int k = t; k < half; k += NT) {
+      const float2 zp = zq[half + k], zm = zq[half - k];
+      o0[k] = make_float2(0.5f * (zp.x + zm.x), 0.5f * (zp.y - zm.y));
+      o1[k] = make_float2(0.5f * (zp.y + zm.y), -0.5f * (zp.x - zm.x));
     }
   }
 }
@@ -388,13 +418,14 @@ inline int rows_per_cta(int rows, int planes, int per_sm) {
   return int(std::min<long long>(r, rows));
 }
 
-template <int N>
-cudaError_t band_rows_resist_n(const float2* q, int clips, int planes, int crop, const float2* tw, float thr,
-                               float* img, float* iblur, uint8_t* printed, const PlaneOut& po, cudaStream_t st) {
-  const int rpc = rows_per_cta(N, clips * planes, 2048 / Plan<N>::NT), grid = (N + rpc - 1) / rpc;
-  auto kern = 2 * crop <= N ? k_band_rows_resist<N, true> : k_band_rows_resist<N, false>;
-  kern<<<dim3(grid, clips * planes), Plan<N>::NT, 0, st>>>(q, crop, tw, thr, img, iblur, printed, planes, po, rpc);
-  return cudaGetLastError();
+template <int N, bool RESIST>
+cudaError_t band_rows_n(const float2* q, int clips, int planes, int h, float scale, const float2* tw, float thr,
+                        float* img, float* iblur, uint8_t* printed, const PlaneOut& po, cudaStream_t st) {
+  const int units = RESIST ? N : N / 2;
+  const int per = rows_per_cta(units, clips * planes, 2048 / Plan<N>::NT), grid = (units + per - 1) / per;
+  auto kern = 4 * h <= N ? k_band_rows<N, true, RESIST> : k_band_rows<N, false, RESIST>;
+  return launch_pdl(kern, dim3(grid, clips * planes), Plan<N>::NT, 0, st, q, h, scale, tw, thr, img, iblur, printed,
+                    planes, po, per);
 }
 
 template <int N>
@@ -407,60 +438,46 @@ cudaError_t resist_grad_rows_n(const float2* band, int planes, int crop, const f
   auto kern = 2 * crop <= N ? k_resist_grad_rows<N, true> : k_resist_grad_rows<N, false>;
   cudaError_t e = smem_attrs(kern, sm);
   if (e != cudaSuccess) return e;
-  kern<<<dim3(grid, planes), Plan<N>::NT, sm, st>>>(band, crop, tw, target, planes_per_clip, weight, beta, thr, rowbuf,
-                                                    partial, ppc);
-  return cudaGetLastError();
+  return launch_pdl(kern, dim3(grid, planes), Plan<N>::NT, sm, st, band, crop, tw, target, planes_per_clip, weight,
+                    beta, thr, rowbuf, partial, ppc);
 }
 
-template <int N>
-cudaError_t band_rows_real_n(const float2* q, int clips, int planes, int crop, float scale, const float2* tw,
-                             float* out, const PlaneOut& po, cudaStream_t st) {
-  const int rpc = rows_per_cta(N, clips * planes, 2048 / Plan<N>::NT), grid = (N + rpc - 1) / rpc;
-  auto kern = 2 * crop <= N ? k_band_rows_real<N, true> : k_band_rows_real<N, false>;
-  kern<<<dim3(grid, clips * planes), Plan<N>::NT, 0, st>>>(q, crop, scale, tw, out, planes, po, rpc);
-  return cudaGetLastError();
+template <int N, int W, bool MIRROR>
+cudaError_t mask_cols_w(const float2* rowbuf, int b, int crop, int cols, int ld, const float2* tw, const float* gain,
+                        float2* mhat, cudaStream_t st) {
+  const size_t sm = sizeof(float2) * (N + size_t(W) * ((PadLen<N>::value + 15) / 16 * 16 + 16 / W));
+  cudaError_t e = smem_attrs(k_mask_cols<N, W, MIRROR>, sm);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_mask_cols<N, W, MIRROR>, dim3((cols + W - 1) / W, b), Plan<N>::NT * W, sm, st, rowbuf, crop,
+                    cols, ld, tw, gain, mhat);
 }
 
-template <int N>
-size_t col_smem_bytes() {
-  return sizeof(float2) * (N + ColW<N>::W * ColLD<N>::value);
-}
+// Half rows of the mask spectrum (whole: with k = crop/2) or of any real plane.
+inline int half_cols(int crop, bool whole) { return crop / 2 + (whole ? 1 : 0); }
+inline int half_ld(int crop, bool whole) { return crop / 2 + (whole ? 8 : 0); }
 
 template <int N>
 cudaError_t mask_cols_n(const float2* rowbuf, int b, int crop, const float2* tw, float2* mhat, const float* gain,
-                        bool gain_real, cudaStream_t st) {
-  const size_t sm = col_smem_bytes<N>();
-  cudaError_t e = smem_attrs(k_mask_cols<N>, sm);
-  if (e != cudaSuccess) return e;
-  k_mask_cols<N><<<dim3(crop / ColW<N>::W, b), Plan<N>::NT * ColW<N>::W, sm, st>>>(rowbuf, crop, tw, gain, mhat,
-                                                                                   gain_real ? 1 : 0);
-  return cudaGetLastError();
+                        bool whole, cudaStream_t st) {
+  const int cols = half_cols(crop, whole), ld = half_ld(crop, whole);
+  // 8 columns a CTA (64-byte pieces of a row); 4 (whole 32-byte sectors) while that leaves SMs without a CTA
+  const bool few = (long long)b * ((cols + 7) / 8) < 152;
+  if (whole)
+    return few ? mask_cols_w<N, 4, true>(rowbuf, b, crop, cols, ld, tw, gain, mhat, st)
+               : mask_cols_w<N, 8, true>(rowbuf, b, crop, cols, ld, tw, gain, mhat, st);
+  return few ? mask_cols_w<N, 4, false>(rowbuf, b, crop, cols, ld, tw, gain, mhat, st)
+             : mask_cols_w<N, 8, false>(rowbuf, b, crop, cols, ld, tw, gain, mhat, st);
 }
 
 template <int N>
-cudaError_t mask_rows_n(const float* m, int b, int crop, const float2* tw, float2* rowbuf, cudaStream_t st) {
+cudaError_t mask_rows_n(const float* m, int b, int crop, const float2* tw, float2* rowbuf, bool whole,
+                        cudaStream_t st) {
   const size_t smr = sizeof(float2) * (2 * N + PadLen<N>::value + 1);
   cudaError_t e = smem_attrs(k_mask_rows<N>, smr);
   if (e != cudaSuccess) return e;
   const int ppc = rows_per_cta(N / 2, b, 2048 / Plan<N>::NT);
-  k_mask_rows<N><<<dim3((N / 2 + ppc - 1) / ppc, b), Plan<N>::NT, smr, st>>>(m, crop, tw, rowbuf, ppc);
-  return cudaGetLastError();
-}
-
-template <int N>
-cudaError_t mask_spectrum_n(const float* m, int b, int crop, const float2* tw, float2* rowbuf, float2* mhat,
-                            const float* gain, bool gain_real, cudaStream_t st) {
-  const size_t smr = sizeof(float2) * (2 * N + PadLen<N>::value + 1);
-  cudaError_t e = smem_attrs(k_mask_rows<N>, smr);
-  if (e != cudaSuccess) return e;
-  const int ppc = rows_per_cta(N / 2, b, 2048 / Plan<N>::NT);
-  k_mask_rows<N><<<dim3((N / 2 + ppc - 1) / ppc, b), Plan<N>::NT, smr, st>>>(m, crop, tw, rowbuf, ppc);
-  const size_t sm = col_smem_bytes<N>();
-  e = smem_attrs(k_mask_cols<N>, sm);
-  if (e != cudaSuccess) return e;
-  k_mask_cols<N><<<dim3(crop / ColW<N>::W, b), Plan<N>::NT * ColW<N>::W, sm, st>>>(rowbuf, crop, tw, gain, mhat,
-                                                                                   gain_real ? 1 : 0);
-  return cudaGetLastError();
+  return launch_pdl(k_mask_rows<N>, dim3((N / 2 + ppc - 1) / ppc, b), Plan<N>::NT, smr, st, m, crop, tw, rowbuf,
+                    half_cols(crop, whole), half_ld(crop, whole), ppc);
 }
 
 template <int N>
@@ -469,12 +486,19 @@ cudaError_t stage1_n(const float2* mhat, const float2* phi, int nk, int crop, co
   return launch_stage1_cols<N, Stage1W<N>::W>(mhat, phi, nk, crop, tw, OutC64{t1, N, crop}, st, clips);
 }
 
+// Only the columns u >= 0 of nk spectra (index u + crop/2), written as half rows.
+template <int N>
+cudaError_t stage1_half_n(const float2* spec, int nk, int crop, const float2* tw, float2* q, int ld,
+                          cudaStream_t st) {
+  return launch_stage1_cols<N, Stage1W<N>::W>(spec, nullptr, nk, crop, tw, OutHalf{q, N, crop / 2, ld}, st, 1,
+                                              crop / 2);
+}
+
 template <int N>
 cudaError_t stage2_n(const float2* t1, const FieldSet& fs, int clips, int crop, float dose, const float2* tw,
                      float* img, const PlaneOut& po, cudaStream_t st) {
   auto kern = 2 * crop <= N ? k_stage2<N, true> : k_stage2<N, false>;
-  kern<<<dim3(N, clips * fs.planes), Plan<N>::NT, 0, st>>>(t1, fs, crop, dose, tw, img, po);
-  return cudaGetLastError();
+  return launch_pdl(kern, dim3(N, clips * fs.planes), Plan<N>::NT, 0, st, t1, fs, crop, dose, tw, img, po);
 }
 
 // Transform sizes of the full grid (powers of two) ...
@@ -521,30 +545,28 @@ bool fft_twiddle_table(int n, float2* out) {
 }
 
 cudaError_t launch_mask_spectrum(const float* m, int b, int n, int crop, const float2* tw, float2* rowbuf,
-                                 float2* mhat, cudaStream_t st, const float* gain, bool gain_real) {
-#define CALL(N) mask_spectrum_n<N>(m, b, crop, tw, rowbuf, mhat, gain, gain_real, st)
-  LITHO_DISPATCH_NC(n, CALL)
-#undef CALL
+                                 float2* mhat, cudaStream_t st) {
+  cudaError_t e = launch_mask_rows(m, b, n, crop, tw, rowbuf, true, st);
+  return e != cudaSuccess ? e : launch_mask_cols(rowbuf, b, n, crop, tw, mhat, nullptr, true, st);
 }
 
-cudaError_t launch_band_rows_real(const float2* q, int clips, int planes, int n, int crop, float scale,
-                                  const float2* tw, float* out, const PlaneOut& po, cudaStream_t st) {
-#define CALL(N) band_rows_real_n<N>(q, clips, planes, crop, scale, tw, out, po, st)
+cudaError_t launch_band_rows_real(const float2* q, int clips, int planes, int n, int h, float scale, const float2* tw,
+                                  float* out, const PlaneOut& po, cudaStream_t st) {
+#define CALL(N) band_rows_n<N, false>(q, clips, planes, h, scale, tw, 0.f, out, nullptr, nullptr, po, st)
   LITHO_DISPATCH_N(n, CALL)
 #undef CALL
 }
 
-cudaError_t launch_mask_rows(const float* m, int b, int n, int crop, const float2* tw, float2* rowbuf,
+cudaError_t launch_mask_rows(const float* m, int b, int n, int crop, const float2* tw, float2* rowbuf, bool whole,
                              cudaStream_t st) {
-#define CALL(N) mask_rows_n<N>(m, b, crop, tw, rowbuf, st)
+#define CALL(N) mask_rows_n<N>(m, b, crop, tw, rowbuf, whole, st)
   LITHO_DISPATCH_NC(n, CALL)
 #undef CALL
 }
 
 cudaError_t launch_blur_gain(const ResistTaps& taps, int n, int crop, float* gain, cudaStream_t st) {
   if (n < 1 || crop < 1) return cudaErrorInvalidValue;
-  k_blur_gain<<<(crop + 127) / 128, 128, 0, st>>>(taps, n, crop, gain);
-  return cudaGetLastError();
+  return launch_pdl(k_blur_gain, (crop + 127) / 128, 128, 0, st, taps, n, crop, gain);
 }
 
 cudaError_t launch_resist_grad_rows(const float2* band, int planes, int n, int crop, const float2* tw,
@@ -556,15 +578,22 @@ cudaError_t launch_resist_grad_rows(const float2* band, int planes, int n, int c
 #undef CALL
 }
 cudaError_t launch_mask_cols(const float2* rowbuf, int b, int n, int crop, const float2* tw, float2* mhat,
-                             const float* gain, bool gain_real, cudaStream_t st) {
-#define CALL(N) mask_cols_n<N>(rowbuf, b, crop, tw, mhat, gain, gain_real, st)
+                             const float* gain, bool whole, cudaStream_t st) {
+#define CALL(N) mask_cols_n<N>(rowbuf, b, crop, tw, mhat, gain, whole, st)
   LITHO_DISPATCH_NC(n, CALL)
 #undef CALL
 }
-cudaError_t launch_band_rows_resist(const float2* q, int clips, int planes, int n, int crop, const float2* tw,
+cudaError_t launch_band_rows_resist(const float2* q, int clips, int planes, int n, int h, const float2* tw,
                                     float threshold, float* img, float* iblur, uint8_t* printed, const PlaneOut& po,
                                     cudaStream_t st) {
-#define CALL(N) band_rows_resist_n<N>(q, clips, planes, crop, tw, threshold, img, iblur, printed, po, st)
+#define CALL(N) band_rows_n<N, true>(q, clips, planes, h, 1.0f, tw, threshold, img, iblur, printed, po, st)
+  LITHO_DISPATCH_N(n, CALL)
+#undef CALL
+}
+
+cudaError_t launch_stage1_half(const float2* spec, int nk, int n, int crop, const float2* tw, float2* q, int ld,
+                               cudaStream_t st) {
+#define CALL(N) stage1_half_n<N>(spec, nk, crop, tw, q, ld, st)
   LITHO_DISPATCH_N(n, CALL)
 #undef CALL
 }

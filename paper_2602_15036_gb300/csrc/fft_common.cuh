@@ -26,6 +26,7 @@
 
 #include <cmath>
 #include <type_traits>
+#include <utility>
 
 namespace litho {
 
@@ -559,6 +560,60 @@ template <int N> struct ColLD {
 // Stride of the compact band buffers [W][crop] (crop is a multiple of 32).
 template <int N>
 __host__ __device__ __forceinline__ int band_ld(int crop) { return crop + 16 / ColW<N>::W; }
+
+// Programmatic dependent launch.  A kernel that launch_pdl starts may begin as soon as every CTA of the
+// kernel before it on the stream has called pdl_start (or ended): its set-up (twiddle tables, which no
+// kernel writes) overlaps that kernel's last CTAs, and the launch latency is hidden.  pdl_wait then holds
+// it until the kernel before it, and so every earlier one, has finished and its writes are visible:
+// every kernel started this way calls it before it reads or writes anything else in global memory.
+// One 256^2 image (7 kernels) 37 -> 23 us, an ILT step of one 512^2 clip (17 kernels) 160 -> 125 us.
+__device__ __forceinline__ void pdl_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// The pointers to what earlier kernels wrote are named, so that no load through them can be moved ahead
+// of the wait (their values pass through an assembly statement that follows it).
+template <class... T>
+__device__ __forceinline__ void pdl_wait(T&... p) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  (([](auto& q) { asm volatile("" : "+l"(q)); })(p), ...);
+}
+
+// A load of what an earlier kernel wrote, in a kernel started by launch_pdl, through a pointer named to
+// pdl_wait and not written by the kernel: not the read-only path, which may assume that memory does not
+// change while the kernel runs.
+__device__ __forceinline__ float ld_dep(const float* p) {
+  float v;
+  asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float2 ld_dep(const float2* p) {
+  float2 v;
+  asm("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 ld_dep(const float4* p) {
+  float4 v;
+  asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double ld_dep(const double* p) {
+  double v;
+  asm("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 
 // Prefer the largest shared-memory carveout for a kernel that uses a lot of it.
 template <class K>

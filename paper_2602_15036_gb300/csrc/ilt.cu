@@ -45,8 +45,10 @@ __device__ __forceinline__ int freq_of_idx(int idx, int n) { return idx < n / 2 
 
 // m = sigmoid(alpha theta), four values per thread and step (count a multiple of 4, 16-byte aligned)
 __global__ void k_sigmoid(const float4* __restrict__ theta, float alpha, float4* __restrict__ m, size_t count4) {
+  pdl_start();
+  pdl_wait(theta);
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count4; i += (size_t)gridDim.x * blockDim.x) {
-    const float4 t = theta[i];
+    const float4 t = ld_dep(theta + i);
     m[i] = make_float4(1.0f / (1.0f + expf(-alpha * t.x)), 1.0f / (1.0f + expf(-alpha * t.y)),
                        1.0f / (1.0f + expf(-alpha * t.z)), 1.0f / (1.0f + expf(-alpha * t.w)));
   }
@@ -58,6 +60,8 @@ __global__ void __launch_bounds__(256) k_resist_grad(const float* __restrict__ i
                                                      size_t nn, int planes, const __grid_constant__ PlaneWeight weight,
                                                      float beta, float thr, float* __restrict__ q,
                                                      double* __restrict__ partial) {
+  pdl_start();
+  pdl_wait(ib, target);
   const size_t clip = blockIdx.y;
   ib += clip * planes * nn;
   q += clip * planes * nn;
@@ -69,8 +73,8 @@ __global__ void __launch_bounds__(256) k_resist_grad(const float* __restrict__ i
   int pl = int(i / nn);
   size_t pix = i - pl * nn;  // i mod nn and i div nn, carried along instead of recomputed
   for (; i < total; i += stride) {
-    const float z = 1.0f / (1.0f + expf(-beta * (ib[i] - thr)));
-    const float d = z - target[pix], w = weight.w[pl];
+    const float z = 1.0f / (1.0f + expf(-beta * (ld_dep(ib + i) - thr)));
+    const float d = z - ld_dep(target + pix), w = weight.w[pl];
     acc += double(w) * double(d) * double(d);
     q[i] = 2.0f * w * d * beta * z * (1.0f - z);
     pix += stride;
@@ -94,10 +98,12 @@ __global__ void __launch_bounds__(256) k_resist_grad(const float* __restrict__ i
 __global__ void __launch_bounds__(1024) k_reduce_loss(const double* __restrict__ partial, int count,
                                                       double* __restrict__ out, int accumulate) {
   __shared__ double s[1024];
+  pdl_start();
+  pdl_wait(partial);
   partial += (size_t)blockIdx.x * count;
   out += blockIdx.x;
   double a = 0.0;
-  for (int i = threadIdx.x; i < count; i += 1024) a += partial[i];
+  for (int i = threadIdx.x; i < count; i += 1024) a += ld_dep(partial + i);
   s[threadIdx.x] = a;
   __syncthreads();
   for (int w = 512; w > 0; w >>= 1) {
@@ -123,7 +129,9 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_adj_rows(const float2* __restri
   float2* tw = sm;
   float2* bufa = sm + N;
   float2* bufb = sm + N + PadLen<N>::value;
+  pdl_start();
   load_twiddles<N>(tw, tw_g);
+  pdl_wait(t1, g);
   const int y = blockIdx.x, plane = blockIdx.y, t = threadIdx.x, half = crop / 2;
   const int clip = plane / fs.planes, pl = plane - clip * fs.planes;
   float gv[PERL][RL];
@@ -133,7 +141,7 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_adj_rows(const float2* __restri
 #pragma unroll
     for (int q = 0; q < RL; ++q) {
       const int jj = t + p * NT;
-      gv[p][q] = jj < N / RL ? grow[jj + q * (N / RL)] : 0.f;
+      gv[p][q] = jj < N / RL ? ld_dep(grow + jj + q * (N / RL)) : 0.f;
     }
   __syncthreads();
   for (int k = fs.start[pl]; k < fs.start[pl + 1]; ++k) {
@@ -141,7 +149,7 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_adj_rows(const float2* __restri
     const float2* row = t1 + rowoff;
     auto load_band = [&](int, int r, int idx) {
       const int c = (r < PL::R[0] / 2 ? idx : idx - N) + half;  // first pass: idx < N/2 exactly when r < R/2
-      return (c >= 0 && c < crop) ? __ldg(row + c) : make_float2(0.f, 0.f);
+      return (c >= 0 && c < crop) ? ld_dep(row + c) : make_float2(0.f, 0.f);
     };
     auto times_g = [&](int p, int q, int idx, float2 v) {
       bufb[pad16(idx)] = make_float2(v.x * gv[p][q], v.y * gv[p][q]);
@@ -197,7 +205,9 @@ __global__ void __launch_bounds__(32 * kAdjWarps, 2)
   float2* tw2 = tw1 + kAdjTw1;                        // forward pass 2: (r - 1) 32 + l
   float2* bufs = tw2 + kAdjTw2;                       // [warp][2 rows][kAdjBuf]
   float2* stage0 = bufs + kAdjWarps * 2 * kAdjBuf;    // [warp][2 rows][crop]
+  pdl_start();
   for (int i = threadIdx.x; i < kAdjTw1 + kAdjTw2; i += blockDim.x) tw1[i] = tw_g[i];
+  pdl_wait(g);
   __syncthreads();
   const int lane = threadIdx.x % 32, wp = threadIdx.x / 32, half = crop / 2;
   const int y0 = (blockIdx.x * kAdjWarps + wp) * 2, plane = blockIdx.y;
@@ -214,7 +224,7 @@ __global__ void __launch_bounds__(32 * kAdjWarps, 2)
   {
     const float* grow = g + ((size_t)(clip * g_planes + pl) * N + y0 + rsel) * N;
 #pragma unroll
-    for (int q = 0; q < 32; ++q) gv[q] = __ldg(grow + jj + 16 * q);
+    for (int q = 0; q < 32; ++q) gv[q] = ld_dep(grow + jj + 16 * q);
   }
   auto fetch = [&](int k) {  // band rows y0, y0 + 1 of kernel k: 2 x crop/2 pieces of 16 bytes
     const float2* src = t1p + (size_t)k * field + (size_t)y0 * crop;
@@ -346,13 +356,15 @@ __global__ void __launch_bounds__(Plan<N>::NT * AdjW<N>::W, AdjAccInSmem<N>::val
       return acc_r[i];
   };
   const int j0 = clip * period + split * jb, j1 = min(j0 + jb, (clip + 1) * period);
+  pdl_start();
   load_twiddles<N>(tw, tw_g);
+  pdl_wait(u);
   // this thread's first-pass inputs (rows t + r N/R0) of a field, loaded one field ahead
   float2 nxt[R0];
   auto prefetch = [&](int j) {
     const float2* src = u + (size_t)j * N * crop + c0 + g;  // row y at src[y crop]
 #pragma unroll
-    for (int r = 0; r < R0; ++r) nxt[r] = t < NB0 ? __ldg(src + (size_t)(t + r * NB0) * crop) : make_float2(0.f, 0.f);
+    for (int r = 0; r < R0; ++r) nxt[r] = t < NB0 ? ld_dep(src + (size_t)(t + r * NB0) * crop) : make_float2(0.f, 0.f);
   };
   if (j0 < j1) prefetch(j0);
   __syncthreads();
@@ -407,12 +419,14 @@ __global__ void __launch_bounds__(Plan<N>::NT * AdjW<N>::W, AdjAccInSmem<N>::val
 // in `sets`.
 __global__ void k_ones_adjoint(const float2* __restrict__ mhat, const float* __restrict__ power,
                                const __grid_constant__ PlaneOut sets, size_t cc, float n2, float2* __restrict__ s) {
+  pdl_start();
+  pdl_wait(mhat);
   mhat += (size_t)blockIdx.y * cc;
   s += (size_t)blockIdx.y * cc;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < cc; i += (size_t)gridDim.x * blockDim.x) {
     float d = 0.f;
     for (int f = 0; f < sets.out_planes; ++f) d += __ldg(power + sets.list[f] * cc + i);
-    const float2 m = mhat[i];
+    const float2 m = ld_dep(mhat + i);
     s[i] = make_float2(n2 * d * m.x, n2 * d * m.y);
   }
 }
@@ -428,12 +442,14 @@ PlaneOut sets_of(const litho_kernels* h, int f0, int count) {
 // out[i nu + u] = the sum of clip i's upstream planes list[first[u]] ... (blockIdx.y = i nu + u).
 __global__ void k_sum_upstream(const float* __restrict__ up, size_t nn, int nu, const __grid_constant__ PlaneOut planes,
                                float* __restrict__ out) {
+  pdl_start();
+  pdl_wait(up);
   const int clip = blockIdx.y / nu, u = blockIdx.y - clip * nu;
   up += (size_t)clip * planes.out_planes * nn;
   out += (size_t)blockIdx.y * nn;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nn; i += (size_t)gridDim.x * blockDim.x) {
-    float a = up[planes.list[planes.first[u]] * nn + i];
-    for (int d = planes.first[u] + 1; d < planes.first[u + 1]; ++d) a += up[planes.list[d] * nn + i];
+    float a = ld_dep(up + planes.list[planes.first[u]] * nn + i);
+    for (int d = planes.first[u] + 1; d < planes.first[u + 1]; ++d) a += ld_dep(up + planes.list[d] * nn + i);
     out[i] = a;
   }
 }
@@ -441,12 +457,14 @@ __global__ void k_sum_upstream(const float* __restrict__ up, size_t nn, int nu, 
 // s[clip] (+)= sum over the clip's `planes` planes of sk, in order (clip = blockIdx.y).
 __global__ void k_sum_planes(const float2* __restrict__ sk, int planes, size_t cc, float2* __restrict__ s,
                              int accumulate) {
+  pdl_start();
+  pdl_wait(sk);
   sk += (size_t)blockIdx.y * planes * cc;
   s += (size_t)blockIdx.y * cc;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < cc; i += (size_t)gridDim.x * blockDim.x) {
     float2 a = accumulate ? s[i] : make_float2(0.f, 0.f);
     for (int j = 0; j < planes; ++j) {
-      const float2 v = sk[(size_t)j * cc + i];
+      const float2 v = ld_dep(sk + (size_t)j * cc + i);
       a.x += v.x;
       a.y += v.y;
     }
@@ -463,7 +481,9 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_grad_rows(const float2* __restr
   extern __shared__ float2 sm[];
   float2* tw = sm;
   float2* buf = sm + N;
+  pdl_start();
   load_twiddles<N>(tw, tw_g);
+  pdl_wait(qf, m);
   __syncthreads();
   const int y = blockIdx.x, t = threadIdx.x, half = crop / 2;
   const size_t clip = blockIdx.y;  // clip of the group: its band rows, mask and gradient
@@ -473,19 +493,23 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_grad_rows(const float2* __restr
   const float2* row = qf + (size_t)y * crop;
   auto load = [&](int idx) {
     const int c = freq_of_idx(idx, N) + half;
-    return (c >= 0 && c < crop) ? __ldg(row + c) : make_float2(0.f, 0.f);
+    return (c >= 0 && c < crop) ? ld_dep(row + c) : make_float2(0.f, 0.f);
   };
   const float* mr = m ? m + (size_t)y * N : nullptr;
   float* gr = grad + (size_t)y * N;
-  auto use = [&](int, int, int x, float2 v) {
-    if (m) {
-      const float mm = mr[x];
-      gr[x] = scale * v.x * alpha * mm * (1.0f - mm);
-    } else {
-      gr[x] = scale * v.x;  // no chain factor: the gradient with respect to m itself
-    }
+  constexpr int NT = Plan<N>::NT, RL = Plan<N>::R[Plan<N>::P - 1], PERL = PassShape<N, NT, RL>::PER;
+  float mm[PERL][RL];  // the mask at this thread's outputs, loaded while the later passes run
+  auto after_first = [&]() {
+#pragma unroll
+    for (int p = 0; p < PERL; ++p)
+#pragma unroll
+      for (int q = 0; q < RL; ++q) mm[p][q] = m && t + p * NT < N / RL ? ld_dep(mr + t + p * NT + q * (N / RL)) : 0.f;
   };
-  fft_load_use<N, +1>(buf, tw, t, load, use);
+  auto use = [&](int p, int q, int x, float2 v) {
+    // without m no chain factor: the gradient with respect to m itself
+    gr[x] = m ? scale * v.x * alpha * mm[p][q] * (1.0f - mm[p][q]) : scale * v.x;
+  };
+  fft_load_use<N, +1, decltype(load), decltype(use), false>(buf, tw, t, load, use, after_first);
 }
 
 template <int N>
@@ -496,16 +520,14 @@ cudaError_t adj_rows_n(const float2* t1, const FieldSet& fs, int clips, int crop
     const size_t sm = sizeof(float2) * (kAdjTw1 + kAdjTw2 + kAdjWarps * 2 * (size_t(kAdjBuf) + crop));
     cudaError_t e = smem_attrs(k_adj_rows_w512<true>, sm);
     if (e != cudaSuccess) return e;
-    k_adj_rows_w512<true><<<dim3(N / (2 * kAdjWarps), planes), 32 * kAdjWarps, sm, st>>>(t1, fs, crop, g, g_planes,
-                                                                                          tw512, u);
-    return cudaGetLastError();
+    return launch_pdl(k_adj_rows_w512<true>, dim3(N / (2 * kAdjWarps), planes), 32 * kAdjWarps, sm, st, t1, fs, crop,
+                      g, g_planes, tw512, u);
   }
   const size_t sm = sizeof(float2) * (N + 2 * PadLen<N>::value);
   auto kern = 2 * crop <= N ? k_adj_rows<N, true> : k_adj_rows<N, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  kern<<<dim3(N, planes), Plan<N>::NT, sm, st>>>(t1, fs, crop, g, g_planes, tw, u);
-  return cudaGetLastError();
+  return launch_pdl(kern, dim3(N, planes), Plan<N>::NT, sm, st, t1, fs, crop, g, g_planes, tw, u);
 }
 
 template <int N>
@@ -519,8 +541,8 @@ cudaError_t adj_cols_n(const float2* u, const float2* phi, int crop, const float
   cudaError_t e = smem_attrs(k_adj_cols<N>, sm);
   if (e != cudaSuccess) return e;
   const int splits = adj_col_splits(period);
-  k_adj_cols<N><<<dim3(crop / W, clips * splits), Plan<N>::NT * W, sm, st>>>(u, phi, crop, tw, part, period, splits);
-  return cudaGetLastError();
+  return launch_pdl(k_adj_cols<N>, dim3(crop / W, clips * splits), Plan<N>::NT * W, sm, st, u, phi, crop, tw, part,
+                    period, splits);
 }
 
 template <int N>
@@ -529,8 +551,8 @@ cudaError_t grad_rows_n(const float2* qf, int crop, float scale, const float* m,
   const size_t sm = sizeof(float2) * (N + PadLen<N>::value);
   cudaError_t e = cudaFuncSetAttribute(k_grad_rows<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  k_grad_rows<N><<<dim3(N, clips), Plan<N>::NT, sm, st>>>(qf, crop, scale, m, alpha, tw, grad, grad_stride);
-  return cudaGetLastError();
+  return launch_pdl(k_grad_rows<N>, dim3(N, clips), Plan<N>::NT, sm, st, qf, crop, scale, m, alpha, tw, grad,
+                    grad_stride);
 }
 
 #define ILT_DISPATCH(n, CALL)              \
@@ -695,16 +717,15 @@ litho_status ai_channels(const litho_kernels* h, const float* target, int b, dou
       LITHO_TRY_CUDA(launch_stage2_fft(L.t1, fs, g, NE, C, float(dose), twe, coarse ? L.ic : dst,
                                        coarse ? one : channel1, st, h->d_tw32, h->d_tw512, rows2 ? L.mid : nullptr, C2));
       if (coarse) {
-        if (!rows2) LITHO_TRY_CUDA(launch_mask_rows(L.ic, g, NE, C2, twe, L.mid, st));
-        LITHO_TRY_CUDA(launch_interp_cols(L.mid, g, NE, N, C2, twe, h->d_tw, nullptr, L.big, st));
-        LITHO_TRY_CUDA(launch_band_rows_real(L.big, g, 1, N, C2, 1.0f, h->d_tw, dst, channel1, st));
+        if (!rows2) LITHO_TRY_CUDA(launch_mask_rows(L.ic, g, NE, C2, twe, L.mid, false, st));
+        LITHO_TRY_CUDA(launch_interp_cols(L.mid, g, NE, N, C, twe, h->d_tw, nullptr, true, L.big, st));
+        LITHO_TRY_CUDA(launch_band_rows_real(L.big, g, 1, N, C, 1.0f, h->d_tw, dst, channel1, st));
       }
     }
     {  // channel 2: the adjoint applied to dL/dI = 1, in closed form (k_ones_adjoint)
       ProfScope ps(kStageIltBackward, st, 3);
-      k_ones_adjoint<<<dim3(128, g), 256, 0, st>>>(L.mhat, h->d_power, sets_of(h, focus, 1), size_t(C) * C,
-                                                   float(double(N) * double(N)), L.s);
-      LITHO_TRY_CUDA(cudaGetLastError());
+      LITHO_TRY_CUDA(launch_pdl(k_ones_adjoint, dim3(128, g), 256, 0, st, L.mhat, h->d_power, sets_of(h, focus, 1),
+                                size_t(C) * C, float(double(N) * double(N)), L.s));
       LITHO_TRY_CUDA(launch_stage1_fft(L.s, nullptr, g, N, C, h->d_tw, L.qf, st));
       LITHO_TRY_CUDA(launch_grad_rows(N, L.qf, C, scale, nullptr, 0.f, h->d_tw, x + (size_t(c0) * 3 + 2) * nn, g,
                                       (long long)3 * nn, st));
@@ -809,8 +830,8 @@ litho_status litho_ilt_grad(const litho_kernels* h, const float* theta_dev, cons
       {
         const size_t c4 = size_t(g) * nn / 4;  // nn = N^2 with N >= 32: a multiple of 4
         const int blocks = int(std::min<size_t>((c4 + 255) / 256, 4096));
-        k_sigmoid<<<blocks, 256, 0, st>>>(reinterpret_cast<const float4*>(theta_dev + c0 * nn), float(mask_steep),
-                                          reinterpret_cast<float4*>(L.m), c4);
+        LITHO_TRY_CUDA(launch_pdl(k_sigmoid, blocks, 256, 0, st, reinterpret_cast<const float4*>(theta_dev + c0 * nn),
+                                  float(mask_steep), reinterpret_cast<float4*>(L.m), c4));
       }
       LITHO_TRY_CUDA(cudaGetLastError());
       LITHO_TRY_CUDA(launch_mask_spectrum(L.m, g, N, C, h->d_tw, L.rowbuf, L.mhat, st));
@@ -827,19 +848,20 @@ litho_status litho_ilt_grad(const litho_kernels* h, const float* theta_dev, cons
         LITHO_TRY_CUDA(launch_stage2_fft(L.t1, fs, g, NE, C, float(dose), twe, coarse ? L.ic : L.img, each, st,
                                          h->d_tw32, h->d_tw512, rows2 ? L.mid : nullptr, C2));
         if (coarse) {  // the blurred image straight from the interpolation (blur applied to the spectrum)
-          if (!rows2) LITHO_TRY_CUDA(launch_mask_rows(L.ic, gp, NE, C2, twe, L.mid, st));
-          LITHO_TRY_CUDA(launch_interp_cols(L.mid, gp, NE, N, C2, twe, h->d_tw, L.gain, L.big, st));
+          if (!rows2) LITHO_TRY_CUDA(launch_mask_rows(L.ic, gp, NE, C2, twe, L.mid, false, st));
+          LITHO_TRY_CUDA(launch_interp_cols(L.mid, gp, NE, N, C, twe, h->d_tw, L.gain, false, L.big, st));
           // blurred rows, resist, dL/dI and its row spectra on the 2C band (into the free image
           // buffer), partial losses per row pair
           LITHO_TRY_CUDA(launch_resist_grad_rows(L.big, gp, N, C2, h->d_tw, target_dev + c0 * nn, PU, weight,
                                                  float(resist_steep), float(threshold), qrows, L.partial, st));
-          k_reduce_loss<<<g, 1024, 0, st>>>(L.partial, PU * N / 2, L.loss + c0, u0 > 0 ? 1 : 0);
+          LITHO_TRY_CUDA(launch_pdl(k_reduce_loss, g, 1024, 0, st, L.partial, PU * N / 2, L.loss + c0,
+                                    u0 > 0 ? 1 : 0));
         } else {
           LITHO_TRY_CUDA(launch_resist(L.img, gp, N, taps, float(threshold), L.blur, nullptr, st));
-          k_resist_grad<<<dim3(kPartials, g), 256, 0, st>>>(L.blur, target_dev + c0 * nn, nn, PU, weight,
-                                                           float(resist_steep), float(threshold), L.img, L.partial);
-          LITHO_TRY_CUDA(cudaGetLastError());
-          k_reduce_loss<<<g, 1024, 0, st>>>(L.partial, kPartials, L.loss + c0, u0 > 0 ? 1 : 0);
+          LITHO_TRY_CUDA(launch_pdl(k_resist_grad, dim3(kPartials, g), 256, 0, st, L.blur, target_dev + c0 * nn, nn,
+                                    PU, weight, float(resist_steep), float(threshold), L.img, L.partial));
+          LITHO_TRY_CUDA(launch_pdl(k_reduce_loss, g, 1024, 0, st, L.partial, kPartials, L.loss + c0,
+                                    u0 > 0 ? 1 : 0));
         }
         LITHO_TRY_CUDA(cudaGetLastError());
       }
@@ -847,18 +869,17 @@ litho_status litho_ilt_grad(const litho_kernels* h, const float* theta_dev, cons
         ProfScope ps(kStageIltBackward, st, coarse ? 6 : 4);
         const float* gsrc = L.blur;
         if (coarse) {  // low-pass of g (x) q: the spectrum of q on the 2C band times the blur's transfer function
-          LITHO_TRY_CUDA(launch_mask_cols(qrows, gp, N, C2, h->d_tw, L.spec, L.gain, true, st));
-          LITHO_TRY_CUDA(launch_stage1_fft(L.spec, nullptr, gp, NE, C2, twe, L.mid, st));
-          LITHO_TRY_CUDA(launch_band_rows_real(L.mid, g, PU, NE, C2, lp_scale, twe, L.ic, each, st));
+          LITHO_TRY_CUDA(launch_mask_cols(qrows, gp, N, C2, h->d_tw, L.spec, L.gain, false, st));
+          LITHO_TRY_CUDA(launch_stage1_half(L.spec, gp, NE, C2, twe, L.mid, C, st));
+          LITHO_TRY_CUDA(launch_band_rows_real(L.mid, g, PU, NE, C, lp_scale, twe, L.ic, each, st));
           gsrc = L.ic;
         } else {
           LITHO_TRY_CUDA(launch_resist(L.img, gp, N, taps, float(threshold), L.blur, nullptr, st));
         }
         LITHO_TRY_CUDA(launch_adj_rows(NE, L.t1, fs, g, C, gsrc, PU, twe, L.u, st, h->d_tw512));
         LITHO_TRY_CUDA(launch_adj_cols(NE, L.u, psi, C, twe, L.sk, g, fs.fields(), st));
-        k_sum_planes<<<dim3(256, g), 256, 0, st>>>(L.sk, adj_col_splits(fs.fields()), size_t(C) * C, L.s,
-                                                   u0 > 0 ? 1 : 0);
-        LITHO_TRY_CUDA(cudaGetLastError());
+        LITHO_TRY_CUDA(launch_pdl(k_sum_planes, dim3(256, g), 256, 0, st, L.sk, adj_col_splits(fs.fields()),
+                                  size_t(C) * C, L.s, u0 > 0 ? 1 : 0));
       }
     }
     ProfScope ps(kStageIltBackward, st, 2);
@@ -922,9 +943,8 @@ litho_status litho_intensity_vjp(const litho_kernels* h, const float* mask_dev, 
     const int g = std::min(G, b - c0);
     LITHO_TRY_CUDA(launch_mask_spectrum(mask_dev + c0 * nn, g, N, C, h->d_tw, L.rowbuf, L.mhat, st));
     if (!upstream_dev) {  // dL/dI = 1 on every pixel of the selected planes: the closed form
-      k_ones_adjoint<<<dim3(128, g), 256, 0, st>>>(L.mhat, h->d_power, sets_of(h, f_first, f_count), size_t(C) * C,
-                                                   float(double(N) * double(N)), L.s);
-      LITHO_TRY_CUDA(cudaGetLastError());
+      LITHO_TRY_CUDA(launch_pdl(k_ones_adjoint, dim3(128, g), 256, 0, st, L.mhat, h->d_power,
+                                sets_of(h, f_first, f_count), size_t(C) * C, float(double(N) * double(N)), L.s));
     }
     for (int f0 = f_first; upstream_dev && f0 < f_first + f_count; f0 += P) {
       int p = std::min(P, f_first + f_count - f0);
@@ -946,16 +966,16 @@ litho_status litho_intensity_vjp(const litho_kernels* h, const float* mask_dev, 
         planes.first[i + 1] = (unsigned char)at;
       }
       if (!in_order) {  // planes with the same fields: their upstreams add up
-        k_sum_upstream<<<dim3(unsigned(std::min<size_t>((nn + 255) / 256, 1024)), g * nu), 256, 0, st>>>(up, nn, nu,
-                                                                                                       planes, L.img);
-        LITHO_TRY_CUDA(cudaGetLastError());
+        LITHO_TRY_CUDA(launch_pdl(k_sum_upstream, dim3(unsigned(std::min<size_t>((nn + 255) / 256, 1024)), g * nu),
+                                  256, 0, st, up, nn, nu, planes, L.img));
         up = L.img;
         p = nu;
       }
       if (coarse) {
-        LITHO_TRY_CUDA(launch_mask_spectrum(up, g * p, N, C2, h->d_tw, L.big, L.spec, st));
-        LITHO_TRY_CUDA(launch_stage1_fft(L.spec, nullptr, g * p, NE, C2, twe, L.mid, st));
-        LITHO_TRY_CUDA(launch_band_rows_real(L.mid, g, p, NE, C2, lp_scale, twe, L.ic, plane_out_identity(p), st));
+        LITHO_TRY_CUDA(launch_mask_rows(up, g * p, N, C2, h->d_tw, L.big, false, st));
+        LITHO_TRY_CUDA(launch_mask_cols(L.big, g * p, N, C2, h->d_tw, L.spec, nullptr, false, st));
+        LITHO_TRY_CUDA(launch_stage1_half(L.spec, g * p, NE, C2, twe, L.mid, C, st));
+        LITHO_TRY_CUDA(launch_band_rows_real(L.mid, g, p, NE, C, lp_scale, twe, L.ic, plane_out_identity(p), st));
         up = L.ic;
       }
       // sets that follow one another in the kernel set share their launches
@@ -967,9 +987,8 @@ litho_status litho_intensity_vjp(const litho_kernels* h, const float* mask_dev, 
         LITHO_TRY_CUDA(
             launch_adj_rows(NE, L.t1, fs, g, C, up + size_t(r0) * NE * NE, p, twe, L.u, st, h->d_tw512));
         LITHO_TRY_CUDA(launch_adj_cols(NE, L.u, psi, C, twe, L.sk, g, fs.fields(), st));
-        k_sum_planes<<<dim3(256, g), 256, 0, st>>>(L.sk, adj_col_splits(fs.fields()), size_t(C) * C, L.s,
-                                                   f0 > f_first || r0 > 0 ? 1 : 0);
-        LITHO_TRY_CUDA(cudaGetLastError());
+        LITHO_TRY_CUDA(launch_pdl(k_sum_planes, dim3(256, g), 256, 0, st, L.sk, adj_col_splits(fs.fields()),
+                                  size_t(C) * C, L.s, f0 > f_first || r0 > 0 ? 1 : 0));
       }
     }
     LITHO_TRY_CUDA(launch_stage1_fft(L.s, nullptr, g, N, C, h->d_tw, L.qf, st));

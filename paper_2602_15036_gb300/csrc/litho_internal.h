@@ -158,19 +158,27 @@ PlaneOut plane_out_identity(int planes);
 // ---- launchers (fft.cu) ---------------------------------------------------------------------
 // The N-entry per-pass twiddle table the FFT kernels expect (false if n unsupported).
 bool fft_twiddle_table(int n, float2* out);
-// Mask spectrum: m[b][n][n] -> mhat[b][C][C] = N^-2 DFT(m) on the crop.  rowbuf: [b][n][C].
-// With `gain` [C] the stored value is mhat (1 + i gain[v] gain[u]) (blur channel, see fft.cu),
-// or with gain_real mhat gain[v] gain[u] (the spectrum of the blurred plane).
+// Mask spectrum: m[b][n][n] -> mhat[b][C][C] = N^-2 DFT(m) on the crop.  rowbuf: [b][n][C/2 + 8].
 cudaError_t launch_mask_spectrum(const float* m, int b, int n, int crop, const float2* tw, float2* rowbuf,
-                                 float2* mhat, cudaStream_t st, const float* gain = nullptr, bool gain_real = false);
-// Row pass of the mask spectrum alone: rowbuf[b][n][C] = row DFT of m, crop columns kept.
-cudaError_t launch_mask_rows(const float* m, int b, int n, int crop, const float2* tw, float2* rowbuf, cudaStream_t st);
-// Column pass of the interpolation from an nc grid to an n grid (interp.cu):
-// q[p][n][c2] = inverse transform on n of the crop c2 of nc^-2 x forward
-// transform on nc of rspec[p][nc][c2] (times 1 + i gain[v] gain[u] with gain).
+                                 float2* mhat, cudaStream_t st);
+// Its two passes.  Row DFTs of real planes, the frequencies u >= 0: rowbuf[b][n][C/2], index u, or (whole:
+// with u = C/2) [b][n][C/2 + 8].
+cudaError_t launch_mask_rows(const float* m, int b, int n, int crop, const float2* tw, float2* rowbuf, bool whole,
+                             cudaStream_t st);
+// Column DFTs times n^-2 on the crop.  whole: mhat[b][C][C]; else only its columns u >= 0 (index u + C/2),
+// times gain[v] gain[u] with gain [C].
+cudaError_t launch_mask_cols(const float2* rowbuf, int b, int n, int crop, const float2* tw, float2* mhat,
+                             const float* gain, bool whole, cudaStream_t st);
+// Column pass of the interpolation from an nc grid to an n grid (interp.cu), for half rows of h columns
+// rspec[p][nc][h]: q[p][n][h] = the inverse transform on n of the crop 2h of nc^-2 x the forward transform
+// on nc; with gain [2h] the same times gain[v] gain[u] (the blur's half rows), or with `image` too both,
+// q[p][n][2][h].
 bool interp_cols_supported(int nc, int n);
-cudaError_t launch_interp_cols(const float2* rspec, int planes, int nc, int n, int c2, const float2* tw_nc,
-                               const float2* tw_n, const float* gain, float2* q, cudaStream_t st);
+cudaError_t launch_interp_cols(const float2* rspec, int planes, int nc, int n, int h, const float2* tw_nc,
+                               const float2* tw_n, const float* gain, bool image, float2* q, cudaStream_t st);
+// Inverse column transform of the columns u >= 0 of spectra spec[nk][C][C]: half rows q[nk][n][ld] (ld >= C/2).
+cudaError_t launch_stage1_half(const float2* spec, int nk, int n, int crop, const float2* tw, float2* q, int ld,
+                               cudaStream_t st);
 // Stage 1 (band multiply + inverse DFT over v): for kernels psi[nk][C][C],
 // t1[j][y][c] = sum_v mhat[v][c] psi_j[v][c] e^{+2 pi i v y/N}, j in [0, nk).
 // psi == NULL transforms nk spectra mhat[j][C][C] themselves.  With kernels,
@@ -184,9 +192,9 @@ cudaError_t launch_stage1_fft(const float2* mhat, const float2* psi, int nk, int
 // (planes of n^2).  With tw32 (the kernel set's d_tw32) a 1024-point row takes
 // the warp-per-row radix-32 kernel, with tw512 (d_tw512) 512-point rows the
 // two-rows-per-warp kernel.  spec (with tw32 only): instead of the image, each
-// image row's forward transform on the spec_crop frequencies |u| < spec_crop/2,
-// laid out as launch_mask_rows writes them ([clips][planes][n][spec_crop]);
-// img is not written.
+// image row's forward transform on the frequencies u in [0, spec_crop/2), laid
+// out as launch_mask_rows writes them ([clips][planes][n][spec_crop/2]); img
+// is not written.
 cudaError_t launch_stage2_fft(const float2* t1, const FieldSet& fs, int clips, int n, int crop, float dose,
                               const float2* tw, float* img, const PlaneOut& po, cudaStream_t st,
                               const float2* tw32 = nullptr, const float2* tw512 = nullptr, float2* spec = nullptr,
@@ -229,18 +237,21 @@ size_t ai_channels_bytes(const litho_kernels* h, int b);
 litho_status ai_channels(const litho_kernels* h, const float* target, int b, double dose, int focus, bool coarse,
                          float* x, void* workspace, cudaStream_t st);
 
-// out[plane][y][x] = scale Re(sum_c q[p][y][c] e^{+2 pi i u_c x/N}) for band rows q[p][N][C] of `clips` x `planes`
-// planes p; plane p of a clip goes to its planes of `po`.
-cudaError_t launch_band_rows_real(const float2* q, int clips, int planes, int n, int crop, float scale,
-                                  const float2* tw, float* out, const PlaneOut& po, cudaStream_t st);
+// Image rows from half band rows q[p][n][h] of `clips` x `planes` planes p, times scale; plane p of a clip
+// goes to its planes of `po` in out.
+cudaError_t launch_band_rows_real(const float2* q, int clips, int planes, int n, int h, float scale, const float2* tw,
+                                  float* out, const PlaneOut& po, cudaStream_t st);
 
 struct ResistTaps;
 // gain[i] = sum_a g[a] cos(2 pi (i - crop/2) a / n): the blur's transfer function on the crop.
 cudaError_t launch_blur_gain(const ResistTaps& taps, int n, int crop, float* gain, cudaStream_t st);
-// Band rows carrying the blur channel: z = sum_c q[p][y][c] e^{+2 pi i u_c x/N};
-// img = Re z (skipped when NULL), iblur = Im z, printed = [Im z >= threshold] (skipped when NULL).
+// Image and blur rows from their half band rows q[p][n][2][h]: img (skipped when NULL), iblur, printed =
+// [iblur >= threshold] (skipped when NULL).
+cudaError_t launch_band_rows_resist(const float2* q, int clips, int planes, int n, int h, const float2* tw,
+                                    float threshold, float* img, float* iblur, uint8_t* printed, const PlaneOut& po,
+                                    cudaStream_t st);
 // ILT forward end on the coarse grid, per pair of full-grid rows: blurred rows from the
-// band rows, sigmoid resist, dL/dI and its row spectra on the crop (rowbuf, as
+// blur's half band rows, sigmoid resist, dL/dI and its half row spectra (rowbuf, as
 // launch_mask_rows), and one FP64 partial loss per row pair at partial[plane][pair]
 // (planes x n/2 doubles).  Plane p uses target clip p / planes_per_clip and counts weight.w[p mod planes_per_clip]
 // times (the focus planes that share its image).
@@ -250,12 +261,6 @@ struct PlaneWeight {
 cudaError_t launch_resist_grad_rows(const float2* band, int planes, int n, int crop, const float2* tw,
                                     const float* target, int planes_per_clip, const PlaneWeight& weight, float beta,
                                     float thr, float2* rowbuf, double* partial, cudaStream_t st);
-// Column half of launch_mask_spectrum on row spectra already in rowbuf.
-cudaError_t launch_mask_cols(const float2* rowbuf, int b, int n, int crop, const float2* tw, float2* mhat,
-                             const float* gain, bool gain_real, cudaStream_t st);
-cudaError_t launch_band_rows_resist(const float2* q, int clips, int planes, int n, int crop, const float2* tw,
-                                    float threshold, float* img, float* iblur, uint8_t* printed, const PlaneOut& po,
-                                    cudaStream_t st);
 
 // ---- rectangle rasterisation (raster.cu) -----------------------------------------------------
 long long raster_tiles_per_rect(int max_side);

@@ -87,11 +87,13 @@ __global__ void __launch_bounds__(Plan<N>::NT * W, Stage1Pipe<Out>::kMinBlocks)
   float2* const blk0 = buf + W * LD;  // Phi (or spectrum) blocks [crop][W], double-buffered
   auto blk = [&](int s) { return blk0 + s * W * crop; };
   const int clip = Out::kRowWise ? blockIdx.y : blockIdx.x, cblk = Out::kRowWise ? blockIdx.x : blockIdx.y;
-  const int tid = threadIdx.x, u0 = cblk * W, half = crop / 2;
+  const int tid = threadIdx.x, u0 = out.first() + cblk * W, half = crop / 2;
   const int j0 = blockIdx.z * jb, j1 = min(nk, j0 + jb), jofs = clip * nk;
   if (j0 >= j1) return;
   mhat += (size_t)clip * crop * crop;
+  pdl_start();
   load_twiddles<N>(tw, tw_g);
+  if (!phi) pdl_wait(mhat);  // the spectra come from the kernel before; Phi is the kernel set's
   const float2* src_base = phi ? phi : mhat;  // the per-j operand
   auto issue = [&](int j, float2* dst) {  // W/2 16-byte pieces per row
     const float2* src = src_base + (size_t)j * crop * crop + u0;
@@ -102,6 +104,7 @@ __global__ void __launch_bounds__(Plan<N>::NT * W, Stage1Pipe<Out>::kMinBlocks)
     cp_async_commit();
   };
   issue(j0, blk(0));
+  if (phi) pdl_wait(mhat);
   const int g = tid % W, t = tid / W;
   auto band_row = [&](int idx) { return (idx < N / 2 ? idx : idx - N) + half; };  // crop row of index idx
   float2 mreg[R0];  // mask spectrum at this thread's first-pass inputs (column u0 + g)
@@ -109,7 +112,7 @@ __global__ void __launch_bounds__(Plan<N>::NT * W, Stage1Pipe<Out>::kMinBlocks)
   for (int r = 0; r < R0; ++r) {
     const int c = band_row(t + r * NB0);
     const bool zero = !phi || t >= NB0 || c < 0 || c >= crop || (BANDED && r >= R0 / 4 && r < 3 * R0 / 4);
-    mreg[r] = zero ? make_float2(0.f, 0.f) : __ldg(mhat + (size_t)c * crop + u0 + g);
+    mreg[r] = zero ? make_float2(0.f, 0.f) : ld_dep(mhat + (size_t)c * crop + u0 + g);
   }
   constexpr bool kSingle = Stage1Pipe<Out>::kBuffers == 1;
   for (int j = j0; j < j1; ++j) {
@@ -144,7 +147,7 @@ __global__ void __launch_bounds__(Plan<N>::NT * W, Stage1Pipe<Out>::kMinBlocks)
       }
     } else {
       float2* const col = out.column(jofs + j, u0 + g);  // element y at col[y crop]
-      auto use = [&](int, int, int y, float2 v) { col[y * crop] = v; };
+      auto use = [&](int, int, int y, float2 v) { col[y * out.ld(crop)] = v; };
       fft_load_use<N, +1, decltype(load), decltype(use), BANDED>(buf + g * LD, tw, t, load, use, refill);
     }
   }
@@ -152,7 +155,7 @@ __global__ void __launch_bounds__(Plan<N>::NT * W, Stage1Pipe<Out>::kMinBlocks)
 
 template <int N, int W, class Out, bool BANDED>
 cudaError_t launch_stage1_cols_t(const float2* mhat, const float2* phi, int nk, int crop, const float2* tw, Out out,
-                                 cudaStream_t st, int clips) {
+                                 cudaStream_t st, int clips, int c_first) {
   // Kernels per CTA: runs of kernels as long as possible (each CTA loads its
   // twiddles and mask values once and starts its copy pipeline once), split
   // so that the CTAs fill whole waves: the fewest waves x (kernels per CTA
@@ -167,7 +170,8 @@ cudaError_t launch_stage1_cols_t(const float2* mhat, const float2* phi, int nk, 
               ? v
               : 152;
   }
-  const long long ctas = (long long)clips * (crop / W), slots = (long long)Stage1Pipe<Out>::kMinBlocks * sms;
+  const int blocks = (crop - c_first) / W;
+  const long long ctas = (long long)clips * blocks, slots = (long long)Stage1Pipe<Out>::kMinBlocks * sms;
   int jblocks = 1;
   long long best = -1;
   for (int jb = 1; jb <= std::min(nk, 32); ++jb) {
@@ -183,20 +187,19 @@ cudaError_t launch_stage1_cols_t(const float2* mhat, const float2* phi, int nk, 
   const size_t sm = sizeof(float2) * Stage1Shape<N, W>::smem_elems(crop, Stage1Pipe<Out>::kBuffers);
   cudaError_t e = smem_attrs(k_stage1_cols<N, W, Out, BANDED>, sm);
   if (e != cudaSuccess) return e;
-  const dim3 grid = Out::kRowWise ? dim3(crop / W, clips, (nk + JB - 1) / JB) : dim3(clips, crop / W, (nk + JB - 1) / JB);
-  k_stage1_cols<N, W, Out, BANDED><<<grid, Plan<N>::NT * W, sm, st>>>(mhat, phi, crop, nk, JB, tw, out);
-  return cudaGetLastError();
+  const dim3 grid = Out::kRowWise ? dim3(blocks, clips, (nk + JB - 1) / JB) : dim3(clips, blocks, (nk + JB - 1) / JB);
+  return launch_pdl(k_stage1_cols<N, W, Out, BANDED>, grid, Plan<N>::NT * W, sm, st, mhat, phi, crop, nk, JB, tw, out);
 }
 
 // W columns per CTA (a divisor of 32; crop is a multiple of 32).  `clips`
 // spectra mhat[clips][C][C] share the kernels (clips must be 1 without them).
-// A crop of at most N/2 takes the banded first pass.
+// A crop of at most N/2 takes the banded first pass.  Columns from c_first on (a multiple of W).
 template <int N, int W, class Out>
 cudaError_t launch_stage1_cols(const float2* mhat, const float2* phi, int nk, int crop, const float2* tw, Out out,
-                               cudaStream_t st, int clips = 1) {
+                               cudaStream_t st, int clips = 1, int c_first = 0) {
   if (clips < 1 || (!phi && clips != 1)) return cudaErrorInvalidValue;
-  if (2 * crop <= N) return launch_stage1_cols_t<N, W, Out, true>(mhat, phi, nk, crop, tw, out, st, clips);
-  return launch_stage1_cols_t<N, W, Out, false>(mhat, phi, nk, crop, tw, out, st, clips);
+  if (2 * crop <= N) return launch_stage1_cols_t<N, W, Out, true>(mhat, phi, nk, crop, tw, out, st, clips, c_first);
+  return launch_stage1_cols_t<N, W, Out, false>(mhat, phi, nk, crop, tw, out, st, clips, c_first);
 }
 
 }  // namespace litho

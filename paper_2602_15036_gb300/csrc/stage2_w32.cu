@@ -47,9 +47,9 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int PENDING>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory"); }
 
-// SPEC: instead of the image row, its forward transform cropped to the c2
-// frequencies |u| < c2/2 (index u + c2/2 of row y of plane p in `spec`, plane
-// stride 1024 c2), as the first step of the exact Fourier interpolation:
+// SPEC: instead of the image row, its forward transform cropped to the c2/2
+// frequencies u in [0, c2/2) (a half row: index u of row y of plane p in
+// `spec`), as the first step of the exact Fourier interpolation:
 // the row x = lane + 32 q is already where the four-step forward transform
 // wants it (pass 1 over q, twiddle e^{-2 pi i lane u1 / 1024}, exchange,
 // pass 2 over the lanes, output u1 + 32 u2 in lane u1).
@@ -62,7 +62,9 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
   float2* tw2 = reinterpret_cast<float2*>(smem_raw);  // w^(r l) at (r - 1) 32 + l
   float2* rowbuf = tw2 + (kR - 1) * kR;                // [kWarps][kRowLd]
   float2* stage0 = rowbuf + kWarps * kRowLd;           // [kWarps][crop]
+  pdl_start();
   for (int i = threadIdx.x; i < (kR - 1) * kR; i += blockDim.x) tw2[i] = tw2_g[i];
+  pdl_wait();
   __syncthreads();
   const int lane = threadIdx.x % 32, wp = threadIdx.x / 32;
   const int y = blockIdx.x * kWarps + wp, plane = blockIdx.y, half = crop / 2;
@@ -130,12 +132,12 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
 #pragma unroll
     for (int l = 0; l < kR; ++l) v[l] = buf[lane + (kR + 1) * l];
     dft32<-1, false>(v);
-    float2* srow = spec + (size_t)plane * kN * c2 + (size_t)y * c2;
     const int h2 = c2 / 2;
+    float2* srow = spec + ((size_t)plane * kN + y) * h2;
 #pragma unroll
-    for (int u2 = 0; u2 < kR; ++u2) {
-      const int u = lane + kR * u2, us = u < kN / 2 ? u : u - kN;
-      if (us >= -h2 && us < h2) srow[us + h2] = v[u2];
+    for (int u2 = 0; u2 < kR / 2; ++u2) {
+      const int u = lane + kR * u2;
+      if (u < h2) srow[u] = v[u2];
     }
   } else {
     for (int d = po.first[pl]; d < po.first[pl + 1]; ++d) {
@@ -153,8 +155,8 @@ cudaError_t launch_w32_k(const float2* t1, const FieldSet& fs, int clips, int cr
   const size_t sm = sizeof(float2) * ((kR - 1) * kR + kWarps * kRowLd + size_t(kWarps) * crop);
   cudaError_t e = smem_attrs(k_stage2_w32<BANDED, kWarps, SPEC>, sm);
   if (e != cudaSuccess) return e;
-  k_stage2_w32<BANDED, kWarps, SPEC><<<grid, 32 * kWarps, sm, st>>>(t1, fs, crop, dose, tw2, img, po, spec, c2);
-  return cudaGetLastError();
+  return launch_pdl(k_stage2_w32<BANDED, kWarps, SPEC>, grid, 32 * kWarps, sm, st, t1, fs, crop, dose, tw2, img, po,
+                    spec, c2);
 }
 
 template <int kWarps>
@@ -186,7 +188,9 @@ __global__ void __launch_bounds__(32 * kW512Warps, 2)
   float2* tw = reinterpret_cast<float2*>(smem_raw);  // (r - 1) 16 + j
   float2* bufs = tw + 31 * 16;                        // [warp][2 rows][kW512Buf]
   float2* stage0 = bufs + kW512Warps * 2 * kW512Buf;  // [warp][2 rows][crop]
+  pdl_start();
   for (int i = threadIdx.x; i < 31 * 16; i += blockDim.x) tw[i] = tw_g[i];
+  pdl_wait();
   __syncthreads();
   const int lane = threadIdx.x % 32, wp = threadIdx.x / 32, half = crop / 2;
   const int y0 = (blockIdx.x * kW512Warps + wp) * 2, plane = blockIdx.y;
@@ -275,8 +279,7 @@ cudaError_t launch_stage2_w512(const float2* t1, const FieldSet& fs, int clips, 
                               : k_stage2_w512<false>;
   cudaError_t e = smem_attrs(kern, sm);
   if (e != cudaSuccess) return e;
-  kern<<<grid, 32 * kW512Warps, sm, st>>>(t1, fs, crop, dose, tw512, img, po);
-  return cudaGetLastError();
+  return launch_pdl(kern, grid, 32 * kW512Warps, sm, st, t1, fs, crop, dose, tw512, img, po);
 }
 
 cudaError_t launch_stage2_w32(const float2* t1, const FieldSet& fs, int clips, int n, int crop, float dose,
