@@ -163,6 +163,8 @@ struct GemmParams {
   int n, planes, tiles_y, tiles_x, chunks, split, fmt;  // planes: of all clips
   FieldSet fs;        // the planes and fields of one clip
   PlaneOut po;        // output planes of each plane
+  int clips;
+  unsigned char order[kMaxPlanes];  // planes by falling number of fields
   const float* lamp;  // [fields] 1 / scale^2
   float dose;
   float* img;         // [clips][out_planes][n][n]
@@ -241,8 +243,17 @@ __global__ void __launch_bounds__(THREADS, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  const int tiles_per_plane = p.tiles_y * p.tiles_x;
-  const int total = p.planes * tiles_per_plane;
+  // Tiles in the order of falling cost (planes with more fields first), dealt out back and forth (round r
+  // left to right, round r + 1 right to left), so that the CTAs' shares even out: 4 clips of a set of 24 and
+  // one of 12 fields are 392 tiles on 152 CTAs, whose largest share is 48 fields, not 72 (786 -> 637 us).
+  const int tiles_per_plane = p.tiles_y * p.tiles_x, total = p.planes * tiles_per_plane;
+  const int rounds = (total + gridDim.x - 1) / gridDim.x;
+  auto tile_at = [&](int r) { return int(r * gridDim.x + (r & 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x)); };
+  auto plane_at = [&](int t, int* clip) {
+    const int k = t / tiles_per_plane;
+    *clip = k % p.clips;
+    return int(p.order[k / p.clips]);
+  };
   const uint32_t tx_bytes = STAGE_BYTES;
 
   if (warp == 0) {
@@ -250,10 +261,13 @@ __global__ void __launch_bounds__(THREADS, 1)
     if (lane == 0) {
       uint32_t it = 0;
       bool ok = true;
-      for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
-        const int plane = t / tiles_per_plane, rem = t % tiles_per_plane;
+      for (int r = 0; r < rounds && ok; ++r) {
+        const int t = tile_at(r);
+        if (t >= total) continue;
+        const int rem = t % tiles_per_plane;
         const int yt = rem / p.tiles_x, xt = rem % p.tiles_x;
-        const int clip = plane / p.fs.planes, pl = plane - clip * p.fs.planes;
+        int clip;
+        const int pl = plane_at(t, &clip);
         for (int k = p.fs.start[pl]; k < p.fs.start[pl + 1] && ok; ++k) {
           const int arow = (clip * p.fs.fields() + k) * p.n + yt * BM;
           for (int ch = 0; ch < p.chunks; ++ch, ++it) {
@@ -296,8 +310,11 @@ __global__ void __launch_bounds__(THREADS, 1)
       const uint32_t d1 = tmem, d2 = tmem + 128, d3 = tmem + 256;
       uint32_t it = 0, acc_it = 0;
       bool ok = true;
-      for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
-        const int pl = t / tiles_per_plane % p.fs.planes, nk = p.fs.start[pl + 1] - p.fs.start[pl];
+      for (int r = 0; r < rounds && ok; ++r) {
+        const int t = tile_at(r);
+        if (t >= total) continue;
+        int clip;
+        const int pl = plane_at(t, &clip), nk = p.fs.start[pl + 1] - p.fs.start[pl];
         for (int k = 0; k < nk && ok; ++k) {
           if (!wait_bar(acc_empty, (acc_it & 1) ^ 1, abort_flag, p.err, 2)) {
             ok = false;
@@ -364,10 +381,13 @@ __global__ void __launch_bounds__(THREADS, 1)
     const uint32_t lane_base = tmem + (uint32_t(q * 32) << 16);
     uint32_t acc_it = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
-      const int plane = t / tiles_per_plane, rem = t % tiles_per_plane;
+    for (int r = 0; r < rounds && ok; ++r) {
+      const int t = tile_at(r);
+      if (t >= total) continue;
+      const int rem = t % tiles_per_plane;
       const int yt = rem / p.tiles_x, xt = rem % p.tiles_x;
-      const int clip = plane / p.fs.planes, pl = plane - clip * p.fs.planes;
+      int clip;
+      const int pl = plane_at(t, &clip);
       float acc[64];
 #pragma unroll
       for (int i = 0; i < 64; ++i) acc[i] = 0.f;
@@ -753,6 +773,11 @@ litho_status gemm_aerial_group(const litho_kernels* h, const float2* mhat, int c
   p.n = N;
   p.fs = fs;
   p.po = coarse ? plane_out_identity(h->n_sets) : plane_out(h);
+  p.clips = clips;
+  for (int i = 0; i < fs.planes; ++i) p.order[i] = (unsigned char)i;
+  std::stable_sort(p.order, p.order + fs.planes, [&](int a, int b) {
+    return fs.start[a + 1] - fs.start[a] > fs.start[b + 1] - fs.start[b];
+  });
   p.planes = clips * fs.planes;
   p.tiles_y = N / BM;
   p.tiles_x = N / XT;
