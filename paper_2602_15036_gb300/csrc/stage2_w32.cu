@@ -289,7 +289,12 @@ cudaError_t launch_stage2_w32(const float2* t1, const FieldSet& fs, int clips, i
   if (spec && (c2 < 2 || c2 > kN || c2 % 2 != 0)) return cudaErrorInvalidValue;
   // 12 warps per CTA: one CTA of 384 threads fits the SM's registers (about 160 per thread);
   // measured on the 2048^2 workload's 1024-point rows: 5.90 ms per step against 6.29 with 8
-  // warps and 6.04 with 16 (128 registers)
+  // warps and 6.04 with 16 (128 registers).  A plane or two leave SMs without a CTA, or a second wave
+  // nearly empty: 7 warps then (147 CTAs a plane; one plane of 12 fields 32.0 -> 24.4 us).  A wave takes
+  // about (warps + 4) units of time.
+  const long long planes = (long long)clips * fs.planes;
+  auto cost = [&](int warps) { return (planes * ((kN + warps - 1) / warps) + 151) / 152 * (warps + 4); };
+  if (cost(7) < cost(12)) return launch_w32_t<7>(t1, fs, clips, crop, dose, tw2, img, po, st, spec, c2);
   return launch_w32_t<12>(t1, fs, clips, crop, dose, tw2, img, po, st, spec, c2);
 }
 
