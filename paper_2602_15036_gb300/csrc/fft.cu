@@ -30,9 +30,9 @@ __device__ __forceinline__ int freq_of(int idx, int n) { return idx < n / 2 ? id
 
 // ---- mask spectrum, pass 1: two real rows per complex transform ----------------------------
 // z = m[y0] + i m[y1]; Z = DFT(z); X(u) = (Z(u) + conj Z(-u))/2, Y(u) = (Z(u) - conj Z(-u))/(2i),
-// written for u in [0, cols) with row stride ld.
-template <int N>
-__global__ void __launch_bounds__(Plan<N>::NT) k_mask_rows(const float* __restrict__ m, int crop,
+// written for u in [0, cols) with row stride ld.  SIGMOID: the mask is sigmoid(alpha m) (the ILT's theta).
+template <int N, bool SIGMOID>
+__global__ void __launch_bounds__(Plan<N>::NT) k_mask_rows(const float* __restrict__ m, float alpha, int crop,
                                                             const float2* __restrict__ tw_g,
                                                             float2* __restrict__ rowbuf, int cols, int ld,
                                                             int pairs_per_cta) {
@@ -55,6 +55,7 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_mask_rows(const float* __restri
     for (int r = 0; r < R0; ++r)
       nxt[r] = t < NB0 ? make_float2(ld_dep(r0 + t + r * NB0), ld_dep(r0 + N + t + r * NB0)) : make_float2(0.f, 0.f);
   };
+  auto value = [&](float2 v) { return SIGMOID ? make_float2(sigmoidf(alpha * v.x), sigmoidf(alpha * v.y)) : v; };
   const int pr0 = blockIdx.x * pairs_per_cta, pr1 = min(N / 2, (blockIdx.x + 1) * pairs_per_cta);
   if (pr0 < pr1) prefetch(pr0);
   // pairs [pr0, pr1): the next pair's first pass writes buf only after a
@@ -64,7 +65,7 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_mask_rows(const float* __restri
     float2 cur[R0];
 #pragma unroll
     for (int r = 0; r < R0; ++r) cur[r] = nxt[r];
-    auto load = [&](int, int r, int) { return cur[r]; };
+    auto load = [&](int, int r, int) { return value(cur[r]); };
     auto use = [&](int, int, int idx, float2 v) {
       const int u = freq_of(idx, N);
       if (u >= -half && u <= half) zc[u + half] = v;
@@ -138,16 +139,15 @@ __global__ void __launch_bounds__(Plan<N>::NT * W) k_mask_cols(const float2* __r
 // exactly in integers before cospi.
 __global__ void k_blur_gain(ResistTaps taps, int n, int crop, float* __restrict__ gain) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  pdl_start();
-  pdl_wait();
-  if (i >= crop) return;
+  pdl_start();  // the sum needs nothing from the kernel before: only the store waits for it
   const int f = i - crop / 2, r = taps.radius;
   float acc = taps.g[r];
   for (int a = 1; a <= r; ++a) {
     const long long e = ((long long)f * a % n + n) % n;  // f a mod n, in [0, n)
     acc = fmaf(2.0f * taps.g[r + a], cospif(2.0f * float(e) / float(n)), acc);
   }
-  gain[i] = acc;
+  pdl_wait();
+  if (i < crop) gain[i] = acc;
 }
 
 // ---- stage 1: band multiply + inverse transform over v (stage1.cuh), FP32 output ------------------
@@ -175,21 +175,31 @@ struct OutHalf {
 };
 
 // ---- stage 2 (FP32 path): one image row per CTA, all kernels of the plane ------------------------
+// Rows of up to 256 points are one warp's: kGroups warps share the plane's kernels (warp w takes kernels w,
+// w + kGroups, ...) and their sums are added in order, so that a row's chain of transforms, which a small
+// call waits for, is that much shorter (2 planes of 256^2, 8 and 4 fields: 11.1 -> 7.9 us).
+template <int N>
+struct Stage2Groups {
+  static constexpr int value = Plan<N>::NT == 32 ? 2 : 1;
+};
+
 template <int N, bool BANDED>
-__global__ void __launch_bounds__(Plan<N>::NT, 512 / Plan<N>::NT) k_stage2(const float2* __restrict__ t1, const __grid_constant__ FieldSet fs,
-                                                        int crop, float dose, const float2* __restrict__ tw_g,
-                                                        float* __restrict__ img, const __grid_constant__ PlaneOut po) {
+__global__ void __launch_bounds__(Plan<N>::NT * Stage2Groups<N>::value, 512 / Plan<N>::NT / Stage2Groups<N>::value)
+    k_stage2(const float2* __restrict__ t1, const __grid_constant__ FieldSet fs, int crop, float dose,
+             const float2* __restrict__ tw_g, float* __restrict__ img, const __grid_constant__ PlaneOut po) {
   using PL = Plan<N>;
-  constexpr int NT = PL::NT;
+  constexpr int NT = PL::NT, G = Stage2Groups<N>::value;
   constexpr int RL = PL::R[PL::P - 1];
   constexpr int PERL = PassShape<N, NT, RL>::PER;
-  __shared__ float2 buf[PadLen<N>::value];
+  __shared__ float2 bufs[G][PadLen<N>::value];
   __shared__ float2 tw[N];
+  __shared__ float part[G > 1 ? G - 1 : 1][G > 1 ? N : 1];
   pdl_start();
   load_twiddles<N>(tw, tw_g);
   pdl_wait(t1);
   __syncthreads();
-  const int y = blockIdx.x, plane = blockIdx.y, t = threadIdx.x, half = crop / 2;
+  const int y = blockIdx.x, plane = blockIdx.y, t = threadIdx.x % NT, grp = threadIdx.x / NT, half = crop / 2;
+  float2* buf = bufs[grp];
   const int clip = plane / fs.planes, pl = plane - clip * fs.planes, nk = fs.start[pl + 1] - fs.start[pl];
   const float2* base = t1 + ((size_t)(clip * fs.fields() + fs.start[pl]) * N + y) * crop;
   float acc[PERL][RL];
@@ -203,17 +213,34 @@ __global__ void __launch_bounds__(Plan<N>::NT, 512 / Plan<N>::NT) k_stage2(const
   constexpr bool kMid = MidTwiddles<N, +1>::kUsable && N >= 2048;
   MidTwiddles<N, +1> mid;
   if constexpr (kMid) mid.load(tw, t);
-  for (int j = 0; j < nk; ++j) {
+  for (int j0 = 0; j0 < nk; j0 += G) {
+    const int j = j0 + grp;
+    const bool live = G == 1 || j < nk;  // every warp runs every round (block barriers)
     const float2* row = base + (size_t)j * N * crop;
     auto load = [&](int, int r, int idx) {
       const int c = (r < PL::R[0] / 2 ? idx : idx - N) + half;  // first pass: idx < N/2 exactly when r < R/2
-      return (c >= 0 && c < crop) ? ld_dep(row + c) : make_float2(0.f, 0.f);
+      return (live && c >= 0 && c < crop) ? ld_dep(row + c) : make_float2(0.f, 0.f);
     };
     auto use = [&](int p, int q, int, float2 v) { acc[p][q] = fmaf(v.x, v.x, fmaf(v.y, v.y, acc[p][q])); };
     if constexpr (kMid)
       fft_load_use_mid<N, +1, decltype(load), decltype(use), BANDED>(buf, tw, t, load, use, mid);
     else
       fft_load_use<N, +1, decltype(load), decltype(use), BANDED>(buf, tw, t, load, use);
+  }
+  if constexpr (G > 1) {
+#pragma unroll
+    for (int p = 0; p < PERL; ++p)
+#pragma unroll
+      for (int q = 0; q < RL; ++q)
+        if (grp > 0 && t + p * NT < N / RL) part[grp - 1][t + p * NT + q * (N / RL)] = acc[p][q];
+    __syncthreads();
+    if (grp > 0) return;
+#pragma unroll
+    for (int p = 0; p < PERL; ++p)
+#pragma unroll
+      for (int q = 0; q < RL; ++q)
+        for (int w = 0; w < G - 1; ++w)
+          if (t + p * NT < N / RL) acc[p][q] += part[w][t + p * NT + q * (N / RL)];
   }
   for (int d = po.first[pl]; d < po.first[pl + 1]; ++d) {
     float* out = img + ((size_t)(clip * po.out_planes + po.list[d]) * N + y) * N;
@@ -401,23 +428,6 @@ __global__ void __launch_bounds__(Plan<N>::NT, N >= 512 ? 640 / Plan<N>::NT : 1)
   }
 }
 
-// Rows per CTA for the one-row-per-transform kernels: enough CTAs for about
-// eight waves of `per_sm` CTAs per SM, each CTA reusing its twiddle table
-// for its rows.
-inline int rows_per_cta(int rows, int planes, int per_sm) {
-  static int sms = 0;  // the same GPU model throughout a process
-  if (!sms) {
-    int dev = 0, v = 0;
-    sms = cudaGetDevice(&dev) == cudaSuccess &&
-                  cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0
-              ? v
-              : 152;
-  }
-  const long long want = 8LL * sms * per_sm;
-  const long long r = std::max<long long>(1, ((long long)rows * planes) / want);
-  return int(std::min<long long>(r, rows));
-}
-
 template <int N, bool RESIST>
 cudaError_t band_rows_n(const float2* q, int clips, int planes, int h, float scale, const float2* tw, float thr,
                         float* img, float* iblur, uint8_t* printed, const PlaneOut& po, cudaStream_t st) {
@@ -470,13 +480,14 @@ cudaError_t mask_cols_n(const float2* rowbuf, int b, int crop, const float2* tw,
 }
 
 template <int N>
-cudaError_t mask_rows_n(const float* m, int b, int crop, const float2* tw, float2* rowbuf, bool whole,
+cudaError_t mask_rows_n(const float* m, bool sigmoid, float alpha, int b, int crop, const float2* tw, float2* rowbuf, bool whole,
                         cudaStream_t st) {
   const size_t smr = sizeof(float2) * (2 * N + PadLen<N>::value + 1);
-  cudaError_t e = smem_attrs(k_mask_rows<N>, smr);
+  auto kern = sigmoid ? k_mask_rows<N, true> : k_mask_rows<N, false>;
+  cudaError_t e = smem_attrs(kern, smr);
   if (e != cudaSuccess) return e;
   const int ppc = rows_per_cta(N / 2, b, 2048 / Plan<N>::NT);
-  return launch_pdl(k_mask_rows<N>, dim3((N / 2 + ppc - 1) / ppc, b), Plan<N>::NT, smr, st, m, crop, tw, rowbuf,
+  return launch_pdl(kern, dim3((N / 2 + ppc - 1) / ppc, b), Plan<N>::NT, smr, st, m, alpha, crop, tw, rowbuf,
                     half_cols(crop, whole), half_ld(crop, whole), ppc);
 }
 
@@ -498,7 +509,8 @@ template <int N>
 cudaError_t stage2_n(const float2* t1, const FieldSet& fs, int clips, int crop, float dose, const float2* tw,
                      float* img, const PlaneOut& po, cudaStream_t st) {
   auto kern = 2 * crop <= N ? k_stage2<N, true> : k_stage2<N, false>;
-  return launch_pdl(kern, dim3(N, clips * fs.planes), Plan<N>::NT, 0, st, t1, fs, crop, dose, tw, img, po);
+  return launch_pdl(kern, dim3(N, clips * fs.planes), Plan<N>::NT * Stage2Groups<N>::value, 0, st, t1, fs, crop, dose,
+                    tw, img, po);
 }
 
 // Transform sizes of the full grid (powers of two) ...
@@ -559,9 +571,20 @@ cudaError_t launch_band_rows_real(const float2* q, int clips, int planes, int n,
 
 cudaError_t launch_mask_rows(const float* m, int b, int n, int crop, const float2* tw, float2* rowbuf, bool whole,
                              cudaStream_t st) {
-#define CALL(N) mask_rows_n<N>(m, b, crop, tw, rowbuf, whole, st)
+#define CALL(N) mask_rows_n<N>(m, false, 0.f, b, crop, tw, rowbuf, whole, st)
   LITHO_DISPATCH_NC(n, CALL)
 #undef CALL
+}
+
+cudaError_t launch_sigmoid_spectrum(const float* theta, float alpha, int b, int n, int crop, const float2* tw,
+                                    float2* rowbuf, float2* mhat, cudaStream_t st) {
+  auto rows = [&]() {
+#define CALL(N) mask_rows_n<N>(theta, true, alpha, b, crop, tw, rowbuf, true, st)
+    LITHO_DISPATCH_N(n, CALL)
+#undef CALL
+  };
+  const cudaError_t e = rows();
+  return e != cudaSuccess ? e : launch_mask_cols(rowbuf, b, n, crop, tw, mhat, nullptr, true, st);
 }
 
 cudaError_t launch_blur_gain(const ResistTaps& taps, int n, int crop, float* gain, cudaStream_t st) {

@@ -24,11 +24,14 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 #include <utility>
 
 namespace litho {
+
+__device__ __forceinline__ float sigmoidf(float x) { return 1.0f / (1.0f + expf(-x)); }
 
 // Complex arithmetic on the packed two-lane FP32 instructions of sm_100+
 // (one instruction for both components, each rounded as the scalar form).
@@ -621,6 +624,23 @@ inline cudaError_t smem_attrs(K kernel, size_t bytes) {
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+}
+
+// Rows per CTA for the one-row-per-transform kernels: enough CTAs for about
+// eight waves of `per_sm` CTAs per SM, each CTA reusing its twiddle table
+// for its rows.
+inline int rows_per_cta(int rows, int planes, int per_sm) {
+  static int sms = 0;  // the same GPU model throughout a process
+  if (!sms) {
+    int dev = 0, v = 0;
+    sms = cudaGetDevice(&dev) == cudaSuccess &&
+                  cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0
+              ? v
+              : 152;
+  }
+  const long long want = 8LL * sms * per_sm;
+  const long long r = std::max<long long>(1, ((long long)rows * planes) / want);
+  return int(std::min<long long>(r, rows));
 }
 
 // Stage the twiddle table (N entries, see above) into shared memory.

@@ -13,18 +13,17 @@
 //   dL/dm(x) = 2 D N^-2 Re sum_u S(u) e^{+2 pi i u.x/N},  dL/dtheta = dL/dm a m (1 - m).
 //
 // Kernels (per clip, for a group of P focus planes at a time):
-//   k_sigmoid        m from theta
-//   (mask spectrum, stage 1, stage 2, resist blur: shared with the forward path)
+//   (mask spectrum of sigmoid(a theta), stage 1, stage 2, resist blur: shared with the forward path)
 //   k_resist_grad    Z, q and per-block FP64 partial sums of (Z - target)^2
 //                    (coarse grid: k_resist_grad_rows, per row pair, with the
 //                    forward row spectra of q)
-//   k_reduce_loss    fixed-order FP64 sum of the partials (deterministic)
 //   k_adj_rows       per image row: E_fk from the stage-1 field (inverse FFT),
 //                    times G_f, forward FFT, crop columns -> U_fk[y][c]
 //   k_adj_cols       per crop column block and run of a clip's fields: forward
 //                    FFT over y, crop rows, times conj(Psi), summed over
 //                    the run in registers -> one partial S per run
-//   k_sum_planes     S = sum of a clip's runs in fixed order
+//   k_sum_planes     S = sum of a clip's runs in fixed order, and the fixed-order
+//                    FP64 sum of its loss partials (deterministic)
 //   k_grad_rows      band-to-full inverse of S along x (after stage 1 along y),
 //                    real part, chain factor -> dL/dtheta
 // The fields E are never stored: each backward row recomputes E_fk from the
@@ -42,17 +41,6 @@ namespace {
 constexpr int kPartials = 1024;  // blocks of k_resist_grad, fixed for a deterministic reduction
 
 __device__ __forceinline__ int freq_of_idx(int idx, int n) { return idx < n / 2 ? idx : idx - n; }
-
-// m = sigmoid(alpha theta), four values per thread and step (count a multiple of 4, 16-byte aligned)
-__global__ void k_sigmoid(const float4* __restrict__ theta, float alpha, float4* __restrict__ m, size_t count4) {
-  pdl_start();
-  pdl_wait(theta);
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count4; i += (size_t)gridDim.x * blockDim.x) {
-    const float4 t = ld_dep(theta + i);
-    m[i] = make_float4(1.0f / (1.0f + expf(-alpha * t.x)), 1.0f / (1.0f + expf(-alpha * t.y)),
-                       1.0f / (1.0f + expf(-alpha * t.z)), 1.0f / (1.0f + expf(-alpha * t.w)));
-  }
-}
 
 // Clip blockIdx.y: its `planes` planes of ib and q, its target, its
 // kPartials partial sums (the same partition for every group size).
@@ -94,29 +82,11 @@ __global__ void __launch_bounds__(256) k_resist_grad(const float* __restrict__ i
   }
 }
 
-// Clip blockIdx.x: out[clip] (+)= the fixed-order sum of its `count` partials.
-__global__ void __launch_bounds__(1024) k_reduce_loss(const double* __restrict__ partial, int count,
-                                                      double* __restrict__ out, int accumulate) {
-  __shared__ double s[1024];
-  pdl_start();
-  pdl_wait(partial);
-  partial += (size_t)blockIdx.x * count;
-  out += blockIdx.x;
-  double a = 0.0;
-  for (int i = threadIdx.x; i < count; i += 1024) a += ld_dep(partial + i);
-  s[threadIdx.x] = a;
-  __syncthreads();
-  for (int w = 512; w > 0; w >>= 1) {
-    if (threadIdx.x < w) s[threadIdx.x] += s[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *out = (accumulate ? *out : 0.0) + s[0];
-}
-
 // Backward rows: for every kernel of the plane, E = inverse FFT of the band row
 // T[y][:], P = G[y][:] E, U[y][c] = forward FFT of P on the crop columns.
 // Planes of a clip and their fields as in `fs`; plane pl of clip i takes G at plane i g_planes + pl of g.
 // BANDED (2 crop <= N): the band row's zero half is skipped in the first pass.
+// CTA z of gridDim.z takes every gridDim.z-th field of its plane (the fields are independent).
 template <int N, bool BANDED>
 __global__ void __launch_bounds__(Plan<N>::NT) k_adj_rows(const float2* __restrict__ t1,
                                                           const __grid_constant__ FieldSet fs, int crop,
@@ -144,7 +114,7 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_adj_rows(const float2* __restri
       gv[p][q] = jj < N / RL ? ld_dep(grow + jj + q * (N / RL)) : 0.f;
     }
   __syncthreads();
-  for (int k = fs.start[pl]; k < fs.start[pl + 1]; ++k) {
+  for (int k = fs.start[pl] + blockIdx.z; k < fs.start[pl + 1]; k += gridDim.z) {
     const size_t rowoff = ((size_t)(clip * fs.fields() + k) * N + y) * crop;
     const float2* row = t1 + rowoff;
     auto load_band = [&](int, int r, int idx) {
@@ -231,8 +201,9 @@ __global__ void __launch_bounds__(32 * kAdjWarps, 2)
     for (int i = lane; i < crop; i += 32) adj_cp16(stage + 2 * i, src + 2 * i);
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  if (nk > 0) fetch(0);
-  for (int k = 0; k < nk; ++k) {
+  const int kz = gridDim.z;
+  if (int(blockIdx.z) < nk) fetch(blockIdx.z);
+  for (int k = blockIdx.z; k < nk; k += kz) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncwarp();
     // inverse pass 1 for both rows (lane l: x[l + 32 r])
@@ -251,8 +222,8 @@ __global__ void __launch_bounds__(32 * kAdjWarps, 2)
         }
       }
     }
-    __syncwarp();  // both band rows are in registers: the staging buffer takes kernel k + 1
-    if (k + 1 < nk) fetch(k + 1);
+    __syncwarp();  // both band rows are in registers: the staging buffer takes the next kernel
+    if (k + kz < nk) fetch(k + kz);
 #pragma unroll
     for (int row = 0; row < 2; ++row) {
       dft_reg<16, +1, BANDED>(a[row]);
@@ -316,11 +287,12 @@ template <int N> struct AdjW { static constexpr int W = Plan<N>::NT <= 64 ? 8 : 
 // cost the 1024-point one (twice the slots); so shared memory up to 512.
 template <int N> struct AdjAccInSmem { static constexpr bool value = N <= 512; };
 
-// Runs of fields per clip in the adjoint columns: at most 8, of equal length
-// but for the last (a function of the clip's field count alone, so a clip's
-// sums do not depend on how many clips a launch holds).
+// Runs of fields per clip in the adjoint columns: one field each for up to 16
+// fields (a small call's chain of transforms is then one long: 12 fields of 256^2 13.6 -> 10.0 us), else at most
+// 8 runs of equal length but for the last.  A function of the clip's field
+// count alone, so a clip's sums do not depend on how many clips a launch holds.
 int adj_col_splits(int period) {
-  const int per = std::max(1, (period + 7) / 8);
+  const int per = period <= 16 ? 1 : (period + 7) / 8;
   return std::max(1, (period + per - 1) / per);
 }
 
@@ -454,14 +426,34 @@ __global__ void k_sum_upstream(const float* __restrict__ up, size_t nn, int nu, 
   }
 }
 
-// s[clip] (+)= sum over the clip's `planes` planes of sk, in order (clip = blockIdx.y).
-__global__ void k_sum_planes(const float2* __restrict__ sk, int planes, size_t cc, float2* __restrict__ s,
-                             int accumulate) {
+// s[clip] (+)= sum over the clip's `planes` planes of sk, in order (clip = blockIdx.y).  With `partial`, the
+// last block of a clip forms its loss instead: loss[clip] (+)= the fixed-order FP64 sum of its `count`
+// partials (a kernel of its own took a launch's 6 us of every small step).
+__global__ void __launch_bounds__(256) k_sum_planes(const float2* __restrict__ sk, int planes, size_t cc,
+                                                    float2* __restrict__ s, int accumulate,
+                                                    const double* __restrict__ partial, int count,
+                                                    double* __restrict__ loss) {
   pdl_start();
-  pdl_wait(sk);
+  pdl_wait(sk, partial);
+  const int blocks = gridDim.x - (partial ? 1 : 0);
+  if (int(blockIdx.x) == blocks) {
+    __shared__ double w[8];
+    partial += (size_t)blockIdx.y * count;
+    double a = 0.0;
+    for (int i = threadIdx.x; i < count; i += blockDim.x) a += ld_dep(partial + i);
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+    if (threadIdx.x % 32 == 0) w[threadIdx.x / 32] = a;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = accumulate ? loss[blockIdx.y] : 0.0;
+      for (int i = 0; i < 8; ++i) t += w[i];
+      loss[blockIdx.y] = t;
+    }
+    return;
+  }
   sk += (size_t)blockIdx.y * planes * cc;
   s += (size_t)blockIdx.y * cc;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < cc; i += (size_t)gridDim.x * blockDim.x) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < cc; i += (size_t)blocks * blockDim.x) {
     float2 a = accumulate ? s[i] : make_float2(0.f, 0.f);
     for (int j = 0; j < planes; ++j) {
       const float2 v = ld_dep(sk + (size_t)j * cc + i);
@@ -472,62 +464,86 @@ __global__ void k_sum_planes(const float2* __restrict__ sk, int planes, size_t c
   }
 }
 
-// Final rows: grad[y][x] = scale Re(sum_c Q[y][c] e^{2 pi i u_c x/N}) a m (1 - m).
-template <int N>
+// The adjoint columns' runs of g clips into s; with partial, the clips' losses too.
+cudaError_t launch_sum_planes(const float2* sk, int runs, size_t cc, float2* s, int accumulate, int g,
+                              const double* partial, int count, double* loss, cudaStream_t st) {
+  const unsigned blocks = unsigned(std::min<size_t>(256, (cc + 255) / 256)) + (partial ? 1 : 0);
+  return launch_pdl(k_sum_planes, dim3(blocks, g), 256, 0, st, sk, runs, cc, s, accumulate, partial, count, loss);
+}
+
+// Final rows: grad[y][x] = scale Re(sum_c Q[y][c] e^{2 pi i u_c x/N}), times a m (1 - m) with theta (m =
+// sigmoid(a theta)).  rows_per_cta rows per CTA share its twiddle table.  BANDED: 2 crop <= N.
+template <int N, bool BANDED>
 __global__ void __launch_bounds__(Plan<N>::NT) k_grad_rows(const float2* __restrict__ qf, int crop, float scale,
-                                                           const float* __restrict__ m, float alpha,
+                                                           const float* __restrict__ theta, float alpha,
                                                            const float2* __restrict__ tw_g, float* __restrict__ grad,
-                                                           long long grad_stride) {
+                                                           long long grad_stride, int rows_per_cta) {
   extern __shared__ float2 sm[];
   float2* tw = sm;
   float2* buf = sm + N;
   pdl_start();
   load_twiddles<N>(tw, tw_g);
-  pdl_wait(qf, m);
+  pdl_wait(qf, theta);
   __syncthreads();
-  const int y = blockIdx.x, t = threadIdx.x, half = crop / 2;
-  const size_t clip = blockIdx.y;  // clip of the group: its band rows, mask and gradient
-  qf += clip * N * crop;
-  if (m) m += clip * N * N;
-  grad += clip * grad_stride;
-  const float2* row = qf + (size_t)y * crop;
-  auto load = [&](int idx) {
-    const int c = freq_of_idx(idx, N) + half;
-    return (c >= 0 && c < crop) ? ld_dep(row + c) : make_float2(0.f, 0.f);
-  };
-  const float* mr = m ? m + (size_t)y * N : nullptr;
-  float* gr = grad + (size_t)y * N;
+  const int t = threadIdx.x, half = crop / 2;
+  const size_t clip = blockIdx.y;  // clip of the group: its band rows, theta and gradient
   constexpr int NT = Plan<N>::NT, RL = Plan<N>::R[Plan<N>::P - 1], PERL = PassShape<N, NT, RL>::PER;
-  float mm[PERL][RL];  // the mask at this thread's outputs, loaded while the later passes run
-  auto after_first = [&]() {
+  for (int y = blockIdx.x * rows_per_cta; y < min(N, int(blockIdx.x + 1) * rows_per_cta); ++y) {
+    const float2* row = qf + (clip * N + y) * crop;
+    const float* th = theta ? theta + (clip * N + y) * N : nullptr;
+    auto load = [&](int, int r, int idx) {
+      const int c = (r < Plan<N>::R[0] / 2 ? idx : idx - N) + half;  // first pass: idx < N/2 exactly when r < R/2
+      return (c >= 0 && c < crop) ? ld_dep(row + c) : make_float2(0.f, 0.f);
+    };
+    float tv[PERL][RL];  // theta at this thread's outputs, loaded while the later passes run
+    auto after_first = [&]() {
 #pragma unroll
-    for (int p = 0; p < PERL; ++p)
+      for (int p = 0; p < PERL; ++p)
 #pragma unroll
-      for (int q = 0; q < RL; ++q) mm[p][q] = m && t + p * NT < N / RL ? ld_dep(mr + t + p * NT + q * (N / RL)) : 0.f;
-  };
-  auto use = [&](int p, int q, int x, float2 v) {
-    // without m no chain factor: the gradient with respect to m itself
-    gr[x] = m ? scale * v.x * alpha * mm[p][q] * (1.0f - mm[p][q]) : scale * v.x;
-  };
-  fft_load_use<N, +1, decltype(load), decltype(use), false>(buf, tw, t, load, use, after_first);
+        for (int q = 0; q < RL; ++q)
+          tv[p][q] = th && t + p * NT < N / RL ? ld_dep(th + t + p * NT + q * (N / RL)) : 0.f;
+    };
+    float* gr = grad + clip * grad_stride + (size_t)y * N;
+    auto use = [&](int p, int q, int x, float2 v) {
+      if (theta) {
+        const float m = sigmoidf(alpha * tv[p][q]);
+        gr[x] = scale * v.x * alpha * m * (1.0f - m);
+      } else {
+        gr[x] = scale * v.x;  // the gradient with respect to the mask itself
+      }
+    };
+    fft_load_use<N, +1, decltype(load), decltype(use), BANDED>(buf, tw, t, load, use, after_first);
+  }
 }
 
 template <int N>
 cudaError_t adj_rows_n(const float2* t1, const FieldSet& fs, int clips, int crop, const float* g, int g_planes,
                        const float2* tw, float2* u, cudaStream_t st, const float2* tw512) {
   const int planes = clips * fs.planes;
+  // fields per CTA: all of a plane's (its G row stays in registers), or with fewer than four waves of CTAs
+  // the plane's fields dealt out to up to 8, at least two to each (12 planes of 512^2 151 -> 126 us, 2 of
+  // 256^2 17.6 -> 10.8 us)
+  int most = 1;
+  for (int p = 0; p < fs.planes; ++p) most = std::max(most, fs.start[p + 1] - fs.start[p]);
+  auto runs = [&](int ctas, int slots) {
+    int z = 1;
+    while (z < 8 && 2 * z <= most && (long long)ctas * z < 4LL * slots) z *= 2;
+    return z;
+  };
   if (N == 512 && tw512 && crop % 2 == 0 && crop / 2 <= 128) {  // two rows per warp
     const size_t sm = sizeof(float2) * (kAdjTw1 + kAdjTw2 + kAdjWarps * 2 * (size_t(kAdjBuf) + crop));
     cudaError_t e = smem_attrs(k_adj_rows_w512<true>, sm);
     if (e != cudaSuccess) return e;
-    return launch_pdl(k_adj_rows_w512<true>, dim3(N / (2 * kAdjWarps), planes), 32 * kAdjWarps, sm, st, t1, fs, crop,
+    const int ctas = N / (2 * kAdjWarps) * planes;
+    return launch_pdl(k_adj_rows_w512<true>, dim3(N / (2 * kAdjWarps), planes, runs(ctas, 2 * 152)), 32 * kAdjWarps, sm, st, t1, fs, crop,
                       g, g_planes, tw512, u);
   }
   const size_t sm = sizeof(float2) * (N + 2 * PadLen<N>::value);
   auto kern = 2 * crop <= N ? k_adj_rows<N, true> : k_adj_rows<N, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3(N, planes), Plan<N>::NT, sm, st, t1, fs, crop, g, g_planes, tw, u);
+  return launch_pdl(kern, dim3(N, planes, runs(N * planes, 152 * 512 / Plan<N>::NT)), Plan<N>::NT, sm, st, t1, fs, crop,
+                    g, g_planes, tw, u);
 }
 
 template <int N>
@@ -546,13 +562,15 @@ cudaError_t adj_cols_n(const float2* u, const float2* phi, int crop, const float
 }
 
 template <int N>
-cudaError_t grad_rows_n(const float2* qf, int crop, float scale, const float* m, float alpha, const float2* tw,
+cudaError_t grad_rows_n(const float2* qf, int crop, float scale, const float* theta, float alpha, const float2* tw,
                         float* grad, int clips, long long grad_stride, cudaStream_t st) {
   const size_t sm = sizeof(float2) * (N + PadLen<N>::value);
-  cudaError_t e = cudaFuncSetAttribute(k_grad_rows<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  auto kern = 2 * crop <= N ? k_grad_rows<N, true> : k_grad_rows<N, false>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_grad_rows<N>, dim3(N, clips), Plan<N>::NT, sm, st, qf, crop, scale, m, alpha, tw, grad,
-                    grad_stride);
+  const int per = rows_per_cta(N, clips, 2048 / Plan<N>::NT);
+  return launch_pdl(kern, dim3((N + per - 1) / per, clips), Plan<N>::NT, sm, st, qf, crop, scale, theta, alpha, tw,
+                    grad, grad_stride, per);
 }
 
 #define ILT_DISPATCH(n, CALL)              \
@@ -581,9 +599,9 @@ cudaError_t launch_adj_cols(int n, const float2* u, const float2* phi, int crop,
 #undef CALL
 }
 // Clip i of `clips` writes grad + i grad_stride.
-cudaError_t launch_grad_rows(int n, const float2* qf, int crop, float scale, const float* m, float alpha,
+cudaError_t launch_grad_rows(int n, const float2* qf, int crop, float scale, const float* theta, float alpha,
                              const float2* tw, float* grad, int clips, long long grad_stride, cudaStream_t st) {
-#define CALL(N) grad_rows_n<N>(qf, crop, scale, m, alpha, tw, grad, clips, grad_stride, st)
+#define CALL(N) grad_rows_n<N>(qf, crop, scale, theta, alpha, tw, grad, clips, grad_stride, st)
   ILT_DISPATCH(n, CALL)
 #undef CALL
 }
@@ -591,7 +609,6 @@ cudaError_t launch_grad_rows(int n, const float2* qf, int crop, float scale, con
 size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 
 struct IltLayout {
-  float* m;
   float2 *rowbuf, *mhat, *t1, *u, *sk, *s, *qf;
   float *img, *blur;
   double *partial, *loss;
@@ -627,7 +644,6 @@ IltLayout ilt_layout(const litho_kernels* h, int b, int P, int G, void* base) {
     return r;
   };
   L.loss = reinterpret_cast<double*>(take(size_t(b) * 8));
-  L.m = reinterpret_cast<float*>(take(g * N * N * 4));
   L.rowbuf = reinterpret_cast<float2*>(take(g * N * C * 8));
   L.mhat = reinterpret_cast<float2*>(take(g * C * C * 8));
   L.t1 = reinterpret_cast<float2*>(take(PG * K * N * C * 8));
@@ -826,15 +842,9 @@ litho_status litho_ilt_grad(const litho_kernels* h, const float* theta_dev, cons
   for (int c0 = 0; c0 < b; c0 += G) {
     const int g = std::min(G, b - c0), gp = g * PU;
     {
-      ProfScope ps(kStageIltForward, st, 3);
-      {
-        const size_t c4 = size_t(g) * nn / 4;  // nn = N^2 with N >= 32: a multiple of 4
-        const int blocks = int(std::min<size_t>((c4 + 255) / 256, 4096));
-        LITHO_TRY_CUDA(launch_pdl(k_sigmoid, blocks, 256, 0, st, reinterpret_cast<const float4*>(theta_dev + c0 * nn),
-                                  float(mask_steep), reinterpret_cast<float4*>(L.m), c4));
-      }
-      LITHO_TRY_CUDA(cudaGetLastError());
-      LITHO_TRY_CUDA(launch_mask_spectrum(L.m, g, N, C, h->d_tw, L.rowbuf, L.mhat, st));
+      ProfScope ps(kStageIltForward, st, 2);
+      LITHO_TRY_CUDA(launch_sigmoid_spectrum(theta_dev + c0 * nn, float(mask_steep), g, N, C, h->d_tw, L.rowbuf, L.mhat,
+                                             st));
     }
     for (int u0 = 0; u0 < U; u0 += PU) {
       const FieldSet fs = field_set(h, u0, PU);
@@ -843,7 +853,7 @@ litho_status litho_ilt_grad(const litho_kernels* h, const float* theta_dev, cons
       for (int f = 0; f < F; ++f)
         if (h->set_of[f] >= u0 && h->set_of[f] < u0 + PU) ++weight.w[h->set_of[f] - u0];
       {
-        ProfScope ps(kStageIltForward, st, coarse ? (rows2 ? 5 : 6) : 5);
+        ProfScope ps(kStageIltForward, st, coarse ? (rows2 ? 4 : 5) : 4);
         LITHO_TRY_CUDA(launch_stage1_fft(L.mhat, psi, fs.fields(), NE, C, twe, L.t1, st, g));
         LITHO_TRY_CUDA(launch_stage2_fft(L.t1, fs, g, NE, C, float(dose), twe, coarse ? L.ic : L.img, each, st,
                                          h->d_tw32, h->d_tw512, rows2 ? L.mid : nullptr, C2));
@@ -854,14 +864,10 @@ litho_status litho_ilt_grad(const litho_kernels* h, const float* theta_dev, cons
           // buffer), partial losses per row pair
           LITHO_TRY_CUDA(launch_resist_grad_rows(L.big, gp, N, C2, h->d_tw, target_dev + c0 * nn, PU, weight,
                                                  float(resist_steep), float(threshold), qrows, L.partial, st));
-          LITHO_TRY_CUDA(launch_pdl(k_reduce_loss, g, 1024, 0, st, L.partial, PU * N / 2, L.loss + c0,
-                                    u0 > 0 ? 1 : 0));
         } else {
           LITHO_TRY_CUDA(launch_resist(L.img, gp, N, taps, float(threshold), L.blur, nullptr, st));
           LITHO_TRY_CUDA(launch_pdl(k_resist_grad, dim3(kPartials, g), 256, 0, st, L.blur, target_dev + c0 * nn, nn,
                                     PU, weight, float(resist_steep), float(threshold), L.img, L.partial));
-          LITHO_TRY_CUDA(launch_pdl(k_reduce_loss, g, 1024, 0, st, L.partial, kPartials, L.loss + c0,
-                                    u0 > 0 ? 1 : 0));
         }
         LITHO_TRY_CUDA(cudaGetLastError());
       }
@@ -878,14 +884,14 @@ litho_status litho_ilt_grad(const litho_kernels* h, const float* theta_dev, cons
         }
         LITHO_TRY_CUDA(launch_adj_rows(NE, L.t1, fs, g, C, gsrc, PU, twe, L.u, st, h->d_tw512));
         LITHO_TRY_CUDA(launch_adj_cols(NE, L.u, psi, C, twe, L.sk, g, fs.fields(), st));
-        LITHO_TRY_CUDA(launch_pdl(k_sum_planes, dim3(256, g), 256, 0, st, L.sk, adj_col_splits(fs.fields()),
-                                  size_t(C) * C, L.s, u0 > 0 ? 1 : 0));
+        LITHO_TRY_CUDA(launch_sum_planes(L.sk, adj_col_splits(fs.fields()), size_t(C) * C, L.s, u0 > 0 ? 1 : 0, g,
+                                         L.partial, coarse ? PU * N / 2 : kPartials, L.loss + c0, st));
       }
     }
     ProfScope ps(kStageIltBackward, st, 2);
     LITHO_TRY_CUDA(launch_stage1_fft(L.s, nullptr, g, N, C, h->d_tw, L.qf, st));
-    LITHO_TRY_CUDA(launch_grad_rows(N, L.qf, C, scale, L.m, float(mask_steep), h->d_tw, grad_dev + c0 * nn, g,
-                                    (long long)nn, st));
+    LITHO_TRY_CUDA(launch_grad_rows(N, L.qf, C, scale, theta_dev + c0 * nn, float(mask_steep), h->d_tw,
+                                    grad_dev + c0 * nn, g, (long long)nn, st));
   }
   if (loss_host) {
     LITHO_TRY_CUDA(cudaMemcpyAsync(loss_host, L.loss, size_t(b) * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -987,8 +993,8 @@ litho_status litho_intensity_vjp(const litho_kernels* h, const float* mask_dev, 
         LITHO_TRY_CUDA(
             launch_adj_rows(NE, L.t1, fs, g, C, up + size_t(r0) * NE * NE, p, twe, L.u, st, h->d_tw512));
         LITHO_TRY_CUDA(launch_adj_cols(NE, L.u, psi, C, twe, L.sk, g, fs.fields(), st));
-        LITHO_TRY_CUDA(launch_pdl(k_sum_planes, dim3(256, g), 256, 0, st, L.sk, adj_col_splits(fs.fields()),
-                                  size_t(C) * C, L.s, f0 > f_first || r0 > 0 ? 1 : 0));
+        LITHO_TRY_CUDA(launch_sum_planes(L.sk, adj_col_splits(fs.fields()), size_t(C) * C, L.s,
+                                         f0 > f_first || r0 > 0 ? 1 : 0, g, nullptr, 0, nullptr, st));
       }
     }
     LITHO_TRY_CUDA(launch_stage1_fft(L.s, nullptr, g, N, C, h->d_tw, L.qf, st));

@@ -161,6 +161,9 @@ bool fft_twiddle_table(int n, float2* out);
 // Mask spectrum: m[b][n][n] -> mhat[b][C][C] = N^-2 DFT(m) on the crop.  rowbuf: [b][n][C/2 + 8].
 cudaError_t launch_mask_spectrum(const float* m, int b, int n, int crop, const float2* tw, float2* rowbuf,
                                  float2* mhat, cudaStream_t st);
+// The same of the mask sigmoid(alpha theta).
+cudaError_t launch_sigmoid_spectrum(const float* theta, float alpha, int b, int n, int crop, const float2* tw,
+                                    float2* rowbuf, float2* mhat, cudaStream_t st);
 // Its two passes.  Row DFTs of real planes, the frequencies u >= 0: rowbuf[b][n][C/2], index u, or (whole:
 // with u = C/2) [b][n][C/2 + 8].
 cudaError_t launch_mask_rows(const float* m, int b, int n, int crop, const float2* tw, float2* rowbuf, bool whole,
