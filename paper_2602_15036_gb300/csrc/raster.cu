@@ -27,8 +27,9 @@ namespace {
 
 constexpr int kTile = 16;
 constexpr int kScanThreads = 1024, kScanRun = 4;  // tiles a thread of the scan takes in a row
-// tile kernel: a warp per tile with a 64-piece cache (larger lists are read from global memory)
-constexpr int kRastWarps = 8, kTileCache = 64, kTilePix = kTile * kTile;
+// tile kernel: a warp per tile with a 64-piece cache (larger lists are read from global memory); four
+// tiles a CTA, since a CTA waits for its slowest tile (eight: 783 us against 718)
+constexpr int kRastWarps = 4, kTileCache = 64, kTilePix = kTile * kTile;
 
 // Pieces of rectangle r (x0, y0, x1, y1) after the shift into [0, n) and the
 // split at n; calls f(piece) for each nonempty one.
@@ -178,7 +179,7 @@ __device__ __forceinline__ float overlap(const float4& p, float px, float py) {
 // measure them: one or two pieces in closed form (A + B - A B), the rest, pooled over the CTA's
 // tiles, by the sweep of pixel_area.  The tile is put together in shared memory and written by rows.
 // 64 clips of 2048^2, 18 k rectangles each:
-// 2062 -> 783 us (a CTA of 64 threads per tile that tested every pixel against every piece and
+// 2062 -> 718 us (a CTA of 64 threads per tile that tested every pixel against every piece and
 // swept every grey pixel).
 template <bool VEC>
 __global__ void __launch_bounds__(32 * kRastWarps) k_rast_tiles(const float4* __restrict__ list,
