@@ -387,7 +387,8 @@ __global__ void __launch_bounds__(Plan<N>::NT * AdjW<N>::W, AdjAccInSmem<N>::val
 // exactly (on the coarse grid too: there G is the constant (N/nc)^2 and the
 // transforms are on nc).  No field is transformed.  The sum over a plane's
 // kernels does not depend on the mask: the kernel set keeps it (`power`, per
-// set, rounded once from FP64).  Clip blockIdx.y; the planes' sets are listed
+// set, rounded once from FP64; even in the frequency unless the set has an edge,
+// since only the real part of the result's transform is taken).  Clip blockIdx.y; the planes' sets are listed
 // in `sets`.
 __global__ void k_ones_adjoint(const float2* __restrict__ mhat, const float* __restrict__ power,
                                const __grid_constant__ PlaneOut sets, size_t cc, float n2, float2* __restrict__ s) {
@@ -725,11 +726,11 @@ litho_status ai_channels(const litho_kernels* h, const float* target, int b, dou
   const bool rows2 = coarse && h->d_tw32 && stage2_w32_supported(NE, C);
   for (int c0 = 0; c0 < b; c0 += G) {
     const int g = std::min(G, b - c0);
+    float* dst = x + size_t(c0) * 3 * nn;
     {  // channel 1: the aerial image of the targets (interpolated from the coarse grid)
       ProfScope ps(kStageIltForward, st, coarse ? (rows2 ? 6 : 7) : 4);
       LITHO_TRY_CUDA(launch_mask_spectrum(target + c0 * nn, g, N, C, h->d_tw, L.rowbuf, L.mhat, st));
       LITHO_TRY_CUDA(launch_stage1_fft(L.mhat, psi, fs.fields(), NE, C, twe, L.t1, st, g));
-      float* dst = x + size_t(c0) * 3 * nn;
       LITHO_TRY_CUDA(launch_stage2_fft(L.t1, fs, g, NE, C, float(dose), twe, coarse ? L.ic : dst,
                                        coarse ? one : channel1, st, h->d_tw32, h->d_tw512, rows2 ? L.mid : nullptr, C2));
       if (coarse) {
@@ -739,12 +740,19 @@ litho_status ai_channels(const litho_kernels* h, const float* target, int b, dou
       }
     }
     {  // channel 2: the adjoint applied to dL/dI = 1, in closed form (k_ones_adjoint)
+      PlaneOut channel2 = channel1;
+      channel2.list[0] = 2;
       ProfScope ps(kStageIltBackward, st, 3);
       LITHO_TRY_CUDA(launch_pdl(k_ones_adjoint, dim3(128, g), 256, 0, st, L.mhat, h->d_power, sets_of(h, focus, 1),
                                 size_t(C) * C, float(double(N) * double(N)), L.s));
-      LITHO_TRY_CUDA(launch_stage1_fft(L.s, nullptr, g, N, C, h->d_tw, L.qf, st));
-      LITHO_TRY_CUDA(launch_grad_rows(N, L.qf, C, scale, nullptr, 0.f, h->d_tw, x + (size_t(c0) * 3 + 2) * nn, g,
-                                      (long long)3 * nn, st));
+      if (h->edge) {
+        LITHO_TRY_CUDA(launch_stage1_fft(L.s, nullptr, g, N, C, h->d_tw, L.qf, st));
+        LITHO_TRY_CUDA(launch_grad_rows(N, L.qf, C, scale, nullptr, 0.f, h->d_tw, x + (size_t(c0) * 3 + 2) * nn, g,
+                                        (long long)3 * nn, st));
+      } else {  // S(-u) = conj S(u): half the columns, two rows to a transform
+        LITHO_TRY_CUDA(launch_stage1_half(L.s, g, N, C, h->d_tw, L.qf, C / 2, st));
+        LITHO_TRY_CUDA(launch_band_rows_real(L.qf, g, 1, N, C / 2, scale, h->d_tw, dst, channel2, st));
+      }
     }
   }
   return LITHO_OK;
@@ -996,6 +1004,12 @@ litho_status litho_intensity_vjp(const litho_kernels* h, const float* mask_dev, 
         LITHO_TRY_CUDA(launch_sum_planes(L.sk, adj_col_splits(fs.fields()), size_t(C) * C, L.s,
                                          f0 > f_first || r0 > 0 ? 1 : 0, g, nullptr, 0, nullptr, st));
       }
+    }
+    if (!upstream_dev && !h->edge) {  // the closed form's S(-u) = conj S(u)
+      LITHO_TRY_CUDA(launch_stage1_half(L.s, g, N, C, h->d_tw, L.qf, C / 2, st));
+      LITHO_TRY_CUDA(launch_band_rows_real(L.qf, g, 1, N, C / 2, scale, h->d_tw, dm_dev + c0 * nn,
+                                           plane_out_identity(1), st));
+      continue;
     }
     LITHO_TRY_CUDA(launch_stage1_fft(L.s, nullptr, g, N, C, h->d_tw, L.qf, st));
     LITHO_TRY_CUDA(launch_grad_rows(N, L.qf, C, scale, nullptr, 0.f, h->d_tw, dm_dev + c0 * nn, g, (long long)nn,

@@ -111,9 +111,11 @@ __global__ void __launch_bounds__(256) k_add_power(const double2* __restrict__ p
   const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (i < cc) dsum[i] += lam * (phi[i].x * phi[i].x + phi[i].y * phi[i].y);
 }
-__global__ void __launch_bounds__(256) k_round(const double* __restrict__ x, size_t n, float* __restrict__ y) {
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (i < n) y[i] = float(x[i]);
+// y = x rounded, or with `even` (x(u) + x(-u))/2.
+__global__ void __launch_bounds__(256) k_round(const double* __restrict__ x, int crop, int even,
+                                               float* __restrict__ y) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < crop * crop) y[i] = float(even ? 0.5 * (x[i] + x[mirror(i, crop)]) : x[i]);
 }
 
 // Eigenvalues (descending) and eigenvectors (columns of v) of a real symmetric
@@ -232,6 +234,8 @@ litho_status build(litho_kernels* h) {
   } else {
     LITHO_TRY_CUDA(cudaMalloc(&phi64.p, cc * sizeof(double2)));  // one kernel at a time
   }
+  // C = n: every frequency has its mirror, but u = -C/2 is left out of half spectra
+  h->edge = C == h->n || std::find(edge.begin(), edge.end(), 1) != edge.end();
   auto gram = [&](int fa, int fb, std::vector<double>* out) -> litho_status {
     std::vector<double4> g(size_t(K) * K);
     k_gram<<<dim3(K, K), 256>>>(phi64.as<double2>() + fa * plane_len, phi64.as<double2>() + fb * plane_len, C,
@@ -321,7 +325,7 @@ litho_status build(litho_kernels* h) {
       LITHO_TRY_CUDA(cudaMemcpy(d_beta, t.beta.data(), t.beta.size() * sizeof(double2), cudaMemcpyHostToDevice));
       k_combine<<<dim3(blocks, t.kernels), 256>>>(phi64.as<double2>() + t.plane * plane_len, K, C, d_alpha, d_beta, psi);
     }
-    k_round<<<blocks, 256>>>(power.as<double>(), cc, h->d_power + u * cc);
+    k_round<<<blocks, 256>>>(power.as<double>(), C, h->edge ? 0 : 1, h->d_power + u * cc);
     LITHO_TRY_CUDA(cudaGetLastError());
   }
   LITHO_TRY_CUDA(cudaStreamSynchronize(nullptr));  // the set is read from any stream afterwards

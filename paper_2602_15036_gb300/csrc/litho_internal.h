@@ -112,7 +112,8 @@ struct litho_kernels {
   int n_sets = 0, set_start[litho::kMaxPlanes + 1] = {};
   unsigned char set_of[litho::kMaxPlanes] = {};
   float2* d_psi = nullptr;                 // [set_start[n_sets]][C][C]
-  float* d_power = nullptr;                // [n_sets][C][C]: sum_k lam_k |Phi_k|^2
+  float* d_power = nullptr;                // [n_sets][C][C]: sum_k lam_k |Phi_k|^2 (without edge: made even in u)
+  bool edge = true;                        // a kernel may be nonzero at u = -C/2, whose mirror is off the crop
   float2* d_tw = nullptr;                  // FFT twiddle table for N
   int nc = 0;                              // FP32 FFT coarse grid: smallest power of two >= 2 crop (0: not below N)
   float2* d_twc = nullptr;                 // FFT twiddle table for nc
