@@ -489,15 +489,16 @@ struct MidTwiddles {
 };
 
 // fft_load_use with the middle pass's twiddles from `mid` (same result).
-template <int N, int SIGN, class Load, class Use, bool BANDED = false>
+template <int N, int SIGN, class Load, class Use, bool BANDED = false, class Hook = NoHook>
 __device__ __forceinline__ void fft_load_use_mid(float2* buf, const float2* tw, int t, Load& load, Use& use,
-                                                 const MidTwiddles<N, SIGN>& mid) {
+                                                 const MidTwiddles<N, SIGN>& mid, const Hook& after_first = Hook()) {
   using PL = Plan<N>;
   using M = MidTwiddles<N, SIGN>;
   static_assert(M::kUsable, "middle-pass twiddles are per thread only when NT is a multiple of the stride");
   constexpr int NT = PL::NT, R = M::R, NS = M::NS;
   using S = PassShape<N, NT, R>;
   pass_to_smem<N, NT, PL::R[0], 1, SIGN, 0, false, Load, BANDED>(buf, tw, t, load);
+  after_first();
   float2 v[S::PER][R];
 #pragma unroll
   for (int p = 0; p < S::PER; ++p) {
