@@ -158,8 +158,9 @@ struct OutC64 {
   __device__ __forceinline__ int first() const { return 0; }  // first crop column, and the rows' stride
   __device__ __forceinline__ int ld(int c) const { return c; }
   __device__ __forceinline__ float2* column(int j, int c) const { return t1 + (size_t)j * n * crop + c; }
+  __device__ float scale(int) const { return 1.f; }
   template <int W>
-  __device__ void store_row(int, int, int, const float2 (&)[W]) const {}
+  __device__ void store_row(int, int, int, float, const float2 (&)[W]) const {}
 };
 
 // The columns u >= 0 alone, as half rows of stride `stride` (any spectra, no kernels).
@@ -170,8 +171,9 @@ struct OutHalf {
   __device__ __forceinline__ int first() const { return half; }
   __device__ __forceinline__ int ld(int) const { return stride; }
   __device__ __forceinline__ float2* column(int j, int c) const { return q + (size_t)j * n * stride + (c - half); }
+  __device__ float scale(int) const { return 1.f; }
   template <int W>
-  __device__ void store_row(int, int, int, const float2 (&)[W]) const {}
+  __device__ void store_row(int, int, int, float, const float2 (&)[W]) const {}
 };
 
 // ---- stage 2 (FP32 path): one image row per CTA, all kernels of the plane ------------------------

@@ -537,12 +537,14 @@ __device__ __forceinline__ void fft_smem(float2* buf, const float2* tw, int t) {
 // shared memory (padded layout, natural order on return).  Ends with a barrier.
 // NTX: the threads that share the transform (default: the plan's own; more
 // threads take the butterflies of a pass in fewer rounds).
-template <int N, int SIGN, class Load, bool BANDED = false, int NTX = Plan<N>::NT>
-__device__ __forceinline__ void fft_load_smem(float2* buf, const float2* tw, int t, Load& load) {
+template <int N, int SIGN, class Load, bool BANDED = false, int NTX = Plan<N>::NT, class Hook = NoHook>
+__device__ __forceinline__ void fft_load_smem(float2* buf, const float2* tw, int t, Load& load,
+                                              const Hook& after_first = Hook()) {
   using PL = Plan<N>;
   constexpr int NT = NTX;
   SmemLoadUnused none;
   pass_to_smem<N, NT, PL::R[0], 1, SIGN, 0, false, Load, BANDED>(buf, tw, t, load);
+  after_first();
   if constexpr (PL::P == 2) {
     pass_to_smem<N, NT, PL::R[1], PL::R[0], SIGN, TwOff<N>::p1, true>(buf, tw, t, none);
   } else {

@@ -471,44 +471,43 @@ template <int MODE>
 struct OutSplit {
   static constexpr bool kRowWise = true;
   __device__ __forceinline__ int first() const { return 0; }
-  __device__ float2* column(int, int) const { return nullptr; }
   void* hi;
   void* lo;
   void* sum;
   const float* scales;
-  int n, crop, nk;  // row j of the operand belongs to kernel j mod nk
+  int n, crop;
+  __device__ __forceinline__ float scale(int k) const { return __ldg(scales + k); }  // of kernel k
   template <int W>
-  __device__ __forceinline__ void store_row(int j, int y, int c0, const float2 (&v)[W]) const {
+  __device__ __forceinline__ void store_row(int j, int y, int c0, float s, const float2 (&v)[W]) const {
     static_assert(W % 4 == 0 && CH % W == 0, "column block");
     const size_t o = ((size_t)j * n + y) * (size_t)(2 * crop) + (size_t)(c0 / CH) * KE + (c0 % CH);
-    const float s = scales[j % nk];
-    uint32_t rh[W], rl[W], ih[W], il[W], sh[W], sl[W];
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-      split16<MODE>(v[w].x, s, rh[w], rl[w]);
-      split16<MODE>(v[w].y, s, ih[w], il[w]);
-      split16<MODE>(v[w].x + v[w].y, s, sh[w], sl[w]);
-    }
     // one store per part and row: W 16-bit values, 16 bytes for W = 8 (fewer L2 write transactions)
-    auto put = [&](void* base, size_t off, const uint32_t (&x)[W]) {
+    auto put = [&](void* base, size_t off, const uint32_t (&x)[W / 2]) {
       uint16_t* d = static_cast<uint16_t*>(base) + off;
       if constexpr (W == 8) {
-        *reinterpret_cast<uint4*>(d) = make_uint4(x[0] | (x[1] << 16), x[2] | (x[3] << 16), x[4] | (x[5] << 16),
-                                                  x[6] | (x[7] << 16));
+        *reinterpret_cast<uint4*>(d) = make_uint4(x[0], x[1], x[2], x[3]);
       } else {
 #pragma unroll
-        for (int q = 0; q < W / 4; ++q)
-          reinterpret_cast<uint2*>(d)[q] = make_uint2(x[4 * q] | (x[4 * q + 1] << 16), x[4 * q + 2] | (x[4 * q + 3] << 16));
+        for (int q = 0; q < W / 4; ++q) reinterpret_cast<uint2*>(d)[q] = make_uint2(x[2 * q], x[2 * q + 1]);
       }
     };
-    put(hi, o, rh);
-    put(hi, o + CH, ih);
-    if (MODE == kFP16X3 || MODE == kBF16X3) {
-      put(lo, o, rl);
-      put(lo, o + CH, il);
-      put(sum, o, sh);
-      put(sum, o + CH, sl);
-    }
+    // the parts one after another, so that only one part's halves are live
+    auto part = [&](auto&& value, void* hi_base, size_t hi_off, void* lo_base, size_t lo_off) {
+      uint32_t h[W / 2], l[W / 2];
+#pragma unroll
+      for (int q = 0; q < W / 2; ++q) {
+        uint32_t h0, l0, h1, l1;
+        split16<MODE>(value(v[2 * q]), s, h0, l0);
+        split16<MODE>(value(v[2 * q + 1]), s, h1, l1);
+        h[q] = h0 | (h1 << 16);
+        l[q] = l0 | (l1 << 16);
+      }
+      put(hi_base, hi_off, h);
+      if (MODE == kFP16X3 || MODE == kBF16X3) put(lo_base, lo_off, l);
+    };
+    part([](float2 x) { return x.x; }, hi, o, lo, o);
+    part([](float2 x) { return x.y; }, hi, o + CH, lo, o + CH);
+    if (MODE == kFP16X3 || MODE == kBF16X3) part([](float2 x) { return x.x + x.y; }, sum, o, sum, o + CH);
   }
 };
 
@@ -517,7 +516,7 @@ template <int N, int MODE>
 cudaError_t stage1_split_n(const float2* mhat, const float2* phi, int nk, int crop, const float2* tw,
                            const float* scales, void* a_hi, void* a_lo, void* a_s, int clips, cudaStream_t st) {
   return launch_stage1_cols<N, Stage1W<N>::W>(mhat, phi, nk, crop, tw,
-                                           OutSplit<MODE>{a_hi, a_lo, a_s, scales, N, crop, nk}, st, clips);
+                                           OutSplit<MODE>{a_hi, a_lo, a_s, scales, N, crop}, st, clips);
 }
 
 template <int MODE>

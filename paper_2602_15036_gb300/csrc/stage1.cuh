@@ -4,10 +4,9 @@
 //
 // A CTA keeps the twiddle table in shared memory and loops over a run of kernels;
 // the next kernel's Phi block is copied in with cp.async while the current
-// block's W column transforms run.  The FP32 output takes one block buffer,
-// refilled as soon as the first pass (the only one that reads the block) is
-// done, so that two CTAs fit an SM's shared memory; the split 16-bit output
-// keeps two buffers.  The band multiply happens in
+// block's W column transforms run.  One block buffer, refilled as soon as the
+// first pass (the only one that reads the block) is done, so that two CTAs fit
+// an SM's shared memory (Stage1Pipe).  The band multiply happens in
 // the first pass's load: the mask-spectrum values a thread multiplies are
 // the same for every kernel, so they are loaded once into registers.
 // Without kernels (phi == NULL) each j transforms its own spectrum mhat[j].
@@ -65,16 +64,19 @@ struct Stage1Shape {
   }
 };
 
-// Block buffers and CTAs per SM the launch bounds ask for: the FP32 output
-// single-buffers its Phi block and runs two CTAs per SM.
-template <class Out>
+// Block buffers and CTAs per SM the launch bounds ask for: one buffer and two
+// CTAs, except for the split output at 896 points, whose radix-7 pass and
+// 16-bit packing spill at 64 registers (4 clips of 36 kernels 482 -> 708 us; at
+// 512 points two CTAs take a call of 4 clips of 9 kernels from 149 to 138 us).
+template <int N, class Out>
 struct Stage1Pipe {
-  static constexpr int kBuffers = Out::kRowWise ? 2 : 1;
-  static constexpr int kMinBlocks = Out::kRowWise ? 1 : 2;
+  static constexpr bool kOne = Out::kRowWise && N == 896;
+  static constexpr int kBuffers = kOne ? 2 : 1;
+  static constexpr int kMinBlocks = kOne ? 1 : 2;
 };
 
 template <int N, int W, class Out, bool BANDED>
-__global__ void __launch_bounds__(Plan<N>::NT * W, Stage1Pipe<Out>::kMinBlocks)
+__global__ void __launch_bounds__(Plan<N>::NT * W, Stage1Pipe<N, Out>::kMinBlocks)
     k_stage1_cols(const float2* __restrict__ mhat, const float2* __restrict__ phi, int crop, int nk, int jb,
                   const float2* __restrict__ tw_g, Out out) {
   constexpr int NT = Plan<N>::NT, LD = Stage1Shape<N, W>::LD, T = W * NT;
@@ -114,7 +116,7 @@ __global__ void __launch_bounds__(Plan<N>::NT * W, Stage1Pipe<Out>::kMinBlocks)
     const bool zero = !phi || t >= NB0 || c < 0 || c >= crop || (BANDED && r >= R0 / 4 && r < 3 * R0 / 4);
     mreg[r] = zero ? make_float2(0.f, 0.f) : ld_dep(mhat + (size_t)c * crop + u0 + g);
   }
-  constexpr bool kSingle = Stage1Pipe<Out>::kBuffers == 1;
+  constexpr bool kSingle = Stage1Pipe<N, Out>::kBuffers == 1;
   for (int j = j0; j < j1; ++j) {
     const int s = kSingle ? 0 : (j - j0) & 1;
     if (!kSingle && j + 1 < j1) {
@@ -137,13 +139,14 @@ __global__ void __launch_bounds__(Plan<N>::NT * W, Stage1Pipe<Out>::kMinBlocks)
       return phi ? cmul(mreg[r], b[c * W]) : b[c * W];
     };
     if constexpr (Out::kRowWise) {
-      fft_load_smem<N, +1, decltype(load), BANDED>(buf + g * LD, tw, t, load);
+      fft_load_smem<N, +1, decltype(load), BANDED>(buf + g * LD, tw, t, load, refill);
       // one thread per output row writes the block's W consecutive columns
+      const float scale = out.scale(j);
       for (int y = tid; y < N; y += T) {
         float2 v[W];
 #pragma unroll
         for (int w = 0; w < W; ++w) v[w] = buf[w * LD + pad16(y)];
-        out.template store_row<W>(jofs + j, y, u0, v);
+        out.template store_row<W>(jofs + j, y, u0, scale, v);
       }
     } else {
       float2* const col = out.column(jofs + j, u0 + g);  // element y at col[y crop]
@@ -171,7 +174,7 @@ cudaError_t launch_stage1_cols_t(const float2* mhat, const float2* phi, int nk, 
               : 152;
   }
   const int blocks = (crop - c_first) / W;
-  const long long ctas = (long long)clips * blocks, slots = (long long)Stage1Pipe<Out>::kMinBlocks * sms;
+  const long long ctas = (long long)clips * blocks, slots = (long long)Stage1Pipe<N, Out>::kMinBlocks * sms;
   int jblocks = 1;
   long long best = -1;
   for (int jb = 1; jb <= std::min(nk, 32); ++jb) {
@@ -184,7 +187,7 @@ cudaError_t launch_stage1_cols_t(const float2* mhat, const float2* phi, int nk, 
     }
   }
   const int JB = (nk + jblocks - 1) / jblocks;
-  const size_t sm = sizeof(float2) * Stage1Shape<N, W>::smem_elems(crop, Stage1Pipe<Out>::kBuffers);
+  const size_t sm = sizeof(float2) * Stage1Shape<N, W>::smem_elems(crop, Stage1Pipe<N, Out>::kBuffers);
   cudaError_t e = smem_attrs(k_stage1_cols<N, W, Out, BANDED>, sm);
   if (e != cudaSuccess) return e;
   const dim3 grid = Out::kRowWise ? dim3(blocks, clips, (nk + JB - 1) / JB) : dim3(clips, blocks, (nk + JB - 1) / JB);
