@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(Plan<N>::NT * W) k_mask_cols(const float2* __r
   const int b = blockIdx.y, tid = threadIdx.x, g = tid % W, t = tid / W, k = blockIdx.x * W + g, half = crop / 2;
   const bool live = k < cols;
   const float2* src = rowbuf + (size_t)b * N * ld + k;
-  auto load = [&](int, int, int y) { return live ? ld_dep(src + (size_t)y * ld) : make_float2(0.f, 0.f); };
+  auto load = [&](int, int, int y) { return ld_dep_if(src + (size_t)y * ld, live); };
   const float scale = 1.0f / (float(N) * float(N));
   const float gu = gain && live ? scale * ld_dep(gain + half + k) : scale;
   float2* dst = mhat + (size_t)b * crop * crop;
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(Plan<N>::NT * Stage2Groups<N>::value, 512 / Pl
     for (int r = 0; r < R0; ++r) {
       const int c = t + r * NB0 - (r < R0 / 2 ? 0 : N) + half;  // index t + r N/R0 < N/2 exactly when r < R0/2
       const bool zero = (BANDED && r >= R0 / 4 && r < 3 * R0 / 4) || t >= NB0 || j >= nk || c < 0 || c >= crop;
-      nxt[r] = zero ? make_float2(0.f, 0.f) : ld_dep(row + c);
+      nxt[r] = ld_dep_if(row + c, !zero);
     }
   };
   prefetch(grp);
@@ -280,8 +280,7 @@ __global__ void __launch_bounds__(Plan<N>::NT * Stage2Groups<N>::value, 512 / Pl
 // Element u of A + i B from the half rows a, b of `h` columns.
 __device__ __forceinline__ float2 two_rows(const float2* __restrict__ a, const float2* __restrict__ b, int h, int u) {
   const int k = u < 0 ? -u : u;
-  if (k >= h) return make_float2(0.f, 0.f);
-  const float2 x = ld_dep(a + k), y = ld_dep(b + k);
+  const float2 x = ld_dep_if(a + k, k < h), y = ld_dep_if(b + k, k < h);
   return u < 0 ? make_float2(x.x + y.y, y.x - x.y) : make_float2(x.x - y.y, x.y + y.x);
 }
 

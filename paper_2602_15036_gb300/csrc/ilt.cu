@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_adj_rows(const float2* __restri
     const float2* row = t1 + rowoff;
     auto load_band = [&](int, int r, int idx) {
       const int c = (r < PL::R[0] / 2 ? idx : idx - N) + half;  // first pass: idx < N/2 exactly when r < R/2
-      return (c >= 0 && c < crop) ? ld_dep(row + c) : make_float2(0.f, 0.f);
+      return ld_dep_if(row + c, c >= 0 && c < crop);
     };
     auto times_g = [&](int p, int q, int idx, float2 v) {
       bufb[pad16(idx)] = make_float2(v.x * gv[p][q], v.y * gv[p][q]);
@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_grad_rows(const float2* __restr
     const float* th = theta ? theta + (clip * N + y) * N : nullptr;
     auto load = [&](int, int r, int idx) {
       const int c = (r < Plan<N>::R[0] / 2 ? idx : idx - N) + half;  // first pass: idx < N/2 exactly when r < R/2
-      return (c >= 0 && c < crop) ? ld_dep(row + c) : make_float2(0.f, 0.f);
+      return ld_dep_if(row + c, c >= 0 && c < crop);
     };
     float tv[PERL][RL];  // theta at this thread's outputs, loaded while the later passes run
     auto after_first = [&]() {
