@@ -15,6 +15,7 @@
 #include <cmath>
 #include <cstdint>
 
+#include "fft_common.cuh"
 #include "litho_internal.h"
 
 namespace litho {
@@ -29,32 +30,14 @@ unsigned blocks_per_clip(int b, size_t items) {
   return unsigned(std::max<size_t>(1, std::min(want, (items + kReduceThreads - 1) / kReduceThreads)));
 }
 
-// Floats as unsigned integers of the same order, for integer atomics.
-__device__ __forceinline__ unsigned ordered(float x) {
-  const unsigned u = __float_as_uint(x);
-  return u & 0x80000000u ? ~u : u | 0x80000000u;
-}
-__device__ __forceinline__ float from_ordered(unsigned u) {
-  return __uint_as_float(u & 0x80000000u ? u & 0x7fffffffu : ~u);
-}
-
-// X[c][0] = target[c]; clip blockIdx.y.
-template <class T>
-__global__ void __launch_bounds__(kReduceThreads) k_copy_channel(const T* __restrict__ src, T* __restrict__ x,
-                                                                 size_t n) {
-  src += (size_t)blockIdx.y * n;
-  x += (size_t)blockIdx.y * 3 * n;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    x[i] = src[i];
-}
-
-// Extremes of channels 1 and 2 of X[b][3][nn] (clip blockIdx.y, channel 1 + blockIdx.z) into
-// ext[channel - 1] = (min, max), as ordered integers: ~0 and 0 on entry.  nn is a multiple of 4.
+// Extremes of one channel of X[b][3][nn] (clip blockIdx.y; x at the channel) into *ext = (min, max), as
+// ordered integers: (~0, 0) on entry.  nn is a multiple of 4.  For the channels whose rows are not written
+// by k_band_rows, which folds them in as it goes.
 __global__ void __launch_bounds__(kReduceThreads) k_minmax(const float4* __restrict__ x, size_t nn4,
                                                            uint2* __restrict__ ext) {
   __shared__ float smin[kReduceThreads / 32], smax[kReduceThreads / 32];
   float lo = FLT_MAX, hi = -FLT_MAX;
-  const float4* src = x + (size_t(blockIdx.y) * 3 + 1 + blockIdx.z) * nn4;
+  const float4* src = x + size_t(blockIdx.y) * 3 * nn4;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nn4; i += (size_t)gridDim.x * blockDim.x) {
     const float4 v = src[i];
     lo = fminf(lo, fminf(fminf(v.x, v.y), fminf(v.z, v.w)));
@@ -74,8 +57,8 @@ __global__ void __launch_bounds__(kReduceThreads) k_minmax(const float4* __restr
       lo = fminf(lo, smin[w]);
       hi = fmaxf(hi, smax[w]);
     }
-    atomicMin(&ext[blockIdx.z].x, ordered(lo));
-    atomicMax(&ext[blockIdx.z].y, ordered(hi));
+    atomicMin(&ext->x, ordered(lo));
+    atomicMax(&ext->y, ordered(hi));
   }
 }
 
@@ -184,25 +167,20 @@ litho_status litho_ai_inputs(const litho_kernels* h, const float* target_dev, in
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t nn = size_t(h->n) * h->n;
   uint2* ext = reinterpret_cast<uint2*>(static_cast<char*>(workspace_dev) + up256(ai_channels_bytes(h, b)));
-  {
-    ProfScope ps(kStageIltForward, st, 1);
-    const bool vec = ((reinterpret_cast<uintptr_t>(target_dev) | reinterpret_cast<uintptr_t>(x_dev)) & 15) == 0;
-    if (vec)
-      k_copy_channel<<<dim3(blocks_per_clip(b, nn / 4), b), kReduceThreads, 0, st>>>(
-          reinterpret_cast<const float4*>(target_dev), reinterpret_cast<float4*>(x_dev), nn / 4);
-    else
-      k_copy_channel<<<dim3(blocks_per_clip(b, nn), b), kReduceThreads, 0, st>>>(target_dev, x_dev, nn);
-    LITHO_TRY_CUDA(cudaGetLastError());
-  }
-  s = ai_channels(h, target_dev, b, dose, focus, (int(prec) & LITHO_GRID_COARSE) != 0, x_dev, workspace_dev, st);
-  if (s != LITHO_OK) return s;
-  ProfScope ps(kStageIltReduce, st, 2);
   for (int ch = 0; ch < 2; ++ch) {  // (~0, 0): nothing seen yet
     LITHO_TRY_CUDA(cudaMemsetAsync(&ext[ch].x, 0xff, sizeof(unsigned), st));
     LITHO_TRY_CUDA(cudaMemsetAsync(&ext[ch].y, 0, sizeof(unsigned), st));
   }
+  bool found[2];
+  s = ai_channels(h, target_dev, b, dose, focus, (int(prec) & LITHO_GRID_COARSE) != 0, x_dev, workspace_dev, ext, found,
+                  st);
+  if (s != LITHO_OK) return s;
+  ProfScope ps(kStageIltReduce, st, 1);
+  for (int ch = 0; ch < 2; ++ch)
+    if (!found[ch])
+      k_minmax<<<dim3(blocks_per_clip(b, nn / 4), b), kReduceThreads, 0, st>>>(
+          reinterpret_cast<const float4*>(x_dev + (1 + ch) * nn), nn / 4, ext + ch);
   const dim3 grid(blocks_per_clip(2 * b, nn / 4), b, 2);
-  k_minmax<<<grid, kReduceThreads, 0, st>>>(reinterpret_cast<const float4*>(x_dev), nn / 4, ext);
   k_normalize<<<grid, kReduceThreads, 0, st>>>(reinterpret_cast<float4*>(x_dev), nn / 4, ext);
   LITHO_TRY_CUDA(cudaGetLastError());
   return LITHO_OK;

@@ -13,6 +13,7 @@
 //   t1      [j][N][C] c64   stage-1 field T_j[y][u] = sum_v mhat[v][u] Phi_j[v][u] e^{2 pi i v y/N}
 //   img     [plane][N][N] f32
 #include <algorithm>
+#include <cfloat>
 
 #include "fft_common.cuh"
 #include "litho_internal.h"
@@ -30,12 +31,15 @@ __device__ __forceinline__ int freq_of(int idx, int n) { return idx < n / 2 ? id
 
 // ---- mask spectrum, pass 1: two real rows per complex transform ----------------------------
 // z = m[y0] + i m[y1]; Z = DFT(z); X(u) = (Z(u) + conj Z(-u))/2, Y(u) = (Z(u) - conj Z(-u))/(2i),
-// written for u in [0, cols) with row stride ld.  SIGMOID: the mask is sigmoid(alpha m) (the ILT's theta).
-template <int N, bool SIGMOID>
+// written for u in [0, cols) with row stride ld.  Mask: m; Sigmoid: sigmoid(alpha m) (the ILT's theta); Copy:
+// m, which is also written to copy + b copy_stride on the way (the AI input's first channel).
+enum class RowInput { Mask, Sigmoid, Copy };
+template <int N, RowInput IN>
 __global__ void __launch_bounds__(Plan<N>::NT) k_mask_rows(const float* __restrict__ m, float alpha, int crop,
                                                             const float2* __restrict__ tw_g,
                                                             float2* __restrict__ rowbuf, int cols, int ld,
-                                                            int pairs_per_cta) {
+                                                            int pairs_per_cta, float* __restrict__ copy,
+                                                            size_t copy_stride) {
   extern __shared__ float2 smem[];
   float2* tw = smem;
   float2* buf = smem + N;
@@ -55,7 +59,9 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_mask_rows(const float* __restri
     for (int r = 0; r < R0; ++r)
       nxt[r] = t < NB0 ? make_float2(ld_dep(r0 + t + r * NB0), ld_dep(r0 + N + t + r * NB0)) : make_float2(0.f, 0.f);
   };
-  auto value = [&](float2 v) { return SIGMOID ? make_float2(sigmoidf(alpha * v.x), sigmoidf(alpha * v.y)) : v; };
+  auto value = [&](float2 v) {
+    return IN == RowInput::Sigmoid ? make_float2(sigmoidf(alpha * v.x), sigmoidf(alpha * v.y)) : v;
+  };
   const int pr0 = blockIdx.x * pairs_per_cta, pr1 = min(N / 2, (blockIdx.x + 1) * pairs_per_cta);
   if (pr0 < pr1) prefetch(pr0);
   // pairs [pr0, pr1): the next pair's first pass writes buf only after a
@@ -65,6 +71,14 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_mask_rows(const float* __restri
     float2 cur[R0];
 #pragma unroll
     for (int r = 0; r < R0; ++r) cur[r] = nxt[r];
+    if (IN == RowInput::Copy && t < NB0) {
+      float* c0 = copy + b * copy_stride + (size_t)y0 * N + t;
+#pragma unroll
+      for (int r = 0; r < R0; ++r) {
+        c0[r * NB0] = cur[r].x;
+        c0[N + r * NB0] = cur[r].y;
+      }
+    }
     auto load = [&](int, int r, int) { return value(cur[r]); };
     auto use = [&](int, int, int idx, float2 v) {
       const int u = freq_of(idx, N);
@@ -287,13 +301,15 @@ __device__ __forceinline__ float2 two_rows(const float2* __restrict__ a, const f
 // Band rows q of h columns two by two (unit i: rows 2 i and 2 i + 1 of q).  RESIST: the two are a row's image
 // and its blur: img = Re (skipped when NULL), iblur = Im, printed = [Im >= threshold] (skipped when NULL).
 // Otherwise they are two rows of the image: img rows 2 i and 2 i + 1, times scale.  Plane p of `planes`
-// per clip goes to its planes of `po`.  Bound by HBM (the rows written).
+// per clip goes to its planes of `po`.  With ext (image rows only) the extremes of what is written are
+// folded into ext = (min, max) as ordered integers.  Bound by HBM (the rows written).
 template <int N, bool BANDED, bool RESIST>
 __global__ void __launch_bounds__(Plan<N>::NT) k_band_rows(const float2* __restrict__ q, int h, float scale,
                                                            const float2* __restrict__ tw_g, float thr,
                                                            float* __restrict__ img, float* __restrict__ iblur,
                                                            uint8_t* __restrict__ printed, int planes,
-                                                           const __grid_constant__ PlaneOut po, int units_per_cta) {
+                                                           const __grid_constant__ PlaneOut po, int units_per_cta,
+                                                           uint2* __restrict__ ext) {
   constexpr int NT = Plan<N>::NT, RL = Plan<N>::R[Plan<N>::P - 1], PERL = PassShape<N, NT, RL>::PER;
   constexpr int UNITS = RESIST ? N : N / 2;
   __shared__ float2 buf[PadLen<N>::value];
@@ -304,6 +320,7 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_band_rows(const float2* __restr
   __syncthreads();
   const int p = blockIdx.y, t = threadIdx.x, clip = p / planes, pl = p - clip * planes;
   const int d0 = po.first[pl], d1 = po.first[pl + 1];
+  float lo = FLT_MAX, hi = -FLT_MAX;
   for (int i = blockIdx.x * units_per_cta; i < min(UNITS, (blockIdx.x + 1) * units_per_cta); ++i) {
     const float2* row = q + ((size_t)p * UNITS + i) * 2 * h;
     auto load = [&](int, int r, int idx) {  // first pass: idx < N/2 exactly when r < R/2
@@ -325,11 +342,31 @@ __global__ void __launch_bounds__(Plan<N>::NT) k_band_rows(const float2* __restr
               iblur[at] = res[pp][qq].y;
               if (printed) printed[at] = res[pp][qq].y >= thr ? 1 : 0;
             } else {
-              img[at] = scale * res[pp][qq].x;
-              img[at + N] = scale * res[pp][qq].y;
+              const float a = scale * res[pp][qq].x, b = scale * res[pp][qq].y;
+              img[at] = a;
+              img[at + N] = b;
+              lo = fminf(lo, fminf(a, b));
+              hi = fmaxf(hi, fmaxf(a, b));
             }
           }
         }
+    }
+  }
+  if (!RESIST && ext) {
+    for (int o = 16; o > 0; o >>= 1) {
+      lo = fminf(lo, __shfl_down_sync(0xffffffffu, lo, o));
+      hi = fmaxf(hi, __shfl_down_sync(0xffffffffu, hi, o));
+    }
+    __shared__ float2 warp_ext[(NT + 31) / 32];
+    if (t % 32 == 0) warp_ext[t / 32] = make_float2(lo, hi);
+    __syncthreads();
+    if (t == 0) {
+      for (int w = 1; w < (NT + 31) / 32; ++w) {
+        lo = fminf(lo, warp_ext[w].x);
+        hi = fmaxf(hi, warp_ext[w].y);
+      }
+      atomicMin(&ext->x, ordered(lo));
+      atomicMax(&ext->y, ordered(hi));
     }
   }
 }
@@ -446,12 +483,13 @@ __global__ void __launch_bounds__(Plan<N>::NT, N >= 512 ? 640 / Plan<N>::NT : 1)
 
 template <int N, bool RESIST>
 cudaError_t band_rows_n(const float2* q, int clips, int planes, int h, float scale, const float2* tw, float thr,
-                        float* img, float* iblur, uint8_t* printed, const PlaneOut& po, cudaStream_t st) {
+                        float* img, float* iblur, uint8_t* printed, const PlaneOut& po, cudaStream_t st,
+                        uint2* ext = nullptr) {
   const int units = RESIST ? N : N / 2;
   const int per = rows_per_cta(units, clips * planes, 2048 / Plan<N>::NT), grid = (units + per - 1) / per;
   auto kern = 4 * h <= N ? k_band_rows<N, true, RESIST> : k_band_rows<N, false, RESIST>;
   return launch_pdl(kern, dim3(grid, clips * planes), Plan<N>::NT, 0, st, q, h, scale, tw, thr, img, iblur, printed,
-                    planes, po, per);
+                    planes, po, per, ext);
 }
 
 template <int N>
@@ -496,15 +534,17 @@ cudaError_t mask_cols_n(const float2* rowbuf, int b, int crop, const float2* tw,
 }
 
 template <int N>
-cudaError_t mask_rows_n(const float* m, bool sigmoid, float alpha, int b, int crop, const float2* tw, float2* rowbuf, bool whole,
-                        cudaStream_t st) {
+cudaError_t mask_rows_n(const float* m, RowInput in, float alpha, int b, int crop, const float2* tw, float2* rowbuf,
+                        bool whole, cudaStream_t st, float* copy = nullptr, size_t copy_stride = 0) {
   const size_t smr = sizeof(float2) * (2 * N + PadLen<N>::value + 1);
-  auto kern = sigmoid ? k_mask_rows<N, true> : k_mask_rows<N, false>;
+  auto kern = in == RowInput::Sigmoid ? k_mask_rows<N, RowInput::Sigmoid>
+              : in == RowInput::Copy  ? k_mask_rows<N, RowInput::Copy>
+                                      : k_mask_rows<N, RowInput::Mask>;
   cudaError_t e = smem_attrs(kern, smr);
   if (e != cudaSuccess) return e;
   const int ppc = rows_per_cta(N / 2, b, 2048 / Plan<N>::NT);
   return launch_pdl(kern, dim3((N / 2 + ppc - 1) / ppc, b), Plan<N>::NT, smr, st, m, alpha, crop, tw, rowbuf,
-                    half_cols(crop, whole), half_ld(crop, whole), ppc);
+                    half_cols(crop, whole), half_ld(crop, whole), ppc, copy, copy_stride);
 }
 
 template <int N>
@@ -579,15 +619,15 @@ cudaError_t launch_mask_spectrum(const float* m, int b, int n, int crop, const f
 }
 
 cudaError_t launch_band_rows_real(const float2* q, int clips, int planes, int n, int h, float scale, const float2* tw,
-                                  float* out, const PlaneOut& po, cudaStream_t st) {
-#define CALL(N) band_rows_n<N, false>(q, clips, planes, h, scale, tw, 0.f, out, nullptr, nullptr, po, st)
+                                  float* out, const PlaneOut& po, cudaStream_t st, uint2* ext) {
+#define CALL(N) band_rows_n<N, false>(q, clips, planes, h, scale, tw, 0.f, out, nullptr, nullptr, po, st, ext)
   LITHO_DISPATCH_N(n, CALL)
 #undef CALL
 }
 
 cudaError_t launch_mask_rows(const float* m, int b, int n, int crop, const float2* tw, float2* rowbuf, bool whole,
                              cudaStream_t st) {
-#define CALL(N) mask_rows_n<N>(m, false, 0.f, b, crop, tw, rowbuf, whole, st)
+#define CALL(N) mask_rows_n<N>(m, RowInput::Mask, 0.f, b, crop, tw, rowbuf, whole, st)
   LITHO_DISPATCH_NC(n, CALL)
 #undef CALL
 }
@@ -595,7 +635,18 @@ cudaError_t launch_mask_rows(const float* m, int b, int n, int crop, const float
 cudaError_t launch_sigmoid_spectrum(const float* theta, float alpha, int b, int n, int crop, const float2* tw,
                                     float2* rowbuf, float2* mhat, cudaStream_t st) {
   auto rows = [&]() {
-#define CALL(N) mask_rows_n<N>(theta, true, alpha, b, crop, tw, rowbuf, true, st)
+#define CALL(N) mask_rows_n<N>(theta, RowInput::Sigmoid, alpha, b, crop, tw, rowbuf, true, st)
+    LITHO_DISPATCH_N(n, CALL)
+#undef CALL
+  };
+  const cudaError_t e = rows();
+  return e != cudaSuccess ? e : launch_mask_cols(rowbuf, b, n, crop, tw, mhat, nullptr, true, st);
+}
+
+cudaError_t launch_mask_spectrum_copy(const float* m, int b, int n, int crop, const float2* tw, float2* rowbuf,
+                                      float2* mhat, float* copy, size_t copy_stride, cudaStream_t st) {
+  auto rows = [&]() {
+#define CALL(N) mask_rows_n<N>(m, RowInput::Copy, 0.f, b, crop, tw, rowbuf, true, st, copy, copy_stride)
     LITHO_DISPATCH_N(n, CALL)
 #undef CALL
   };

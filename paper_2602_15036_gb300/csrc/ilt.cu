@@ -707,7 +707,7 @@ double* ilt_loss_device(const litho_kernels* h, int b, void* workspace, size_t w
 size_t ai_channels_bytes(const litho_kernels* h, int b) { return ilt_layout(h, b, 1, ilt_group(h, b), nullptr).bytes; }
 
 litho_status ai_channels(const litho_kernels* h, const float* target, int b, double dose, int focus, bool coarse,
-                         float* x, void* workspace, cudaStream_t st) {
+                         float* x, void* workspace, uint2* ext, bool found[2], cudaStream_t st) {
   const int G = ilt_group(h, b), N = h->n, C = h->crop;
   IltLayout L = ilt_layout(h, b, 1, G, workspace);
   const size_t nn = size_t(N) * N;
@@ -724,19 +724,21 @@ litho_status ai_channels(const litho_kernels* h, const float* target, int b, dou
   const float scale = float(2.0 * dose / (double(N) * double(N)));
   // a 1024-point coarse grid: the warp-per-row stage 2 writes the coarse image's row spectra itself
   const bool rows2 = coarse && h->d_tw32 && stage2_w32_supported(NE, C);
+  found[0] = coarse;
+  found[1] = !h->edge;
   for (int c0 = 0; c0 < b; c0 += G) {
     const int g = std::min(G, b - c0);
     float* dst = x + size_t(c0) * 3 * nn;
     {  // channel 1: the aerial image of the targets (interpolated from the coarse grid)
       ProfScope ps(kStageIltForward, st, coarse ? (rows2 ? 6 : 7) : 4);
-      LITHO_TRY_CUDA(launch_mask_spectrum(target + c0 * nn, g, N, C, h->d_tw, L.rowbuf, L.mhat, st));
+      LITHO_TRY_CUDA(launch_mask_spectrum_copy(target + c0 * nn, g, N, C, h->d_tw, L.rowbuf, L.mhat, dst, 3 * nn, st));
       LITHO_TRY_CUDA(launch_stage1_fft(L.mhat, psi, fs.fields(), NE, C, twe, L.t1, st, g));
       LITHO_TRY_CUDA(launch_stage2_fft(L.t1, fs, g, NE, C, float(dose), twe, coarse ? L.ic : dst,
                                        coarse ? one : channel1, st, h->d_tw32, h->d_tw512, rows2 ? L.mid : nullptr, C2));
       if (coarse) {
         if (!rows2) LITHO_TRY_CUDA(launch_mask_rows(L.ic, g, NE, C2, twe, L.mid, false, st));
         LITHO_TRY_CUDA(launch_interp_cols(L.mid, g, NE, N, C, twe, h->d_tw, nullptr, true, L.big, st));
-        LITHO_TRY_CUDA(launch_band_rows_real(L.big, g, 1, N, C, 1.0f, h->d_tw, dst, channel1, st));
+        LITHO_TRY_CUDA(launch_band_rows_real(L.big, g, 1, N, C, 1.0f, h->d_tw, dst, channel1, st, ext));
       }
     }
     {  // channel 2: the adjoint applied to dL/dI = 1, in closed form (k_ones_adjoint)
@@ -751,7 +753,7 @@ litho_status ai_channels(const litho_kernels* h, const float* target, int b, dou
                                         (long long)3 * nn, st));
       } else {  // S(-u) = conj S(u): half the columns, two rows to a transform
         LITHO_TRY_CUDA(launch_stage1_half(L.s, g, N, C, h->d_tw, L.qf, C / 2, st));
-        LITHO_TRY_CUDA(launch_band_rows_real(L.qf, g, 1, N, C / 2, scale, h->d_tw, dst, channel2, st));
+        LITHO_TRY_CUDA(launch_band_rows_real(L.qf, g, 1, N, C / 2, scale, h->d_tw, dst, channel2, st, ext + 1));
       }
     }
   }

@@ -165,6 +165,9 @@ cudaError_t launch_mask_spectrum(const float* m, int b, int n, int crop, const f
 // The same of the mask sigmoid(alpha theta).
 cudaError_t launch_sigmoid_spectrum(const float* theta, float alpha, int b, int n, int crop, const float2* tw,
                                     float2* rowbuf, float2* mhat, cudaStream_t st);
+// The mask spectrum, the masks also copied to copy + i copy_stride.
+cudaError_t launch_mask_spectrum_copy(const float* m, int b, int n, int crop, const float2* tw, float2* rowbuf,
+                                      float2* mhat, float* copy, size_t copy_stride, cudaStream_t st);
 // Its two passes.  Row DFTs of real planes, the frequencies u >= 0: rowbuf[b][n][C/2], index u, or (whole:
 // with u = C/2) [b][n][C/2 + 8].
 cudaError_t launch_mask_rows(const float* m, int b, int n, int crop, const float2* tw, float2* rowbuf, bool whole,
@@ -232,19 +235,20 @@ void adj512_table(float2* out);
 // Device address of the per-clip FP64 losses inside an ILT workspace (ilt.cu).
 double* ilt_loss_device(const litho_kernels* h, int b, void* workspace, size_t workspace_bytes);
 
-// Channels 1 and 2 of Eq. (9) before normalisation (ilt.cu): for b targets
-// at focus plane `focus`, x[c][1] = the aerial image and x[c][2] = the
-// gradient of the plane's total intensity with respect to the mask pixels
-// (x: [b][3][n][n]), in groups of clips; `coarse` evaluates the fields and
-// the adjoint on the coarse grid.  Workspace: ai_channels_bytes(h, b).
+// The channels of Eq. (9) before normalisation (ilt.cu): for b targets at focus plane `focus`, x[c][0] = the
+// target, x[c][1] = the aerial image and x[c][2] = the gradient of the plane's total intensity with
+// respect to the mask pixels (x: [b][3][n][n]), in groups of clips; `coarse` evaluates the fields and the
+// adjoint on the coarse grid.  The extremes of channels 1 and 2 are folded into ext[0] and ext[1] (ordered
+// integers, (~0, 0) on entry) where a kernel writes the channel by rows; found[i] tells.  Workspace:
+// ai_channels_bytes(h, b).
 size_t ai_channels_bytes(const litho_kernels* h, int b);
 litho_status ai_channels(const litho_kernels* h, const float* target, int b, double dose, int focus, bool coarse,
-                         float* x, void* workspace, cudaStream_t st);
+                         float* x, void* workspace, uint2* ext, bool found[2], cudaStream_t st);
 
 // Image rows from half band rows q[p][n][h] of `clips` x `planes` planes p, times scale; plane p of a clip
-// goes to its planes of `po` in out.
+// goes to its planes of `po` in out.  ext: its (min, max) are updated as ordered integers.
 cudaError_t launch_band_rows_real(const float2* q, int clips, int planes, int n, int h, float scale, const float2* tw,
-                                  float* out, const PlaneOut& po, cudaStream_t st);
+                                  float* out, const PlaneOut& po, cudaStream_t st, uint2* ext = nullptr);
 
 struct ResistTaps;
 // gain[i] = sum_a g[a] cos(2 pi (i - crop/2) a / n): the blur's transfer function on the crop.
