@@ -16,6 +16,7 @@
 // (32 x 128 strips that loaded 2R + 1 shared values per pixel and row).
 #include <cmath>
 
+#include "fft_common.cuh"
 #include "litho_internal.h"
 
 namespace litho {
@@ -34,6 +35,8 @@ __global__ void __launch_bounds__(kThreads, R > 10 ? 2 : 3) k_resist(const float
   static_assert(SH % GROUPS == 0, "whole row groups");
   __shared__ __align__(16) float hb[ROWS * TW];  // horizontally blurred rows
   const int x0 = blockIdx.x * TW, y0 = blockIdx.y * SH;
+  pdl_start();
+  pdl_wait(img);
   const size_t plane = (size_t)blockIdx.z * n * n;
   const float* src = img + plane;
   // rows: hb[ry][x] = sum_a g[a] I[y0 + ry - R][x0 + x - a]
@@ -48,14 +51,14 @@ __global__ void __launch_bounds__(kThreads, R > 10 ? 2 : 3) k_resist(const float
       int gx = xs - HR + 4 * q;
       gx += gx < 0 ? n : gx >= n ? -n : 0;
       if constexpr (ALIGNED) {
-        const float4 v = __ldg(reinterpret_cast<const float4*>(row + gx));
+        const float4 v = ld_dep(reinterpret_cast<const float4*>(row + gx));
         w[4 * q] = v.x;
         w[4 * q + 1] = v.y;
         w[4 * q + 2] = v.z;
         w[4 * q + 3] = v.w;
       } else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) w[4 * q + e] = __ldg(row + gx + e);
+        for (int e = 0; e < 4; ++e) w[4 * q + e] = ld_dep(row + gx + e);
       }
     }
     float o[8];
@@ -100,59 +103,106 @@ __global__ void __launch_bounds__(kThreads, R > 10 ? 2 : 3) k_resist(const float
   }
 }
 
-// Any radius, taps in a loop: a 32 x SH strip and its halo in shared memory, a warp per row for the
-// horizontal sums, a thread per column for the vertical ones.
-template <int SH>
-__global__ void __launch_bounds__(kThreads) k_resist_any(const float* __restrict__ img, int n,
-                                                         const __grid_constant__ ResistTaps taps, float thr,
-                                                         float* __restrict__ iblur, uint8_t* __restrict__ printed) {
-  constexpr int SW = 32, WARPS = kThreads / 32, PER = SH / WARPS;
+// Any radius.  A CTA takes 32 x SH pixels; the tile and its periodic halo go to shared memory, rows at an odd
+// pitch, so that lanes on different rows, and lanes on different columns, read different banks.  Each
+// thread forms eight neighbouring outputs (of a row, then of a column) from a window of 15 values that
+// moves by eight taps at a time: one shared-memory load per eight FMAs, taps in the order of the fixed radii.
+// 265 planes of 1024^2: 28.3 -> 4.46 ms at R = 40, 6.33 -> 2.85 ms at R = 20 (a load for every FMA); bound by
+// the FP32 pipe and the shared-memory loads of the halo rows.
+
+// o[j] = sum over t of taps.g[t] s[(j + 2 r - t) stride], t = 0 .. 2 r.
+__device__ __forceinline__ void blur8(const float* s, int stride, const ResistTaps& taps, float (&o)[8]) {
+  const int last = 2 * taps.radius;
+  float w[15];  // w[m] = s[last - 8 c - 7 + m] in chunk c
+#pragma unroll
+  for (int m = 0; m < 15; ++m) w[m] = last - 7 + m >= 0 ? s[(last - 7 + m) * stride] : 0.f;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) o[j] = 0.f;
+  int t0 = 0;
+  for (; t0 + 15 <= last; t0 += 8) {  // whole chunks, and the next one's eight values exist
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float g = taps.g[t0 + i];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) o[j] = fmaf(g, w[j - i + 7], o[j]);
+    }
+#pragma unroll
+    for (int m = 14; m >= 8; --m) w[m] = w[m - 8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) w[m] = s[(last - t0 - 15 + m) * stride];
+  }
+  for (; t0 <= last; t0 += 8) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      if (t0 + i > last) break;
+      const float g = taps.g[t0 + i];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) o[j] = fmaf(g, w[j - i + 7], o[j]);
+    }
+#pragma unroll
+    for (int m = 14; m >= 8; --m) w[m] = w[m - 8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      const int k = last - t0 - 15 + m;
+      w[m] = k >= 0 ? s[k * stride] : 0.f;
+    }
+  }
+}
+
+template <int W, int SH, int NT>
+__global__ void __launch_bounds__(NT) k_resist_any(const float* __restrict__ img, int n,
+                                                   const __grid_constant__ ResistTaps taps, float thr,
+                                                   float* __restrict__ iblur, uint8_t* __restrict__ printed) {
   extern __shared__ float sm[];
-  const int r = taps.radius, rows_in = SH + 2 * r, wi = SW + 2 * r;
-  float* tile = sm;               // [rows_in][wi] the strip and its periodic halo
-  float* hb = sm + rows_in * wi;  // [rows_in][SW] horizontally blurred rows
+  const int r = taps.radius, rows = SH + 2 * r, wi = W + 2 * r, pitch = wi | 1, hp = W + 1;
+  float* tile = sm;                // [rows][pitch]
+  float* hb = sm + rows * pitch;   // [rows][hp] horizontally blurred rows
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int plane = blockIdx.z, x0 = blockIdx.x * SW, y0 = blockIdx.y * SH;
-  const float* src = img + (size_t)plane * n * n;
-  for (int ry = warp; ry < rows_in; ry += WARPS) {  // r < n/2: one wrap at most
+  const int x0 = blockIdx.x * W, y0 = blockIdx.y * SH;
+  pdl_start();
+  pdl_wait(img);
+  const size_t plane = (size_t)blockIdx.z * n * n;
+  const float* src = img + plane;
+  for (int ry = warp; ry < rows; ry += NT / 32) {  // r < n/2: one wrap at most
     int gy = y0 + ry - r;
     gy += gy < 0 ? n : gy >= n ? -n : 0;
     for (int rx = lane; rx < wi; rx += 32) {
       int gx = x0 + rx - r;
       gx += gx < 0 ? n : gx >= n ? -n : 0;
-      tile[ry * wi + rx] = __ldg(src + (size_t)gy * n + gx);
+      tile[ry * pitch + rx] = ld_dep(src + (size_t)gy * n + gx);
     }
   }
   __syncthreads();
-  for (int ry = warp; ry < rows_in; ry += WARPS) {
-    const float* t = tile + ry * wi + lane + r;
-    float acc = 0.f;
-    for (int a = -r; a <= r; ++a) acc = fmaf(taps.g[a + r], t[-a], acc);
-    hb[ry * SW + lane] = acc;
+  float o[8];
+  for (int i = threadIdx.x; i < rows * (W / 8); i += NT) {  // lanes on rows
+    const int seg = i / rows, ry = i - seg * rows;
+    blur8(tile + ry * pitch + 8 * seg, 1, taps, o);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) hb[ry * hp + 8 * seg + j] = o[j];
   }
   __syncthreads();
-  const int yy = warp * PER;
-  float* dst = iblur + (size_t)plane * n * n;
-  uint8_t* pr = printed ? printed + (size_t)plane * n * n : nullptr;
-  for (int i = 0; i < PER; ++i) {
-    const float* c = hb + (yy + i + r) * SW + lane;
-    float acc = 0.f;
-    for (int a = -r; a <= r; ++a) acc = fmaf(taps.g[a + r], c[-a * SW], acc);
-    const size_t o = (size_t)(y0 + yy + i) * n + x0 + lane;
-    dst[o] = acc;
-    if (pr) pr[o] = acc >= thr ? 1 : 0;
+  for (int i = threadIdx.x; i < W * (SH / 8); i += NT) {  // lanes on columns
+    const int x = i % W, y = i / W * 8;
+    blur8(hb + y * hp + x, hp, taps, o);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const size_t at = plane + (size_t)(y0 + y + j) * n + x0 + x;
+      iblur[at] = o[j];
+      if (printed) printed[at] = o[j] >= thr ? 1 : 0;
+    }
   }
 }
 
-template <int SH>
+size_t any_bytes(int r, int w, int sh) { return sizeof(float) * (sh + 2 * r) * (((w + 2 * r) | 1) + w + 1); }
+
+template <int W, int SH, int NT>
 cudaError_t launch_any(const float* img, int planes, int n, const ResistTaps& taps, float thr, float* iblur,
                        uint8_t* printed, cudaStream_t st) {
-  const int r = taps.radius;
-  const size_t sm = sizeof(float) * ((SH + 2 * r) * (32 + 2 * r) + (SH + 2 * r) * 32);
-  cudaError_t e = cudaFuncSetAttribute(k_resist_any<SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  const size_t sm = any_bytes(taps.radius, W, SH);  // 199 KB at radius 64 for 32 x 128
+  cudaError_t e = cudaFuncSetAttribute(k_resist_any<W, SH, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  k_resist_any<SH><<<dim3(n / 32, n / SH, planes), kThreads, sm, st>>>(img, n, taps, thr, iblur, printed);
-  return cudaGetLastError();
+  return launch_pdl(k_resist_any<W, SH, NT>, dim3(n / W, n / SH, planes), NT, sm, st, img, n, taps, thr, iblur,
+                    printed);
 }
 
 template <int R>
@@ -160,20 +210,16 @@ cudaError_t launch_r(const float* img, int planes, int n, const ResistTaps& taps
                      uint8_t* printed, cudaStream_t st) {
   const bool aligned = (reinterpret_cast<uintptr_t>(img) & 15) == 0 && (reinterpret_cast<uintptr_t>(iblur) & 7) == 0 &&
                        (reinterpret_cast<uintptr_t>(printed) & 1) == 0;
-#define RUN(TW, SH, A) \
-  k_resist<R, TW, SH, A><<<dim3(n / TW, n / SH, planes), kThreads, 0, st>>>(img, n, taps, thr, iblur, printed)
+#define RUN(TW, SH, A)                                                                                            \
+  return launch_pdl(k_resist<R, TW, SH, A>, dim3(n / TW, n / SH, planes), kThreads, 0, st, img, n, taps, thr, iblur, \
+                    printed)
   // 128-row tiles read (128 + 2R)/128 of the rows; with fewer than two of them per SM, 32-row tiles
   // fill the chip instead
-  if (!aligned)
-    RUN(32, 32, false);
-  else if (n % 128 == 0 && (long long)planes * (n / 64) * (n / 128) >= 304)
-    RUN(64, 128, true);
-  else if (n % 64 == 0)
-    RUN(64, 32, true);
-  else
-    RUN(32, 32, true);
+  if (!aligned) RUN(32, 32, false);
+  if (n % 128 == 0 && (long long)planes * (n / 64) * (n / 128) >= 304) RUN(64, 128, true);
+  if (n % 64 == 0) RUN(64, 32, true);
+  RUN(32, 32, true);
 #undef RUN
-  return cudaGetLastError();
 }
 
 }  // namespace
@@ -208,8 +254,16 @@ cudaError_t launch_resist(const float* img, int planes, int n, const ResistTaps&
     R_CASE(11) R_CASE(12)
 #undef R_CASE
     default:
-      return n % 128 == 0 ? launch_any<128>(img, planes, n, taps, threshold, iblur, printed, st)
-                          : launch_any<32>(img, planes, n, taps, threshold, iblur, printed, st);
+      if (n % 128 != 0) return launch_any<32, 32, 512>(img, planes, n, taps, threshold, iblur, printed, st);
+      // two tiles per SM while they fit (radius 36); then one, by twice the threads, and wide enough
+      // for less of a halo where that fits (radius 55) and fills the chip.  265 planes of 1024^2, 32 and 64 wide:
+      // 2840 and 3251 us at R = 20, 8627 (by 512 threads) and 4455 at R = 40; 64 of 2048^2 at R = 64, by 512 and
+      // 1024 threads: 9.98 and 8.12 ms
+      if (2 * any_bytes(taps.radius, 32, 128) <= 226 * 1024)
+        return launch_any<32, 128, 512>(img, planes, n, taps, threshold, iblur, printed, st);
+      if (any_bytes(taps.radius, 64, 128) <= 227 * 1024 && (long long)planes * (n / 64) * (n / 128) >= 152)
+        return launch_any<64, 128, 1024>(img, planes, n, taps, threshold, iblur, printed, st);
+      return launch_any<32, 128, 1024>(img, planes, n, taps, threshold, iblur, printed, st);
   }
 }
 

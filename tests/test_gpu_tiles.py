@@ -14,9 +14,9 @@ from oracle import resist as OR
 pytestmark = pytest.mark.gpu
 
 
-# radius 1, 5, 10, 12 (register windows) and 13, 30 (loop); 128-, 64- and 32-wide tiles, few and many planes
+# radius 1, 5, 10, 12 (register windows) and 13, 15, 30, 45, 64 (loop); 128-, 64- and 32-wide tiles, few and many planes
 @pytest.mark.parametrize("n,planes", [(32, 3), (96, 2), (64, 5), (128, 1), (256, 40), (192, 3)])
-@pytest.mark.parametrize("radius", [1, 5, 10, 12, 13, 30])
+@pytest.mark.parametrize("radius", [1, 5, 10, 12, 13, 15, 30, 45, 64])
 def test_blur_tiles(litho_lib, cuda, n, planes, radius):
     import torch
     if 2 * radius >= n:
@@ -90,9 +90,10 @@ def test_contour_rows(litho_lib, cuda, n):
         assert np.all(np.abs(seg[start[p]:start[p + 1]] - want) <= 1e-5 + 2.5e-7 * np.abs(want))
 
 
-def test_epe_wraps_outside_the_grid(litho_lib, cuda):
+# rows of whole 16-byte pieces, and not
+@pytest.mark.parametrize("n", [96, 90])
+def test_epe_wraps_outside_the_grid(litho_lib, cuda, n):
     import torch
-    n = 96
     img = (0.5 + 0.4 * np.sin(2 * np.pi * np.mgrid[0:n, 0:n][1] * 3 / n) * np.cos(2 * np.pi * np.mgrid[0:n, 0:n][0] * 2 / n))
     img = img.astype(np.float32)
     st = synth.Stream(2)
