@@ -92,6 +92,8 @@ __global__ void __launch_bounds__(kReduceThreads) k_print(const float* __restric
                                                           uint4* __restrict__ z_print,
                                                           unsigned long long* __restrict__ out) {
   __shared__ unsigned warp_sum[kReduceThreads / 32];
+  pdl_start();
+  pdl_wait(img, z_round);
   const size_t base = size_t(blockIdx.y) * pieces;
   unsigned c = 0;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < pieces; i += (size_t)gridDim.x * blockDim.x) {
@@ -101,9 +103,9 @@ __global__ void __launch_bounds__(kReduceThreads) k_print(const float* __restric
       float4 v;
       const float* s = img + (base + i) * 16 + 4 * q;
       if constexpr (VEC)
-        v = __ldg(reinterpret_cast<const float4*>(s));
+        v = ld_dep(reinterpret_cast<const float4*>(s));
       else
-        v = make_float4(__ldg(s), __ldg(s + 1), __ldg(s + 2), __ldg(s + 3));
+        v = make_float4(ld_dep(s), ld_dep(s + 1), ld_dep(s + 2), ld_dep(s + 3));
       z[q] = unsigned(v.x >= thr) | unsigned(v.y >= thr) << 8 | unsigned(v.z >= thr) << 16 | unsigned(v.w >= thr) << 24;
     }
     z_print[base + i] = make_uint4(z[0], z[1], z[2], z[3]);
@@ -214,14 +216,14 @@ litho_status litho_print_images(const float* target_dev, const float* intensity_
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t nn = size_t(n) * n;
   ProfScope ps(kStageResist, st, 2);
-  LITHO_TRY_CUDA(launch_resist(target_dev, b, n, taps, float(tau_round), blur_dev, z_round_dev, st));
   if (loss_dev) LITHO_TRY_CUDA(cudaMemsetAsync(loss_dev, 0, size_t(b) * sizeof(int64_t), st));
+  LITHO_TRY_CUDA(launch_resist(target_dev, b, n, taps, float(tau_round), blur_dev, z_round_dev, st));
   const size_t pieces = nn / 16;
   const dim3 grid(blocks_per_clip(b, pieces), b);
   auto kern = (reinterpret_cast<uintptr_t>(intensity_dev) & 15) == 0 ? k_print<true> : k_print<false>;
-  kern<<<grid, kReduceThreads, 0, st>>>(intensity_dev, float(tau_print), reinterpret_cast<const uint4*>(z_round_dev),
-                                        pieces, reinterpret_cast<uint4*>(z_print_dev),
-                                        reinterpret_cast<unsigned long long*>(loss_dev));
+  LITHO_TRY_CUDA(launch_pdl(kern, grid, kReduceThreads, 0, st, intensity_dev, float(tau_print),
+                            reinterpret_cast<const uint4*>(z_round_dev), pieces, reinterpret_cast<uint4*>(z_print_dev),
+                            reinterpret_cast<unsigned long long*>(loss_dev)));
   LITHO_TRY_CUDA(cudaGetLastError());
   return LITHO_OK;
 }

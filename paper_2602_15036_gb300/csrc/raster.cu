@@ -19,6 +19,7 @@
 // The result does not depend on the order of a tile's list.
 #include <cstdint>
 
+#include "fft_common.cuh"
 #include "litho_internal.h"
 
 namespace litho {
@@ -50,6 +51,8 @@ __global__ void k_rast_bin(const float4* __restrict__ rects, const long long* __
                            long long max_rects, float max_side, int* __restrict__ count, const int* __restrict__ tile_start,
                            const long long* __restrict__ clip_base, int* __restrict__ cursor,
                            float4* __restrict__ list, int* __restrict__ bad) {
+  pdl_start();
+  pdl_wait(rects, rect_start, tile_start, clip_base);
   const int c = blockIdx.y, tiles = n / kTile;
   if (!FILL && blockIdx.x == 0 && threadIdx.x == 0 && rect_start[c + 1] - rect_start[c] > max_rects) bad[c] = 1;
   const long long r = rect_start[c] + (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -82,6 +85,8 @@ __global__ void k_rast_bin(const float4* __restrict__ rects, const long long* __
 __global__ void __launch_bounds__(kScanThreads) k_rast_scan(const int* __restrict__ count, int tiles2, int* __restrict__ tile_start,
                                                             int* __restrict__ cursor, int* __restrict__ total) {
   __shared__ int warp_sums[kScanThreads / 32];
+  pdl_start();
+  pdl_wait(count);
   const int c = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const size_t base = (size_t)c * tiles2;
   int run = 0;
@@ -125,6 +130,8 @@ __global__ void __launch_bounds__(kScanThreads) k_rast_scan(const int* __restric
 
 // Offsets of the clips' lists: clip_base[c] = sum of the totals before c.
 __global__ void k_rast_base(const int* __restrict__ total, int b, long long* __restrict__ clip_base) {
+  pdl_start();
+  pdl_wait(total);
   long long run = 0;
   for (int c = 0; c < b; ++c) {
     clip_base[c] = run;
@@ -194,6 +201,8 @@ __global__ void __launch_bounds__(32 * kRastWarps) k_rast_tiles(const float4* __
   __shared__ unsigned short pool[kRastWarps * kTilePix];  // warp << 8 | pixel
   __shared__ const float4* pieces[kRastWarps];
   __shared__ int n_pieces[kRastWarps], n_pool;
+  pdl_start();
+  pdl_wait(list, count, tile_start, clip_base, bad);
   const int tiles = n / kTile, c = blockIdx.y, lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   const int t0 = blockIdx.x * kRastWarps, t = t0 + wp;
   const bool live = t < tiles * tiles;
@@ -346,20 +355,21 @@ cudaError_t launch_raster(const float4* rects, const long long* rect_start, int 
   if (e != cudaSuccess) return e;
   if (max_rects > 0) {
     const dim3 grid(unsigned((max_rects + 255) / 256), b);
-    k_rast_bin<false><<<grid, 256, 0, st>>>(rects, rect_start, n, max_rects, float(max_side), L.count, nullptr, nullptr,
-                                            nullptr, nullptr, L.bad);
+    e = launch_pdl(k_rast_bin<false>, grid, 256, 0, st, rects, rect_start, n, max_rects, float(max_side), L.count,
+                   nullptr, nullptr, nullptr, nullptr, L.bad);
   }
-  k_rast_scan<<<b, kScanThreads, 0, st>>>(L.count, int(tiles2), L.tile_start, L.cursor, L.total);
-  k_rast_base<<<1, 1, 0, st>>>(L.total, b, L.clip_base);
-  if (max_rects > 0) {
+  if (e == cudaSuccess)
+    e = launch_pdl(k_rast_scan, b, kScanThreads, 0, st, L.count, int(tiles2), L.tile_start, L.cursor, L.total);
+  if (e == cudaSuccess) e = launch_pdl(k_rast_base, 1, 1, 0, st, L.total, b, L.clip_base);
+  if (e == cudaSuccess && max_rects > 0) {
     const dim3 grid(unsigned((max_rects + 255) / 256), b);
-    k_rast_bin<true><<<grid, 256, 0, st>>>(rects, rect_start, n, max_rects, float(max_side), L.count, L.tile_start,
-                                           L.clip_base, L.cursor, L.list, L.bad);
+    e = launch_pdl(k_rast_bin<true>, grid, 256, 0, st, rects, rect_start, n, max_rects, float(max_side), L.count,
+                   L.tile_start, L.clip_base, L.cursor, L.list, L.bad);
   }
   auto kern = (reinterpret_cast<uintptr_t>(mask) & 15) == 0 ? k_rast_tiles<true> : k_rast_tiles<false>;
-  kern<<<dim3(unsigned((tiles2 + kRastWarps - 1) / kRastWarps), b), 32 * kRastWarps, 0, st>>>(
-      L.list, L.count, L.tile_start, L.clip_base, L.bad, n, mask);
-  return cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  return launch_pdl(kern, dim3(unsigned((tiles2 + kRastWarps - 1) / kRastWarps), b), 32 * kRastWarps, 0, st, L.list,
+                    L.count, L.tile_start, L.clip_base, L.bad, n, mask);
 }
 
 }  // namespace litho
