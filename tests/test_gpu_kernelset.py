@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 
 import synth
+from oracle import ai as OA
 from oracle import ilt as OL
 from oracle import imaging as OI
 from tests.gpu_util import DUV_ANNULAR, DUV_QUAD21, oracle_kernel_set
@@ -103,3 +104,19 @@ def test_gradients_match_the_given_kernels(litho_lib, cuda, name, precision):
                 g = [up[i, f] if given is not None else np.ones((n, n)) for f in range(f0, f0 + count)]
                 ref = OL.intensity_vjp(m64[i], pairs[f0:f0 + count], g)
                 assert np.linalg.norm(dm[i] - ref) <= 1e-4 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("precision", ["fft32", "fft32/coarse"])
+@pytest.mark.parametrize("name", ["through focus", "random", "edge"])
+def test_ai_inputs_match_the_given_kernels(litho_lib, cuda, name, precision):
+    """Extremes found by the band-row kernel, or (full grid, edge kernels) by a pass over the channel."""
+    import torch
+    n, b = 128, 5
+    lam, phi = _set(name, n)
+    kern = litho_lib.litho_upload_kernels(n, PIXEL, lam, phi)
+    targets = np.stack([synth.random_rect_mask(n, seed=70 + i, count=15) for i in range(b)]).astype(np.float32)
+    x = litho_lib.litho_ai_inputs(kern, torch.from_numpy(targets).to(cuda), focus=0, precision=precision).cpu().numpy()
+    ref, _, _ = OA.ai_channels(targets, lam[0], phi[0])
+    assert np.array_equal(x[:, 0], targets)
+    assert np.abs(x[:, 1] - ref[:, 1]).max() <= 1e-5
+    assert np.abs(x[:, 2] - ref[:, 2]).max() <= 1e-4
