@@ -486,7 +486,7 @@ cudaError_t band_rows_n(const float2* q, int clips, int planes, int h, float sca
                         float* img, float* iblur, uint8_t* printed, const PlaneOut& po, cudaStream_t st,
                         uint2* ext = nullptr) {
   const int units = RESIST ? N : N / 2;
-  const int per = rows_per_cta(units, clips * planes, 2048 / Plan<N>::NT), grid = (units + per - 1) / per;
+  const int per = rows_per_cta(units, clips * planes, Plan<N>::NT, 8 * (N + PadLen<N>::value)), grid = (units + per - 1) / per;
   auto kern = 4 * h <= N ? k_band_rows<N, true, RESIST> : k_band_rows<N, false, RESIST>;
   return launch_pdl(kern, dim3(grid, clips * planes), Plan<N>::NT, 0, st, q, h, scale, tw, thr, img, iblur, printed,
                     planes, po, per, ext);
@@ -498,7 +498,7 @@ cudaError_t resist_grad_rows_n(const float2* band, int planes, int crop, const f
                                double* partial, cudaStream_t st) {
   static_assert(Plan<N>::NT % 32 == 0, "whole warps");
   const size_t sm = sizeof(float2) * (N + PadLen<N>::value + (GradRowsShape<N>::kRegs ? crop + 1 : N + 1));
-  const int ppc = rows_per_cta(N / 2, planes, 2048 / Plan<N>::NT), grid = (N / 2 + ppc - 1) / ppc;
+  const int ppc = rows_per_cta(N / 2, planes, Plan<N>::NT, sm), grid = (N / 2 + ppc - 1) / ppc;
   auto kern = 2 * crop <= N ? k_resist_grad_rows<N, true> : k_resist_grad_rows<N, false>;
   cudaError_t e = smem_attrs(kern, sm);
   if (e != cudaSuccess) return e;
@@ -542,7 +542,7 @@ cudaError_t mask_rows_n(const float* m, RowInput in, float alpha, int b, int cro
                                       : k_mask_rows<N, RowInput::Mask>;
   cudaError_t e = smem_attrs(kern, smr);
   if (e != cudaSuccess) return e;
-  const int ppc = rows_per_cta(N / 2, b, 2048 / Plan<N>::NT);
+  const int ppc = rows_per_cta(N / 2, b, Plan<N>::NT, smr);
   return launch_pdl(kern, dim3((N / 2 + ppc - 1) / ppc, b), Plan<N>::NT, smr, st, m, alpha, crop, tw, rowbuf,
                     half_cols(crop, whole), half_ld(crop, whole), ppc, copy, copy_stride);
 }

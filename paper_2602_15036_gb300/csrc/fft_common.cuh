@@ -647,10 +647,11 @@ inline cudaError_t smem_attrs(K kernel, size_t bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
 }
 
-// Rows per CTA for the one-row-per-transform kernels: enough CTAs for about
-// eight waves of `per_sm` CTAs per SM, each CTA reusing its twiddle table
-// for its rows.
-inline int rows_per_cta(int rows, int planes, int per_sm) {
+// Rows per CTA for the one-row-per-transform kernels: CTAs for about four waves at the residency that
+// their threads and shared memory allow, each reusing its twiddle table for its rows.  64 clips of 2048^2 with
+// resist, by waves: 8960 us (1), 8754 (2), 8673 (3), 8647 (4), 8853 (a row per CTA: eight waves of the
+// CTAs that threads alone allow, three times what fits); fewer than two leave a long tail.
+inline int rows_per_cta(int rows, int planes, int threads, size_t smem) {
   static int sms = 0;  // the same GPU model throughout a process
   if (!sms) {
     int dev = 0, v = 0;
@@ -659,7 +660,8 @@ inline int rows_per_cta(int rows, int planes, int per_sm) {
               ? v
               : 152;
   }
-  const long long want = 8LL * sms * per_sm;
+  const int per_sm = std::max<int>(1, std::min<int>(std::min(2048 / threads, 32), int(227 * 1024 / (smem + 1024))));
+  const long long want = 4LL * sms * per_sm;
   const long long r = std::max<long long>(1, ((long long)rows * planes) / want);
   return int(std::min<long long>(r, rows));
 }

@@ -569,7 +569,7 @@ cudaError_t grad_rows_n(const float2* qf, int crop, float scale, const float* th
   auto kern = 2 * crop <= N ? k_grad_rows<N, true> : k_grad_rows<N, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  const int per = rows_per_cta(N, clips, 2048 / Plan<N>::NT);
+  const int per = rows_per_cta(N, clips, Plan<N>::NT, sm);
   return launch_pdl(kern, dim3((N + per - 1) / per, clips), Plan<N>::NT, sm, st, qf, crop, scale, theta, alpha, tw,
                     grad, grad_stride, per);
 }
