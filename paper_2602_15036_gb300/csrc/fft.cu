@@ -8,9 +8,10 @@
 //
 // Data layout (all row-major, x fastest):
 //   mask    [b][N][N] f32
-//   rowbuf  [b][N][C] c64   row DFT of the mask, crop columns only
+//   rowbuf  [b][N][C/2 + 8] c64   row DFT of the mask, the columns 0 <= u <= C/2 (the mask is real)
 //   mhat    [b][C][C] c64   N^-2 DFT(m) on the crop, [v][u]
-//   t1      [j][N][C] c64   stage-1 field T_j[y][u] = sum_v mhat[v][u] Phi_j[v][u] e^{2 pi i v y/N}
+//   t1      [j][N][C] c64   stage-1 field T_j[y][u] = sum_v mhat[v][u] Psi_j[v][u] e^{2 pi i v y/N}
+//   q       [plane][N][..] c64  half band rows of a real plane (0 <= u < h; with a blur, the image's then the blur's)
 //   img     [plane][N][N] f32
 #include <algorithm>
 #include <cfloat>
@@ -191,20 +192,21 @@ struct OutHalf {
 };
 
 // ---- stage 2 (FP32 path): one image row per CTA, all kernels of the plane ------------------------
-// Rows of up to 256 points are one warp's: kGroups warps share the plane's kernels (warp w takes kernels w,
-// w + kGroups, ...) and their sums are added in order, so that a row's chain of transforms, which a small
-// call waits for, is that much shorter (2 planes of 256^2, 8 and 4 fields: 11.1 -> 7.9 us).
+// Rows of up to 256 points are one warp's: G warps share the plane's kernels (warp w takes kernels w, w + G,
+// ...) and their sums are added in order, where a chain of many kernels is what an SM of few rows waits for.  256^2
+// images of one plane and 12 fields, one and two warps a row: 2 clips 19.2 and 18.9 us, 4 28.6 and 20.9, 8 30.3 and
+// 28.5, 12 40.1 and 38.8, 20 59.4 and 59.1; two planes of 5: 1 clip 16.3 and 19.1 us, 20 51.2 and 61.6.
 template <int N>
 struct Stage2Groups {
   static constexpr int value = Plan<N>::NT == 32 ? 2 : 1;
 };
 
-template <int N, bool BANDED>
-__global__ void __launch_bounds__(Plan<N>::NT * Stage2Groups<N>::value, 512 / Plan<N>::NT / Stage2Groups<N>::value)
+template <int N, bool BANDED, int G>
+__global__ void __launch_bounds__(Plan<N>::NT * G, 512 / Plan<N>::NT / G)
     k_stage2(const float2* __restrict__ t1, const __grid_constant__ FieldSet fs, int crop, float dose,
              const float2* __restrict__ tw_g, float* __restrict__ img, const __grid_constant__ PlaneOut po) {
   using PL = Plan<N>;
-  constexpr int NT = PL::NT, G = Stage2Groups<N>::value;
+  constexpr int NT = PL::NT;
   constexpr int RL = PL::R[PL::P - 1];
   constexpr int PERL = PassShape<N, NT, RL>::PER;
   __shared__ float2 bufs[G][PadLen<N>::value];
@@ -564,9 +566,15 @@ cudaError_t stage1_half_n(const float2* spec, int nk, int crop, const float2* tw
 template <int N>
 cudaError_t stage2_n(const float2* t1, const FieldSet& fs, int clips, int crop, float dose, const float2* tw,
                      float* img, const PlaneOut& po, cudaStream_t st) {
-  auto kern = 2 * crop <= N ? k_stage2<N, true> : k_stage2<N, false>;
-  return launch_pdl(kern, dim3(N, clips * fs.planes), Plan<N>::NT * Stage2Groups<N>::value, 0, st, t1, fs, crop, dose,
-                    tw, img, po);
+  const dim3 grid(N, clips * fs.planes);
+  constexpr int G = Stage2Groups<N>::value;
+  const int rows = N * clips * fs.planes;
+  if (G > 1 && fs.fields() >= 8 * fs.planes && rows >= 768 && rows <= 3072) {
+    auto kern = 2 * crop <= N ? k_stage2<N, true, G> : k_stage2<N, false, G>;
+    return launch_pdl(kern, grid, Plan<N>::NT * G, 0, st, t1, fs, crop, dose, tw, img, po);
+  }
+  auto kern = 2 * crop <= N ? k_stage2<N, true, 1> : k_stage2<N, false, 1>;
+  return launch_pdl(kern, grid, Plan<N>::NT, 0, st, t1, fs, crop, dose, tw, img, po);
 }
 
 // Transform sizes of the full grid (powers of two) ...

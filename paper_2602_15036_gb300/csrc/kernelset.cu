@@ -17,7 +17,7 @@
 // assumed about the optics: the Gram matrix of the h decides, in FP64, once
 // per kernel set; a plane that does not reduce keeps sqrt(lam) Phi.
 //
-// Measured (K = 24, planes at -50/0/+50 nm: 36 fields a clip instead of 72):
+// Measured when it was added (K = 24, planes at -50/0/+50 nm: 36 fields a clip instead of 72):
 // 64 clips of 2048^2 with resist 15.50 -> 9.78 ms, 8 clips on the full grid
 // 5.96 -> 3.27 ms, on the tensor cores 5.18 -> 3.12 ms; ILT step of 16 clips
 // of 1024^2, K = 16, 5 planes 3.62 -> 2.16 ms; one 2048^2 clip in focus 149 ->

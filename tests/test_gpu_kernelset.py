@@ -120,3 +120,19 @@ def test_ai_inputs_match_the_given_kernels(litho_lib, cuda, name, precision):
     assert np.array_equal(x[:, 0], targets)
     assert np.abs(x[:, 1] - ref[:, 1]).max() <= 1e-5
     assert np.abs(x[:, 2] - ref[:, 2]).max() <= 1e-4
+
+
+@pytest.mark.parametrize("n", [128, 256])
+@pytest.mark.parametrize("k,rows", [(9, 512), (9, 1024), (8, 2816), (9, 3328), (7, 1024)])
+def test_rows_shared_by_warps(litho_lib, cuda, n, k, rows):
+    """Short rows: one warp a row, or two that share the kernels (odd and even numbers of them)."""
+    import torch
+    b = rows // n
+    lam, phi = _random_set(n, 32, 1, k, False)
+    lam[0, -2:] = lam[0, -3]
+    kern = litho_lib.litho_upload_kernels(n, PIXEL, lam, phi)
+    masks = np.stack([synth.random_rect_mask(n, seed=90 + i, count=12) for i in range(b)])
+    img = litho_lib.litho_aerial(kern, torch.from_numpy(masks).to(cuda), precision="fft32").cpu().numpy()
+    for i in (0, b - 1):
+        ref = OI.socs_image(masks[i].astype(np.float64), lam[0], phi[0])
+        assert np.abs(img[i, 0] - ref).max() <= 1e-5 * max(1.0, ref.max())
