@@ -176,7 +176,7 @@ def fft_group(clips: int, n_focus: int, k: int, ne: int, crop: int) -> int:
     return -(-clips // groups)
 
 
-def stage_models(prec: str, clips: int, n: int, crop: int, n_focus: int, k_eff: int, nc: int, peaks,
+def stage_models(prec: str, clips: int, n: int, crop: int, n_focus: int, k_eff: float, nc: int, peaks,
                  resist_taps: int = 11, k_alloc: int = K) -> dict:
     """stage -> (flops per step, algorithmic DRAM bytes per step).
 
@@ -185,7 +185,8 @@ def stage_models(prec: str, clips: int, n: int, crop: int, n_focus: int, k_eff: 
     writes and reads back, such as the row spectra of a 2D transform, are not
     counted); the kernels Phi count once per launch, since a launch's clips share
     them.  Flops count 5 m log2 m per m-point complex transform and 6 per complex
-    multiply-add of the band multiply."""
+    multiply-add of the band multiply.  k_eff: complex fields evaluated per focus plane (all given
+    kernels where no set reduces)."""
     coarse = prec.endswith("/coarse") and nc > 0
     ne = nc if coarse else n
     fk = n_focus * k_eff
@@ -258,7 +259,7 @@ def ai_models(clips: int, n: int, ne: int, crop: int, k: int, coarse: bool, roun
     (litho_ai_inputs + litho_print_images), counted as in stage_models: ilt_forward = the image
     channel (mask spectrum, stage 1 and 2 per kernel, interpolation), ilt_backward = the adjoint of
     ones (its closed form N^2 sum_k lam_k |Phi_k|^2 mhat, then the band-to-full gradient), ilt_reduce = the two
-    channel normalisations (read, then read and write), resist = the print images (blur of the
+    channel normalisations (read and write), resist = the print images (blur of the
     targets, two thresholds, the L1 count).  Bytes: targets in, the three channels out."""
     fft = lambda m: 5.0 * m * math.log2(m)  # noqa: E731
     c2 = 2 * crop
@@ -272,7 +273,7 @@ def ai_models(clips: int, n: int, ne: int, crop: int, k: int, coarse: bool, roun
     bwd = clips * (k * 4.0 * crop * crop + 4.0 * crop * crop + crop * fft(n) + n * fft(n))
     px = clips * n * n
     return {"ilt_forward": (fwd, px * 4.0 + px * 8.0), "ilt_backward": (bwd, px * 4.0),
-            "ilt_reduce": (px * 2 * 3.0, px * 2 * 12.0),
+            "ilt_reduce": (px * 2 * 3.0, px * 2 * 8.0),
             "resist": (px * 4.0 * round_taps, px * (4.0 + 4.0 + 4.0 + 1.0 + 1.0))}
 
 
@@ -569,8 +570,7 @@ def run_aerial(args, ctx):
     torch = ctx.torch
     clips = args.clips
     kern = P.litho_make_kernels(P.make_optics(**OPTICS), N, PIXEL, FOCUS, K)
-    info = kern.info()
-    k_eff = min(K, min(info["rank"]))
+    k_eff = kern.fields() / len(FOCUS)  # fields evaluated per plane, on average
     c = kern.crop
     masks_np = np.stack([synth.manhattan_mask(N, seed=s) for s in clip_seeds(ctx.rank, clips)])
     masks = torch.from_numpy(masks_np).to(ctx.dev)
@@ -730,7 +730,7 @@ def run_ilt(args, ctx):
     cap = max(1, min(clips, int((2 << 30) // per_clip)))
     group = -(-clips // -(-clips // cap))
     roofs = rooflines(prof, args.steps + args.warmup,
-                      ilt_models(clips, n, ne or n, kern.crop, len(focus), k, bool(ne) and ne < n, group), peaks)
+                      ilt_models(clips, n, ne or n, kern.crop, len(focus), kern.fields() / len(focus), bool(ne) and ne < n, group), peaks)
     dominant = max(roofs.items(), key=lambda kv: kv[1]["ms_per_step"])
     roof = dict(dominant[1], kernel=dominant[0], traffic=None,
                 peak_source=f"derived ALU peak; {peak_src} HBM copy bandwidth")
@@ -902,7 +902,7 @@ def run_ai(args, ctx):
     peaks, peak_src = _peaks()
     ne = kern.grid(prec) if prec.endswith("/coarse") else N
     round_taps = 2 * math.ceil(4 * 20.0 / PIXEL) + 1
-    roofs = rooflines(prof, args.steps, ai_models(clips, N, ne or N, kern.crop, K, bool(ne) and ne < N, round_taps),
+    roofs = rooflines(prof, args.steps, ai_models(clips, N, ne or N, kern.crop, kern.fields(), bool(ne) and ne < N, round_taps),
                       peaks)
     dominant = max(roofs.items(), key=lambda kv: kv[1]["ms_per_step"])
     roof = dict(dominant[1], kernel=dominant[0], traffic=None,

@@ -147,6 +147,10 @@ litho_status litho_kernels_info(const litho_kernels* h, int* n, int* crop, int* 
  * ignored for that path).  Either output may be NULL. */
 litho_status litho_kernels_grid(const litho_kernels* h, int* nc_fft, int* nc_tensor);
 
+/* How many complex fields per clip the device evaluates for all focus planes: at most
+ * n_focus k, fewer where a plane's kernels reduce or planes share a set. */
+litho_status litho_kernels_fields(const litho_kernels* h, int* fields);
+
 /* Copies the FP64 kernels phi[n_focus][k][crop][crop][2] back to the host. */
 litho_status litho_kernels_phi(const litho_kernels* h, double* phi_host);
 

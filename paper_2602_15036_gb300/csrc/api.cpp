@@ -309,6 +309,12 @@ litho_status litho_kernels_grid(const litho_kernels* h, int* nc_fft, int* nc_ten
   return LITHO_OK;
 }
 
+litho_status litho_kernels_fields(const litho_kernels* h, int* fields) {
+  LITHO_REQUIRE(h && fields, "null argument");
+  *fields = h->set_start[h->n_sets];
+  return LITHO_OK;
+}
+
 litho_status litho_kernels_phi(const litho_kernels* h, double* phi_host) {
   LITHO_REQUIRE(h && phi_host, "null argument");
   std::memcpy(phi_host, h->phi_host.data(), h->phi_host.size() * sizeof(double));

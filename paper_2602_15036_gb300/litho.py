@@ -72,6 +72,7 @@ _SIGS = {
     "litho_kernels_info": (c_int, [c_void_p, POINTER(c_int), POINTER(c_int), POINTER(c_int), POINTER(c_int),
                                    POINTER(c_int), POINTER(c_double), POINTER(c_double), POINTER(c_double)]),
     "litho_kernels_grid": (c_int, [c_void_p, POINTER(c_int), POINTER(c_int)]),
+    "litho_kernels_fields": (c_int, [c_void_p, POINTER(c_int)]),
     "litho_kernels_phi": (c_int, [c_void_p, POINTER(c_double)]),
     "litho_free_kernels": (None, [c_void_p]),
     "litho_aerial_workspace_size": (c_int, [c_void_p, c_int, c_int, POINTER(c_size_t)]),
@@ -196,6 +197,12 @@ class Kernels:
         fft, tc = c_int(), c_int()
         _check(lib().litho_kernels_grid(self.handle, byref(fft), byref(tc)))
         return fft.value if precision.split("/")[0] == "fft32" else tc.value
+
+    def fields(self) -> int:
+        """Complex fields per clip the device evaluates, over all focus planes (at most n_focus k)."""
+        out = c_int()
+        _check(lib().litho_kernels_fields(self.handle, byref(out)))
+        return out.value
 
     def close(self):
         if self.handle is not None and self.handle.value:
