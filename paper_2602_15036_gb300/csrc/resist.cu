@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kThreads, R > 10 ? 2 : 3) k_resist(const float
   }
 }
 
-// Any radius.  A CTA takes 32 x SH pixels; the tile and its periodic halo go to shared memory, rows at an odd
+// Any radius.  A CTA takes W x SH pixels; the tile and its periodic halo go to shared memory, rows at an odd
 // pitch, so that lanes on different rows, and lanes on different columns, read different banks.  Each
 // thread forms eight neighbouring outputs (of a row, then of a column) from a window of 15 values that
 // moves by eight taps at a time: one shared-memory load per eight FMAs, taps in the order of the fixed radii.
