@@ -192,13 +192,15 @@ struct OutHalf {
 };
 
 // ---- stage 2 (FP32 path): one image row per CTA, all kernels of the plane ------------------------
-// Rows of up to 256 points are one warp's: G warps share the plane's kernels (warp w takes kernels w, w + G,
-// ...) and their sums are added in order, where a chain of many kernels is what an SM of few rows waits for.  256^2
-// images of one plane and 12 fields, one and two warps a row: 2 clips 19.2 and 18.9 us, 4 28.6 and 20.9, 8 30.3 and
-// 28.5, 12 40.1 and 38.8, 20 59.4 and 59.1; two planes of 5: 1 clip 16.3 and 19.1 us, 20 51.2 and 61.6.
+// Rows of up to 256 points are one warp's: two warps share the plane's kernels (G = 2, half of them each), where a
+// chain of many kernels is what an SM of few rows waits for.  256^2 images of one plane and 12 fields, one and
+// two warps a row: 2 clips 19.2 and 18.9 us, 4 28.6 and 20.9, 8 30.3 and 28.5, 12 40.1 and 38.8, 20 59.4 and
+// 59.1; two planes of 5: 1 clip 16.3 and 19.1 us, 20 51.2 and 61.6.
+// How many warps there are depends on the clips of the launch, a clip's bits must not: these rows' sums are
+// always those of the first half of the fields and of the rest, whether two warps form them or one after the other.
 template <int N>
-struct Stage2Groups {
-  static constexpr int value = Plan<N>::NT == 32 ? 2 : 1;
+struct Stage2Halves {
+  static constexpr bool value = Plan<N>::NT == 32;
 };
 
 template <int N, bool BANDED, int G>
@@ -211,7 +213,7 @@ __global__ void __launch_bounds__(Plan<N>::NT * G, 512 / Plan<N>::NT / G)
   constexpr int PERL = PassShape<N, NT, RL>::PER;
   __shared__ float2 bufs[G][PadLen<N>::value];
   __shared__ float2 tw[N];
-  __shared__ float part[G > 1 ? G - 1 : 1][G > 1 ? N : 1];
+  __shared__ float part[G > 1 ? N : 1];
   pdl_start();
   load_twiddles<N>(tw, tw_g);
   pdl_wait(t1);
@@ -220,11 +222,14 @@ __global__ void __launch_bounds__(Plan<N>::NT * G, 512 / Plan<N>::NT / G)
   float2* buf = bufs[grp];
   const int clip = plane / fs.planes, pl = plane - clip * fs.planes, nk = fs.start[pl + 1] - fs.start[pl];
   const float2* base = t1 + ((size_t)(clip * fs.fields() + fs.start[pl]) * N + y) * crop;
-  float acc[PERL][RL];
+  static_assert(G == 1 || (G == 2 && Stage2Halves<N>::value), "two warps take the halves of the fields");
+  constexpr bool kFold = Stage2Halves<N>::value && G == 1;  // this warp forms both halves' sums
+  const int nh = (nk + 1) / 2, j0 = grp * nh, rounds = G == 2 ? nh : nk;
+  float acc[PERL][RL], first[PERL][RL];
 #pragma unroll
   for (int p = 0; p < PERL; ++p)
 #pragma unroll
-    for (int q = 0; q < RL; ++q) acc[p][q] = 0.f;
+    for (int q = 0; q < RL; ++q) acc[p][q] = first[p][q] = 0.f;
   // middle-pass twiddles in registers: measured faster for 2048-point rows,
   // slower for 1024 (where the registers they take cost more than the
   // shared-memory reads they save)
@@ -245,14 +250,25 @@ __global__ void __launch_bounds__(Plan<N>::NT * G, 512 / Plan<N>::NT / G)
       nxt[r] = ld_dep_if(row + c, !zero);
     }
   };
-  prefetch(grp);
-  for (int j0 = 0; j0 < nk; j0 += G) {  // every warp runs every round (block barriers)
+  prefetch(j0);
+  for (int i = 0; i < rounds; ++i) {  // every warp runs every round (block barriers)
+    if constexpr (kFold) {
+      if (i == nh) {
+#pragma unroll
+        for (int p = 0; p < PERL; ++p)
+#pragma unroll
+          for (int q = 0; q < RL; ++q) {
+            first[p][q] = acc[p][q];
+            acc[p][q] = 0.f;
+          }
+      }
+    }
     float2 cur[R0];
 #pragma unroll
     for (int r = 0; r < R0; ++r) cur[r] = nxt[r];
     auto load = [&](int, int r, int) { return cur[r]; };
     auto after_first = [&]() {
-      if (j0 + G < nk) prefetch(j0 + G + grp);
+      if (i + 1 < rounds) prefetch(j0 + i + 1);
     };
     auto use = [&](int p, int q, int, float2 v) { acc[p][q] = fmaf(v.x, v.x, fmaf(v.y, v.y, acc[p][q])); };
     if constexpr (kMid)
@@ -260,20 +276,25 @@ __global__ void __launch_bounds__(Plan<N>::NT * G, 512 / Plan<N>::NT / G)
     else
       fft_load_use<N, +1, decltype(load), decltype(use), BANDED>(buf, tw, t, load, use, after_first);
   }
+  if constexpr (kFold) {
+#pragma unroll
+    for (int p = 0; p < PERL; ++p)
+#pragma unroll
+      for (int q = 0; q < RL; ++q) acc[p][q] = first[p][q] + acc[p][q];
+  }
   if constexpr (G > 1) {
 #pragma unroll
     for (int p = 0; p < PERL; ++p)
 #pragma unroll
       for (int q = 0; q < RL; ++q)
-        if (grp > 0 && t + p * NT < N / RL) part[grp - 1][t + p * NT + q * (N / RL)] = acc[p][q];
+        if (grp > 0 && t + p * NT < N / RL) part[t + p * NT + q * (N / RL)] = acc[p][q];
     __syncthreads();
     if (grp > 0) return;
 #pragma unroll
     for (int p = 0; p < PERL; ++p)
 #pragma unroll
       for (int q = 0; q < RL; ++q)
-        for (int w = 0; w < G - 1; ++w)
-          if (t + p * NT < N / RL) acc[p][q] += part[w][t + p * NT + q * (N / RL)];
+        if (t + p * NT < N / RL) acc[p][q] += part[t + p * NT + q * (N / RL)];
   }
   for (int d = po.first[pl]; d < po.first[pl + 1]; ++d) {
     float* out = img + ((size_t)(clip * po.out_planes + po.list[d]) * N + y) * N;
@@ -567,7 +588,7 @@ template <int N>
 cudaError_t stage2_n(const float2* t1, const FieldSet& fs, int clips, int crop, float dose, const float2* tw,
                      float* img, const PlaneOut& po, cudaStream_t st) {
   const dim3 grid(N, clips * fs.planes);
-  constexpr int G = Stage2Groups<N>::value;
+  constexpr int G = Stage2Halves<N>::value ? 2 : 1;
   const int rows = N * clips * fs.planes;
   if (G > 1 && fs.fields() >= 8 * fs.planes && rows >= 768 && rows <= 3072) {
     auto kern = 2 * crop <= N ? k_stage2<N, true, G> : k_stage2<N, false, G>;

@@ -136,3 +136,40 @@ def test_rows_shared_by_warps(litho_lib, cuda, n, k, rows):
     for i in (0, b - 1):
         ref = OI.socs_image(masks[i].astype(np.float64), lam[0], phi[0])
         assert np.abs(img[i, 0] - ref).max() <= 1e-5 * max(1.0, ref.max())
+
+
+# grids whose rows one or two warps take by the number of rows of the launch, and whose row kernels have
+# several shapes by the number of planes; 12 and 24 fields of one and three planes
+@pytest.mark.parametrize("n,k,focus,counts", [(256, 24, [0.0], (1, 4, 16)), (128, 24, [0.0], (1, 8, 30)),
+                                              (512, 16, [-40.0, 0.0, 40.0], (1, 2, 5)),
+                                              (1024, 12, [0.0, 30.0], (1, 5))])
+@pytest.mark.parametrize("precision", ["fft32", "fft32/coarse"])
+def test_images_do_not_depend_on_the_number_of_clips(litho_lib, cuda, n, k, focus, counts, precision):
+    import torch
+    lam, phi = oracle_kernel_set(DUV_ANNULAR, n, PIXEL, focus, k)
+    kern = litho_lib.litho_upload_kernels(n, PIXEL, lam, phi)
+    masks = np.stack([synth.random_rect_mask(n, seed=30 + i, count=n // 6) for i in range(max(counts))])
+    m = torch.from_numpy(masks).to(cuda)
+    alone = [litho_lib.litho_aerial_resist(kern, m[i:i + 1].contiguous(), precision=precision) for i in range(len(m))]
+    for b in counts[1:]:
+        img, blur, printed = litho_lib.litho_aerial_resist(kern, m[:b].contiguous(), precision=precision)
+        for i in range(b):
+            assert torch.equal(img[i], alone[i][0][0]), (b, i)
+            assert torch.equal(blur[i], alone[i][1][0]) and torch.equal(printed[i], alone[i][2][0]), (b, i)
+
+
+@pytest.mark.parametrize("n,k,focus,counts", [(512, 16, [-40.0, 0.0, 40.0], (1, 2)), (256, 24, [0.0], (1, 5)),
+                                              (128, 16, [-30.0, 0.0, 30.0], (1, 9))])
+@pytest.mark.parametrize("precision", ["fft32", "fft32/coarse"])
+def test_ilt_does_not_depend_on_the_number_of_clips(litho_lib, cuda, n, k, focus, counts, precision):
+    import torch
+    lam, phi = oracle_kernel_set(DUV_ANNULAR, n, PIXEL, focus, k)
+    kern = litho_lib.litho_upload_kernels(n, PIXEL, lam, phi)
+    clips = [synth.ilt_clip(n, PIXEL, seed=60 + i) for i in range(counts[-1])]
+    theta = torch.from_numpy(np.stack([c[0] for c in clips])).to(cuda)
+    target = torch.from_numpy(np.stack([c[1] for c in clips])).to(cuda)
+    grad, loss = litho_lib.litho_ilt_grad(kern, theta, target, precision=precision)
+    for i in range(counts[-1]):
+        g, lo = litho_lib.litho_ilt_grad(kern, theta[i:i + 1].contiguous(), target[i:i + 1].contiguous(),
+                                         precision=precision)
+        assert torch.equal(grad[i], g[0]) and loss[i] == lo[0], i

@@ -237,3 +237,26 @@ def test_queued_requests_of_one_key_run_as_batches(litho_lib, cuda):
         else:
             g, lo = L.litho_ilt_grad(kern, xd, torch.from_numpy(tg[None]).to(cuda), precision="fft32/coarse")
             assert np.array_equal(out, g.cpu().numpy()[0]) and loss[0] == lo[0]
+
+
+def test_batched_images_of_many_kernels_equal_requests_alone(litho_lib, cuda):
+    """Eight images of 24 kernels queue behind a slow request and run as one batch: each is bit for bit
+    the image of the same request run alone (12 fields: the rows of 4 to 12 clips are shared by two warps)."""
+    import torch
+    L = litho_lib
+    srv = L.Server(16 << 30, max_slots=1, max_queue=64)
+    opt = L.make_optics(**DUV)
+    masks = [synth.random_rect_mask(256, seed=500 + i) for i in range(8)]
+    t, _ = srv.submit("image", opt, 256, 8.0, 0.0, 24, masks[0], np.zeros_like(masks[0]))  # builds the kernel set
+    assert srv.poll(t, 60000) == L.OK
+    srv.inject_fault(2)
+    hold, _ = srv.submit("image", opt, 256, 8.0, 0.0, 24, masks[0], np.zeros_like(masks[0]))
+    outs = [np.zeros_like(m) for m in masks]
+    tickets = [srv.submit("image", opt, 256, 8.0, 0.0, 24, m, o)[0] for m, o in zip(masks, outs)]
+    status, _ = _wait_all(srv, L, [hold] + tickets, timeout_s=120)
+    assert all(v == L.OK for v in status.values()), status
+    assert srv.stats()["max_batch"] == len(masks)
+    srv.close()
+    kern = L.litho_make_kernels(opt, 256, 8.0, [0.0], 24)
+    for m, o in zip(masks, outs):
+        assert np.array_equal(o, L.litho_aerial(kern, torch.from_numpy(m[None]).to(cuda)).cpu().numpy()[0, 0])
