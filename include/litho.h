@@ -478,6 +478,11 @@ litho_status litho_serve_create(size_t hbm_budget_bytes, int max_slots, int max_
 /* EBUSY if the queue is full; EINVAL if the request's footprint exceeds the
  * whole budget or its fields are invalid. */
 litho_status litho_serve_submit(litho_server* s, const litho_request* req, uint64_t* ticket);
+/* 1 when the device may read (writable: and write) all `bytes` at `host` as
+ * they stand: page-locked to the last byte in one allocation or registration,
+ * at the same address.  Small requests' buffers of this kind are copied by
+ * kernels, other page-locked ones by the copy engines.  Host query only. */
+int litho_host_range_mapped(const void* host, size_t bytes, int writable);
 /* OK when done (output written), ECANCELED, ETIMEOUT if still pending after
  * timeout_ms (0 = just check), EINVAL for an unknown ticket, or the request's
  * own error status.  Never blocks longer than timeout_ms. */

@@ -26,6 +26,8 @@
 // calls give each clip the same result as the clip imaged alone, bit for
 // bit, and all device kernels are deterministic, so a request's result does
 // not depend on what it ran with.
+#include <cuda.h>
+
 #include <algorithm>
 #include <atomic>
 #include <chrono>
@@ -79,7 +81,7 @@ struct Req {
   double t_submit = 0, t_done = 0;
   int slot = -1;
   bool in_pinned = false, out_pinned = false;  // caller buffers usable for DMA directly
-  bool mapped = true;                          // ... and those that are, addressable by the device as they stand
+  bool mapped = true;                          // ... and those that are, a kernel's to read or write to their last byte
   size_t stage_in = 0, stage_out = 0;          // offsets in the slot's pinned staging
 };
 
@@ -94,9 +96,41 @@ double work_px(const litho_request& r) { return double(r.n) * r.n * (r.kind == L
 // requests, so small requests are not held behind them.
 constexpr double kSmallBatchWork = 2.0 * 1024.0 * 1024.0;
 
-// True for page-locked (cudaHostAlloc / cudaHostRegister) host memory; *mapped is cleared when a kernel
-// cannot address it by the same pointer.
-bool is_pinned(const void* p, bool* mapped) {
+// True when the `bytes` at p all lie in one page-locked allocation or registration that the device addresses by
+// the same pointers and may read (write): only then may a kernel touch them.  A copy by the runtime may be
+// asked for a range that runs past a registration (it checks, and fails or stages); a kernel would fault.
+bool range_mapped(const void* p, size_t bytes, bool write) {
+  using Query = CUresult (*)(void*, CUpointer_attribute, CUdeviceptr);
+  static const Query query = []() -> Query {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      return reinterpret_cast<Query>(f);
+    cudaGetLastError();
+    return nullptr;
+  }();
+  cudaPointerAttributes a;
+  if (!query || !p || bytes == 0 || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (a.type != cudaMemoryTypeHost || a.devicePointer != p) return false;
+  const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+  CUdeviceptr start = 0;
+  size_t size = 0;
+  unsigned access = 0;
+  if (query(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, at) != CUDA_SUCCESS ||
+      query(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, at) != CUDA_SUCCESS ||
+      query(&access, CU_POINTER_ATTRIBUTE_ACCESS_FLAGS, at) != CUDA_SUCCESS)
+    return false;
+  const unsigned need = write ? CU_POINTER_ATTRIBUTE_ACCESS_FLAG_READWRITE : CU_POINTER_ATTRIBUTE_ACCESS_FLAG_READ;
+  return (access & need) == need && at >= start && size >= bytes && at - start <= size - bytes;
+}
+
+// True for page-locked (cudaHostAlloc / cudaHostRegister) host memory at p; *mapped is cleared unless a
+// kernel may read (write) all `bytes` of it.
+bool is_pinned(const void* p, size_t bytes, bool write, bool* mapped) {
   if (!p) return true;
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -104,7 +138,7 @@ bool is_pinned(const void* p, bool* mapped) {
     return false;
   }
   if (a.type != cudaMemoryTypeHost) return false;
-  if (a.devicePointer != p) *mapped = false;
+  if (!range_mapped(p, bytes, write)) *mapped = false;
   return true;
 }
 
@@ -551,6 +585,10 @@ litho_status litho_serve_create(size_t hbm_budget_bytes, int max_slots, int max_
   return LITHO_OK;
 }
 
+int litho_host_range_mapped(const void* host, size_t bytes, int writable) {
+  return range_mapped(host, bytes, writable != 0) ? 1 : 0;
+}
+
 litho_status litho_serve_submit(litho_server* s, const litho_request* req, uint64_t* ticket) {
   if (!s || !req || !ticket) {
     set_error("null argument");
@@ -586,9 +624,10 @@ litho_status litho_serve_submit(litho_server* s, const litho_request* req, uint6
   q->key = kernel_key(q->r, q->custom);
   q->bkey = batch_key(q->r, q->key);
   // pinned caller buffers are copied by DMA directly; pageable ones through the slot's staging
-  q->in_pinned = is_pinned(r.input_host, &q->mapped) &&
-                 (r.kind != LITHO_REQ_ILT_STEP || is_pinned(r.target_host, &q->mapped));
-  q->out_pinned = is_pinned(r.output_host, &q->mapped);
+  const size_t plane = size_t(r.n) * r.n * sizeof(float);
+  q->in_pinned = is_pinned(r.input_host, plane, false, &q->mapped) &&
+                 (r.kind != LITHO_REQ_ILT_STEP || is_pinned(r.target_host, plane, false, &q->mapped));
+  q->out_pinned = is_pinned(r.output_host, plane, true, &q->mapped);
   std::lock_guard<std::mutex> lk(s->mu);
   if (s->stop) {
     set_error("server is shutting down");

@@ -112,6 +112,7 @@ _SIGS = {
                                c_int, c_void_p, POINTER(c_double), c_void_p, c_size_t, c_void_p]),
     "litho_serve_create": (c_int, [c_size_t, c_int, c_int, POINTER(c_void_p)]),
     "litho_serve_submit": (c_int, [c_void_p, POINTER(litho_request), POINTER(c_uint64)]),
+    "litho_host_range_mapped": (c_int, [c_void_p, c_size_t, c_int]),
     "litho_serve_poll": (c_int, [c_void_p, c_uint64, c_int]),
     "litho_serve_cancel": (c_int, [c_void_p, c_uint64]),
     "litho_serve_stats": (c_int, [c_void_p, POINTER(litho_serve_stats_t)]),
@@ -588,6 +589,11 @@ def litho_ilt_grad(kern: Kernels, theta, target, dose=1.0, mask_steep=4.0, resis
                                 loss.ctypes.data_as(POINTER(c_double)) if want_loss else None,
                                 c_void_p(workspace.data_ptr()), workspace.numel(), _stream_ptr(stream)))
     return grad, loss
+
+
+def litho_host_range_mapped(address: int, nbytes: int, writable: bool) -> bool:
+    """Whether a kernel may read (write) all `nbytes` of host memory at `address`."""
+    return bool(lib().litho_host_range_mapped(c_void_p(address), nbytes, int(writable)))
 
 
 class Server:

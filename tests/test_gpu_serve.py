@@ -260,3 +260,27 @@ def test_batched_images_of_many_kernels_equal_requests_alone(litho_lib, cuda):
     kern = L.litho_make_kernels(opt, 256, 8.0, [0.0], 24)
     for m, o in zip(masks, outs):
         assert np.array_equal(o, L.litho_aerial(kern, torch.from_numpy(m[None]).to(cuda)).cpu().numpy()[0, 0])
+
+
+def test_only_whole_page_locked_ranges_are_a_kernels(litho_lib, cuda):
+    """Host queries only: a buffer that runs past its registration, or starts before it, is not for a kernel."""
+    import torch
+    L = litho_lib
+    pinned = torch.zeros(4096).pin_memory()
+    at = pinned.data_ptr()
+    assert L.litho_host_range_mapped(at, 4 * 4096, True) and L.litho_host_range_mapped(at + 400, 4096, False)
+    assert not L.litho_host_range_mapped(at, 0, False)
+    room = np.zeros(1 << 20, dtype=np.uint8)
+    base = (room.ctypes.data + 65535) // 65536 * 65536
+    span = 4 * 65536
+    assert not L.litho_host_range_mapped(base, span, False)  # pageable
+    rt = torch.cuda.cudart()
+    assert int(rt.cudaHostRegister(base, span, 0)) == 0
+    try:
+        assert L.litho_host_range_mapped(base, span, True) and L.litho_host_range_mapped(base + span - 16, 16, True)
+        assert not L.litho_host_range_mapped(base, span + 4, False)
+        assert not L.litho_host_range_mapped(base + span - 16, 32, True)
+        assert not L.litho_host_range_mapped(base - 16, 32, False)
+    finally:
+        assert int(rt.cudaHostUnregister(base)) == 0
+    assert not L.litho_host_range_mapped(base, span, False)
