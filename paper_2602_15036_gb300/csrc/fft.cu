@@ -539,6 +539,14 @@ cudaError_t mask_cols_w(const float2* rowbuf, int b, int crop, int cols, int ld,
                     cols, ld, tw, gain, mhat);
 }
 
+template <int N>
+cudaError_t load_mask_cols_n() {
+  cudaError_t e = load_kernel(k_mask_cols<N, 4, true>);
+  if (e == cudaSuccess) e = load_kernel(k_mask_cols<N, 8, true>);
+  if (e == cudaSuccess) e = load_kernel(k_mask_cols<N, 4, false>);
+  return e != cudaSuccess ? e : load_kernel(k_mask_cols<N, 8, false>);
+}
+
 // Half rows of the mask spectrum (whole: with k = crop/2) or of any real plane.
 inline int half_cols(int crop, bool whole) { return crop / 2 + (whole ? 1 : 0); }
 inline int half_ld(int crop, bool whole) { return crop / 2 + (whole ? 8 : 0); }
@@ -596,6 +604,15 @@ cudaError_t stage2_n(const float2* t1, const FieldSet& fs, int clips, int crop, 
   }
   auto kern = 2 * crop <= N ? k_stage2<N, true, 1> : k_stage2<N, false, 1>;
   return launch_pdl(kern, grid, Plan<N>::NT, 0, st, t1, fs, crop, dose, tw, img, po);
+}
+
+template <int N>
+cudaError_t load_stage2_n(int crop) {
+  if constexpr (Stage2Halves<N>::value) {
+    cudaError_t e = load_kernel(2 * crop <= N ? k_stage2<N, true, 1> : k_stage2<N, false, 1>);
+    return e != cudaSuccess ? e : load_kernel(2 * crop <= N ? k_stage2<N, true, 2> : k_stage2<N, false, 2>);
+  }
+  return cudaSuccess;  // one shape
 }
 
 // Transform sizes of the full grid (powers of two) ...
@@ -723,6 +740,24 @@ cudaError_t launch_stage1_fft(const float2* mhat, const float2* phi, int nk, int
 #define CALL(N) stage1_n<N>(mhat, phi, nk, crop, tw, t1, st, clips)
   LITHO_DISPATCH_N(n, CALL)
 #undef CALL
+}
+
+cudaError_t load_clip_shapes(int n, int nc, int crop) {
+  auto cols = [&](int m) {
+#define CALL(N) load_mask_cols_n<N>()
+    LITHO_DISPATCH_NC(m, CALL)
+#undef CALL
+  };
+  auto rows = [&](int m) {
+    if (stage2_w32_supported(m, crop)) return load_stage2_w32(crop);
+#define CALL(N) load_stage2_n<N>(crop)
+    LITHO_DISPATCH_N(m, CALL)
+#undef CALL
+  };
+  cudaError_t e = cols(n);
+  if (e == cudaSuccess) e = rows(n);
+  if (e == cudaSuccess && nc > 0) e = rows(nc);
+  return e;
 }
 
 cudaError_t launch_stage2_fft(const float2* t1, const FieldSet& fs, int clips, int n, int crop, float dose,

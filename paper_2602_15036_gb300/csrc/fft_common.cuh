@@ -647,6 +647,13 @@ inline cudaError_t smem_attrs(K kernel, size_t bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
 }
 
+// Loads a kernel now: the runtime loads one at its first launch, and that waits for the work in flight.
+template <class K>
+inline cudaError_t load_kernel(K kernel) {
+  cudaFuncAttributes a;
+  return cudaFuncGetAttributes(&a, kernel);
+}
+
 // Rows per CTA for the one-row-per-transform kernels: CTAs for about four waves at the residency that
 // their threads and shared memory allow, each reusing its twiddle table for its rows.  64 clips of 2048^2 with
 // resist, by waves: 8960 us (1), 8754 (2), 8673 (3), 8647 (4), 8853 (a row per CTA: eight waves of the

@@ -219,6 +219,11 @@ cudaError_t launch_stage2_w32(const float2* t1, const FieldSet& fs, int clips, i
                               const float2* tw2, float* img, const PlaneOut& po, cudaStream_t st,
                               float2* spec = nullptr, int c2 = 0);
 
+// Loads the kernels that the FP32 calls of an n-point set with a crop and a coarse grid nc (0: none) choose
+// between by the number of their clips (the mask spectrum's columns, stage 2 and the spectra of the ILT's dL/dI).
+cudaError_t load_clip_shapes(int n, int nc, int crop);
+cudaError_t load_stage2_w32(int crop);
+
 // A device-side delay of about `ms` milliseconds on `st` (util.cu): one
 // thread spinning on the SM clock for a fixed number of cycles, which always
 // ends.  The slow request of the serving tests.

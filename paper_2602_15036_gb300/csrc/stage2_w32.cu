@@ -169,6 +169,14 @@ cudaError_t launch_w32_t(const float2* t1, const FieldSet& fs, int clips, int cr
 #undef W32
 }
 
+template <bool BANDED>
+cudaError_t load_w32() {
+  cudaError_t e = load_kernel(k_stage2_w32<BANDED, 7, false>);
+  if (e == cudaSuccess) e = load_kernel(k_stage2_w32<BANDED, 12, false>);
+  if (e == cudaSuccess) e = load_kernel(k_stage2_w32<BANDED, 7, true>);
+  return e != cudaSuccess ? e : load_kernel(k_stage2_w32<BANDED, 12, true>);
+}
+
 // The same stage 2 for 512-point rows, two rows per warp (512 = 16 x 32):
 // lane l takes x[l + 32 r] of both rows for the first (radix-16) pass; in the
 // second (radix-32) pass lanes 0-15 take row A and lanes 16-31 row B, lane j
@@ -259,6 +267,8 @@ __global__ void __launch_bounds__(32 * kW512Warps, 2)
 
 // crop: even (16-byte row pieces) and at most 512 (staging buffers within shared memory)
 bool stage2_w32_supported(int n, int crop) { return n == kN && crop >= 2 && crop <= kN / 2 && crop % 2 == 0; }
+
+cudaError_t load_stage2_w32(int crop) { return crop / 2 <= kN / 4 ? load_w32<true>() : load_w32<false>(); }
 
 void stage2_w32_table(float2* out) {
   for (int r = 1; r < kR; ++r)
