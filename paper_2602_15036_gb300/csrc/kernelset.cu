@@ -14,8 +14,8 @@
 // unaberrated pupil and a centrosymmetric source the TCC is real and even,
 // each h or h' is zero up to a phase, and half the transforms suffice.  Planes
 // whose Q agree (+z and -z of such a system) share one set.  Nothing is
-// assumed about the optics: the Gram matrix of the h decides, in FP64, once
-// per kernel set; a plane that does not reduce keeps sqrt(lam) Phi.
+// assumed about the optics: the Gram matrices of the h decide, in FP64, once
+// per kernel set, and relative to each kernel's own weight; a plane that does not reduce keeps sqrt(lam) Phi.
 //
 // Measured when it was added (K = 24, planes at -50/0/+50 nm: 36 fields a clip instead of 72):
 // 64 clips of 2048^2 with resist 15.50 -> 9.78 ms, 8 clips on the full grid
@@ -34,8 +34,12 @@ namespace {
 
 constexpr int kMaxReduceK = 64;                       // kernels per plane the reduction considers (2 K-square Jacobi)
 constexpr size_t kMaxReduceBytes = size_t(2) << 30;   // FP64 kernels held on the device while the set is built
-constexpr double kRankTol = 1e-12;                    // eigenvalues of Q below this share of the largest are rounding
-constexpr double kSameTol = 3.552713678800501e-15;    // 2^-48: planes with |Q - Q'|_F <= 2^-24 |Q|_F share a set
+// A field is left out, and two planes share a set, only where no kernel's own image misses it, however little the
+// kernel weighs beside the others: a mask whose spectrum the strong kernels do not pass is imaged by the weak one alone.
+constexpr double kRankTol = 1e-12;   // eigenvalues of Q below this share of the largest may be left out ...
+constexpr double kOwnTol = 0x1p-26;  // ... when that takes no more than this share from any kernel's own weight,
+constexpr double kNoise = 1e-14;     // or they are rounding (and below what FP32 fields of the largest leave)
+constexpr int kSpanBlocks = 64;      // partial sums per kernel in k_span
 
 // Crop index of -u: entry 0 is u = -C/2, its own mirror on a full-width crop
 // (C = N) and required to be zero otherwise.
@@ -97,6 +101,37 @@ __global__ void __launch_bounds__(256) k_combine(const double2* __restrict__ phi
     im += a.x * x.y + a.y * x.x + b.y * y.x - b.x * y.y;
   }
   psi[(size_t)p * cc + i] = make_float2(float(re), float(im));
+}
+
+// part[k][block] = its share of sum_u |root_k Phi_k(u) - sum_l alpha[k][l] Psi_l(u) + beta[k][l] conj Psi_l(-u)|^2:
+// what of kernel k (of phi) the kernels psi do not span.  blockIdx.y = k.
+__global__ void __launch_bounds__(256) k_span(const double2* __restrict__ phi, const double* __restrict__ root,
+                                              const double2* __restrict__ psi, int nk, int crop,
+                                              const double2* __restrict__ alpha, const double2* __restrict__ beta,
+                                              double* __restrict__ part) {
+  const int cc = crop * crop, k = blockIdx.y;
+  const double r = root[k];
+  double sum = 0.0;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < cc; i += gridDim.x * blockDim.x) {
+    const int m = mirror(i, crop);
+    double re = r * phi[(size_t)k * cc + i].x, im = r * phi[(size_t)k * cc + i].y;
+    for (int l = 0; l < nk; ++l) {
+      const double2 x = psi[(size_t)l * cc + i], y = psi[(size_t)l * cc + m];
+      const double2 a = alpha[k * nk + l], b = beta[k * nk + l];
+      re -= a.x * x.x - a.y * x.y + b.x * y.x + b.y * y.y;
+      im -= a.x * x.y + a.y * x.x + b.y * y.x - b.x * y.y;
+    }
+    sum += re * re + im * im;
+  }
+  __shared__ double w[8];
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+  if (threadIdx.x % 32 == 0) w[threadIdx.x / 32] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int i = 0; i < 8; ++i) t += w[i];
+    part[(size_t)k * gridDim.x + blockIdx.x] = t;
+  }
 }
 
 // One kernel that is kept: psi = root Phi.
@@ -194,6 +229,29 @@ double sum_sq(const std::vector<double>& a) {
   return s;
 }
 
+// The two real fields' share of kernel k in Q: |h_2k|^2 + |h_2k+1|^2.
+double own_weight(const std::vector<double>& g, int nk, int k) {
+  return g[size_t(2 * k) * (2 * nk) + 2 * k] + g[size_t(2 * k + 1) * (2 * nk) + 2 * k + 1];
+}
+
+// How many eigenvectors of Q (ev descending, columns of v) its image needs.
+int kept_rank(const std::vector<double>& g, int nk, const std::vector<double>& ev, const std::vector<double>& v) {
+  const int n = 2 * nk;
+  std::vector<double> taken(nk, 0.0);  // from each kernel's weight by the eigenvectors left out
+  int r = n;
+  for (; r > 0 && ev[r - 1] <= kRankTol * ev[0]; --r) {
+    if (ev[r - 1] <= kNoise * ev[0]) continue;
+    bool missed = false;
+    for (int k = 0; k < nk; ++k) {
+      const double a = v[size_t(2 * k) * n + r - 1], b = v[size_t(2 * k + 1) * n + r - 1];
+      taken[k] += ev[r - 1] * (a * a + b * b);
+      missed = missed || taken[k] > kOwnTol * own_weight(g, nk, k);
+    }
+    if (missed) break;
+  }
+  return r;
+}
+
 struct DeviceBuffer {
   void* p = nullptr;
   ~DeviceBuffer() { cudaFree(p); }
@@ -214,11 +272,13 @@ litho_status build(litho_kernels* h) {
     int plane;                         // its first focus plane
     bool reduced = false;
     std::vector<double> gram;          // 2K x 2K, when the plane can be reduced or shared
+    std::vector<double> ev, v;         // its eigenvalues (descending) and eigenvectors, the first `rank` of them needed
+    int rank = 0;
     std::vector<double2> alpha, beta;  // [kernels][K] when reduced
     int kernels = 0;
   };
   std::vector<Set> sets;
-  DeviceBuffer phi64, gram_d, flag_d, coef, power;
+  DeviceBuffer phi64, gram_d, flag_d, coef, root_d, span_d, power;
   const bool whole = K <= kMaxReduceK && F * plane_len * sizeof(double2) <= kMaxReduceBytes;
   std::vector<int> edge(F, 1);
   if (whole) {
@@ -226,6 +286,9 @@ litho_status build(litho_kernels* h) {
     LITHO_TRY_CUDA(cudaMemcpy(phi64.p, host, F * plane_len * sizeof(double2), cudaMemcpyHostToDevice));
     LITHO_TRY_CUDA(cudaMalloc(&gram_d.p, size_t(K) * K * sizeof(double4)));
     LITHO_TRY_CUDA(cudaMalloc(&coef.p, size_t(2) * K * K * sizeof(double2)));
+    LITHO_TRY_CUDA(cudaMalloc(&span_d.p, size_t(K) * kSpanBlocks * sizeof(double)));
+    LITHO_TRY_CUDA(cudaMalloc(&root_d.p, root.size() * sizeof(double)));
+    LITHO_TRY_CUDA(cudaMemcpy(root_d.p, root.data(), root.size() * sizeof(double), cudaMemcpyHostToDevice));
     LITHO_TRY_CUDA(cudaMalloc(&flag_d.p, F * sizeof(int)));
     LITHO_TRY_CUDA(cudaMemset(flag_d.p, 0, F * sizeof(int)));
     if (C < h->n) k_edge<<<F * K, 128>>>(phi64.as<double2>(), C, K, flag_d.as<int>());
@@ -245,6 +308,66 @@ litho_status build(litho_kernels* h) {
     *out = real_gram(g, &root[size_t(fa) * K], K, &root[size_t(fb) * K], K);
     return LITHO_OK;
   };
+  // a h_2k + b h_2k+1 = root ((a - i b) Phi + (a + i b) conj Phi(-u))/2 for complex a, b
+  auto upload_coef = [&](const std::vector<double2>& alpha, const std::vector<double2>& beta) -> litho_status {
+    double2* d = coef.as<double2>();
+    LITHO_TRY_CUDA(cudaMemcpy(d, alpha.data(), alpha.size() * sizeof(double2), cudaMemcpyHostToDevice));
+    LITHO_TRY_CUDA(cudaMemcpy(d + size_t(K) * K, beta.data(), beta.size() * sizeof(double2), cudaMemcpyHostToDevice));
+    return LITHO_OK;
+  };
+  // Whether plane f (its Gram matrix g) has the image of set e: in the basis of e's needed eigenvectors E_j =
+  // sum_i v_ij h_i / sqrt(ev_j), plane f's form is diag(ev), entry by entry relative to the entry's own
+  // eigenvalues, and every kernel of f lies in their span (formed point by point: the difference of two
+  // norms would leave rounding the size of the bound).
+  auto same = [&](const Set& e, int f, const std::vector<double>& g, bool* out) -> litho_status {
+    *out = false;
+    const int n = 2 * K, r = e.rank;
+    std::vector<double> x;
+    litho_status s = gram(e.plane, f, &x);
+    if (s != LITHO_OK) return s;
+    std::vector<double> c(size_t(r) * n, 0.0);  // c[j][l] = <E_j, h'_l>
+    for (int j = 0; j < r; ++j) {
+      for (int i = 0; i < n; ++i) {
+        const double w = e.v[size_t(i) * n + j] / std::sqrt(e.ev[j]);
+        for (int l = 0; l < n; ++l) c[size_t(j) * n + l] += w * x[size_t(i) * n + l];
+      }
+      for (int q = 0; q <= j; ++q) {
+        double d = q == j ? -e.ev[j] : 0.0;
+        for (int l = 0; l < n; ++l) d += c[size_t(j) * n + l] * c[size_t(q) * n + l];
+        if (!(std::fabs(d) <= kOwnTol * std::sqrt(e.ev[j] * e.ev[q]))) return LITHO_OK;
+      }
+    }
+    std::vector<double2> alpha(size_t(K) * K), beta(size_t(K) * K);
+    std::vector<double> d(size_t(n) * 2);  // kernel k of f = sum_i (d[i][0] + i d[i][1]) h_i of e
+    for (int k = 0; k < K; ++k) {
+      std::fill(d.begin(), d.end(), 0.0);
+      for (int j = 0; j < r; ++j)
+        for (int i = 0; i < n; ++i) {
+          const double w = e.v[size_t(i) * n + j] / std::sqrt(e.ev[j]);
+          d[2 * i] += w * c[size_t(j) * n + 2 * k];
+          d[2 * i + 1] += w * c[size_t(j) * n + 2 * k + 1];
+        }
+      for (int l = 0; l < K; ++l) {
+        const double *a = &d[4 * l], *b = &d[4 * l + 2], w = 0.5 * root[size_t(e.plane) * K + l];
+        alpha[size_t(k) * K + l] = make_double2(w * (a[0] + b[1]), w * (a[1] - b[0]));
+        beta[size_t(k) * K + l] = make_double2(w * (a[0] - b[1]), w * (a[1] + b[0]));
+      }
+    }
+    if ((s = upload_coef(alpha, beta)) != LITHO_OK) return s;
+    k_span<<<dim3(kSpanBlocks, K), 256>>>(phi64.as<double2>() + f * plane_len, root_d.as<double>() + size_t(f) * K,
+                                          phi64.as<double2>() + e.plane * plane_len, K, C, coef.as<double2>(),
+                                          coef.as<double2>() + size_t(K) * K, span_d.as<double>());
+    LITHO_TRY_CUDA(cudaGetLastError());
+    std::vector<double> part(size_t(K) * kSpanBlocks);
+    LITHO_TRY_CUDA(cudaMemcpy(part.data(), span_d.p, part.size() * sizeof(double), cudaMemcpyDeviceToHost));
+    for (int k = 0; k < K; ++k) {
+      double left = 0.0;
+      for (int i = 0; i < kSpanBlocks; ++i) left += part[size_t(k) * kSpanBlocks + i];
+      if (!(left <= kOwnTol * kOwnTol * own_weight(g, K, k))) return LITHO_OK;
+    }
+    *out = true;
+    return LITHO_OK;
+  };
   for (int f = 0; f < F; ++f) {
     Set t;
     t.plane = f;
@@ -252,19 +375,20 @@ litho_status build(litho_kernels* h) {
     for (int k = 0; k < K; ++k) nonzero += root[size_t(f) * K + k] > 0.0;
     t.kernels = nonzero;
     int shared = -1;
-    if (!edge[f]) {
+    for (size_t e = 0; e < sets.size() && shared < 0; ++e)
+      if (nonzero == 0 && sets[e].kernels == 0) shared = int(e);  // dark planes
+    if (shared < 0 && !edge[f]) {
       litho_status s = gram(f, f, &t.gram);
       if (s != LITHO_OK) return s;
       const double na = sum_sq(t.gram);
       if (!std::isfinite(na)) t.gram.clear();
       for (size_t e = 0; e < sets.size() && shared < 0 && !t.gram.empty(); ++e) {
-        if (sets[e].gram.empty()) continue;
+        if (sets[e].rank == 0) continue;
         const double nb = sum_sq(sets[e].gram);
         if (std::fabs(na - nb) > 1e-6 * std::max(na, nb)) continue;
-        std::vector<double> x;
-        if ((s = gram(sets[e].plane, f, &x)) != LITHO_OK) return s;
-        // |Q - Q'|^2 = |G|^2 + |G'|^2 - 2 |X|^2
-        if (na + nb - 2.0 * sum_sq(x) <= kSameTol * std::max(na, nb)) shared = int(e);
+        bool equal;
+        if ((s = same(sets[e], f, t.gram, &equal)) != LITHO_OK) return s;
+        if (equal) shared = int(e);
       }
     }
     if (shared >= 0) {
@@ -272,19 +396,18 @@ litho_status build(litho_kernels* h) {
       continue;
     }
     h->set_of[f] = (unsigned char)sets.size();
-    std::vector<double> a = t.gram, ev, v;
-    if (!a.empty() && jacobi(a, 2 * K, ev, v) && ev[0] > 0.0) {
-      int r = 0;
-      while (r < 2 * K && ev[r] > kRankTol * ev[0]) ++r;
+    std::vector<double> a = t.gram;
+    if (!a.empty() && jacobi(a, 2 * K, t.ev, t.v) && t.ev[0] > 0.0) {
+      const int r = t.rank = kept_rank(t.gram, K, t.ev, t.v);
       if ((r + 1) / 2 < nonzero) {
         t.reduced = true;
         t.kernels = (r + 1) / 2;
         t.alpha.resize(size_t(t.kernels) * K);
         t.beta.resize(size_t(t.kernels) * K);
-        auto at = [&](int row, int col) { return col < r ? v[size_t(row) * (2 * K) + col] : 0.0; };
+        auto at = [&](int row, int col) { return col < r ? t.v[size_t(row) * (2 * K) + col] : 0.0; };
         for (int q = 0; q < t.kernels; ++q)
           for (int k = 0; k < K; ++k) {
-            // eigenvectors (a1, b1) and (a2, b2) on h_2k, h_2k+1; a h + b h' = root ((a - i b) Phi + (a + i b) conj Phi(-u))/2
+            // eigenvectors (a1, b1) and (a2, b2) on h_2k, h_2k+1, the second times i
             const double a1 = at(2 * k, 2 * q), b1 = at(2 * k + 1, 2 * q);
             const double a2 = at(2 * k, 2 * q + 1), b2 = at(2 * k + 1, 2 * q + 1), w = 0.5 * root[size_t(f) * K + k];
             t.alpha[size_t(q) * K + k] = make_double2(w * (a1 + b2), w * (a2 - b1));
@@ -319,11 +442,10 @@ litho_status build(litho_kernels* h) {
       k_add_power<<<blocks, 256>>>(src, h->lambda[size_t(t.plane) * K + k], cc, power.as<double>());
     }
     if (t.reduced) {
-      double2* d_alpha = coef.as<double2>();
-      double2* d_beta = d_alpha + size_t(K) * K;
-      LITHO_TRY_CUDA(cudaMemcpy(d_alpha, t.alpha.data(), t.alpha.size() * sizeof(double2), cudaMemcpyHostToDevice));
-      LITHO_TRY_CUDA(cudaMemcpy(d_beta, t.beta.data(), t.beta.size() * sizeof(double2), cudaMemcpyHostToDevice));
-      k_combine<<<dim3(blocks, t.kernels), 256>>>(phi64.as<double2>() + t.plane * plane_len, K, C, d_alpha, d_beta, psi);
+      const litho_status cs = upload_coef(t.alpha, t.beta);
+      if (cs != LITHO_OK) return cs;
+      k_combine<<<dim3(blocks, t.kernels), 256>>>(phi64.as<double2>() + t.plane * plane_len, K, C, coef.as<double2>(),
+                                                      coef.as<double2>() + size_t(K) * K, psi);
     }
     k_round<<<blocks, 256>>>(power.as<double>(), C, h->edge ? 0 : 1, h->d_power + u * cc);
     LITHO_TRY_CUDA(cudaGetLastError());

@@ -173,3 +173,38 @@ def test_ilt_does_not_depend_on_the_number_of_clips(litho_lib, cuda, n, k, focus
         g, lo = litho_lib.litho_ilt_grad(kern, theta[i:i + 1].contiguous(), target[i:i + 1].contiguous(),
                                          precision=precision)
         assert torch.equal(grad[i], g[0]) and loss[i] == lo[0], i
+
+
+@pytest.mark.parametrize("name,fields", [("nominal", 4), ("one kernel", 1), ("through focus", 8 + 4),
+                                         ("reordered", 5 + 5 + 3), ("repeated", 6 + 3), ("dark plane", 5),
+                                         ("random", 4 + 2), ("edge", 1)])
+def test_planes_reduce_and_share(litho_lib, cuda, name, fields):
+    """In focus K kernels of one phase are K real fields, ceil(K/2) complex ones; +z and -z share a set."""
+    lam, phi = _set(name, 256)
+    assert litho_lib.litho_upload_kernels(256, PIXEL, lam, phi).fields() == fields
+
+
+def test_planes_of_a_large_crop_share(litho_lib, cuda):
+    opt = litho_lib.make_optics(kind="quadrupole", src_grid=41, pole_sigma=0.8, pole_radius=0.1)
+    assert litho_lib.litho_make_kernels(opt, 2048, PIXEL, [-50.0, 0.0, 50.0], 24).fields() == 24 + 12
+
+
+@pytest.mark.parametrize("precision", ["fft32", "fft32/coarse"])
+@pytest.mark.parametrize("lams", [[[1.0, 1e-13]], [[1.0, 0.0], [1.0, 1e-9]], [[1.0, 1e-9], [1.0, 0.0]],
+                                  [[1.0, 1e-9], [1.0, 1.001e-9]]])
+def test_a_weak_kernel_that_images_alone(litho_lib, cuda, lams, precision):
+    """A clear mask passes the weak kernel (zero frequency) alone: each plane's image is that kernel's lambda,
+    exactly but for the rounding of a few products (1e-6), however little it adds to the plane's Gram matrix."""
+    import torch
+    n, c = 64, 32
+    lam = np.array(lams)
+    rng = np.random.default_rng(1)
+    phi = np.zeros(lam.shape + (c, c), dtype=np.complex128)
+    strong = rng.standard_normal((c, c)) + 1j * rng.standard_normal((c, c))
+    strong[0, :] = strong[:, 0] = strong[c // 2, c // 2] = 0.0
+    phi[:, 0] = strong / np.linalg.norm(strong)
+    phi[:, 1, c // 2, c // 2] = 1.0
+    kern = litho_lib.litho_upload_kernels(n, PIXEL, lam, phi)
+    img = litho_lib.litho_aerial(kern, torch.ones(1, n, n, device=cuda), precision=precision)[0].cpu().numpy()
+    for f in range(len(lam)):
+        assert np.abs(img[f] - lam[f, 1]).max() <= 1e-6 * lam[f, 1]
