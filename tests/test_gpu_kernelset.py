@@ -208,3 +208,23 @@ def test_a_weak_kernel_that_images_alone(litho_lib, cuda, lams, precision):
     img = litho_lib.litho_aerial(kern, torch.ones(1, n, n, device=cuda), precision=precision)[0].cpu().numpy()
     for f in range(len(lam)):
         assert np.abs(img[f] - lam[f, 1]).max() <= 1e-6 * lam[f, 1]
+
+
+def test_adjoint_of_thousands_of_clips(litho_lib, cuda):
+    """4500 clips of 16 fields in one group: 72000 runs of fields in the adjoint's columns."""
+    import torch
+    n, b = 32, 4500
+    lam, phi = _random_set(n, 32, 1, 16, False)
+    lam[0, -2:] = lam[0, -3]
+    kern = litho_lib.litho_upload_kernels(n, PIXEL, lam, phi)
+    gen = torch.Generator(device=cuda).manual_seed(4)
+    theta = torch.rand((b, n, n), device=cuda, generator=gen) - 0.5
+    target = (torch.rand((b, n, n), device=cuda, generator=gen) > 0.5).float()
+    grad, loss = litho_lib.litho_ilt_grad(kern, theta, target, sigma_nm=6.0)
+    up = torch.rand((b, 1, n, n), device=cuda, generator=gen)
+    dm = litho_lib.litho_intensity_vjp(kern, target, up)
+    for i in (0, 4095, b - 1):
+        g, lo = litho_lib.litho_ilt_grad(kern, theta[i:i + 1].contiguous(), target[i:i + 1].contiguous(), sigma_nm=6.0)
+        assert torch.equal(grad[i], g[0]) and loss[i] == lo[0]
+        d = litho_lib.litho_intensity_vjp(kern, target[i:i + 1].contiguous(), up[i:i + 1].contiguous())
+        assert torch.equal(dm[i], d[0])
