@@ -16,10 +16,13 @@ namespace litho {
 // thread-local error message behind litho_last_error()
 void set_error(const char* fmt, ...);
 
+// The runtime keeps a failed call's error until it is read: it is read here, so that the next call's check
+// (ours, or that of another library on this thread) does not report it again.
 #define LITHO_TRY_CUDA(expr)                                                                   \
   do {                                                                                         \
     cudaError_t e_ = (expr);                                                                   \
     if (e_ != cudaSuccess) {                                                                   \
+      cudaGetLastError();                                                                      \
       ::litho::set_error("%s failed: %s (%s:%d)", #expr, cudaGetErrorString(e_), __FILE__, __LINE__); \
       return LITHO_ECUDA;                                                                      \
     }                                                                                          \

@@ -338,6 +338,7 @@ litho_status launch(litho_server* s, Slot& sl, litho_kernels* h, int fault, std:
   const size_t ws_bytes = sl.footprint - plane * (ilt ? 3 : 2);
   auto fail = [&](litho_status code, const char* what) {
     *err = what;
+    cudaGetLastError();  // not the next batch's
     cudaFreeAsync(d, sl.stream);
     return code;
   };

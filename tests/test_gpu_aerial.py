@@ -169,3 +169,19 @@ def test_aerial_plus_resist_edge_placement_config1(litho_lib, cuda):
         epe = OR.edge_placement_difference(ref, ib[i, 0].astype(np.float64), 0.3, pixel)
         assert epe <= 0.1, epe
         assert len(OR.crossings(ref, 0.3, 1)[0]) > 50
+
+
+def test_a_refused_launch_leaves_no_error_behind(litho_lib, cuda):
+    """65536 planes are more than a grid axis holds: the call is refused, the next ones are not."""
+    import torch
+    n = 32
+    planes = torch.rand((65536, n, n), device=cuda)
+    with pytest.raises(litho_lib.LithoError) as e:
+        litho_lib.litho_resist(planes, 8.0, 6.0, 0.5)
+    assert e.value.status == litho_lib.ECUDA
+    lam, phi = oracle_kernel_set(DUV_ANNULAR, n, 8.0, [0.0], 3)
+    kern = litho_lib.litho_upload_kernels(n, 8.0, lam, phi)
+    m = synth.random_rect_mask(n, seed=3, count=4)
+    img = litho_lib.litho_aerial(kern, torch.from_numpy(m[None]).to(cuda)).cpu().numpy()[0, 0]
+    assert np.abs(img - OI.socs_image(m.astype(np.float64), lam[0], phi[0])).max() <= 1e-5
+    assert litho_lib.litho_contours(planes[:1].contiguous(), 0.5)[0].shape[1] == 4
