@@ -33,7 +33,7 @@ namespace litho {
 namespace {
 
 constexpr int kMaxReduceK = 64;                       // kernels per plane the reduction considers (2 K-square Jacobi)
-constexpr size_t kMaxReduceBytes = size_t(2) << 30;   // FP64 kernels held on the device while the set is built
+constexpr size_t kMaxReduceBytes = size_t(2) << 30;   // FP64 kernels held on the device at once while the set is built
 // A field is left out, and two planes share a set, only where no kernel's own image misses it, however little the
 // kernel weighs beside the others: a mask whose spectrum the strong kernels do not pass is imaged by the weak one alone.
 constexpr double kRankTol = 1e-12;   // eigenvalues of Q below this share of the largest may be left out ...
@@ -261,7 +261,9 @@ struct DeviceBuffer {
   }
 };
 
-litho_status build(litho_kernels* h) {
+// whole: all FP64 kernels on the device at once, so that planes can be reduced and shared; otherwise one kernel
+// at a time.  *no_memory tells whether a failure was for want of device memory.
+litho_status build(litho_kernels* h, bool whole, bool* no_memory) {
   const int F = h->n_focus, K = h->k, C = h->crop;
   const size_t cc = size_t(C) * C, plane_len = size_t(K) * cc;
   const double2* host = reinterpret_cast<const double2*>(h->phi_host.data());
@@ -279,23 +281,30 @@ litho_status build(litho_kernels* h) {
   };
   std::vector<Set> sets;
   DeviceBuffer phi64, gram_d, flag_d, coef, root_d, span_d, power;
-  const bool whole = K <= kMaxReduceK && F * plane_len * sizeof(double2) <= kMaxReduceBytes;
+  *no_memory = false;
+  auto alloc = [&](void* p, size_t bytes) -> litho_status {
+    const cudaError_t e = cudaMalloc(static_cast<void**>(p), bytes);
+    *no_memory = e == cudaErrorMemoryAllocation;
+    LITHO_TRY_CUDA(e);
+    return LITHO_OK;
+  };
   std::vector<int> edge(F, 1);
+  litho_status st;
   if (whole) {
-    LITHO_TRY_CUDA(cudaMalloc(&phi64.p, F * plane_len * sizeof(double2)));
+    if ((st = alloc(&phi64.p, F * plane_len * sizeof(double2))) != LITHO_OK) return st;
     LITHO_TRY_CUDA(cudaMemcpy(phi64.p, host, F * plane_len * sizeof(double2), cudaMemcpyHostToDevice));
-    LITHO_TRY_CUDA(cudaMalloc(&gram_d.p, size_t(K) * K * sizeof(double4)));
-    LITHO_TRY_CUDA(cudaMalloc(&coef.p, size_t(2) * K * K * sizeof(double2)));
-    LITHO_TRY_CUDA(cudaMalloc(&span_d.p, size_t(K) * kSpanBlocks * sizeof(double)));
-    LITHO_TRY_CUDA(cudaMalloc(&root_d.p, root.size() * sizeof(double)));
+    if ((st = alloc(&gram_d.p, size_t(K) * K * sizeof(double4))) != LITHO_OK) return st;
+    if ((st = alloc(&coef.p, size_t(2) * K * K * sizeof(double2))) != LITHO_OK) return st;
+    if ((st = alloc(&span_d.p, size_t(K) * kSpanBlocks * sizeof(double))) != LITHO_OK) return st;
+    if ((st = alloc(&root_d.p, root.size() * sizeof(double))) != LITHO_OK) return st;
     LITHO_TRY_CUDA(cudaMemcpy(root_d.p, root.data(), root.size() * sizeof(double), cudaMemcpyHostToDevice));
-    LITHO_TRY_CUDA(cudaMalloc(&flag_d.p, F * sizeof(int)));
+    if ((st = alloc(&flag_d.p, F * sizeof(int))) != LITHO_OK) return st;
     LITHO_TRY_CUDA(cudaMemset(flag_d.p, 0, F * sizeof(int)));
     if (C < h->n) k_edge<<<F * K, 128>>>(phi64.as<double2>(), C, K, flag_d.as<int>());
     LITHO_TRY_CUDA(cudaGetLastError());
     LITHO_TRY_CUDA(cudaMemcpy(edge.data(), flag_d.p, F * sizeof(int), cudaMemcpyDeviceToHost));
   } else {
-    LITHO_TRY_CUDA(cudaMalloc(&phi64.p, cc * sizeof(double2)));  // one kernel at a time
+    if ((st = alloc(&phi64.p, cc * sizeof(double2))) != LITHO_OK) return st;
   }
   // C = n: every frequency has its mirror, but u = -C/2 is left out of half spectra
   h->edge = C == h->n || std::find(edge.begin(), edge.end(), 1) != edge.end();
@@ -422,9 +431,9 @@ litho_status build(litho_kernels* h) {
   h->set_start[0] = 0;
   for (int u = 0; u < h->n_sets; ++u) h->set_start[u + 1] = h->set_start[u] + sets[u].kernels;
   const size_t total = std::max(1, h->set_start[h->n_sets]);
-  LITHO_TRY_CUDA(cudaMalloc(&h->d_psi, total * cc * sizeof(float2)));
-  LITHO_TRY_CUDA(cudaMalloc(&h->d_power, h->n_sets * cc * sizeof(float)));
-  LITHO_TRY_CUDA(cudaMalloc(&power.p, cc * sizeof(double)));
+  if ((st = alloc(&h->d_psi, total * cc * sizeof(float2))) != LITHO_OK) return st;
+  if ((st = alloc(&h->d_power, h->n_sets * cc * sizeof(float))) != LITHO_OK) return st;
+  if ((st = alloc(&power.p, cc * sizeof(double))) != LITHO_OK) return st;
   const unsigned blocks = unsigned((cc + 255) / 256);
   for (int u = 0; u < h->n_sets; ++u) {
     const Set& t = sets[u];
@@ -458,7 +467,18 @@ litho_status build(litho_kernels* h) {
 
 litho_status build_kernel_set(litho_kernels* h) {
   try {
-    return build(h);
+    const size_t bytes = h->phi_host.size() * sizeof(double);
+    const bool whole = h->k <= kMaxReduceK && bytes <= kMaxReduceBytes;
+    bool no_memory;
+    litho_status s = build(h, whole, &no_memory);
+    if (s != LITHO_OK && whole && no_memory) {  // beside a nearly full device: the set as given, no scratch of its size
+      cudaFree(h->d_psi);
+      cudaFree(h->d_power);
+      h->d_psi = nullptr;
+      h->d_power = nullptr;
+      s = build(h, false, &no_memory);
+    }
+    return s;
   } catch (const std::bad_alloc&) {
     set_error("host allocation failed while building the kernel set");
     return LITHO_ENOMEM;

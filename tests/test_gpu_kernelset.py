@@ -228,3 +228,26 @@ def test_adjoint_of_thousands_of_clips(litho_lib, cuda):
         assert torch.equal(grad[i], g[0]) and loss[i] == lo[0]
         d = litho_lib.litho_intensity_vjp(kern, target[i:i + 1].contiguous(), up[i:i + 1].contiguous())
         assert torch.equal(dm[i], d[0])
+
+
+def test_upload_beside_a_nearly_full_device(litho_lib, cuda):
+    """Room for the set (134 MB of FP32 kernels) but not for its FP64 kernels (268 MB) beside it: uploaded as given."""
+    import torch
+    n, c, k, room = 1024, 512, 64, 240 << 20
+    rng = np.random.default_rng(3)
+    phi = (rng.standard_normal((1, k, c, c)) + 1j * rng.standard_normal((1, k, c, c))) / c
+    phi[..., 0, :] = phi[..., :, 0] = 0.0
+    lam = np.full((1, k), 1.0 / k)
+    mask = torch.from_numpy(synth.random_rect_mask(n, seed=2, count=200)[None]).to(cuda)
+    want = litho_lib.litho_aerial(litho_lib.litho_upload_kernels(n, PIXEL, lam, phi), mask)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    full = torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device=cuda)
+    assert (150 << 20) < torch.cuda.mem_get_info()[0] < (260 << 20)
+    try:
+        kern = litho_lib.litho_upload_kernels(n, PIXEL, lam, phi)
+    finally:
+        del full
+        torch.cuda.empty_cache()
+    assert kern.fields() == k
+    assert torch.equal(litho_lib.litho_aerial(kern, mask), want)
