@@ -105,12 +105,12 @@ __global__ void __launch_bounds__(256) k_combine(const double2* __restrict__ phi
 
 // part[k][block] = its share of sum_u |root_k Phi_k(u) - sum_l alpha[k][l] Psi_l(u) + beta[k][l] conj Psi_l(-u)|^2:
 // what of kernel k (of phi) the kernels psi do not span.  blockIdx.y = k.
-__global__ void __launch_bounds__(256) k_span(const double2* __restrict__ phi, const double* __restrict__ root,
-                                              const double2* __restrict__ psi, int nk, int crop,
-                                              const double2* __restrict__ alpha, const double2* __restrict__ beta,
+__global__ void __launch_bounds__(256) k_span(const double2* __restrict__ phi, const double2* __restrict__ psi, int nk,
+                                              int crop, const double2* __restrict__ alpha,
+                                              const double2* __restrict__ beta, const double2* __restrict__ root,
                                               double* __restrict__ part) {
   const int cc = crop * crop, k = blockIdx.y;
-  const double r = root[k];
+  const double r = root[k].x;
   double sum = 0.0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < cc; i += gridDim.x * blockDim.x) {
     const int m = mirror(i, crop);
@@ -252,13 +252,45 @@ int kept_rank(const std::vector<double>& g, int nk, const std::vector<double>& e
   return r;
 }
 
-struct DeviceBuffer {
-  void* p = nullptr;
-  ~DeviceBuffer() { cudaFree(p); }
-  template <class T>
-  T* as() const {
-    return static_cast<T*>(p);
+// Device memory while a set is built, and the stream it is built on: a set may be built beside running work (the
+// server's builder thread), for which neither cudaFree nor a copy on the default stream should wait.  The pool is
+// its own, so that nothing of it stays reserved.
+class Scratch {
+ public:
+  cudaStream_t st = nullptr;
+  Scratch() = default;
+  Scratch(const Scratch&) = delete;
+  Scratch& operator=(const Scratch&) = delete;
+  ~Scratch() {
+    if (base_) cudaFreeAsync(base_, st);
+    if (st) cudaStreamSynchronize(st);
+    if (pool_) cudaMemPoolDestroy(pool_);
+    if (st) cudaStreamDestroy(st);
   }
+  cudaError_t open(int device, size_t bytes) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaMemPoolCreate(&pool_, &props);
+    return e != cudaSuccess ? e : cudaMallocFromPoolAsync(&base_, bytes, pool_, st);
+  }
+  template <class T>
+  T* at(size_t offset) const {
+    return reinterpret_cast<T*>(static_cast<char*>(base_) + offset);
+  }
+  // Copies that the host waits for: the other end is pageable.
+  cudaError_t up(void* dst, const void* src, size_t bytes) { return copy(dst, src, bytes, cudaMemcpyHostToDevice); }
+  cudaError_t down(void* dst, const void* src, size_t bytes) { return copy(dst, src, bytes, cudaMemcpyDeviceToHost); }
+
+ private:
+  cudaError_t copy(void* dst, const void* src, size_t bytes, cudaMemcpyKind kind) {
+    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, kind, st);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(st);
+  }
+  cudaMemPool_t pool_ = nullptr;
+  void* base_ = nullptr;
 };
 
 // whole: all FP64 kernels on the device at once, so that planes can be reduced and shared; otherwise one kernel
@@ -280,48 +312,59 @@ litho_status build(litho_kernels* h, bool whole, bool* no_memory) {
     int kernels = 0;
   };
   std::vector<Set> sets;
-  DeviceBuffer phi64, gram_d, flag_d, coef, root_d, span_d, power;
-  *no_memory = false;
-  auto alloc = [&](void* p, size_t bytes) -> litho_status {
-    const cudaError_t e = cudaMalloc(static_cast<void**>(p), bytes);
+  size_t bytes = 0;
+  auto place = [&](size_t b) {
+    const size_t at = bytes;
+    bytes += (b + 255) / 256 * 256;
+    return at;
+  };
+  const size_t kk = size_t(K) * K, o_phi = place((whole ? F * plane_len : cc) * sizeof(double2)),
+               o_power = place(cc * sizeof(double)), o_gram = place(whole ? kk * sizeof(double4) : 0),
+               o_coef = place(whole ? (2 * kk + K) * sizeof(double2) : 0),
+               o_span = place(whole ? size_t(K) * kSpanBlocks * sizeof(double) : 0), o_flag = place(F * sizeof(int));
+  Scratch sc;
+  // an allocation's status
+  auto memory = [&](cudaError_t e) -> litho_status {
     *no_memory = e == cudaErrorMemoryAllocation;
     LITHO_TRY_CUDA(e);
     return LITHO_OK;
   };
+  litho_status st = memory(sc.open(h->device, bytes));
+  if (st != LITHO_OK) return st;
+  double2 *phi64 = sc.at<double2>(o_phi), *coef = sc.at<double2>(o_coef);  // coef: alpha, beta, roots (see upload_coef)
+  double4* gram_d = sc.at<double4>(o_gram);
+  double *power = sc.at<double>(o_power), *span_d = sc.at<double>(o_span);
+  int* flag_d = sc.at<int>(o_flag);
   std::vector<int> edge(F, 1);
-  litho_status st;
   if (whole) {
-    if ((st = alloc(&phi64.p, F * plane_len * sizeof(double2))) != LITHO_OK) return st;
-    LITHO_TRY_CUDA(cudaMemcpy(phi64.p, host, F * plane_len * sizeof(double2), cudaMemcpyHostToDevice));
-    if ((st = alloc(&gram_d.p, size_t(K) * K * sizeof(double4))) != LITHO_OK) return st;
-    if ((st = alloc(&coef.p, size_t(2) * K * K * sizeof(double2))) != LITHO_OK) return st;
-    if ((st = alloc(&span_d.p, size_t(K) * kSpanBlocks * sizeof(double))) != LITHO_OK) return st;
-    if ((st = alloc(&root_d.p, root.size() * sizeof(double))) != LITHO_OK) return st;
-    LITHO_TRY_CUDA(cudaMemcpy(root_d.p, root.data(), root.size() * sizeof(double), cudaMemcpyHostToDevice));
-    if ((st = alloc(&flag_d.p, F * sizeof(int))) != LITHO_OK) return st;
-    LITHO_TRY_CUDA(cudaMemset(flag_d.p, 0, F * sizeof(int)));
-    if (C < h->n) k_edge<<<F * K, 128>>>(phi64.as<double2>(), C, K, flag_d.as<int>());
-    LITHO_TRY_CUDA(cudaGetLastError());
-    LITHO_TRY_CUDA(cudaMemcpy(edge.data(), flag_d.p, F * sizeof(int), cudaMemcpyDeviceToHost));
-  } else {
-    if ((st = alloc(&phi64.p, cc * sizeof(double2))) != LITHO_OK) return st;
+    LITHO_TRY_CUDA(sc.up(phi64, host, F * plane_len * sizeof(double2)));
+    if (C < h->n) {
+      LITHO_TRY_CUDA(cudaMemsetAsync(flag_d, 0, F * sizeof(int), sc.st));
+      k_edge<<<F * K, 128, 0, sc.st>>>(phi64, C, K, flag_d);
+      LITHO_TRY_CUDA(cudaGetLastError());
+      LITHO_TRY_CUDA(sc.down(edge.data(), flag_d, F * sizeof(int)));
+    } else {
+      edge.assign(F, 0);
+    }
   }
   // C = n: every frequency has its mirror, but u = -C/2 is left out of half spectra
   h->edge = C == h->n || std::find(edge.begin(), edge.end(), 1) != edge.end();
   auto gram = [&](int fa, int fb, std::vector<double>* out) -> litho_status {
     std::vector<double4> g(size_t(K) * K);
-    k_gram<<<dim3(K, K), 256>>>(phi64.as<double2>() + fa * plane_len, phi64.as<double2>() + fb * plane_len, C,
-                                gram_d.as<double4>());
+    k_gram<<<dim3(K, K), 256, 0, sc.st>>>(phi64 + fa * plane_len, phi64 + fb * plane_len, C, gram_d);
     LITHO_TRY_CUDA(cudaGetLastError());
-    LITHO_TRY_CUDA(cudaMemcpy(g.data(), gram_d.p, g.size() * sizeof(double4), cudaMemcpyDeviceToHost));
+    LITHO_TRY_CUDA(sc.down(g.data(), gram_d, g.size() * sizeof(double4)));
     *out = real_gram(g, &root[size_t(fa) * K], K, &root[size_t(fb) * K], K);
     return LITHO_OK;
   };
-  // a h_2k + b h_2k+1 = root ((a - i b) Phi + (a + i b) conj Phi(-u))/2 for complex a, b
-  auto upload_coef = [&](const std::vector<double2>& alpha, const std::vector<double2>& beta) -> litho_status {
-    double2* d = coef.as<double2>();
-    LITHO_TRY_CUDA(cudaMemcpy(d, alpha.data(), alpha.size() * sizeof(double2), cudaMemcpyHostToDevice));
-    LITHO_TRY_CUDA(cudaMemcpy(d + size_t(K) * K, beta.data(), beta.size() * sizeof(double2), cudaMemcpyHostToDevice));
+  // a h_2k + b h_2k+1 = root ((a - i b) Phi + (a + i b) conj Phi(-u))/2 for complex a, b: alpha from coef[0],
+  // beta from coef[K^2], and plane f's roots from coef[2 K^2].
+  std::vector<double2> ab(whole ? 2 * kk + K : 0);
+  auto upload_coef = [&](const std::vector<double2>& alpha, const std::vector<double2>& beta, int f) -> litho_status {
+    std::copy(alpha.begin(), alpha.end(), ab.begin());
+    std::copy(beta.begin(), beta.end(), ab.begin() + kk);
+    for (int k = 0; k < K; ++k) ab[2 * kk + k] = make_double2(root[size_t(f) * K + k], 0.0);
+    LITHO_TRY_CUDA(sc.up(coef, ab.data(), ab.size() * sizeof(double2)));
     return LITHO_OK;
   };
   // Whether plane f (its Gram matrix g) has the image of set e: in the basis of e's needed eigenvectors E_j =
@@ -362,13 +405,12 @@ litho_status build(litho_kernels* h, bool whole, bool* no_memory) {
         beta[size_t(k) * K + l] = make_double2(w * (a[0] - b[1]), w * (a[1] + b[0]));
       }
     }
-    if ((s = upload_coef(alpha, beta)) != LITHO_OK) return s;
-    k_span<<<dim3(kSpanBlocks, K), 256>>>(phi64.as<double2>() + f * plane_len, root_d.as<double>() + size_t(f) * K,
-                                          phi64.as<double2>() + e.plane * plane_len, K, C, coef.as<double2>(),
-                                          coef.as<double2>() + size_t(K) * K, span_d.as<double>());
+    if ((s = upload_coef(alpha, beta, f)) != LITHO_OK) return s;
+    k_span<<<dim3(kSpanBlocks, K), 256, 0, sc.st>>>(phi64 + f * plane_len, phi64 + e.plane * plane_len, K, C, coef,
+                                                    coef + kk, coef + 2 * kk, span_d);
     LITHO_TRY_CUDA(cudaGetLastError());
     std::vector<double> part(size_t(K) * kSpanBlocks);
-    LITHO_TRY_CUDA(cudaMemcpy(part.data(), span_d.p, part.size() * sizeof(double), cudaMemcpyDeviceToHost));
+    LITHO_TRY_CUDA(sc.down(part.data(), span_d, part.size() * sizeof(double)));
     for (int k = 0; k < K; ++k) {
       double left = 0.0;
       for (int i = 0; i < kSpanBlocks; ++i) left += part[size_t(k) * kSpanBlocks + i];
@@ -431,35 +473,31 @@ litho_status build(litho_kernels* h, bool whole, bool* no_memory) {
   h->set_start[0] = 0;
   for (int u = 0; u < h->n_sets; ++u) h->set_start[u + 1] = h->set_start[u] + sets[u].kernels;
   const size_t total = std::max(1, h->set_start[h->n_sets]);
-  if ((st = alloc(&h->d_psi, total * cc * sizeof(float2))) != LITHO_OK) return st;
-  if ((st = alloc(&h->d_power, h->n_sets * cc * sizeof(float))) != LITHO_OK) return st;
-  if ((st = alloc(&power.p, cc * sizeof(double))) != LITHO_OK) return st;
+  if ((st = memory(cudaMalloc(&h->d_psi, total * cc * sizeof(float2)))) != LITHO_OK) return st;
+  if ((st = memory(cudaMalloc(&h->d_power, h->n_sets * cc * sizeof(float)))) != LITHO_OK) return st;
   const unsigned blocks = unsigned((cc + 255) / 256);
   for (int u = 0; u < h->n_sets; ++u) {
     const Set& t = sets[u];
     float2* psi = h->d_psi + h->set_start[u] * cc;
-    LITHO_TRY_CUDA(cudaMemset(power.p, 0, cc * sizeof(double)));
+    LITHO_TRY_CUDA(cudaMemsetAsync(power, 0, cc * sizeof(double), sc.st));
     int at = 0;
     for (int k = 0; k < K; ++k) {
       const double r = root[size_t(t.plane) * K + k];
       if (r == 0.0) continue;
-      const double2* src = phi64.as<double2>() + (whole ? t.plane * plane_len + k * cc : 0);
-      if (!whole)
-        LITHO_TRY_CUDA(cudaMemcpy(phi64.p, host + t.plane * plane_len + k * cc, cc * sizeof(double2),
-                                  cudaMemcpyHostToDevice));
-      if (!t.reduced) k_scale<<<blocks, 256>>>(src, r, cc, psi + (at++) * cc);
-      k_add_power<<<blocks, 256>>>(src, h->lambda[size_t(t.plane) * K + k], cc, power.as<double>());
+      const double2* src = phi64 + (whole ? t.plane * plane_len + k * cc : 0);
+      if (!whole) LITHO_TRY_CUDA(sc.up(phi64, host + t.plane * plane_len + k * cc, cc * sizeof(double2)));
+      if (!t.reduced) k_scale<<<blocks, 256, 0, sc.st>>>(src, r, cc, psi + (at++) * cc);
+      k_add_power<<<blocks, 256, 0, sc.st>>>(src, h->lambda[size_t(t.plane) * K + k], cc, power);
     }
     if (t.reduced) {
-      const litho_status cs = upload_coef(t.alpha, t.beta);
-      if (cs != LITHO_OK) return cs;
-      k_combine<<<dim3(blocks, t.kernels), 256>>>(phi64.as<double2>() + t.plane * plane_len, K, C, coef.as<double2>(),
-                                                      coef.as<double2>() + size_t(K) * K, psi);
+      if ((st = upload_coef(t.alpha, t.beta, t.plane)) != LITHO_OK) return st;
+      k_combine<<<dim3(blocks, t.kernels), 256, 0, sc.st>>>(phi64 + t.plane * plane_len, K, C, coef,
+                                                            coef + kk, psi);
     }
-    k_round<<<blocks, 256>>>(power.as<double>(), C, h->edge ? 0 : 1, h->d_power + u * cc);
+    k_round<<<blocks, 256, 0, sc.st>>>(power, C, h->edge ? 0 : 1, h->d_power + u * cc);
     LITHO_TRY_CUDA(cudaGetLastError());
   }
-  LITHO_TRY_CUDA(cudaStreamSynchronize(nullptr));  // the set is read from any stream afterwards
+  LITHO_TRY_CUDA(cudaStreamSynchronize(sc.st));  // the set is read from any stream afterwards
   return LITHO_OK;
 }
 

@@ -251,3 +251,20 @@ def test_upload_beside_a_nearly_full_device(litho_lib, cuda):
         torch.cuda.empty_cache()
     assert kern.fields() == k
     assert torch.equal(litho_lib.litho_aerial(kern, mask), want)
+
+
+def test_upload_does_not_wait_for_running_work(litho_lib, cuda):
+    """A set of two planes, one reduced, is built while another stream is busy for a second or so."""
+    import torch
+    lam, phi = oracle_kernel_set(DUV_ANNULAR, 256, PIXEL, [0.0, 30.0, -30.0], 12)
+    keep = [litho_lib.litho_upload_kernels(256, PIXEL, lam, phi)]  # its kernels are loaded
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(2_000_000_000)
+        done = torch.cuda.Event()
+        done.record()
+    keep.append(litho_lib.litho_upload_kernels(256, PIXEL, lam, phi))
+    assert not done.query()
+    side.synchronize()
+    assert keep[1].fields() == 6 + 12
