@@ -255,8 +255,8 @@ cudaError_t launch_resist(const float* img, int planes, int n, const ResistTaps&
 #undef R_CASE
     default:
       if (n % 128 != 0) return launch_any<32, 32, 512>(img, planes, n, taps, threshold, iblur, printed, st);
-      // two tiles per SM while they fit (radius 36); then one, by twice the threads, and wide enough
-      // for less of a halo where that fits (radius 55) and fills the chip.  265 planes of 1024^2, 32 and 64 wide:
+      // two tiles per SM while they fit (radius 37); then one, by twice the threads, and wide enough
+      // for less of a halo where that fits (radius 56) and fills the chip.  265 planes of 1024^2, 32 and 64 wide:
       // 2840 and 3251 us at R = 20, 8627 (by 512 threads) and 4455 at R = 40; 64 of 2048^2 at R = 64, by 512 and
       // 1024 threads: 9.98 and 8.12 ms
       if (2 * any_bytes(taps.radius, 32, 128) <= 226 * 1024)

@@ -38,6 +38,21 @@ def test_blur_tiles(litho_lib, cuda, n, planes, radius):
         assert np.abs(first[p] - OR.blur(img[p], sigma, pixel)).max() <= 1e-6
 
 
+# the last radius of two tiles per SM and the first of one, the last and the first that the wide tile does not
+# hold; planes enough for the wide tile, and not
+@pytest.mark.parametrize("n,planes", [(256, 20), (128, 1)])
+@pytest.mark.parametrize("radius", [37, 38, 56, 57])
+def test_blur_tile_widths(litho_lib, cuda, n, planes, radius):
+    import torch
+    pixel, sigma = 8.0, 8.0 * (radius - 0.5) / 4.0
+    img = synth.random_field((planes, n, n), seed=radius, lo=0.0, hi=1.0).astype(np.float32)
+    ib, pr = litho_lib.litho_resist(torch.from_numpy(img).to(cuda), pixel, sigma, 0.5)
+    ib = ib.cpu().numpy()
+    assert np.array_equal(pr.cpu().numpy(), (ib >= np.float32(0.5)).astype(np.uint8))
+    for p in (0, planes - 1):
+        assert np.abs(ib[p] - OR.blur(img[p], sigma, pixel)).max() <= 1e-6
+
+
 @pytest.mark.parametrize("n,b", [(32, 3), (96, 1), (256, 2)])
 def test_print_counts(litho_lib, cuda, n, b):
     import torch
