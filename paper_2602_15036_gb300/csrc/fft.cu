@@ -195,7 +195,11 @@ struct OutHalf {
 // Rows of up to 256 points are one warp's: two warps share the plane's kernels (G = 2, half of them each), where a
 // chain of many kernels is what an SM of few rows waits for.  256^2 images of one plane and 12 fields, one and
 // two warps a row: 2 clips 19.2 and 18.9 us, 4 28.6 and 20.9, 8 30.3 and 28.5, 12 40.1 and 38.8, 20 59.4 and
-// 59.1; two planes of 5: 1 clip 16.3 and 19.1 us, 20 51.2 and 61.6.
+// 59.1; two planes of 5: 1 clip 16.3 and 19.1 us, 20 51.2 and 61.6.  Whole calls by rows, 12 fields: 256 points
+// 1024 rows 28.5 and 20.8, 2048 30.0 and 28.3, 3072 39.7 and 38.8, 4096 47.4 and 48.8; 128 points 20.1 and 17.8,
+// 21.9 and 20.8, 28.0 and 27.8, 32.6 and 34.6; 64 points 2048 rows 20.1 and 18.1, 3072 24.2 and 24.1, 4096 27.8
+// and 28.7; 8 fields of 128 points 2048 rows 17.4 and 17.2, 3072 21.7 and 22.2.  Below 768 rows the launches take
+// longer than the chain.
 // How many warps there are depends on the clips of the launch, a clip's bits must not: these rows' sums are
 // always those of the first half of the fields and of the rest, whether two warps form them or one after the other.
 template <int N>

@@ -526,22 +526,6 @@ __device__ __forceinline__ void fft_load_use_mid(float2* buf, const float2* tw, 
   pass_last<N, NT, PL::R[2], PL::R[0] * PL::R[1], SIGN, TwOff<N>::p2>(buf, tw, t, use);
 }
 
-// Full transform in place in shared memory (padded layout on entry and on
-// return, natural order).  Ends with a barrier.
-template <int N, int SIGN>
-__device__ __forceinline__ void fft_smem(float2* buf, const float2* tw, int t) {
-  using PL = Plan<N>;
-  constexpr int NT = PL::NT;
-  SmemLoadUnused none;
-  pass_to_smem<N, NT, PL::R[0], 1, SIGN, 0, true>(buf, tw, t, none);
-  if constexpr (PL::P == 2) {
-    pass_to_smem<N, NT, PL::R[1], PL::R[0], SIGN, TwOff<N>::p1, true>(buf, tw, t, none);
-  } else {
-    pass_to_smem<N, NT, PL::R[1], PL::R[0], SIGN, TwOff<N>::p1, true>(buf, tw, t, none);
-    pass_to_smem<N, NT, PL::R[2], PL::R[0] * PL::R[1], SIGN, TwOff<N>::p2, true>(buf, tw, t, none);
-  }
-}
-
 // Full transform with the first pass from `load` and every pass's output in
 // shared memory (padded layout, natural order on return).  Ends with a barrier.
 // NTX: the threads that share the transform (default: the plan's own; more
@@ -561,20 +545,6 @@ __device__ __forceinline__ void fft_load_smem(float2* buf, const float2* tw, int
     pass_to_smem<N, NT, PL::R[2], PL::R[0] * PL::R[1], SIGN, TwOff<N>::p2, true>(buf, tw, t, none);
   }
 }
-
-// Columns per CTA for the column-transform kernels (W transforms of
-// Plan<N>::NT threads each): 8, so that a CTA loads its twiddle table for
-// many columns, except at 512 points (4 columns, several CTAs per SM).
-template <int N> struct ColW { static constexpr int W = N == 512 ? 4 : 8; };
-// Column stride in shared memory: the padded length rounded up to 16 complex
-// values plus 16/W, so that a half-warp of the cooperative copies (w fastest,
-// W columns x 16/W rows) touches 16 different 8-byte bank pairs.
-template <int N> struct ColLD {
-  static constexpr int value = (PadLen<N>::value + 15) / 16 * 16 + 16 / ColW<N>::W;
-};
-// Stride of the compact band buffers [W][crop] (crop is a multiple of 32).
-template <int N>
-__host__ __device__ __forceinline__ int band_ld(int crop) { return crop + 16 / ColW<N>::W; }
 
 // Programmatic dependent launch.  A kernel that launch_pdl starts may begin as soon as every CTA of the
 // kernel before it on the stream has called pdl_start (or ended): its set-up (twiddle tables, which no
