@@ -306,7 +306,8 @@ template <int N>
 __global__ void __launch_bounds__(Plan<N>::NT * AdjW<N>::W, AdjAccInSmem<N>::value ? 2 : 1) k_adj_cols(const float2* __restrict__ u,
                                                                         const float2* __restrict__ phi,
                                                                         int crop, const float2* __restrict__ tw_g,
-                                                                        float2* __restrict__ part, int period) {
+                                                                        float2* __restrict__ part, int period,
+                                                                        int splits) {
   constexpr int W = AdjW<N>::W, NT = Plan<N>::NT, LD = (PadLen<N>::value + 15) / 16 * 16 + 16 / W;
   constexpr int RL = Plan<N>::R[Plan<N>::P - 1], PERL = PassShape<N, NT, RL>::PER;
   constexpr int T = NT * W;
@@ -317,7 +318,7 @@ __global__ void __launch_bounds__(Plan<N>::NT * AdjW<N>::W, AdjAccInSmem<N>::val
   constexpr int R0 = Plan<N>::R[0], NB0 = N / R0;
   static_assert(PassShape<N, NT, R0>::PER == 1, "one first-pass butterfly per thread");
   const int tid = threadIdx.x, g = tid % W, t = tid / W, c0 = blockIdx.x * W, half = crop / 2;
-  const int splits = gridDim.y, split = blockIdx.y, clip = blockIdx.z, jb = (period + splits - 1) / splits;
+  const int clip = blockIdx.y / splits, split = blockIdx.y % splits, jb = (period + splits - 1) / splits;
   float2* acc_s = buf + W * LD;  // kSmem: this thread's PERL x RL sums at (pp RL + q) T + tid
   float2 acc_r[kSmem ? 1 : PERL * RL];
   auto acc = [&](int i) -> float2& {
@@ -364,7 +365,7 @@ __global__ void __launch_bounds__(Plan<N>::NT * AdjW<N>::W, AdjAccInSmem<N>::val
     fft_load_use<N, -1, decltype(load), decltype(use), false>(buf + g * LD, tw, t, load, use, after_first);
   }
   // the last pass's output positions of this thread: idx = jj + q N/RL, jj = t + pp NT
-  float2* dst = part + ((size_t)clip * splits + split) * crop * crop + c0 + g;  // crop row cv at dst[cv crop]
+  float2* dst = part + (size_t)blockIdx.y * crop * crop + c0 + g;  // crop row cv at dst[cv crop]
 #pragma unroll
   for (int pp = 0; pp < PERL; ++pp) {
     const int jj = t + pp * NT;
@@ -556,9 +557,14 @@ cudaError_t adj_cols_n(const float2* u, const float2* phi, int crop, const float
   const size_t sm = sizeof(float2) * (N + W * LD + (AdjAccInSmem<N>::value ? size_t(PERL) * RL * Plan<N>::NT * W : 0));
   cudaError_t e = smem_attrs(k_adj_cols<N>, sm);
   if (e != cudaSuccess) return e;
-  // clips on a grid axis of their own: clips x runs of a call of thousands of clips are more than an axis holds
-  return launch_pdl(k_adj_cols<N>, dim3(crop / W, adj_col_splits(period), clips), Plan<N>::NT * W, sm, st, u, phi, crop,
-                    tw, part, period);
+  // runs of all clips on one grid axis, which holds 65535: thousands of clips take more than one launch
+  // (clips on an axis of their own: VJP of 4 clips of 1024^2 358.0 -> 360.1 us, of 2 of 2048^2 766 -> 773)
+  const int splits = adj_col_splits(period), most = 65535 / splits;
+  for (int c = 0; c < clips && e == cudaSuccess; c += most)
+    e = launch_pdl(k_adj_cols<N>, dim3(crop / W, std::min(most, clips - c) * splits), Plan<N>::NT * W, sm, st,
+                   u + size_t(c) * period * N * crop, phi, crop, tw, part + size_t(c) * splits * crop * crop, period,
+                   splits);
+  return e;
 }
 
 template <int N>
