@@ -624,19 +624,24 @@ inline cudaError_t load_kernel(K kernel) {
   return cudaFuncGetAttributes(&a, kernel);
 }
 
+// SMs of the GPU (the same model throughout a process), asked for once, by whichever thread comes first.
+inline int sm_count() {
+  static const int sms = [] {
+    int dev = 0, v = 0;
+    return cudaGetDevice(&dev) == cudaSuccess &&
+                   cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0
+               ? v
+               : 152;
+  }();
+  return sms;
+}
+
 // Rows per CTA for the one-row-per-transform kernels: CTAs for about four waves at the residency that
 // their threads and shared memory allow, each reusing its twiddle table for its rows.  64 clips of 2048^2 with
 // resist, by waves: 8960 us (1), 8754 (2), 8673 (3), 8647 (4), 8853 (a row per CTA: eight waves of the
 // CTAs that threads alone allow, three times what fits); fewer than two leave a long tail.
 inline int rows_per_cta(int rows, int planes, int threads, size_t smem) {
-  static int sms = 0;  // the same GPU model throughout a process
-  if (!sms) {
-    int dev = 0, v = 0;
-    sms = cudaGetDevice(&dev) == cudaSuccess &&
-                  cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0
-              ? v
-              : 152;
-  }
+  const int sms = sm_count();
   const int per_sm = std::max<int>(1, std::min<int>(std::min(2048 / threads, 32), int(227 * 1024 / (smem + 1024))));
   const long long want = 4LL * sms * per_sm;
   const long long r = std::max<long long>(1, ((long long)rows * planes) / want);

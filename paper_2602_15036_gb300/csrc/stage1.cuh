@@ -165,16 +165,8 @@ cudaError_t launch_stage1_cols_t(const float2* mhat, const float2* phi, int nk, 
   // + half a kernel of set-up).
   // (One run per CTA block leaves, e.g., 448 CTAs on 304 slots: a second wave
   // half empty for a whole CTA's time.)
-  static int sms = 0;  // the same GPU model throughout a process; a racing first call stores the same value
-  if (!sms) {
-    int dev = 0, v = 0;
-    sms = cudaGetDevice(&dev) == cudaSuccess &&
-                  cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0
-              ? v
-              : 152;
-  }
   const int blocks = (crop - c_first) / W;
-  const long long ctas = (long long)clips * blocks, slots = (long long)Stage1Pipe<N, Out>::kMinBlocks * sms;
+  const long long ctas = (long long)clips * blocks, slots = (long long)Stage1Pipe<N, Out>::kMinBlocks * sm_count();
   int jblocks = 1;
   long long best = -1;
   for (int jb = 1; jb <= std::min(nk, 32); ++jb) {
