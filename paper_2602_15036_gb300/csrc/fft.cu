@@ -4,7 +4,7 @@
 //
 // Paper Section III.A: the object spectrum O(f) of Eq. (1) (thin-mask reading:
 // the mask's DFT), and the SOCS image of Eq. (4), I = sum_k lam_k |O (x) phi_k|^2,
-// evaluated as E_k = IDFT(M . Phi_k) restricted to the C x C band crop.
+// evaluated as E_j = IDFT(M . Psi_j) restricted to the C x C band crop (Psi: kernelset.cu).
 //
 // Data layout (all row-major, x fastest):
 //   mask    [b][N][N] f32

@@ -1,9 +1,9 @@
 // Stage 1 of the SOCS evaluation (paper Eq. (4)): band multiply and inverse
-// transform over the y frequency, T_j[y][c] = sum_v mhat[v][c] Phi_j[v][c] e^{+2 pi i v y/N},
+// transform over the y frequency, T_j[y][c] = sum_v mhat[v][c] Psi_j[v][c] e^{+2 pi i v y/N},
 // for a block of W crop columns c and a run of kernels j.
 //
 // A CTA keeps the twiddle table in shared memory and loops over a run of kernels;
-// the next kernel's Phi block is copied in with cp.async while the current
+// the next kernel's Psi block is copied in with cp.async while the current
 // block's W column transforms run.  One block buffer, refilled as soon as the
 // first pass (the only one that reads the block) is done, so that two CTAs fit
 // an SM's shared memory (Stage1Pipe).  The band multiply happens in
@@ -19,7 +19,7 @@
 // in one thread and goes through shared memory.
 //
 // With kernels, one launch can image several clips (grid x = clip, the
-// fastest-varying block index): the CTAs of all clips that need the same Phi
+// fastest-varying block index): the CTAs of all clips that need the same Psi
 // block run side by side, so each block comes from DRAM once and from L2
 // for the other clips.  Clip i writes j + i nk.  The row-wise (split 16-bit)
 // output swaps the two: its W columns fill only part of each 32-byte sector
@@ -44,7 +44,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // Shared memory of a CTA: the twiddle table, W column transforms at stride LD
 // (the padded length rounded up to 16 complex values plus 16/W, so that a
 // half-warp of 16/W transform threads x W columns touches 16 different bank
-// pairs) and two operand blocks [crop][W] in the operand's own row-major
+// pairs) and one or two operand blocks [crop][W] in the operand's own row-major
 // order (a row's W values are one or more whole 16-byte copies; a half-warp
 // reading rows c..c+16/W-1 of all W columns again hits 16 bank pairs).
 // Columns per CTA: as many as fit one CTA of at most 512 threads, since a
@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(Plan<N>::NT * W, Stage1Pipe<N, Out>::kMinBlock
   float2* smem = reinterpret_cast<float2*>(smem_raw);
   float2* tw = smem;
   float2* buf = smem + N;
-  float2* const blk0 = buf + W * LD;  // Phi (or spectrum) blocks [crop][W], double-buffered
+  float2* const blk0 = buf + W * LD;  // Psi (or spectrum) blocks [crop][W], as many as Stage1Pipe has
   auto blk = [&](int s) { return blk0 + s * W * crop; };
   const int clip = Out::kRowWise ? blockIdx.y : blockIdx.x, cblk = Out::kRowWise ? blockIdx.x : blockIdx.y;
   const int tid = threadIdx.x, u0 = out.first() + cblk * W, half = crop / 2;
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(Plan<N>::NT * W, Stage1Pipe<N, Out>::kMinBlock
   mhat += (size_t)clip * crop * crop;
   pdl_start();
   load_twiddles<N>(tw, tw_g);
-  if (!phi) pdl_wait(mhat);  // the spectra come from the kernel before; Phi is the kernel set's
+  if (!phi) pdl_wait(mhat);  // the spectra come from the kernel before; Psi is the kernel set's
   const float2* src_base = phi ? phi : mhat;  // the per-j operand
   auto issue = [&](int j, float2* dst) {  // W/2 16-byte pieces per row
     const float2* src = src_base + (size_t)j * crop * crop + u0;
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(Plan<N>::NT * W, Stage1Pipe<N, Out>::kMinBlock
       cp_async_wait_all();
     }
     // Block j (and, first time round, tw) visible to all threads; every thread
-    // has finished transform j - 1, so buf and the other Phi buffer are free.
+    // has finished transform j - 1, so buf (and, with two, the other block) is free.
     __syncthreads();
     const float2* b = blk(s) + g;
     // single buffer: the first pass has read block j in every thread, so block j + 1 may land
