@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(256) k_ms_count(const unsigned* __restrict__ b
 // segment of the cell), into the warp's queue at the place a warp scan gives it; the queue holds them
 // in output order, and whenever it has 32 the lanes compute one each from the cell's corner pixels.
 // So the crossing arithmetic runs on full warps, and finding the segments costs a few instructions per
-// 32 cells.  48 planes of 2048^2 (15 M segments), all five launches of the contours: 868 -> 440 us (pixel
+// 32 cells.  48 planes of 2048^2 (15 M segments), all launches of the contours: 868 -> 425 us (pixel
 // rows walked twice in 128-cell chunks, rounds of 32 segments per chunk, a third full).
 constexpr int kEmitWarps = 8, kEmitWords = 16, kEmitQueue = 32 + kEmitWords * 64;
 
